@@ -72,10 +72,11 @@ static EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// Tensor map over a [tokens, heads, d] bf16 tensor (d contiguous) with a box of
-// 64 elements x box_heads x box_tokens and the 128-byte swizzle the MMA descriptors expect.
+// Tensor map over a [tokens, heads, d] bf16 tensor (d contiguous) with a box of box_elems (64 or 32) elements x
+// box_heads x box_tokens and the swizzle of the box's row (128 or 64 bytes) that the MMA descriptors expect.
 // Rows past the end of the tensor read as zero.
-static int make_tmap(CUtensorMap* m, const void* base, int64_t tokens, int heads, int d, int box_heads, int box_tokens) {
+static int make_tmap(CUtensorMap* m, const void* base, int64_t tokens, int heads, int d, int box_heads, int box_tokens,
+                     int box_elems = 64) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) {
         snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled entry point not found");
@@ -83,10 +84,11 @@ static int make_tmap(CUtensorMap* m, const void* base, int64_t tokens, int heads
     }
     cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(heads), static_cast<cuuint64_t>(tokens)};
     cuuint64_t strides[2] = {static_cast<cuuint64_t>(d) * 2, static_cast<cuuint64_t>(d) * 2 * heads};
-    cuuint32_t box[3] = {64, static_cast<cuuint32_t>(box_heads), static_cast<cuuint32_t>(box_tokens)};
+    cuuint32_t box[3] = {static_cast<cuuint32_t>(box_elems), static_cast<cuuint32_t>(box_heads), static_cast<cuuint32_t>(box_tokens)};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     box_elems == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled failed with CUresult %d", static_cast<int>(r));
@@ -134,12 +136,11 @@ static QueryPlan plan_query(const pevlm_shape_t* s) {
     q.tok_per_tile = kTile / G;
     q.q_tiles = (s->query_len + q.tok_per_tile - 1) / q.tok_per_tile;
     q.total_kv_tiles = static_cast<int>((L + kTile - 1) / kTile);
-    // Work items are (kv head, pair of query tiles, key split).  The kernel is persistent with one
-    // CTA per SM, so the split count is chosen to give one full wave of the 148 SMs of a B200:
-    // as many splits as fit, never more than there are key tiles.
+    // Work items are (kv head, pair of query tiles, key split), one for each pair of CTAs, so the split count is chosen
+    // to give one full wave of the 74 CTA pairs of a B200: as many splits as fit, never more than there are key tiles.
     const int pairs = (q.q_tiles + 1) / 2;
     const int groups = s->num_kv_heads * (pairs > 0 ? pairs : 1);
-    int want = kNumSms / groups;
+    int want = kNumSms / 2 / groups;
     if (want < 1) want = 1;
     if (want > q.total_kv_tiles) want = q.total_kv_tiles;
     q.tiles_per_split = (q.total_kv_tiles + want - 1) / want;
@@ -343,6 +344,11 @@ static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, 
     const int n_chunks = p.pairs_block > 0 ? (p.pairs_block + p.pair_chunk - 1) / p.pair_chunk : 0;
     p.items_block = p.N * p.Hkv * p.pair_chunk * n_chunks;
     p.n_items = p.items_block + p.Hkv * p.pairs_sink;
+    p.div_per_chunk = make_divisor(p.N * p.Hkv * p.pair_chunk);
+    p.div_pair_chunk = make_divisor(p.pair_chunk);
+    p.div_hkv = make_divisor(p.Hkv);
+    p.div_pairs_sink = make_divisor(p.pairs_sink);
+    p.div_g = make_divisor(p.G);
     p.scale = resolve_scale(s);
     p.scale_log2 = p.scale * 1.4426950408889634f;
     p.wait_limit_ns = kDefaultWaitLimitNs;
@@ -363,16 +369,12 @@ static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, 
         const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(v) + koff;
         const int64_t blk_off = static_cast<int64_t>(p.blk_key0) * p.Hkv * d;
         const int64_t sink_rows = p.S > 0 ? p.S : 1, blk_rows = block_rows_launch > 0 ? block_rows_launch : 1;
-        if ((rc = make_tmap(&m.k_sink, kb, sink_rows, p.Hkv, d, 1, kTile)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&m.v_sink, vb, sink_rows, p.Hkv, d, 1, kTile)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&m.k, kb + blk_off, blk_rows, p.Hkv, d, 1, kTile)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&m.v, vb + blk_off, blk_rows, p.Hkv, d, 1, kTile)) != PEVLM_OK) return rc;
+        if ((rc = make_tmap(&m.k_sink, kb, sink_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+        if ((rc = make_tmap(&m.v_sink, vb, sink_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
+        if ((rc = make_tmap(&m.k, kb + blk_off, blk_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+        if ((rc = make_tmap(&m.v, vb + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
         p.o = static_cast<__nv_bfloat16*>(o) + qoff;
         p.lse = lse ? lse + static_cast<int64_t>(b) * p.Hq * q_rows : nullptr;
-        if (b > 0) {  // every launch starts its work counter at zero; the status word is kept
-            e = cudaMemsetAsync(&p.hdr->work_counter, 0, sizeof(int32_t), st);
-            if (e != cudaSuccess) return cuda_fail(e, "work counter memset");
-        }
         e = launch_attn(p, d, m, st);
         if (e != cudaSuccess) return cuda_fail(e, "prefill attention launch");
     }
@@ -420,6 +422,8 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
     p.n_splits = qp.n_splits;
     p.tiles_per_split = qp.tiles_per_split;
     p.n_items = p.Hkv * ((p.q_tiles + 1) / 2) * p.n_splits;
+    p.div_splits = make_divisor(p.n_splits);
+    p.div_q_pairs = make_divisor((p.q_tiles + 1) / 2);
     p.scale = resolve_scale(s);
     p.scale_log2 = p.scale * 1.4426950408889634f;
     p.wait_limit_ns = kDefaultWaitLimitNs;
@@ -431,14 +435,10 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
         p.part_o = part;
         p.part_lse = part + static_cast<size_t>(p.n_splits) * p.Q * p.Hq * d;
         const int64_t qoff = static_cast<int64_t>(b) * p.Q * p.Hq * d, koff = static_cast<int64_t>(b) * L * p.Hkv * d;
-        if (b > 0) {
-            e = cudaMemsetAsync(&p.hdr->work_counter, 0, sizeof(int32_t), st);
-            if (e != cudaSuccess) return cuda_fail(e, "work counter memset");
-        }
         AttnMaps maps;
         if ((rc = make_tmap(&maps.q, static_cast<const __nv_bfloat16*>(q_question) + qoff, p.Q, p.Hq, d, p.G, p.tok_per_tile)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&maps.k, static_cast<const __nv_bfloat16*>(k_cache) + koff, L, p.Hkv, d, 1, kTile)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&maps.v, static_cast<const __nv_bfloat16*>(v_cache) + koff, L, p.Hkv, d, 1, kTile)) != PEVLM_OK) return rc;
+        if ((rc = make_tmap(&maps.k, static_cast<const __nv_bfloat16*>(k_cache) + koff, L, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+        if ((rc = make_tmap(&maps.v, static_cast<const __nv_bfloat16*>(v_cache) + koff, L, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
         maps.q_tail_block = maps.q; maps.q_tail_sink = maps.q; maps.k_sink = maps.k; maps.v_sink = maps.v;
         e = launch_attn(p, d, maps, st);
         if (e != cudaSuccess) return cuda_fail(e, "question attention launch");
@@ -462,7 +462,7 @@ int pevlm_selftest_wait_expiry(void* workspace, size_t workspace_bytes, int64_t 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, st);
     if (e != cudaSuccess) return cuda_fail(e, "workspace memset");
-    e = launch_wait_selftest(static_cast<WorkspaceHeader*>(workspace), static_cast<uint64_t>(limit_ns), st);
+    e = launch_wait_selftest(static_cast<WorkspaceHeader*>(workspace), static_cast<uint32_t>(limit_ns), st);
     if (e != cudaSuccess) return cuda_fail(e, "wait self-test launch");
     return PEVLM_OK;
 }

@@ -1,53 +1,76 @@
-// Warp-specialised block-masked flash attention for sm_100a (Eq. 1 under the masks of Eq. 3-5).
+// Warp-specialised block-masked flash attention for sm_100a (Eq. 1 under the masks of Eq. 3-5), on CTA pairs.
 //
-// One CTA owns TWO query tiles of 128 rows that share a kv head and a key-tile list (two q
-// heads of one GQA group at the same block position, or two neighbouring positions), so every
-// K/V tile staged in shared memory feeds both.  Roles (12 warps):
-//   warps 0-3   softmax and epilogue of query tile 0: one thread per row; the 128 scores of a key
-//               tile are read from TMEM once, running max/sum kept in fp32, probabilities written
-//               back over the scores as bf16; the rare rescale of the O accumulator (the reference
-//               maximum moves only when a row's maximum grows by more than 2^8) is done in place
-//               by the same threads.  After the item's last key tile the same thread reads its
-//               row of the accumulator in one round trip, releases the accumulator, and writes
-//               the normalised output and the LSE
-//   warps 4-7   the same for query tile 1
-//   warp 8      issues the tcgen05 MMAs: S = Q K^T (both operands from shared memory) and
-//               O += P V (P from TMEM, V from shared memory), ping-ponging between the two
-//               query tiles so one is in the tensor cores while the other is in its softmax
-//   warp 9      work scheduler and TMA producer: takes the next work item from a global
-//               counter, decodes it once into shared memory for the other roles (the decode is
-//               a dozen integer divisions), loads its two Q tiles, then streams K/V tiles
-//               through a 4-slot ring that runs on across items
-//   warps 10-11 idle (they complete the third warpgroup for the register reallocation)
-// The kernel is persistent (one CTA per SM): while the softmax threads write out item k, the
-// producer and the MMA warp already work on item k+1.
-// TMEM (512 columns): S0/P0 [0,128) S1/P1 [128,256) O0 [256,384) O1 [384,512).
-// Every wait is bounded; an expired wait records PEVLM_ETIMEOUT and the CTA still runs to its
+// A pair of CTAs (a cluster of 2, cta_group::2) owns a work item = TWO query tiles of 128 rows that share a kv head and
+// a key-tile list (two q heads of one GQA group at the same block position, or two neighbouring positions); CTA r of the
+// pair owns tile r.  The MMAs span the pair (M = 256): each CTA stages half of every K tile (64 keys) and half of every
+// V tile (D/2 columns), so a pair reads each K/V tile from L2 once and an SM's shared memory holds and delivers half.
+// Per CTA, 16 warps:
+//   warps 0-3, 4-7  two softmax warpgroups, one thread per row, taking the key tiles of the CTA's query tile in turn.
+//               The 128 scores of a key tile are read from TMEM once, the probabilities written back as bf16.  The
+//               running reference maximum of a row passes from one warpgroup to the other through shared memory
+//               (warp to warp); it moves only when the row's maximum grows by more than 2^8, and then the thread
+//               rescales its row of the output accumulator in place (rare).  Each warpgroup keeps the row sum of its
+//               own tiles; the epilogue adds the two
+//   warps 8-11  epilogue: reads the finished accumulator, releases it, writes the normalised output and the LSE
+//   warps 12, 14 (first CTA of the pair) issue the tcgen05 MMAs of both CTAs: warp 12 S = Q K^T (operands from shared
+//               memory), warp 14 O += P V (P from TMEM, V from shared memory).  Neither has to know of the other
+//   warp 13     TMA producer of Q, K and V
+//   warp 15     scheduler: takes work items from the hardware's queue of unlaunched clusters, decodes each once into
+//               shared memory for the other roles (the decode is a dozen integer divisions)
+// TMEM (512 columns): score buffers S0 S1 of 128 columns, probability buffers P0 P1 of 64, accumulator O of D.
+// Probabilities and scores do not share columns, so QK(t + 2) needs nothing but that tile t's scores have been read
+// into registers, which is the first thing its softmax does: the scores of a softmax warpgroup's next tile are ready
+// long before it has finished this one, and neither the tensor pipe's latency nor the hand-offs between the warps are
+// on its path.  QK runs three tiles ahead of PV, over the boundaries of work items too.
+// What bounds it: two softmax warpgroups that never wait take 2,390 cycles for two key tiles beside running MMAs, the
+// MMAs 1,024 a tile (both measured free-running); reached are 1,480 cycles a tile on long work items (1,741 before, with
+// two query tiles and two softmax warpgroups per CTA) and 2,400 with four tiles an item (2,710 before).  On B200, back
+// to back under the 1 kW cap: 50K tokens 1.708 -> 1.546 ms, 12.6K 0.249 -> 0.228, 256-token blocks 0.322 -> 0.296,
+// 8,192-token blocks 4.97 -> 4.54.  Two things took more than the schedule itself:
+//   - the two softmax warps that share a scheduler take turns on its special-function unit (left alone they fall into
+//     step, form their exponentials at the same time and leave the unit idle at the same time: 1,741 cycles a tile);
+//   - instruction fetch.  What a work item runs (all roles, masks and item ends included) has to stay near the size of
+//     the SM's instruction cache: at 73 KB of code four-tile items lost more time to missing instructions than to
+//     anything else (26 % of the fetches missed), 55 KB run them 15 % faster.  Hence one instantiation per mode,
+//     loops that stay loops wherever the registers' indices allow it, waits that expand to little, no divisions.
+// Every wait on an mbarrier is bounded; an expired wait records PEVLM_ETIMEOUT and the CTA still runs to its
 // normal end (waits become short), so TMEM is always released.
 #include "internal.h"
 #include "ptx.cuh"
 
 namespace pevlm {
 
-constexpr int kAttnThreads = 384;
-constexpr int kRing = 4;
+constexpr int kAttnThreads = 512;
+constexpr int kRing = 4;      // K tiles and V tiles in flight
+constexpr int kQkAhead = 3;   // tiles by which QK runs ahead of PV
+constexpr int kItems = 8;     // decoded work items in flight
+constexpr int kSums = 8;      // items whose row sums may be in flight between softmax and epilogue
+constexpr int kClaimAhead = 6;  // tiles before the end of an item's loads at which the next item is claimed
+// pair of exponentials (of 64) after which a softmax warp passes the turn on: the rest overlaps the other warp's start
+// (measured: 16 to 40 within 1 % of each other, 52 and later 4 % slower)
+constexpr int kTurn = 40;
 constexpr float kRescaleThresholdLog2 = 8.0f;  // rescale O only when the row maximum grew by > 2^8
+constexpr uint32_t kTmemP = 2 * kTile;          // first TMEM column of the probability buffers
+constexpr uint32_t kTmemO = kTmemP + kTile;     // of the accumulator
 
 enum WaitId : int {
-    kWaitQ = 11, kWaitFull = 12, kWaitEmpty = 13, kWaitS = 14,
-    kWaitPO = 16, kWaitPV = 17, kWaitItem = 19, kWaitItemFree = 20,
-    kWaitQFree = 21, kWaitOFree = 22
+    kWaitQ = 11, kWaitK = 12, kWaitV = 13, kWaitS = 14, kWaitP = 15, kWaitSRead = 16, kWaitPV = 17, kWaitPFree = 18, kWaitItem = 19,
+    kWaitItemFree = 20, kWaitQFree = 21, kWaitOFree = 22, kWaitKvFree = 23, kWaitSum = 25, kWaitODone = 26,
+    kWaitGo = 27, kWaitClc = 28
 };
 
 template <int D>
 struct AttnSmem {
     static constexpr int kPanels = D / 64;
-    static constexpr int kPanelBytes = kTile * 128;
-    static constexpr int kTileBytes = kPanels * kPanelBytes;
-    static constexpr int kQ0 = 0;
-    static constexpr int kQ1 = kTileBytes;
-    static constexpr int kRing0 = 2 * kTileBytes;
-    static constexpr int kTotal = kRing0 + kRing * kTileBytes;
+    static constexpr int kQPanelBytes = kTile * 128;     // 128 rows of 64 elements
+    static constexpr int kKPanelBytes = kTile / 2 * 128; // this CTA's 64 keys of 64 elements
+    static constexpr int kQBytes = kPanels * kQPanelBytes;
+    static constexpr int kKBytes = kPanels * kKPanelBytes;
+    static constexpr int kVBytes = kTile * D;            // 128 keys of this CTA's D/2 columns
+    static constexpr int kQ = 0;                         // two buffers
+    static constexpr int kK = 2 * kQBytes;
+    static constexpr int kV = kK + kRing * kKBytes;
+    static constexpr int kTotal = kV + kRing * kVBytes;
 };
 
 size_t attn_smem_bytes(int head_dim) {
@@ -60,63 +83,42 @@ size_t attn_smem_bytes(int head_dim) {
 // ntok = the tail's rows); question tiles pack all G heads of the group.
 struct QSlot {
     int valid;
-    int q_tok0, q_head0, row_div, ntok, nheads, qmap, box_rows, limit0, b_end, nt;
+    int q_tok0, q_head0, row_div, ntok, nheads, qmap, box_rows;
+    int limit0;  // last visible key of row token 0, counted from the first key of the own range
+    int end;     // keys of the own range that the tile's rows can see at all
 };
 // Key tiles of an item: first the na tiles of the shared range [0, a_end) (the sink), then the tiles of the own
-// range from global key row b_start on.  The own range is fetched through the block tensor map at row
-// b_coord0 of that map, or, for the sink's own items, through the sink map (own_map = 1).
+// range, nt tiles in all (what the longer of the two query tiles needs; the other one masks its surplus tile).
+// The own range is fetched through the block tensor map at row b_coord0 of that map, or, for the sink's own items,
+// through the sink map (own_map = 1).  n_a, n_b: MMA columns of tile na - 1 and of the last tile; the others have 128.
 struct WorkItem {
-    int kv_head, a_end, b_start, na, split, b_coord0, own_map;
+    int kv_head, a_end, na, nt, n_a, n_b, split, b_coord0, own_map;
     QSlot s[2];
 };
 
-// Optional time stamps (-DPEVLM_TRACE): clock64 at the hand-offs of CTA 0's first work item, key tiles
-// [kTraceJ0, kTraceJ0 + 16), read back through pevlm_debug_trace (see timeline.py).  Events: 0/1 scores of
-// tile 0/1 seen by the softmax, 2/3 probabilities handed over, 4 QK0 issue starts, 5 QK0 issued,
-// 6 probabilities of tile 0 seen by the MMA warp, 7 PV0 issued.  A second table holds, for CTA 0's work items
-// [kTraceK0, kTraceK0 + 16), the events of an item boundary: 0 item taken by the MMA warp, 1 its first QK goes
-// out, 2 its last PV and commits are issued; query tile 0's thread 0: 3 first scores seen, 4 last probabilities
-// handed over, 5 accumulator complete, 6 accumulator released, 7 output stored.
+// Optional accounting (-DPEVLM_TRACE): for the first CTA pair of a launch, the cycles every warp spent in each kind of
+// wait and between the start and the end of its role, read back through pevlm_debug_waits (see timeline.py).
 #ifdef PEVLM_TRACE
-__device__ unsigned g_trace[8][16];
-__device__ unsigned g_trace_item[8][16];
-constexpr int kTraceK0 = 2;
-#define PEVLM_STAMP_ITEM(ev, kk, cond)                                                          \
-    do {                                                                                        \
-        if ((cond) && blockIdx.x == 0 && (kk) >= kTraceK0 && (kk) < kTraceK0 + 16)              \
-            g_trace_item[ev][(kk) - kTraceK0] = static_cast<unsigned>(clock64());               \
-    } while (0)
-constexpr int kTraceJ0 = 8;
-#define PEVLM_STAMP(ev, j, cond)                                                                \
-    do {                                                                                        \
-        if ((cond) && blockIdx.x == 0 && k == 0 && (j) >= kTraceJ0 && (j) < kTraceJ0 + 16)      \
-            g_trace[ev][(j) - kTraceJ0] = static_cast<unsigned>(clock64());                     \
-    } while (0)
-extern "C" int pevlm_debug_trace(unsigned* host_out) {
-    return cudaMemcpyFromSymbol(host_out, g_trace, sizeof(g_trace)) == cudaSuccess ? 0 : -1;
+constexpr int kTraceIds = 32;  // wait ids are below this; index 0 = whole role, 1 = key tiles handled
+__device__ unsigned g_waits[2][16][kTraceIds];
+extern "C" int pevlm_debug_waits(unsigned* host_out) {
+    return cudaMemcpyFromSymbol(host_out, g_waits, sizeof(g_waits)) == cudaSuccess ? 0 : -1;
 }
-extern "C" int pevlm_debug_trace_items(unsigned* host_out) {
-    return cudaMemcpyFromSymbol(host_out, g_trace_item, sizeof(g_trace_item)) == cudaSuccess ? 0 : -1;
-}
-#else
-#define PEVLM_STAMP(ev, j, cond) do {} while (0)
-#define PEVLM_STAMP_ITEM(ev, kk, cond) do {} while (0)
 #endif
-
-// The probabilities of a key tile are handed to the MMA warp in two parts: after the first 32 * kPvSplit keys and
-// at the end of the tile, so the first PV steps run while the softmax still forms the rest (0 = one hand-off).
-// Measured on B200: 2 and 3 within 1 % of each other, both 1-3 % ahead of 0.
-#ifndef PEVLM_PV_SPLIT
-#define PEVLM_PV_SPLIT 2
-#endif
-constexpr int kPvSplit = PEVLM_PV_SPLIT;
 
 __device__ __forceinline__ int cdiv(int a, int b) { return (a + b - 1) / b; }
 
+// a / b for 0 <= a < 2^31 by the multiplier and shift that the host worked out for b
+__device__ __forceinline__ int quotient(int a, const Divisor& b) {
+    return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(a)) * b.mul) >> 31 >> b.shift);
+}
+
+template <int MODE>
 __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem& it) {
     it.split = 0;
-    if (p.mode == 0) {
-        int seg_start, seg_q0, seg_len, tiles, pi, g, tail_rows, tail_heads, tail_tiles, qmap_tail;
+    int own_keys = 0;  // keys of the own range that the longer query tile sees
+    if (MODE == 0) {
+        int seg_q0, seg_len, tiles, pi, g, tail_rows, tail_heads, tail_tiles, qmap_tail;
         if (w < p.items_block) {
             // Order of the items: the pair list of a (block, kv head), heaviest first, is cut into chunks of
             // pair_chunk pairs; chunk-major, then (block, kv head), then the pairs of the chunk.  CTAs that run
@@ -124,13 +126,12 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             // lightest chunk of every (block, kv head) rather than on the last block's whole list.  A pair
             // index past the end of the list (padding of the last chunk) is an empty item.
             const int per_chunk = p.N * p.Hkv * p.pair_chunk;
-            const int r = w % per_chunk;
-            const int combo = r / p.pair_chunk;
-            pi = (w / per_chunk) * p.pair_chunk + r % p.pair_chunk;
-            const int blk = combo / p.Hkv;
-            g = combo % p.Hkv;
-            seg_start = p.blk_key0 + blk * p.B;  // key rows of the block
-            seg_q0 = p.blk_q0 + blk * p.B;       // its rows in q / o
+            const int chunk = quotient(w, p.div_per_chunk), r = w - chunk * per_chunk;
+            const int combo = quotient(r, p.div_pair_chunk);
+            pi = chunk * p.pair_chunk + r - combo * p.pair_chunk;
+            const int blk = quotient(combo, p.div_hkv);
+            g = combo - blk * p.Hkv;
+            seg_q0 = p.blk_q0 + blk * p.B;       // the block's rows in q / o
             seg_len = p.B;
             tiles = p.tiles_block;
             tail_rows = p.tail_rows_block; tail_heads = p.tail_heads_block; tail_tiles = p.tail_tiles_block;
@@ -140,9 +141,8 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             it.own_map = 0;
         } else {
             const int w2 = w - p.items_block;
-            g = w2 / p.pairs_sink;
-            pi = w2 % p.pairs_sink;
-            seg_start = 0;
+            g = quotient(w2, p.div_pairs_sink);
+            pi = w2 - g * p.pairs_sink;
             seg_q0 = 0;
             seg_len = p.S;
             tiles = p.tiles_sink;
@@ -153,13 +153,11 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             it.own_map = 1;
         }
         it.kv_head = g;
-        it.b_start = seg_start;
-        it.na = cdiv(it.a_end, kTile);
         // entries of this (segment, kv head), heaviest first: the packed tail tiles (last tile position of
         // the segment, tail_heads q heads each), then (tile position, q head) for the full positions
         const int full_tiles = tiles - (tail_tiles > 0 ? 1 : 0);
         const int entries = tail_tiles + p.G * full_tiles;
-#pragma unroll
+#pragma unroll 1
         for (int x = 0; x < 2; ++x) {
             const int e = 2 * pi + x;
             QSlot& s = it.s[x];
@@ -175,8 +173,9 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
                 s.box_rows = tail_heads * tail_rows;
             } else {
                 const int e2 = e - tail_tiles;
-                qt = full_tiles - 1 - e2 / p.G;
-                s.q_head0 = g * p.G + e2 % p.G;
+                const int up = quotient(e2, p.div_g);
+                qt = full_tiles - 1 - up;
+                s.q_head0 = g * p.G + e2 - up * p.G;
                 s.row_div = 1;
                 s.ntok = min(kTile, seg_len - qt * kTile);
                 s.nheads = 1;
@@ -184,25 +183,22 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
                 s.box_rows = kTile;
             }
             s.q_tok0 = seg_q0 + qt * kTile;
-            s.limit0 = seg_start + qt * kTile;
-            s.b_end = min(s.limit0 + kTile, seg_start + seg_len);
-            s.nt = s.valid ? it.na + cdiv(s.b_end - it.b_start, kTile) : 0;
+            s.limit0 = qt * kTile;
+            s.end = min(qt * kTile + kTile, seg_len);
+            if (s.valid) own_keys = max(own_keys, s.end);
         }
     } else {
-        it.split = w % p.n_splits;
-        const int rest = w / p.n_splits;
+        const int rest = quotient(w, p.div_splits);
+        it.split = w - rest * p.n_splits;
         const int q_pairs = cdiv(p.q_tiles, 2);
-        const int pi = rest % q_pairs;
-        const int g = rest / q_pairs;
+        const int g = quotient(rest, p.div_q_pairs);
+        const int pi = rest - g * q_pairs;
         it.kv_head = g;
         it.a_end = 0;
-        it.na = 0;
         const int split_lo = it.split * p.tiles_per_split * kTile;
-        const int split_hi = split_lo + p.tiles_per_split * kTile;
-        it.b_start = split_lo;
         it.b_coord0 = split_lo;
         it.own_map = 0;
-#pragma unroll
+#pragma unroll 1
         for (int x = 0; x < 2; ++x) {
             const int qt = 2 * pi + x;
             QSlot& s = it.s[x];
@@ -216,16 +212,34 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             s.nheads = p.G;
             s.qmap = 0;
             s.box_rows = p.G * p.tok_per_tile;
-            s.limit0 = p.n_video + tok0;
-            const int kv_end = p.n_video + tok0 + ntok;  // keys past the last row's limit are never visible
-            s.b_end = min(kv_end, split_hi);
-            s.nt = (s.valid && s.b_end > split_lo) ? cdiv(s.b_end - split_lo, kTile) : 0;
+            s.limit0 = p.n_video + tok0 - split_lo;
+            // keys past the last row's limit are never visible; a split that lies past it altogether still takes
+            // one (wholly masked) tile and leaves the neutral partial
+            s.end = max(0, min(p.n_video + tok0 + ntok - split_lo, p.tiles_per_split * kTile));
+            if (s.valid) own_keys = max(own_keys, max(1, s.end));
         }
     }
+    it.na = cdiv(it.a_end, kTile);
+    it.nt = own_keys > 0 ? it.na + cdiv(own_keys, kTile) : 0;
+    it.n_a = (it.a_end - (it.na - 1) * kTile + 15) & ~15;
+    it.n_b = (own_keys - (it.nt - it.na - 1) * kTile + 15) & ~15;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads, 1)
+// Between the two softmax warps that share a scheduler (warp `quarter` of each warpgroup), hardware barriers of 64
+// threads, one id per direction, all sixteen in use (the kernel has no __syncthreads: the cluster barrier stands at its
+// start and end).  Both warps go through the same tiles whatever happens, so every pass meets its wait; what the passing
+// warp wrote to shared memory before is seen after the wait.  kPassMax: the row maxima of a tile; kPassTurn: the turn on
+// the scheduler's special-function unit.
+constexpr int kPassMax = 0, kPassTurn = 8;
+__device__ __forceinline__ void pass_wait(int what, int wg, int quarter) {
+    asm volatile("bar.sync %0, 64;" ::"r"(what + wg * 4 + quarter) : "memory");
+}
+__device__ __forceinline__ void pass_on(int what, int wg, int quarter) {
+    asm volatile("bar.arrive %0, 64;" ::"r"(what + (wg ^ 1) * 4 + quarter) : "memory");
+}
+
+template <int D, int MODE>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kAttnThreads, 1)
 attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmap_q,
             const __grid_constant__ CUtensorMap tmap_q_tail_block, const __grid_constant__ CUtensorMap tmap_q_tail_sink,
             const __grid_constant__ CUtensorMap tmap_k_sink, const __grid_constant__ CUtensorMap tmap_v_sink,
@@ -233,43 +247,62 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
     using L = AttnSmem<D>;
     constexpr int NP = L::kPanels;
     extern __shared__ uint8_t smem_raw[];
-    // barrier map (uint64 each): [0,2) item_full [2,4) item_free [4,6) q_full [6,8) q_free
-    // [8,12) ring full [12,16) ring empty, then per slot x: [16,18) s_full [18,20) po
-    // [24,26) o_free [26,28) o_done
-    __shared__ uint64_t bars[30];  // [28,30) po_a: first part of a tile's probabilities written
+    // Barriers.  "first": the copy of the pair's first CTA is the one that is used (the MMA warps wait there and both
+    // CTAs arrive); "both": each CTA has its own.
+    struct Bars {
+        uint64_t item_full[kItems], item_free[kItems];  // both: decoded items
+        uint64_t clc;                                   // both: answer of the hardware queue
+        uint64_t clc_read;                              // first: the second CTA has read it
+        uint64_t q_full[2];                             // first
+        uint64_t q_free[2];                             // both
+        uint64_t k_full[kRing], v_full[kRing];          // first: a tile has landed in both CTAs
+        uint64_t s_full[kRing];                         // both: QK(t) is complete: scores there, K tile consumed
+        uint64_t s_read[2];                             // first: scores are in registers
+        uint64_t p_full[2];                             // first: probabilities are written
+        uint64_t pv_done[kRing];                        // both: PV(t) is complete: P and V tile consumed, O up to date
+        uint64_t o_free;                                // first: both CTAs have read it
+        uint64_t sums_full[kSums];                      // both: row sums of an item are in shared memory
+        uint64_t go;                                    // first: the next item may be claimed
+    };
+    __shared__ Bars bars;
+    __shared__ __align__(16) uint4 s_clc;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
-    __shared__ int s_item[2];
-    __shared__ WorkItem s_decoded[2];  // the producer decodes an item once; every role copies it from here
+    __shared__ int s_item[kItems];       // 1 = a work item, -1 = no more work
+    __shared__ WorkItem s_decoded[kItems];
+    __shared__ float s_max[2][kTile];
+    __shared__ float2 s_sums[kSums][2][kTile];  // (row sum, reference maximum) of each warpgroup's tiles
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const int lane = tid & 31;
+    const uint32_t rank = cluster_ctarank();
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t bar0 = smem_u32(&bars[0]);
-    const uint32_t bar_item_full = bar0, bar_item_free = bar0 + 16, bar_q_full = bar0 + 32, bar_q_free = bar0 + 48;
-    const uint32_t bar_full = bar0 + 64, bar_empty = bar0 + 96;
-    const uint32_t bar_s_full = bar0 + 128, bar_po = bar0 + 144;
-    const uint32_t bar_o_free = bar0 + 192, bar_o_done = bar0 + 208, bar_po_a = bar0 + 224;
-    constexpr int kItemConsumers = 1 + 2 * kTile;  // MMA warp + two softmax warpgroups
+    constexpr int kConsumerWarps = 1 + 8 + 4;  // producer, softmax, epilogue; in the first CTA also the MMA warps
 
     if (tid == 0) {
         abort_flag = 0;
+        for (int i = 0; i < kItems; ++i) {
+            mbar_init(smem_u32(&bars.item_full[i]), 1);
+            mbar_init(smem_u32(&bars.item_free[i]), kConsumerWarps + (rank == 0 ? 2 : 0));
+        }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bar_item_full + 8 * i, 1);
-            mbar_init(bar_item_free + 8 * i, kItemConsumers);
-            mbar_init(bar_q_full + 8 * i, 1);
-            mbar_init(bar_q_free + 8 * i, 1);
-            mbar_init(bar_s_full + 8 * i, 1);
-            mbar_init(bar_po + 8 * i, kTile);
-            mbar_init(bar_po_a + 8 * i, kTile);
-            mbar_init(bar_o_free + 8 * i, kTile);
-            mbar_init(bar_o_done + 8 * i, 1);
+            mbar_init(smem_u32(&bars.q_full[i]), 1);
+            mbar_init(smem_u32(&bars.q_free[i]), 1);
+            mbar_init(smem_u32(&bars.s_read[i]), 8);  // 4 warps of each CTA
+            mbar_init(smem_u32(&bars.p_full[i]), 8);
         }
         for (int i = 0; i < kRing; ++i) {
-            mbar_init(bar_full + 8 * i, 1);
-            mbar_init(bar_empty + 8 * i, 1);
+            mbar_init(smem_u32(&bars.k_full[i]), 1);
+            mbar_init(smem_u32(&bars.v_full[i]), 1);
+            mbar_init(smem_u32(&bars.s_full[i]), 1);
+            mbar_init(smem_u32(&bars.pv_done[i]), 1);
         }
+        for (int i = 0; i < kSums; ++i) mbar_init(smem_u32(&bars.sums_full[i]), 8);
+        mbar_init(smem_u32(&bars.o_free), 8);
+        mbar_init(smem_u32(&bars.go), 1);
+        mbar_init(smem_u32(&bars.clc), 1);
+        mbar_init(smem_u32(&bars.clc_read), 1);
         fence_mbar_init();
         tma_prefetch_desc(&tmap_q);
         tma_prefetch_desc(&tmap_q_tail_block);
@@ -279,275 +312,329 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
         tma_prefetch_desc(&tmap_k);
         tma_prefetch_desc(&tmap_v);
     }
-    if (warp == 8) {
+    if (warp == 12) {
         __syncwarp();
-        tmem_alloc(smem_u32(&tmem_base_slot), 512);
+        tmem_alloc_pair(smem_u32(&tmem_base_slot), 512);
     }
     tc_fence_before_sync();
-    __syncthreads();
+    cluster_sync_all();  // also: the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
 
-    auto give_up = [&](int which) {
-        if (atomicCAS(&p.hdr->status, 0, PEVLM_ETIMEOUT) == 0) p.hdr->detail = which * 1000000 + blockIdx.x;
+#ifdef PEVLM_TRACE
+    __shared__ unsigned s_waits[16][kTraceIds];
+    for (int i = lane; i < kTraceIds; i += 32) s_waits[warp][i] = 0;
+    __syncwarp();
+    const unsigned role_start = static_cast<unsigned>(clock64());
+#define PEVLM_WAIT_ACCOUNT(which, call)                                                              \
+    const unsigned before = static_cast<unsigned>(clock64());                                        \
+    call;                                                                                            \
+    if (lane == 0) s_waits[warp][which] += static_cast<unsigned>(clock64()) - before
+#else
+#define PEVLM_WAIT_ACCOUNT(which, call) call
+#endif
+    auto wait = [&](const uint64_t& bar, uint32_t parity, int which) {
+        PEVLM_WAIT_ACCOUNT(which, mbar_wait(smem_u32(&bar), parity, smem_u32(&abort_flag), p.wait_limit_ns, which));
     };
-    auto wait = [&](uint32_t bar, uint32_t parity, int which) {
-        if (!mbar_wait(bar, parity, &abort_flag, p.wait_limit_ns)) give_up(which);
+    auto wait_asleep = [&](const uint64_t& bar, uint32_t parity, int which) {
+        PEVLM_WAIT_ACCOUNT(which, mbar_wait<100>(smem_u32(&bar), parity, smem_u32(&abort_flag), p.wait_limit_ns, which));
     };
-    // consumer side of the item queue: k-th item of this CTA, -1 = no more work
-    auto next_item = [&](int k, WorkItem& it) {
-        wait(bar_item_full + 8 * (k & 1), (k >> 1) & 1, kWaitItem);
-        const int w = s_item[k & 1];
-        if (w >= 0) it = s_decoded[k & 1];
-        mbar_arrive(bar_item_free + 8 * (k & 1));
-        return w;
+    // k-th item of the pair: wait for it, read from s_decoded[k % kItems], then give the slot back (once per warp)
+    auto item_ready = [&](int k) {
+        wait(bars.item_full[k % kItems], (k / kItems) & 1, kWaitItem);
+        return s_item[k % kItems] > 0;
     };
+    auto item_release = [&](int k) { mbar_arrive(smem_u32(&bars.item_free[k % kItems])); };
+    auto wait_s_full = [&](uint32_t t, int which) { wait(bars.s_full[t % kRing], (t / kRing) & 1, which); };
+    auto wait_pv_done = [&](uint32_t t, int which) { wait(bars.pv_done[t % kRing], (t / kRing) & 1, which); };
 
-    // register budget per warpgroup: 2 x 216 (softmax + epilogue) + 56 (TMA/MMA) <= 384 x 168
-    if (warp >= 8) {
-        reg_dealloc<56>();
-      if (warp == 9) {
-        // ------------------------------------------------------------- scheduler + TMA producer
-        if (lane == 0) {
-            int ring_idx = 0;          // K/V tiles loaded so far (ring position), runs on across items
-            int q_loads[2] = {0, 0};   // Q loads per slot so far
-            for (int k = 0;; ++k) {
-                int w = (k == 0) ? static_cast<int>(blockIdx.x)
-                                 : static_cast<int>(gridDim.x) + atomicAdd(&p.hdr->work_counter, 1);
-                if (w >= p.n_items || abort_flag != 0 || *reinterpret_cast<volatile int32_t*>(&p.hdr->status) != 0) w = -1;
-                if (k >= 2) wait(bar_item_free + 8 * (k & 1), ((k >> 1) - 1) & 1, kWaitItemFree);
-                s_item[k & 1] = w;
-                WorkItem it;
-                if (w >= 0) {
-                    decode_item(p, w, it);
-                    s_decoded[k & 1] = it;
+    // register budget per warpgroup: 2 x 184 (softmax) + 96 (epilogue) + 48 (the rest) = 4 x 128
+    if (warp >= 12) {
+        reg_dealloc<48>();
+        if (warp == 15) {
+            // --------------------------------------------------------- scheduler
+            if (lane == 0) {
+                int w = static_cast<int>(blockIdx.x >> 1);
+                int published = 0, asked = 0;
+                if (*reinterpret_cast<volatile int32_t*>(&p.hdr->status) != 0) w = -1;
+                while (true) {
+                    const int slot = published % kItems;
+                    if (published >= kItems) wait_asleep(bars.item_free[slot], (published / kItems - 1) & 1, kWaitItemFree);
+                    bool some = false;
+                    if (w >= 0) {
+                        decode_item<MODE>(p, w, s_decoded[slot]);
+                        some = s_decoded[slot].nt > 0;  // padding of the item list is skipped
+                    }
+                    if (w < 0 || some) {
+                        s_item[slot] = w < 0 ? -1 : 1;
+                        mbar_arrive(smem_u32(&bars.item_full[slot]));  // release: the decoded item is visible
+                        if (w < 0) break;
+                        ++published;
+                        // the next item is claimed when the loads of this one near their end, so that a pair never
+                        // sits on work another one could take
+                        if (rank == 0) wait_asleep(bars.go, (published - 1) & 1, kWaitGo);
+                    }
+                    mbar_arrive_expect_tx(smem_u32(&bars.clc), 16);
+                    if (rank == 0) {
+                        if (asked > 0) wait_asleep(bars.clc_read, (asked - 1) & 1, kWaitClc);
+                        clc_try_cancel(smem_u32(&s_clc), smem_u32(&bars.clc));
+                    }
+                    wait_asleep(bars.clc, asked & 1, kWaitClc);
+                    const int first = clc_first_block(smem_u32(&s_clc));
+                    fence_proxy_async_smem();  // the answer is written again by the asynchronous proxy
+                    if (rank == 1) mbar_arrive_cluster(map_to_cta(smem_u32(&bars.clc_read), 0));
+                    w = (first < 0 || abort_flag != 0) ? -1 : first >> 1;
+                    ++asked;
                 }
-                mbar_arrive(bar_item_full + 8 * (k & 1));  // release: the item and its decoded form are visible
-                if (w < 0) break;
-                const int nt_max = max(it.s[0].nt, it.s[1].nt);
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    if (it.s[x].nt == 0) continue;
-                    if (q_loads[x] > 0) wait(bar_q_free + 8 * x, (q_loads[x] - 1) & 1, kWaitQFree);
-                    mbar_arrive_expect_tx(bar_q_full + 8 * x, static_cast<uint32_t>(NP * it.s[x].box_rows * 128));
-                    const CUtensorMap* qmap = it.s[x].qmap == 0 ? &tmap_q : it.s[x].qmap == 1 ? &tmap_q_tail_block : &tmap_q_tail_sink;
-                    for (int h = 0; h < NP; ++h)
-                        tma_load_3d(smem_base + (x ? L::kQ1 : L::kQ0) + h * L::kPanelBytes, qmap, h * 64,
-                                    it.s[x].q_head0, it.s[x].q_tok0, bar_q_full + 8 * x);
-                    ++q_loads[x];
-                }
-                for (int j = 0; j < nt_max; ++j) {
+            }
+        } else if (warp == 13) {
+            // --------------------------------------------------------- TMA producer: K(s), then V(s - kQkAhead)
+            if (lane == 0) {
+                struct Cursor {
+                    int k, j, nt, na, kv_head, b_coord0, own_map;
+                };
+                auto enter = [&](Cursor& c) {  // the cursor's item; false: no more work
+                    if (!item_ready(c.k)) return false;
+                    const WorkItem& it = s_decoded[c.k % kItems];
+                    c.j = 0; c.nt = it.nt; c.na = it.na;
+                    c.kv_head = it.kv_head; c.b_coord0 = it.b_coord0; c.own_map = it.own_map;
+                    return true;
+                };
+                Cursor kc{}, vc{};
+                int n_a = 0, n_b = 0;
+                bool k_end = false;
+                uint32_t tiles = 0;  // K tiles loaded so far
+#pragma unroll 1
+                for (uint32_t s = 0; !k_end || s < tiles + kQkAhead; ++s) {
+                    if (!k_end && kc.j == kc.nt) {
+                        k_end = !enter(kc);
+                        if (!k_end) {
+                            const WorkItem& it = s_decoded[kc.k % kItems];
+                            const QSlot& q = it.s[rank];
+                            n_a = it.n_a; n_b = it.n_b;
+                            const int qb = kc.k & 1;
+                            if (kc.k >= 2) wait(bars.q_free[qb], ((kc.k >> 1) - 1) & 1, kWaitQFree);
+                            if (rank == 0)
+                                mbar_arrive_expect_tx(smem_u32(&bars.q_full[qb]),
+                                                      static_cast<uint32_t>(NP * 128 * ((it.s[0].valid ? it.s[0].box_rows : 0) +
+                                                                                        (it.s[1].valid ? it.s[1].box_rows : 0))));
+                            if (q.valid) {
+                                const CUtensorMap* qmap = q.qmap == 0 ? &tmap_q : q.qmap == 1 ? &tmap_q_tail_block : &tmap_q_tail_sink;
+                                const uint32_t bar = map_to_cta(smem_u32(&bars.q_full[qb]), 0);
+                                for (int h = 0; h < NP; ++h)
+                                    tma_load_3d_pair(smem_base + L::kQ + qb * L::kQBytes + h * L::kQPanelBytes, qmap, h * 64,
+                                                     q.q_head0, q.q_tok0, bar);
+                            }
+                        }
+                    }
                     // Rows past the end of the sink, and past the end of the block range, are outside their
                     // tensor map and arrive as zeros: a ragged last tile never brings in a neighbour's rows.
-                    const bool shared_range = j < it.na || it.own_map != 0;
-                    const int j0 = j < it.na ? j * kTile : it.b_coord0 + (j - it.na) * kTile;
-#pragma unroll
-                    for (int kv = 0; kv < 2; ++kv) {
-                        const int slot = ring_idx % kRing, use = ring_idx / kRing;
-                        if (use > 0) wait(bar_empty + 8 * slot, (use - 1) & 1, kWaitEmpty);
-                        mbar_arrive_expect_tx(bar_full + 8 * slot, L::kTileBytes);
+                    if (!k_end) {
+                        const int j = kc.j++;
+                        if (rank == 0 && j == max(0, kc.nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
+                        const CUtensorMap* map = (j < kc.na || kc.own_map != 0) ? &tmap_k_sink : &tmap_k;
+                        const int n = j == kc.na - 1 ? n_a : j == kc.nt - 1 ? n_b : kTile;  // this CTA's keys: half of them
+                        const int row = (j < kc.na ? j * kTile : kc.b_coord0 + (j - kc.na) * kTile) + static_cast<int>(rank) * (n >> 1);
+                        const uint32_t slot = tiles % kRing;
+                        if (tiles >= kRing) wait_s_full(tiles - kRing, kWaitKvFree);
+                        if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[slot]), 2 * L::kKBytes);
+                        const uint32_t bar = map_to_cta(smem_u32(&bars.k_full[slot]), 0);
                         for (int h = 0; h < NP; ++h)
-                            tma_load_3d(smem_base + L::kRing0 + slot * L::kTileBytes + h * L::kPanelBytes,
-                                        shared_range ? (kv ? &tmap_v_sink : &tmap_k_sink) : (kv ? &tmap_v : &tmap_k),
-                                        h * 64, it.kv_head, j0, bar_full + 8 * slot);
-                        ++ring_idx;
+                            tma_load_3d_pair(smem_base + L::kK + slot * L::kKBytes + h * L::kKPanelBytes, map, h * 64, kc.kv_head, row, bar);
+                        ++tiles;
+                        if (kc.j == kc.nt) ++kc.k;
+                    }
+                    if (s >= kQkAhead && s - kQkAhead < tiles) {
+                        const uint32_t u = s - kQkAhead;
+                        if (vc.j == vc.nt) {
+                            enter(vc);
+                            item_release(vc.k);
+                        }
+                        const int j = vc.j++;
+                        const CUtensorMap* map = (j < vc.na || vc.own_map != 0) ? &tmap_v_sink : &tmap_v;
+                        const int row = j < vc.na ? j * kTile : vc.b_coord0 + (j - vc.na) * kTile;
+                        const uint32_t slot = u % kRing;
+                        if (u >= kRing) wait_pv_done(u - kRing, kWaitKvFree);
+                        if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[slot]), 2 * L::kVBytes);
+                        tma_load_3d_pair(smem_base + L::kV + slot * L::kVBytes, map, static_cast<int>(rank) * (D / 2), vc.kv_head, row,
+                                         map_to_cta(smem_u32(&bars.v_full[slot]), 0));
+                        if (vc.j == vc.nt) ++vc.k;
                     }
                 }
             }
-        }
-      } else if (warp == 8) {
-        // ------------------------------------------------------------- MMA issuer
-        // All 32 lanes run this loop with warp-uniform values (descriptors and addresses stay in
-        // uniform registers); the MMA and commit instructions themselves go out from one elected lane.
-        int ring_base = 0;        // ring position of this item's K(0)
-        int cnt[2] = {0, 0};      // tiles per slot before this item (phase of s_full / po)
-        int q_uses[2] = {0, 0};   // items in which the slot was active so far
-        for (int k = 0;; ++k) {
-            // every lane reads the item, one lane releases the queue slot
-            wait(bar_item_full + 8 * (k & 1), (k >> 1) & 1, kWaitItem);
-            const int w = s_item[k & 1];
-            WorkItem it;
-            if (w >= 0) it = s_decoded[k & 1];
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_item_free + 8 * (k & 1));
-            if (w < 0) break;
-            PEVLM_STAMP_ITEM(0, k, lane == 0);
-            const int nt[2] = {it.s[0].nt, it.s[1].nt};
-            const int nt_max = max(nt[0], nt[1]);
-            // keys in the last tile of the shared range and of each slot's own range (every other
-            // tile is full)
-            const int na = it.na;
-            const int a_last = it.a_end - (na - 1) * kTile;
-            const int b_last[2] = {it.s[0].b_end - it.b_start - (nt[0] - na - 1) * kTile,
-                                   it.s[1].b_end - it.b_start - (nt[1] - na - 1) * kTile};
-            auto valid_of = [&](int x, int j) { return (j == na - 1) ? a_last : (j == nt[x] - 1) ? b_last[x] : kTile; };
-            auto ring_addr = [&](int idx) { return smem_base + L::kRing0 + ((ring_base + idx) % kRing) * L::kTileBytes; };
-            auto wait_full = [&](int idx) {
-                const int g = ring_base + idx;
-                wait(bar_full + 8 * (g % kRing), (g / kRing) & 1, kWaitFull);
-            };
-            auto commit_empty = [&](int idx) { mma_commit_elect(bar_empty + 8 * ((ring_base + idx) % kRing)); };
-            // S_x = Q_x K(j)^T
-            auto issue_qk = [&](int x, int j) {
-                PEVLM_STAMP(4, j, lane == 0 && x == 0);
-                const int n_mma = (valid_of(x, j) + 15) & ~15;
-                const uint32_t idesc = make_idesc_bf16(kTile, n_mma, false);
-                mma_ss_batch<D / 16>(tmem_base + x * 128, desc_lo(smem_base + (x ? L::kQ1 : L::kQ0), 16),
-                                     desc_lo(ring_addr(2 * j), 16), idesc);
-                PEVLM_STAMP(5, j, lane == 0 && x == 0);
-                mma_commit_elect(bar_s_full + 8 * x);
-                if (j == nt[x] - 1) mma_commit_elect(bar_q_free + 8 * x);  // last use of this Q tile
-            };
-            // O_x += P_x V(j)
-            auto issue_pv = [&](int x, int j) {
-                wait((kPvSplit > 0 ? bar_po_a : bar_po) + 8 * x, (cnt[x] + j) & 1, kWaitPO);
-                PEVLM_STAMP(6, j, lane == 0 && x == 0);
-                // the previous item's output must have left TMEM before O is overwritten
-                if (j == 0 && q_uses[x] > 0) wait(bar_o_free + 8 * x, (q_uses[x] - 1) & 1, kWaitOFree);
-                tc_fence_after_sync();
-                const int nvalid = valid_of(x, j);
-                const uint32_t idesc = make_idesc_bf16(kTile, D, true);
-                const uint32_t sv = ring_addr(2 * j + 1);
-                const uint32_t d_tmem = tmem_base + 256 + x * 128, a_tmem = tmem_base + x * 128;
-                if (kPvSplit > 0) {
-                    // first part (the wait above was for it), then the wait for the rest of the tile
-                    const uint32_t b_lo = desc_lo(sv, L::kPanelBytes);
-                    const int ksteps = (nvalid + 15) >> 4;
-                    constexpr int kFirst = 2 * kPvSplit;
-                    if (nvalid == kTile) {
-                        if (kPvSplit == 1) mma_ts_batch2(d_tmem, a_tmem, b_lo, idesc, j > 0);
-                        if (kPvSplit >= 2) mma_ts_batch4(d_tmem, a_tmem, b_lo, idesc, j > 0);
-                        if (kPvSplit == 3) mma_ts_batch2(d_tmem, a_tmem + 32, b_lo + 512, idesc, 1);
-                    } else {
-                        for (int ks = 0; ks < min(ksteps, kFirst); ++ks)
-                            mma_ts_elect(d_tmem, a_tmem + ks * 8, make_smem_desc_sw128(sv + ks * 2048, L::kPanelBytes, 1024), idesc,
-                                         (j > 0) || (ks > 0));
-                    }
-                    wait(bar_po + 8 * x, (cnt[x] + j) & 1, kWaitPO);
+        } else if (rank == 0 && warp == 12) {
+            // --------------------------------------------------------- S = Q K^T of the pair
+            // All 32 lanes run this loop with warp-uniform values (descriptors and addresses stay in
+            // uniform registers); the MMA and commit instructions themselves go out from one elected lane.
+            uint32_t t = 0;
+#pragma unroll 1
+            for (int k = 0; item_ready(k); ++k) {
+                const WorkItem& it = s_decoded[k % kItems];
+                const int nt = it.nt, na = it.na, n_a = it.n_a, n_b = it.n_b;
+                __syncwarp();
+                if (lane == 0) item_release(k);
+                const uint32_t q_lo = desc_lo(smem_base + L::kQ + (k & 1) * L::kQBytes, 16);
+                wait(bars.q_full[k & 1], (k >> 1) & 1, kWaitQ);
+#pragma unroll 1
+                for (int j = 0; j < nt; ++j, ++t) {
+                    const int n = j == na - 1 ? n_a : j == nt - 1 ? n_b : kTile;
+                    const uint32_t slot = t % kRing;
+                    wait(bars.k_full[slot], (t / kRing) & 1, kWaitK);
+                    if (t >= 2) wait(bars.s_read[t & 1], ((t >> 1) - 1) & 1, kWaitSRead);
                     tc_fence_after_sync();
-                    if (nvalid == kTile) {
-                        if (kPvSplit == 1) mma_ts_batch2(d_tmem, a_tmem + 16, b_lo + 256, idesc, 1);
-                        if (kPvSplit <= 2) mma_ts_batch4(d_tmem, a_tmem + 32, b_lo + 512, idesc, 1);
-                        if (kPvSplit == 3) mma_ts_batch2(d_tmem, a_tmem + 48, b_lo + 768, idesc, 1);
+                    mma_ss_batch<D / 16>(tmem_base + (t & 1) * kTile, q_lo, desc_lo(smem_base + L::kK + slot * L::kKBytes, 16),
+                                         make_idesc_bf16(2 * kTile, n, false));
+                    mma_commit_pair(smem_u32(&bars.s_full[slot]));
+                }
+                mma_commit_pair(smem_u32(&bars.q_free[k & 1]));
+            }
+        } else if (rank == 0 && warp == 14) {
+            // --------------------------------------------------------- O += P V of the pair
+            constexpr uint32_t kIdescPv = make_idesc_bf16(2 * kTile, D, true);
+            const uint32_t d_tmem = tmem_base + kTmemO;
+            uint32_t t = 0;
+#pragma unroll 1
+            for (int k = 0; item_ready(k); ++k) {
+                const WorkItem& it = s_decoded[k % kItems];
+                const int nt = it.nt, na = it.na, n_a = it.n_a, n_b = it.n_b;
+                __syncwarp();
+                if (lane == 0) item_release(k);
+                // the previous item's output must have left TMEM before O is overwritten
+                if (k > 0) wait(bars.o_free, (k - 1) & 1, kWaitOFree);
+#pragma unroll 1
+                for (int j = 0; j < nt; ++j, ++t) {
+                    const int n = j == na - 1 ? n_a : j == nt - 1 ? n_b : kTile;
+                    const uint32_t slot = t % kRing;
+                    const uint32_t v_lo = desc_lo(smem_base + L::kV + slot * L::kVBytes, 0);
+                    const uint32_t a_tmem = tmem_base + kTmemP + (t & 1) * (kTile / 2);
+                    wait(bars.v_full[slot], (t / kRing) & 1, kWaitV);
+                    wait(bars.p_full[t & 1], (t >> 1) & 1, kWaitP);
+                    tc_fence_after_sync();
+                    if (n == kTile) {
+                        mma_ts_batch8<D>(d_tmem, a_tmem, v_lo, kIdescPv, j > 0);
                     } else {
-                        for (int ks = kFirst; ks < ksteps; ++ks)
-                            mma_ts_elect(d_tmem, a_tmem + ks * 8, make_smem_desc_sw128(sv + ks * 2048, L::kPanelBytes, 1024), idesc, 1);
+#pragma unroll 1
+                        for (int ks = 0; ks < (n >> 4); ++ks)
+                            mma_ts_step<D>(d_tmem, a_tmem + ks * 8, v_lo + ks * kVDescStep<D>, kIdescPv, (j > 0) || (ks > 0));
                     }
-                } else if (nvalid == kTile) {
-                    mma_ts_batch8(d_tmem, a_tmem, desc_lo(sv, L::kPanelBytes), idesc, j > 0);
-                } else {
-                    const int ksteps = (nvalid + 15) >> 4;
-                    for (int ks = 0; ks < ksteps; ++ks)
-                        mma_ts_elect(d_tmem, a_tmem + ks * 8, make_smem_desc_sw128(sv + ks * 2048, L::kPanelBytes, 1024), idesc,
-                                     (j > 0) || (ks > 0));
+                    mma_commit_pair(smem_u32(&bars.pv_done[slot]));
                 }
-                PEVLM_STAMP(7, j, lane == 0 && x == 0);
-                // o_done: the item's accumulator is complete (one phase per item, for the epilogue)
-                if (j == nt[x] - 1) mma_commit_elect(bar_o_done + 8 * x);
-            };
-#pragma unroll
-            for (int x = 0; x < 2; ++x)
-                if (nt[x] > 0) wait(bar_q_full + 8 * x, q_uses[x] & 1, kWaitQ);
-            tc_fence_after_sync();
-            // Order on the tensor pipe: QK0(0) QK1(0), then per key tile j: PV0(j) QK0(j+1) PV1(j) QK1(j+1).
-            // While one query tile is in its softmax the other one's MMAs run.  PV_x(j) and QK_x(j+1) go out
-            // back to back: everything they wait for except the probabilities (V(j), K(j+1)) is waited for
-            // before the wait on P_x(j), so the scores of the next tile follow the probabilities of this one
-            // through the pipe without a gap.
-            if (nt_max > 0) {
-                wait_full(0);
-                PEVLM_STAMP_ITEM(1, k, lane == 0);
-                if (nt[0] > 0) issue_qk(0, 0);
-                if (nt[1] > 0) issue_qk(1, 0);
-                commit_empty(0);  // K(0) consumed
-            }
-            for (int j = 0; j < nt_max; ++j) {
-                const bool more = j + 1 < nt_max;
-                wait_full(2 * j + 1);             // V(j)
-                if (more) wait_full(2 * j + 2);   // K(j+1)
-                if (j < nt[0]) {
-                    issue_pv(0, j);
-                    if (j + 1 < nt[0]) issue_qk(0, j + 1);
-                }
-                if (j < nt[1]) {
-                    issue_pv(1, j);
-                    if (j + 1 < nt[1]) issue_qk(1, j + 1);
-                }
-                commit_empty(2 * j + 1);            // V(j) consumed
-                if (more) commit_empty(2 * j + 2);  // K(j+1) consumed
-            }
-            PEVLM_STAMP_ITEM(2, k, lane == 0);
-            ring_base += 2 * nt_max;
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                cnt[x] += nt[x];
-                if (nt[x] > 0) ++q_uses[x];
             }
         }
-      }
-    } else {
-        // ------------------------------------------------------------- softmax and epilogue of slot x
-        reg_alloc<216>();
-        const int x = warp >> 2;
+    } else if (warp >= 8) {
+        // ------------------------------------------------------------- epilogue
+        reg_dealloc<96>();
         const int row = tid & 127;
-        const uint32_t lane_off = static_cast<uint32_t>((warp & 3) * 32) << 16;
-        const uint32_t tS = tmem_base + x * 128 + lane_off;
-        const uint32_t tO = tmem_base + 256 + x * 128 + lane_off;
-        const uint32_t my_s_full = bar_s_full + 8 * x, my_po = bar_po + 8 * x;
-        int cnt = 0;        // tiles of this slot processed so far (phase of s_full)
-        int uses = 0;       // items in which this slot was active so far
-        int ring_base = 0;  // ring position of this item's K(0)
-        for (int k = 0;; ++k) {
-            WorkItem it;
-            const int w = next_item(k, it);
-            if (w < 0) break;
-            // this slot's scalars, in registers
-            const int nt = x ? it.s[1].nt : it.s[0].nt;
-            const int item_ring_base = ring_base;
-            ring_base += 2 * max(it.s[0].nt, it.s[1].nt);
-            const QSlot& qs = x ? it.s[1] : it.s[0];
-            if (!qs.valid) continue;
-            // this thread's row of the query tile
-            // (row_div is 1 for all but packed tiles: no integer division on the way to the item's first scores)
+        const uint32_t tO = tmem_base + kTmemO + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+        const uint32_t o_free_bar = map_to_cta(smem_u32(&bars.o_free), 0);
+        uint32_t t_end = 0;  // tiles up to the end of this item
+#pragma unroll 1
+        for (int k = 0; item_ready(k); ++k) {
+            const WorkItem& it = s_decoded[k % kItems];
+            const QSlot& qs = it.s[rank];
+            t_end += it.nt;
             const int row_tok = qs.row_div == 1 ? row : row / qs.row_div;
             const int row_head = qs.row_div == 1 ? 0 : row - row_tok * qs.row_div;
-            const bool row_ok = (row_tok < qs.ntok) && (row_head < qs.nheads);
+            const bool row_ok = qs.valid && (row_tok < qs.ntok) && (row_head < qs.nheads);
             const int tok = qs.q_tok0 + row_tok;
             const int head = qs.q_head0 + row_head;
-            if (nt == 0) {
-                // question-mode tile with no visible key in this CTA's key range: neutral partial
-                if (p.mode == 1 && row_ok) {
-                    const size_t r = (static_cast<size_t>(it.split) * p.Q + tok) * p.Hq + head;
-                    p.part_lse[r] = -INFINITY;
-                    float4* dst = reinterpret_cast<float4*>(p.part_o + r * D);
-                    for (int c = 0; c < D / 4; ++c) dst[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int split = it.split;
+            __syncwarp();
+            if (lane == 0) item_release(k);
+            wait_asleep(bars.sums_full[k % kSums], (k / kSums) & 1, kWaitSum);
+            const float2 sa = s_sums[k % kSums][0][row], sb = s_sums[k % kSums][1][row];
+            const float m = fmaxf(sa.y, sb.y);
+            const float l = m == -INFINITY ? 0.f
+                                           : sa.x * fast_exp2((sa.y - m) * p.scale_log2) + sb.x * fast_exp2((sb.y - m) * p.scale_log2);
+            const float inv_l = (l > 0.f) ? 1.f / l : 0.f;
+            const float lse_val = (l > 0.f) ? m * p.scale + logf(l) : -INFINITY;
+            wait_pv_done(t_end - 1, kWaitODone);
+            tc_fence_after_sync();
+            // 32 columns at a time, in a loop that stays one; 32 bytes per store: every lane writes whole sectors of
+            // its own row
+            const size_t r = MODE == 0 ? static_cast<size_t>(tok) * p.Hq + head
+                                       : (static_cast<size_t>(split) * p.Q + tok) * p.Hq + head;
+#pragma unroll 1
+            for (int c = 0; c < D / 32; ++c) {
+                uint32_t o[32];
+                tmem_ld32(tO + c * 32, o);
+                tmem_wait_ld();
+                if (c == D / 32 - 1) {  // the accumulator may be written again
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(o_free_bar);
                 }
-                continue;
+                if (MODE == 0) {
+                    uint32_t wd[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        wd[e] = pack_bf16x2(__uint_as_float(o[2 * e]) * inv_l, __uint_as_float(o[2 * e + 1]) * inv_l);
+                    if (row_ok) {
+#pragma unroll
+                        for (int v = 0; v < 2; ++v)
+                            st_global_v8(p.o + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]));
+                    }
+                } else if (row_ok) {
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * inv_l);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) st_global_v8(p.part_o + r * D + c * 32 + v * 8, *reinterpret_cast<uint32_t(*)[8]>(&o[8 * v]));
+                }
             }
-            const int limit0 = x ? it.s[1].limit0 : it.s[0].limit0;
-            const int b_end = x ? it.s[1].b_end : it.s[0].b_end;
-            const int na = it.na, a_end = it.a_end, b_start = it.b_start;
-            const int my_limit = limit0 + row_tok;
-            float m_ref = -INFINITY;  // reference maximum (raw score units) the probabilities are scaled by
+            if (row_ok && MODE == 0 && p.lse) st_global_stream_f32(p.lse + static_cast<size_t>(head) * p.q_rows + tok, lse_val);
+            if (row_ok && MODE == 1) st_global_stream_f32(p.part_lse + r, lse_val);
+        }
+    } else {
+        // ------------------------------------------------------------- softmax, every other key tile
+        reg_alloc<184>();
+        const int wg = warp >> 2, quarter = warp & 3;
+        const int row = tid & 127;
+        const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
+        const uint32_t p_bar = map_to_cta(smem_u32(&bars.p_full[wg]), 0), s_read_bar = map_to_cta(smem_u32(&bars.s_read[wg]), 0);
+        const uint32_t tS = tmem_base + wg * kTile + lane_off, tP = tmem_base + kTmemP + wg * (kTile / 2) + lane_off;
+        const uint32_t tO = tmem_base + kTmemO + lane_off;
+        uint32_t t0 = 0;                // tiles of all items so far
+#pragma unroll 1
+        for (int k = 0; item_ready(k); ++k) {
+            const WorkItem& it = s_decoded[k % kItems];
+            const QSlot& qs = it.s[rank];
+            const int nt = it.nt, na = it.na, a_end = qs.valid ? it.a_end : 0;  // a slot without a tile sees nothing
+            // (row_div is 1 for all but packed tiles: no integer division on the way to the item's first scores)
+            const int row_tok = qs.row_div == 1 ? row : row / qs.row_div;
+            // this row's last visible key and the smallest such key of the tile, counted from the own range's start
+            const int end = qs.valid ? qs.end : 0;
+            const int my_limit = min(qs.limit0 + row_tok, end - 1), limit0 = min(qs.limit0, end - 1);
+            __syncwarp();
+            if (lane == 0) item_release(k);
+            float m_own = -INFINITY;  // reference maximum (raw score units) this warpgroup's row sum is scaled by
             float l_run = 0.f;
-            for (int j = 0; j < nt; ++j, ++cnt) {
-                const int j0 = j < na ? j * kTile : b_start + (j - na) * kTile;
-                const int nvalid = min(kTile, (j < na ? a_end : b_end) - j0);
-                const bool need_mask = (nvalid < kTile) || (j0 + kTile - 1 > limit0);
-                wait(my_s_full, cnt & 1, kWaitS);
-                PEVLM_STAMP(0 + x, j, (tid & 127) == 0);
-                PEVLM_STAMP_ITEM(3, k, tid == 0 && j == 0);
+#pragma unroll 1
+            for (int j = static_cast<int>((t0 ^ static_cast<uint32_t>(wg)) & 1u); j < nt; j += 2) {
+                const uint32_t t = t0 + j;
+                // keys of this tile that the row sees, and that every row of the query tile sees
+                const int max_col = j < na ? a_end - j * kTile : my_limit + 1 - (j - na) * kTile;
+                const bool need_mask = (j < na ? a_end - j * kTile : limit0 + 1 - (j - na) * kTile) < kTile;
+                wait_s_full(t, kWaitS);
                 tc_fence_after_sync();
                 // all 128 scores of the row in registers: one round trip to TMEM
                 uint32_t r[kTile];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) tmem_ld32(tS + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&r[32 * c]));
                 tmem_wait_ld();
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(s_read_bar);
                 if (need_mask) {
-                    const int max_col = min(nvalid, my_limit - j0 + 1);
+                    // by 32 columns: on the diagonal the rows of a warp differ within one such part only, the others are
+                    // visible or hidden as a whole (a compare for each of the 128 columns took 1,200 cycles a tile)
 #pragma unroll
-                    for (int i = 0; i < kTile; ++i)
-                        if (i >= max_col) r[i] = 0xff800000u;  // -inf
+                    for (int c = 0; c < 4; ++c) {
+                        const int cols = max_col - c * 32;  // visible ones of this part
+                        if (__all_sync(0xffffffffu, cols >= 32)) continue;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if (i >= cols) r[c * 32 + i] = 0xff800000u;  // -inf
+                    }
                 }
                 float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -557,145 +644,105 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
                         mx[a] = fmax3(mx[a], __uint_as_float(r[i + 2 * a]), __uint_as_float(r[i + 2 * a + 1]));
                 }
                 const float m_tile = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-                float alpha = 1.f;
-                if ((m_tile - m_ref) * p.scale_log2 > kRescaleThresholdLog2 || m_ref == -INFINITY) {
-                    const float m_new = fmaxf(m_ref, m_tile);
-                    alpha = (m_new == -INFINITY) ? 1.f : fast_exp2((m_ref - m_new) * p.scale_log2);
-                    m_ref = m_new;
+                // the row's reference maximum after tile t - 1 comes from the other warpgroup
+                float m_prev = -INFINITY;
+                if (t > 0) {
+                    pass_wait(kPassMax, wg, quarter);
+                    if (j > 0) m_prev = s_max[wg ^ 1][row];
                 }
-                if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-                    // rare: rescale this row of the O accumulator in place, once PV(j-1) has landed: the
-                    // ring slot of V(j-1) is released by a commit issued after both slots' PV(j-1).
-                    // (S(j) is complete, so that slot's previous release, two tiles back, is too.)
-                    const int gv = item_ring_base + 2 * (j - 1) + 1;
-                    wait(bar_empty + 8 * (gv % kRing), (gv / kRing) & 1, kWaitPV);
+                float m_ref = m_prev;
+                if ((m_tile - m_prev) * p.scale_log2 > kRescaleThresholdLog2 || m_prev == -INFINITY) m_ref = fmaxf(m_prev, m_tile);
+                s_max[wg][row] = m_ref;
+                pass_on(kPassMax, wg, quarter);
+                if (j > 0 && __any_sync(0xffffffffu, m_ref != m_prev)) {
+                    // rare: rescale this row of the O accumulator in place, once PV(t - 1) has landed
+                    const float alpha = m_ref == m_prev ? 1.f : fast_exp2((m_prev - m_ref) * p.scale_log2);
+                    wait_pv_done(t - 1, kWaitPV);
                     tc_fence_after_sync();
-#pragma unroll
-                    for (int c = 0; c < D / 32; ++c) {
-                        uint32_t o[32];
-                        tmem_ld32(tO + c * 32, o);
+#pragma unroll 1
+                    for (int c = 0; c < D / 16; ++c) {
+                        uint32_t o[16];
+                        tmem_ld16(tO + c * 16, o);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                        tmem_st32(tO + c * 32, o);
+                        for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                        tmem_st16(tO + c * 16, o);
                     }
                 }
+                if (t >= 2) wait_pv_done(t - 2, kWaitPFree);  // this probability buffer has been read
+                if (t > 0) pass_wait(kPassTurn, wg, quarter);
                 const float neg_ms = (m_ref == -INFINITY) ? 0.f : -m_ref * p.scale_log2;
-                // probabilities, written over the scores as bf16 pairs (columns [0, 64) of the slot);
-                // scale-and-shift and the row sum run as packed fp32 pairs
+                // probabilities as bf16 pairs; scale-and-shift and the row sum run as packed fp32 pairs
                 const uint64_t scale2 = pack_f32x2(p.scale_log2, p.scale_log2);
                 const uint64_t shift2 = pack_f32x2(neg_ms, neg_ms);
                 uint64_t sm2[4] = {0ull, 0ull, 0ull, 0ull};
+                uint32_t pk[kTile / 2];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    uint32_t pk[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const uint64_t t2 = fma_f32x2(pack_f32x2(__uint_as_float(r[c * 32 + 2 * i]),
-                                                                 __uint_as_float(r[c * 32 + 2 * i + 1])), scale2, shift2);
-                        float t0, t1;
-                        unpack_f32x2(t2, t0, t1);
-                        const float p0 = fast_exp2(t0), p1 = fast_exp2(t1);
-                        sm2[i & 3] = add_f32x2(sm2[i & 3], pack_f32x2(p0, p1));
-                        pk[i] = pack_bf16x2(p0, p1);
-                    }
-                    tmem_st16(tS + c * 16, pk);
-                    if (kPvSplit > 0 && c == kPvSplit - 1) {  // first part of the probabilities is in TMEM
-                        tmem_wait_st();
-                        tc_fence_before_sync();
-                        mbar_arrive(bar_po_a + 8 * x);
-                    }
-                }
-                float sum;
-                {
-                    float a0, a1, b0, b1;
-                    unpack_f32x2(add_f32x2(sm2[0], sm2[1]), a0, a1);
-                    unpack_f32x2(add_f32x2(sm2[2], sm2[3]), b0, b1);
-                    sum = (a0 + a1) + (b0 + b1);
+                for (int i = 0; i < kTile / 2; ++i) {
+                    const uint64_t t2 = fma_f32x2(pack_f32x2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), scale2, shift2);
+                    float e0, e1;
+                    unpack_f32x2(t2, e0, e1);
+                    const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
+                    sm2[i & 3] = add_f32x2(sm2[i & 3], pack_f32x2(p0, p1));
+                    pk[i] = pack_bf16x2(p0, p1);
+                    if (i % 16 == 15) tmem_st16(tP + i - 15, &pk[i - 15]);
+                    if (i == kTurn) pass_on(kPassTurn, wg, quarter);
                 }
                 tmem_wait_st();
                 tc_fence_before_sync();
-                mbar_arrive(my_po);
-                PEVLM_STAMP(2 + x, j, (tid & 127) == 0);
-                PEVLM_STAMP_ITEM(4, k, tid == 0 && j == nt - 1);
-                l_run = l_run * alpha + sum;
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(p_bar);
+                float a0, a1, b0, b1;
+                unpack_f32x2(add_f32x2(sm2[0], sm2[1]), a0, a1);
+                unpack_f32x2(add_f32x2(sm2[2], sm2[3]), b0, b1);
+                const float sum = (a0 + a1) + (b0 + b1);
+                l_run = (m_own == m_ref ? l_run : l_run * fast_exp2((m_own - m_ref) * p.scale_log2)) + sum;
+                m_own = m_ref;
+#ifdef PEVLM_TRACE
+                if (lane == 0) ++s_waits[warp][1];
+#endif
             }
-            // Epilogue, by the same thread (its registers are free now and it would only wait for the next
-            // item's scores): once the last PV has landed, the whole accumulator row goes to registers in one
-            // round trip and the accumulator is released for the next item; normalisation, conversion and the
-            // stores follow while the next item's first QK is already in the tensor pipe.
-            wait(bar_o_done + 8 * x, uses & 1, kWaitPV);
-            PEVLM_STAMP_ITEM(5, k, tid == 0);
-            tc_fence_after_sync();
-            {
-                uint32_t o[D];
-#pragma unroll
-                for (int c = 0; c < D / 32; ++c) tmem_ld32(tO + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&o[32 * c]));
-                tmem_wait_ld();
-                tc_fence_before_sync();
-                mbar_arrive(bar_o_free + 8 * x);
-                PEVLM_STAMP_ITEM(6, k, tid == 0);
-                const float inv_l = (l_run > 0.f) ? 1.f / l_run : 0.f;
-                const float lse_val = (l_run > 0.f) ? m_ref * p.scale + logf(l_run) : -INFINITY;
-                if (row_ok) {
-                    if (p.mode == 0) {
-                        // 32 bytes per store: every lane writes whole sectors of its own row
-                        __nv_bfloat16* dst = p.o + (static_cast<size_t>(tok) * p.Hq + head) * D;
-#pragma unroll
-                        for (int v = 0; v < D / 16; ++v) {
-                            uint32_t wd[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                wd[e] = pack_bf16x2(__uint_as_float(o[v * 16 + 2 * e]) * inv_l,
-                                                    __uint_as_float(o[v * 16 + 2 * e + 1]) * inv_l);
-                            st_global_v8(dst + v * 16, wd);
-                        }
-                        if (p.lse) st_global_stream_f32(p.lse + static_cast<size_t>(head) * p.q_rows + tok, lse_val);
-                    } else {
-                        const size_t r = (static_cast<size_t>(it.split) * p.Q + tok) * p.Hq + head;
-                        float* dst = p.part_o + r * D;
-#pragma unroll
-                        for (int v = 0; v < D / 8; ++v) {
-                            uint32_t wd[8];
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) wd[e] = __float_as_uint(__uint_as_float(o[v * 8 + e]) * inv_l);
-                            st_global_v8(dst + v * 8, wd);
-                        }
-                        st_global_stream_f32(p.part_lse + r, lse_val);
-                    }
-                }
-            }
-            PEVLM_STAMP_ITEM(7, k, tid == 0);
-            ++uses;
+            t0 += nt;
+            s_sums[k % kSums][wg][row] = make_float2(l_run, m_own);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bars.sums_full[k % kSums]));
+        }
+        if (t0 > 0 && static_cast<uint32_t>(wg) == (t0 & 1u)) {  // the last tile's passes
+            pass_wait(kPassMax, wg, quarter);
+            pass_wait(kPassTurn, wg, quarter);
         }
     }
+#ifdef PEVLM_TRACE
+    __syncwarp();
+    if (lane == 0) s_waits[warp][0] = static_cast<unsigned>(clock64()) - role_start;
+    __syncwarp();
+    if (blockIdx.x < 2)
+        for (int i = lane; i < kTraceIds; i += 32) g_waits[blockIdx.x][warp][i] = s_waits[warp][i];
+#endif
     tc_fence_before_sync();
-    __syncthreads();
-    if (warp == 8) {
+    __syncwarp();
+    cluster_sync_all();  // neither CTA leaves, or frees TMEM, while the other may still reach it
+    if (warp == 12) {
         __syncwarp();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc_pair(tmem_base, 512);
     }
+    if (tid == 0 && abort_flag != 0 && atomicCAS(&p.hdr->status, 0, PEVLM_ETIMEOUT) == 0)
+        p.hdr->detail = abort_flag * 1000000 + blockIdx.x;
 }
 
 cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cudaStream_t stream) {
     if (p.n_items <= 0) return cudaSuccess;
     const size_t smem = attn_smem_bytes(head_dim);
-    int dev = 0, sms = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    const int grid = p.n_items < sms ? p.n_items : sms;  // persistent: one CTA per SM
-    if (head_dim == 128) {
-        e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    // one cluster per work item; those that run take the rest from the hardware's queue
+    const unsigned grid = 2u * static_cast<unsigned>(p.n_items);
+    auto go = [&](auto kernel) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
-        attn_kernel<128><<<grid, kAttnThreads, smem, stream>>>(p, m.q, m.q_tail_block, m.q_tail_sink, m.k_sink, m.v_sink, m.k, m.v);
-    } else {
-        e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        attn_kernel<64><<<grid, kAttnThreads, smem, stream>>>(p, m.q, m.q_tail_block, m.q_tail_sink, m.k_sink, m.v_sink, m.k, m.v);
-    }
-    return cudaGetLastError();
+        kernel<<<grid, kAttnThreads, smem, stream>>>(p, m.q, m.q_tail_block, m.q_tail_sink, m.k_sink, m.v_sink, m.k, m.v);
+        return cudaGetLastError();
+    };
+    if (p.mode == 0) return head_dim == 128 ? go(attn_kernel<128, 0>) : go(attn_kernel<64, 0>);
+    return head_dim == 128 ? go(attn_kernel<128, 1>) : go(attn_kernel<64, 1>);
 }
 
 }  // namespace pevlm

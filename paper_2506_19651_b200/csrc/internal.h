@@ -10,16 +10,29 @@
 namespace pevlm {
 
 constexpr int kTile = 128;        // query-tile rows (MMA M) and key-tile columns (MMA N max)
-constexpr int kStatusBytes = 256; // first bytes of every workspace: status word + detail + counters
+constexpr int kStatusBytes = 256; // first bytes of every workspace: status word + detail
 constexpr int kNumSms = 148;      // B200; used only to size the key splits of the question attention
 
 // Workspace header (device memory, first kStatusBytes of the workspace).
 struct WorkspaceHeader {
     int32_t status;  // 0 or PEVLM_ETIMEOUT
     int32_t detail;  // which wait expired (kernel-specific code)
-    int32_t work_counter;
-    int32_t pad[61];
+    int32_t pad[62];
 };
+
+// a / b for 0 <= a < 2^31 without a divide: (a * mul) >> (31 + shift), shift = ceil(log2 b), mul = ceil(2^(31 + shift) / b)
+// < 2^32.  Exact: mul exceeds 2^(31 + shift) / b by less than 1, which adds less than a / 2^(31 + shift) < 1 / b.
+struct Divisor {
+    uint32_t mul;
+    uint32_t shift;
+};
+inline Divisor make_divisor(int b) {  // b = 0 (a quantity the launch does not use) gives quotient 0
+    Divisor d{0, 0};
+    if (b <= 0) return d;
+    while ((1ll << d.shift) < b) ++d.shift;
+    d.mul = static_cast<uint32_t>(((1ull << (31 + d.shift)) + static_cast<uint64_t>(b) - 1) / static_cast<uint64_t>(b));
+    return d;
+}
 
 // What one launch of the attention kernel does.  mode 0: prefill rows (sink + blocks, or
 // full causal); mode 1: question rows against the assembled cache, split over keys.
@@ -47,7 +60,8 @@ struct AttnParams {
     int32_t q_tiles;        // mode 1: ceil(Q / tok_per_tile)
     int32_t n_splits;       // mode 1
     int32_t tiles_per_split;// mode 1
-    uint64_t wait_limit_ns; // longest a single device-side wait may last before the launch reports PEVLM_ETIMEOUT
+    Divisor div_per_chunk, div_pair_chunk, div_hkv, div_pairs_sink, div_g, div_splits, div_q_pairs;  // decode_item
+    uint32_t wait_limit_ns; // longest a single device-side wait may last before the launch reports PEVLM_ETIMEOUT
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
     __nv_bfloat16* o;       // mode 0: [n_video, Hq, d]
@@ -99,7 +113,7 @@ struct AttnMaps {
     CUtensorMap q, q_tail_block, q_tail_sink, k_sink, v_sink, k, v;
 };
 cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cudaStream_t stream);
-cudaError_t launch_wait_selftest(WorkspaceHeader* hdr, uint64_t limit_ns, cudaStream_t stream);
+cudaError_t launch_wait_selftest(WorkspaceHeader* hdr, uint32_t limit_ns, cudaStream_t stream);
 // device address of the built-in scratch array of pevlm_query_attn_noalloc on the current device
 int noalloc_scratch_for_current_device(void** out);
 int check_query_args(const pevlm_shape_t* s, const void* q_question, const void* k_cache, const void* v_cache,

@@ -11,9 +11,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ uint64_t globaltimer_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+// low word of the nanosecond clock: differences up to 4 s
+__device__ __forceinline__ uint32_t globaltimer_lo() {
+    uint32_t t;
+    asm volatile("mov.u32 %0, %globaltimer_lo;" : "=r"(t));
     return t;
 }
 
@@ -30,9 +31,6 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t byt
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
@@ -45,29 +43,96 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
+// Whether the phase is complete, without waiting: issued early, used when the answer has arrived.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+constexpr uint32_t kDefaultWaitLimitNs = 400u * 1000 * 1000;  // 0.4 s
+constexpr uint32_t kAbortGraceNs = 20u * 1000;
+
 // Bounded wait.  `abort_flag` lives in shared memory: once any thread of the CTA has given
 // up on a wait, every later wait in the CTA gives up after a short grace period, so the
 // kernel always runs to its normal end (control flow is never altered by a timeout).
 // `limit_ns` is the longest a single wait may last (a launch parameter: the library's calls pass
-// kDefaultWaitLimitNs, orders of magnitude above any legitimate wait).  Returns false if the wait expired.
-constexpr uint64_t kDefaultWaitLimitNs = 400ull * 1000 * 1000;  // 0.4 s
-constexpr uint64_t kAbortGraceNs = 20ull * 1000;
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint64_t limit_ns) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    uint32_t spins = 0;
+// kDefaultWaitLimitNs, orders of magnitude above any legitimate wait).  The first expiry leaves `which` in the flag.
+// SLEEP_NS > 0 is for waits that are long and not on the critical path: the warp sleeps between its looks, so that it
+// takes no issue slots from the others of its scheduler.
+// Kept short, because it is inlined at two dozen places of the attention kernel, and what that runs per work item has to
+// fit the instruction cache (see there).
+template <unsigned SLEEP_NS = 0>
+__device__ __forceinline__ void mbar_wait_slow(uint32_t bar, uint32_t parity, uint32_t abort_flag, uint32_t limit_ns, int which) {
+    const uint32_t t0 = globaltimer_lo();
     while (true) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((++spins & 63u) == 0) {
-            const uint64_t dt = globaltimer_ns() - t0;
-            const uint64_t lim = (*abort_flag) ? kAbortGraceNs : limit_ns;
-            if (dt > lim) {
-                *abort_flag = 1;
-                return false;
+        if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
+        if (mbar_try_wait(bar, parity)) return;
+        const uint32_t waited = globaltimer_lo() - t0;
+        if (waited > kAbortGraceNs) {
+            int gave_up;
+            asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(gave_up) : "r"(abort_flag) : "memory");
+            if (gave_up != 0 || waited > limit_ns) {
+                if (gave_up == 0) asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(abort_flag), "r"(which) : "memory");
+                return;
             }
         }
     }
+}
+template <unsigned SLEEP_NS = 0>
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_flag, uint32_t limit_ns, int which) {
+    if (!__builtin_expect(mbar_try_wait(bar, parity), 1)) mbar_wait_slow<SLEEP_NS>(bar, parity, abort_flag, limit_ns, which);
+}
+
+// ---------------------------------------------------------------- clusters
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// Address of the same shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Arrive on a barrier of any CTA of the cluster (address from map_to_cta).
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+
+// ---------------------------------------------------------------- work queue of the hardware scheduler
+// One thread asks for a cluster of this grid that has not been launched yet; the 16-byte answer and its
+// completion go to the same offsets in every CTA of the cluster.
+__device__ __forceinline__ void clc_try_cancel(uint32_t result_addr, uint32_t bar) {
+    asm volatile(
+        "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.multicast::cluster::all.b128 [%0], [%1];"
+        ::"r"(result_addr), "r"(bar)
+        : "memory");
+}
+// First block index (x) of the cancelled cluster, or -1 if there was none left.
+__device__ __forceinline__ int clc_first_block(uint32_t result_addr) {
+    int x;
+    asm volatile(
+        "{\n\t.reg .b128 h;\n\t.reg .pred p;\n\t.reg .b32 x, y, z, w;\n\t"
+        "ld.shared.b128 h, [%1];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+        "mov.b32 %0, -1;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, y, z, w}, h;\n\t}"
+        : "=r"(x)
+        : "r"(result_addr)
+        : "memory");
+    return x;
 }
 
 // ---------------------------------------------------------------- fences
@@ -85,63 +150,35 @@ __device__ __forceinline__ void tc_fence_after_sync() {
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
 }
-// 3-D tiled load global -> shared, completion counted in bytes on `bar`.  c0 (innermost)
-// times the element size must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const void* tmap, int c0, int c1, int c2, uint32_t bar) {
+// 3-D tiled load global -> shared by a CTA of a pair.  c0 (innermost) times the element size must be a multiple of
+// 16 bytes.  The data goes to this CTA's shared memory, the bytes are counted on a barrier of either CTA of the pair
+// (`bar` is a cluster address).
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap, int c0, int c1, int c2, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
         " [%0], [%1, {%2, %3, %4}], [%5];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
         : "memory");
 }
 
 // ---------------------------------------------------------------- TMEM
-// One full warp allocates `ncols` (power of two >= 32) TMEM columns; the base address is
-// written to shared memory at `dst`.
-__device__ __forceinline__ void tmem_alloc(uint32_t dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+// One full warp of EACH CTA of a pair allocates `ncols` (power of two >= 32) TMEM columns; the base address is
+// written to that CTA's shared memory at `dst`.
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t dst, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-
-// D[tmem] (+)= A[smem] * B[smem]; one thread issues.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
-        : "memory");
-}
-// D[tmem] (+)= A[tmem] * B[smem]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(static_cast<uint32_t>(accumulate))
-        : "memory");
-}
-// All MMAs issued so far by this thread arrive on `bar` once they have completed.
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// Warp-collective forms: every lane calls them, one elected lane issues.
-__device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
+// All MMAs issued so far by this thread arrive, once they have completed, on the barrier at this offset in both CTAs
+// of the pair.  Warp-collective: every lane calls it, one elected lane issues.
+__device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
     asm volatile(
         "{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
-        "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        "@pe tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+        ::"r"(bar), "h"(static_cast<uint16_t>(3))
         : "memory");
-}
-__device__ __forceinline__ void mma_ts_elect(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p, pe;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-        "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(static_cast<uint32_t>(accumulate)));
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
@@ -160,16 +197,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         : "r"(taddr)
         : "memory");
 }
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
-        ::"r"(taddr),
-          "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
-          "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
-          "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
         : "memory");
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
@@ -183,7 +217,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
 }
 
 // ---------------------------------------------------------------- descriptors
-// Instruction descriptor, kind::f16: bf16 x bf16 -> fp32, M = 128, A K-major.
+// Instruction descriptor, kind::f16: bf16 x bf16 -> fp32, A K-major.
 // bits: [4,6) D format (1 = f32); [7,10) A format (1 = bf16); [10,13) B format; bit 15 A major;
 // bit 16 B major (0 = K-major, 1 = MN-major); [17,23) N >> 3; [24,29) M >> 4.
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int m, int n, bool b_mn_major) {
@@ -191,36 +225,29 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int m, int n, bool b_mn_m
            (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
 }
 
-// Shared-memory matrix descriptor (sm_100 version field = 1), 128-byte swizzle.
-// bits: [0,14) start address >> 4; [16,30) leading byte offset >> 4; [32,46) stride byte
-// offset >> 4; [46,48) version = 1; [61,64) layout (2 = 128-byte swizzle).
-__device__ __forceinline__ uint64_t make_smem_desc_sw128(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFFu) << 16;
-    d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFFu) << 32;
-    d |= 1ull << 46;
-    d |= 2ull << 61;
-    return d;
-}
+// Shared-memory matrix descriptors (64 bits, sm_100 version field = 1): [0,14) start address >> 4; [16,30) leading byte
+// offset >> 4; [32,46) stride byte offset >> 4; [46,48) version = 1; [61,64) layout (2 = 128-byte, 4 = 64-byte swizzle).
 
 // ---- batched MMA issue.  The issuing thread is latency-bound on its own instruction stream,
 // so a whole k-loop goes out as one asm block: descriptors are a constant high word plus a
 // low word (address >> 4 | leading byte offset >> 4 << 16) that only needs an add per step.
+// All MMAs are those of a CTA pair (cta_group::2, M = 256): each CTA holds its 128 rows of A and of the
+// accumulator and half of B's N columns, at the same shared-memory and TMEM addresses.
 constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);  // SBO 1024 B, version 1, 128-byte swizzle
+constexpr uint32_t kDescHiSw64 = (512u >> 4) | (1u << 14) | (4u << 29);    // SBO 512 B, version 1, 64-byte swizzle
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
     return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16);
 }
 
 // These are called by ALL lanes of the issuing warp with warp-uniform operands (so the
 // operands live in uniform registers); one elected lane issues.
-#define PEVLM_MMA_SS_STEP(OFF, PRED)                                              \
-    "add.u32 ta, %1, " #OFF ";\n\tadd.u32 tb, %2, " #OFF ";\n\t"                  \
+#define PEVLM_MMA_SS_STEP(AOFF, BOFF, PRED)                                       \
+    "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                \
     "mov.b64 da, {ta, %3};\n\tmov.b64 db, {tb, %3};\n\t"                          \
-    "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, " PRED ";\n\t"
+    "@pe tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, " PRED ";\n\t"
 
-// D[tmem] = A[smem] * B[smem]^T over head_dim = 16 * KSTEPS; A and B are K-major, 128-byte
-// swizzled tiles whose 64-element column panels are 16 KB apart.  The first step overwrites D.
+// D[tmem] = A[smem] * B[smem]^T over head_dim = 16 * KSTEPS; A (128 rows a CTA) and B (64 rows a CTA) are K-major,
+// 128-byte swizzled tiles in panels of 64 elements (16 KB and 8 KB apart).  The first step overwrites D.
 template <int KSTEPS>
 __device__ __forceinline__ void mma_ss_batch(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
     static_assert(KSTEPS == 4 || KSTEPS == 8, "head_dim 64 or 128");
@@ -228,15 +255,16 @@ __device__ __forceinline__ void mma_ss_batch(uint32_t d_tmem, uint32_t a_lo, uin
         asm volatile(
             "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 da, db;\n\t"
             "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-            PEVLM_MMA_SS_STEP(0, "p0") PEVLM_MMA_SS_STEP(2, "p1") PEVLM_MMA_SS_STEP(4, "p1") PEVLM_MMA_SS_STEP(6, "p1")
-            PEVLM_MMA_SS_STEP(1024, "p1") PEVLM_MMA_SS_STEP(1026, "p1") PEVLM_MMA_SS_STEP(1028, "p1") PEVLM_MMA_SS_STEP(1030, "p1")
+            PEVLM_MMA_SS_STEP(0, 0, "p0") PEVLM_MMA_SS_STEP(2, 2, "p1") PEVLM_MMA_SS_STEP(4, 4, "p1") PEVLM_MMA_SS_STEP(6, 6, "p1")
+            PEVLM_MMA_SS_STEP(1024, 512, "p1") PEVLM_MMA_SS_STEP(1026, 514, "p1") PEVLM_MMA_SS_STEP(1028, 516, "p1")
+            PEVLM_MMA_SS_STEP(1030, 518, "p1")
             "}"
             ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc));
     } else {
         asm volatile(
             "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 da, db;\n\t"
             "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-            PEVLM_MMA_SS_STEP(0, "p0") PEVLM_MMA_SS_STEP(2, "p1") PEVLM_MMA_SS_STEP(4, "p1") PEVLM_MMA_SS_STEP(6, "p1")
+            PEVLM_MMA_SS_STEP(0, 0, "p0") PEVLM_MMA_SS_STEP(2, 2, "p1") PEVLM_MMA_SS_STEP(4, 4, "p1") PEVLM_MMA_SS_STEP(6, 6, "p1")
             "}"
             ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc));
     }
@@ -245,44 +273,49 @@ __device__ __forceinline__ void mma_ss_batch(uint32_t d_tmem, uint32_t a_lo, uin
 #define PEVLM_MMA_TS_STEP(AOFF, BOFF, PRED)                                       \
     "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                \
     "mov.b64 db, {tb, %3};\n\t"                                                   \
-    "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], [ta], db, %4, " PRED ";\n\t"
+    "@pe tcgen05.mma.cta_group::2.kind::f16 [%0], [ta], db, %4, " PRED ";\n\t"
 
-// D[tmem] (+)= A[tmem] * B[smem] over 64 keys (four steps of 16): A = bf16 probabilities, 8
-// TMEM columns per step; B = V rows (MN-major, 16 keys = 2048 bytes per step).  The first step
-// accumulates iff accumulate_first != 0.
-__device__ __forceinline__ void mma_ts_batch4(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
-                                              uint32_t accumulate_first) {
-    asm volatile(
-        "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-        PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 128, "p1") PEVLM_MMA_TS_STEP(16, 256, "p1")
-        PEVLM_MMA_TS_STEP(24, 384, "p1")
-        "}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc), "r"(accumulate_first));
-}
+// B = V rows, MN-major: a CTA holds D/2 columns of all keys of the tile, 128-byte rows (D = 128) or 64-byte rows
+// (D = 64), so 16 keys are 2048 or 1024 bytes.
+template <int D>
+constexpr uint32_t kVDescHi = D == 128 ? kDescHiSw128 : kDescHiSw64;
+template <int D>
+constexpr uint32_t kVDescStep = D == 128 ? 128 : 64;
 
-// Same over 32 keys (two steps).
-__device__ __forceinline__ void mma_ts_batch2(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
-                                              uint32_t accumulate_first) {
-    asm volatile(
-        "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-        PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 128, "p1")
-        "}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc), "r"(accumulate_first));
-}
-
-// Same over 128 keys (eight steps).
+// D[tmem] (+)= A[tmem] * B[smem] over 128 keys (eight steps of 16): A = bf16 probabilities, 8
+// TMEM columns per step.  The first step accumulates iff accumulate_first != 0.
+template <int D>
 __device__ __forceinline__ void mma_ts_batch8(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
                                               uint32_t accumulate_first) {
+    if constexpr (D == 128) {
+        asm volatile(
+            "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
+            "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
+            PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 128, "p1") PEVLM_MMA_TS_STEP(16, 256, "p1")
+            PEVLM_MMA_TS_STEP(24, 384, "p1") PEVLM_MMA_TS_STEP(32, 512, "p1") PEVLM_MMA_TS_STEP(40, 640, "p1")
+            PEVLM_MMA_TS_STEP(48, 768, "p1") PEVLM_MMA_TS_STEP(56, 896, "p1")
+            "}"
+            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kVDescHi<D>), "r"(idesc), "r"(accumulate_first));
+    } else {
+        asm volatile(
+            "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
+            "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
+            PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 64, "p1") PEVLM_MMA_TS_STEP(16, 128, "p1")
+            PEVLM_MMA_TS_STEP(24, 192, "p1") PEVLM_MMA_TS_STEP(32, 256, "p1") PEVLM_MMA_TS_STEP(40, 320, "p1")
+            PEVLM_MMA_TS_STEP(48, 384, "p1") PEVLM_MMA_TS_STEP(56, 448, "p1")
+            "}"
+            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kVDescHi<D>), "r"(idesc), "r"(accumulate_first));
+    }
+}
+
+// One step of 16 keys (ragged key tiles).
+template <int D>
+__device__ __forceinline__ void mma_ts_step(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-        "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-        PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 128, "p1") PEVLM_MMA_TS_STEP(16, 256, "p1")
-        PEVLM_MMA_TS_STEP(24, 384, "p1") PEVLM_MMA_TS_STEP(32, 512, "p1") PEVLM_MMA_TS_STEP(40, 640, "p1")
-        PEVLM_MMA_TS_STEP(48, 768, "p1") PEVLM_MMA_TS_STEP(56, 896, "p1")
-        "}"
-        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc), "r"(accumulate_first));
+        "{\n\t.reg .pred p, pe;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\telect.sync _|pe, 0xffffffff;\n\tmov.b64 db, {%2, %3};\n\t"
+        "@pe tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kVDescHi<D>), "r"(idesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
