@@ -218,7 +218,11 @@ static int rope_common(const pevlm_shape_t* s, const void* q_in, const void* k_i
     p.n_tokens = n_tokens;
     p.Hq = q_in ? s->num_q_heads : 0;
     p.Hkv = k_in ? s->num_kv_heads : 0;
-    p.head_split = 1;
+    p.split_token = n_tokens;
+    p.q_out2 = nullptr;
+    p.v_in = nullptr;
+    p.v_out = nullptr;
+    p.Hv = 0;
     p.sec_end0 = sections ? sections[0] : 0;
     p.sec_end1 = sections ? sections[0] + sections[1] : 0;
     for (int b = 0; b < s->batch; ++b) {

@@ -108,11 +108,6 @@ extern "C" int pevlm_debug_waits(unsigned* host_out) {
 
 __device__ __forceinline__ int cdiv(int a, int b) { return (a + b - 1) / b; }
 
-// a / b for 0 <= a < 2^31 by the multiplier and shift that the host worked out for b
-__device__ __forceinline__ int quotient(int a, const Divisor& b) {
-    return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(a)) * b.mul) >> 31 >> b.shift);
-}
-
 template <int MODE>
 __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem& it) {
     it.split = 0;

@@ -34,6 +34,39 @@ inline Divisor make_divisor(int b) {  // b = 0 (a quantity the launch does not u
     return d;
 }
 
+#ifdef __CUDACC__
+__device__ __forceinline__ int quotient(int a, const Divisor& b) {
+    return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(a)) * b.mul) >> 31 >> b.shift);
+}
+#endif
+
+// Launch of one of the library's kernels behind another.  The kernel may be brought onto the GPU while the one before it
+// in the stream still runs, so that its launch costs nothing; every kernel therefore calls grid_wait() before it touches
+// global memory.  All kernels ask for the same split of the SM's memory (as much shared memory as there is), because an
+// SM has to run empty before it can change the split.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+                                  const Args&... args) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    if (smem > 48 * 1024) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute chained;
+    chained.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    chained.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t config{};
+    config.gridDim = dim3(grid);
+    config.blockDim = dim3(threads);
+    config.dynamicSmemBytes = smem;
+    config.stream = stream;
+    config.attrs = &chained;
+    config.numAttrs = 1;
+    e = cudaLaunchKernelEx(&config, kernel, args...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // What one launch of the attention kernel does.  mode 0: prefill rows (sink + blocks, or
 // full causal); mode 1: question rows against the assembled cache, split over keys.
 struct AttnParams {
@@ -89,7 +122,14 @@ struct RopeParams {
     int64_t first_token;
     int64_t n_tokens;
     int32_t Hq, Hkv;  // heads to process of each tensor (0 = skip tensor)
-    int32_t head_split;  // slots sharing one token's heads (set by launch_rope)
+    // q rows of tokens from split_token on go to the same place counted from q_out2
+    __nv_bfloat16* q_out2;
+    int64_t split_token;
+    const __nv_bfloat16* v_in;  // rows copied along: Hv heads of v_in to v_out (0 = none)
+    __nv_bfloat16* v_out;
+    int32_t Hv;
+    int32_t group;  // tokens per CTA (this and the divisors are set by launch_rope)
+    Divisor div_hq, div_hkv;
     // multimodal RoPE: pos3 != NULL selects it; rotary pair i takes its position from component 0 for
     // i < sec_end0, component 1 for i < sec_end1, else component 2; pos3 is [3, n_tokens]
     const int32_t* pos3;

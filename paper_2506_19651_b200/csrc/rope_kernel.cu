@@ -1,20 +1,36 @@
 // RoPE at global positions (Sec. 3.2.2): every token keeps its original sequential position.
-// HBM-bound elementwise kernel; angle, sine/cosine and rotation in fp64, one rounding
-// fp64 -> fp32 -> bf16 (round to nearest even).  No fused multiply-add in the rotation, so
-// every fp64 operation rounds exactly once.
+// HBM-bound elementwise kernel.  The result is that of the fp64 definition: angle, sine/cosine and rotation in fp64 (no
+// fused multiply-add in the rotation, so every fp64 operation rounds exactly once), then one rounding fp64 -> fp32 ->
+// bf16 (round to nearest even).
+//
+// The CTAs share the tokens out in groups of up to 8 neighbours.  A CTA evaluates a group's angles once (fp64 sincos)
+// into shared memory, one group ahead, and its threads walk over the group's head vectors of Q and K: d/16 threads a
+// vector, 16 bytes of either half each; the vectors of a group are one contiguous range per tensor.  What bounds it: DRAM
+// traffic.  Two things used to stand in the way (numbers for B200, 28/4 heads of 128):
+//   - the fp64 <-> fp32 conversion unit (16 values per clock and SM, 70 % busy at 50K tokens).  The rotation therefore
+//     runs in fp32, with the sine and cosine rounded to fp32, and takes its result only where it cannot differ: with
+//     |cos|, |sin| <= 1 and fp32 rounding (2^-24 relative, half an ulp) of the cosine, the sine, the product b s and the
+//     sum, the error of a c - b s is below 3 * 2^-25 (|a| + |b|) * 1.01 < E = 2^-23 (|a| + |b|), and the rounding to
+//     fp32 and to bf16 is monotone, so if r - E and r + E round to the same bf16, the fp64 value does too.  The remaining
+//     quarter of E covers the rounding of r -+ E itself.  Where they differ (about one head vector of a warp in
+//     sixteen) the thread repeats its eight pairs in fp64;
+//   - the bytes in flight, above all in ranges that do not fill the GPU many times over (12.5K tokens took 73 us where
+//     50K took 148).  The loads go through a ring in shared memory, kRopeRing vectors ahead, over the ends of groups
+//     too, which costs no registers.  A thread reads only what it has fetched itself, so the ring needs no barrier.
+// The V rows of the same tokens can be copied along (V needs no rotation): a third range of vectors.
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace pevlm {
 
 constexpr int kRopeThreads = 256;
-
-constexpr int kRopeCtasPerSm = 4;  // resident CTAs per SM of the long-range form (its register budget: 64)
+constexpr int kRopeCtasPerSm = 3;
+constexpr int kRopeTokens = 8;   // most tokens of a group
+constexpr int kRopeRing = 6;     // vectors a thread has in flight
 
 // 16-byte accesses that do not allocate in L1 (every byte is touched once)
-__device__ __forceinline__ uint4 ld_stream(const __nv_bfloat16* p) {
-    uint4 v;
-    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-    return v;
+__device__ __forceinline__ void fetch16(uint32_t dst, const __nv_bfloat16* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void st_stream(__nv_bfloat16* p, const uint4& v) {
     asm volatile("st.global.L1::no_allocate.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
@@ -24,177 +40,166 @@ __device__ __forceinline__ void st_stream(__nv_bfloat16* p, const uint4& v) {
 __device__ __forceinline__ double bf16_bits_to_f64(uint32_t bits16) {
     return static_cast<double>(__uint_as_float(bits16 << 16));
 }
-// fp64 -> fp32 (round to nearest even) -> bf16 (round to nearest even): two roundings, in this order;
-// the second one is done for two values at once by the packed conversion
-__device__ __forceinline__ uint32_t f64x2_to_bf16x2_bits(double lo, double hi) {
-    const float flo = __double2float_rn(lo), fhi = __double2float_rn(hi);
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(fhi), "f"(flo));
-    return r;
+
+// Two rotation pairs (a0, b0), (a1, b1), packed as bf16 words: outputs of both halves, and whether any of the four could
+// round differently from the exact value.  cs = (cos0, cos1, sin0, sin1).
+__device__ __forceinline__ uint32_t rotate2(uint32_t a, uint32_t b, const float4& cs, uint32_t& out_a, uint32_t& out_b) {
+    const float a0 = __uint_as_float(a << 16), a1 = __uint_as_float(a & 0xffff0000u);
+    const float b0 = __uint_as_float(b << 16), b1 = __uint_as_float(b & 0xffff0000u);
+    const uint64_t A = pack_f32x2(a0, a1), B = pack_f32x2(b0, b1);
+    const uint64_t C = pack_f32x2(cs.x, cs.y), S = pack_f32x2(cs.z, cs.w), nS = pack_f32x2(-cs.z, -cs.w);
+    const uint64_t ra = fma_f32x2(A, C, mul_f32x2(B, nS)), rb = fma_f32x2(B, C, mul_f32x2(A, S));
+    const uint64_t m = pack_f32x2(fabsf(a0) + fabsf(b0), fabsf(a1) + fabsf(b1));
+    const float e = 1.0f / 8388608.0f;  // 2^-23
+    const uint64_t up = pack_f32x2(e, e), down = pack_f32x2(-e, -e);
+    float x0, x1, y0, y1;
+    unpack_f32x2(fma_f32x2(m, up, ra), x0, x1);
+    unpack_f32x2(fma_f32x2(m, down, ra), y0, y1);
+    out_a = pack_bf16x2(x0, x1);
+    const uint32_t other_a = pack_bf16x2(y0, y1);
+    unpack_f32x2(fma_f32x2(m, up, rb), x0, x1);
+    unpack_f32x2(fma_f32x2(m, down, rb), y0, y1);
+    out_b = pack_bf16x2(x0, x1);
+    return (out_a ^ other_a) | (out_b ^ pack_bf16x2(y0, y1));
 }
 
-// A SLOT is a group of d/16 threads that handles one token: a thread owns 8 rotation pairs (elements i0..i0+7
-// and i0+d/2..i0+d/2+7), evaluates their 8 angles once in fp64 (sincos) and then walks over the token's
-// Hq + Hkv head vectors, two 16-byte loads and two 16-byte stores per head; the d/16 threads of a slot read 128
-// contiguous bytes per half head vector, the 16 slots of a CTA take 16 neighbouring tokens (a contiguous 256 KB
-// at 28/4 heads of 128: slots that each streamed a region of their own ran 25 % slower), and CTAs stride over
-// these groups.  The kernel is bound by the bytes it keeps in flight (resident warps x outstanding loads) and
-// registers bound the resident warps, so the (cos, sin) pairs sit in a thread-private column of shared memory
-// rather than in 32 registers (4 resident CTAs per SM instead of 3) and the loads of the next two heads are
-// issued before a head is rotated (template flag LONG).  Short ranges (the question block, a streamed block)
-// take the other form, which keeps the pairs in registers, uses no shared memory and fetches one head at a time:
-// a launch that uses shared memory made the attention launch that follows two launches later start about 9 us
-// later (the SMs change their shared-memory configuration), which a short range cannot pay back.
-// No block-level synchronisation.  The heads of a token can be split over
-// `head_split` slots, each evaluating the token's angles itself, for short token ranges (the question block),
-// so that the launch still fills the machine.
-// MODE 0: one position per token.  MODE 1, 2: the multimodal form, where a rotary pair's section picks the
-// position component; 1 when the section boundaries are multiples of 8 pairs (16/24/24 at d = 128), so that a
-// thread's 8 pairs share one component, 2 in general (a component per pair).
-template <int D, int MODE, bool LONG>
-__global__ void __launch_bounds__(kRopeThreads, LONG ? kRopeCtasPerSm : 1) rope_kernel(const __grid_constant__ RopeParams p) {
-    constexpr int kPrefetch = LONG ? 2 : 0;  // heads whose loads are in flight while one head is rotated
+template <int D>
+struct RopeSmem {
+    static constexpr int kHalf = D / 2;
+    // per token: [pair / 2 of the thread][thread of the vector], so that the threads of a vector read 16 contiguous bytes each
+    float4 cs32[2][kRopeTokens * kHalf / 2];   // (cos0, cos1, sin0, sin1) of two pairs
+    double2 cs64[2][kRopeTokens * kHalf];      // (cos, sin), [pair of the thread][thread of the vector]
+    uint4 ring[kRopeRing][2][kRopeThreads];    // [half of the vector][thread]
+};
+
+template <int D>
+__global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(const __grid_constant__ RopeParams p) {
     constexpr int HALF = D / 2;
-    constexpr int TPT = HALF / 8;                  // threads per slot
-    constexpr int SLOTS_PER_CTA = kRopeThreads / TPT;
-    // [pair of the thread][thread]: conflict-free 16-byte accesses (one dummy element in the short form)
-    __shared__ double2 cs_sn[LONG ? 8 : 1][LONG ? kRopeThreads : 1];
-    double cs[LONG ? 1 : 8], sn[LONG ? 1 : 8];
-    const int v = threadIdx.x % TPT;
+    constexpr int TPV = HALF / 8;                // threads per head vector: 8 rotation pairs each
+    constexpr int SLOTS = kRopeThreads / TPV;    // vectors the CTA has in hand at a time
+    extern __shared__ __align__(16) uint8_t raw[];
+    RopeSmem<D>& sm = *reinterpret_cast<RopeSmem<D>*>(raw);
+    const int v = threadIdx.x % TPV, slot = threadIdx.x / TPV;
     const int i0 = v * 8;
-    const int heads = p.Hq + p.Hkv;
-    const int64_t n_slots = p.n_tokens * p.head_split;
-    const int64_t n_groups = (n_slots + SLOTS_PER_CTA - 1) / SLOTS_PER_CTA;
-    for (int64_t grp = blockIdx.x; grp < n_groups; grp += gridDim.x) {
-        const int64_t slot = grp * SLOTS_PER_CTA + threadIdx.x / TPT;
-        if (slot >= n_slots) continue;
-        const int64_t tok = slot / p.head_split;
-        // this slot's share of the token's heads: a contiguous range
-        const int part = static_cast<int>(slot % p.head_split);
-        const int h_first = part * heads / p.head_split, h_end = (part + 1) * heads / p.head_split;
-        int64_t pos = 0;
-        if (MODE == 0) pos = p.pos_ids ? static_cast<int64_t>(p.pos_ids[tok]) : p.first_token + tok;
-        if (MODE == 1) {
-            const int comp = i0 < p.sec_end0 ? 0 : i0 < p.sec_end1 ? 1 : 2;
-            pos = static_cast<int64_t>(p.pos3[comp * p.n_tokens + tok]);
+    const int heads = p.Hq + p.Hkv + p.Hv;
+
+    // groups of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ... of p.group tokens each
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * p.group;
+    auto size_of = [&](int64_t tok0) { return static_cast<int>(p.n_tokens - tok0 < p.group ? p.n_tokens - tok0 : p.group); };
+    auto angles = [&](int64_t tok0, int buf) {
+        if (tok0 >= p.n_tokens) return;
+        for (int a = threadIdx.x; a < size_of(tok0) * HALF; a += kRopeThreads) {
+            const int t = a / HALF, i = a % HALF;
+            const int64_t tok = tok0 + t;
+            // one position per token, or, multimodal, the component that the rotary pair's section picks
+            const int64_t pos = p.pos3 ? p.pos3[(i < p.sec_end0 ? 0 : i < p.sec_end1 ? 1 : 2) * p.n_tokens + tok]
+                              : p.pos_ids ? p.pos_ids[tok]
+                                          : p.first_token + tok;
+            double sn, cn;
+            sincos(__dmul_rn(static_cast<double>(pos), p.inv_freq[i]), &sn, &cn);
+            const int e = i % 8, w = i / 8;
+            sm.cs64[buf][t * HALF + e * TPV + w] = make_double2(cn, sn);
+            float* f = reinterpret_cast<float*>(&sm.cs32[buf][t * (HALF / 2) + (e / 2) * TPV + w]);
+            f[e % 2] = __double2float_rn(cn);
+            f[2 + e % 2] = __double2float_rn(sn);
         }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            int64_t pe = pos;
-            if (MODE == 2) {  // multimodal: the pair's section picks the temporal, height or width position
-                const int i = i0 + e;
-                const int comp = i < p.sec_end0 ? 0 : i < p.sec_end1 ? 1 : 2;
-                pe = static_cast<int64_t>(p.pos3[comp * p.n_tokens + tok]);
+    };
+    // fetch cursor: kRopeRing vectors ahead of the one that is rotated
+    int64_t f_tok0 = static_cast<int64_t>(blockIdx.x) * p.group;
+    int f_u = slot, f_total = f_tok0 < p.n_tokens ? size_of(f_tok0) * heads : 0, f_ring = 0;
+    auto fetch = [&]() {
+        if (f_tok0 < p.n_tokens) {
+            if (f_u < f_total) {
+                const int nt = size_of(f_tok0), nq = nt * p.Hq, nqk = nq + nt * p.Hkv;
+                const __nv_bfloat16* src = f_u < nq ? p.q_in + (f_tok0 * p.Hq + f_u) * D
+                                         : f_u < nqk ? p.k_in + (f_tok0 * p.Hkv + (f_u - nq)) * D
+                                                     : p.v_in + (f_tok0 * p.Hv + (f_u - nqk)) * D;
+                fetch16(smem_u32(&sm.ring[f_ring][0][threadIdx.x]), src + i0);
+                fetch16(smem_u32(&sm.ring[f_ring][1][threadIdx.x]), src + i0 + HALF);
             }
-            const double ang = __dmul_rn(static_cast<double>(pe), p.inv_freq[i0 + e]);
-            double sv, cv;
-            sincos(ang, &sv, &cv);
-            if (LONG) {
-                cs_sn[e][threadIdx.x] = make_double2(cv, sv);
-            } else {
-                cs[e] = cv;
-                sn[e] = sv;
+            f_u += SLOTS;
+            if (f_u - slot >= f_total) {  // the same for all threads: every thread takes the same number of steps
+                f_tok0 += stride;
+                f_u = slot;
+                f_total = f_tok0 < p.n_tokens ? size_of(f_tok0) * heads : 0;
             }
         }
-        auto addr_of = [&](int h, const __nv_bfloat16*& src, __nv_bfloat16*& dst) {
-            if (h < p.Hq) {
-                const int64_t off = (tok * p.Hq + h) * D;
-                src = p.q_in + off;
-                dst = p.q_out + off;
-            } else {
-                const int64_t off = (tok * p.Hkv + (h - p.Hq)) * D;
-                src = p.k_in + off;
-                dst = p.k_out + off;
-            }
-        };
-        uint4 lo_q[kPrefetch + 1], hi_q[kPrefetch + 1];
-#pragma unroll
-        for (int n = 0; n < kPrefetch; ++n) {
-            const int h = h_first + n;
-            if (h < h_end) {
-                const __nv_bfloat16* src;
+        f_ring = f_ring + 1 == kRopeRing ? 0 : f_ring + 1;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    grid_wait();
+    grid_launch_dependents();
+#pragma unroll 1
+    for (int i = 0; i < kRopeRing - 1; ++i) fetch();
+    int buf = 0, ring = 0;
+    angles(static_cast<int64_t>(blockIdx.x) * p.group, 0);
+    for (int64_t tok0 = static_cast<int64_t>(blockIdx.x) * p.group; tok0 < p.n_tokens; tok0 += stride, buf ^= 1) {
+        __syncthreads();  // this group's angles are there, and nobody reads the previous group's any more
+        angles(tok0 + stride, buf ^ 1);
+        const int nt = size_of(tok0), nq = nt * p.Hq, nqk = nq + nt * p.Hkv, total = nt * heads;
+#pragma unroll 1
+        for (int base = 0; base < total; base += SLOTS) {
+            fetch();
+            asm volatile("cp.async.wait_group %0;" ::"n"(kRopeRing - 1) : "memory");
+            const int u = base + slot;
+            if (u < total) {
+                const uint4 lo = sm.ring[ring][0][threadIdx.x], hi = sm.ring[ring][1][threadIdx.x];
+                uint4 out_lo = lo, out_hi = hi;
                 __nv_bfloat16* dst;
-                addr_of(h, src, dst);
-                lo_q[n] = ld_stream(src + i0);
-                hi_q[n] = ld_stream(src + i0 + HALF);
-            }
-        }
-        for (int h = h_first; h < h_end; ++h) {
-            const __nv_bfloat16* src;
-            __nv_bfloat16* dst;
-            if (h + kPrefetch < h_end) {
-                addr_of(h + kPrefetch, src, dst);
-                lo_q[kPrefetch] = ld_stream(src + i0);
-                hi_q[kPrefetch] = ld_stream(src + i0 + HALF);
-            }
-            addr_of(h, src, dst);
-            const uint4 lo = lo_q[0], hi = hi_q[0];
+                if (u < nqk) {
+                    const bool is_q = u < nq;
+                    const int t = is_q ? quotient(u, p.div_hq) : quotient(u - nq, p.div_hkv);
+                    if (is_q) dst = (tok0 + t < p.split_token ? p.q_out : p.q_out2) + (tok0 * p.Hq + u) * D;
+                    else dst = p.k_out + (tok0 * p.Hkv + (u - nq)) * D;
+                    const uint32_t lw[4] = {lo.x, lo.y, lo.z, lo.w}, hw[4] = {hi.x, hi.y, hi.z, hi.w};
+                    uint32_t ol[4], oh[4], unsure = 0;
 #pragma unroll
-            for (int n = 0; n < kPrefetch; ++n) {
-                lo_q[n] = lo_q[n + 1];
-                hi_q[n] = hi_q[n + 1];
-            }
-            const uint32_t lo_w[4] = {lo.x, lo.y, lo.z, lo.w};
-            const uint32_t hi_w[4] = {hi.x, hi.y, hi.z, hi.w};
-            uint32_t out_lo[4], out_hi[4];
+                    for (int w = 0; w < 4; ++w)
+                        unsure |= rotate2(lw[w], hw[w], sm.cs32[buf][t * (HALF / 2) + w * TPV + v], ol[w], oh[w]);
+                    if (__builtin_expect(unsure != 0, 0)) {
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                double ra[2], rb[2];
+                        for (int w = 0; w < 4; ++w) {
+                            float ra[2], rb[2];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const double a = bf16_bits_to_f64((lo_w[w] >> (16 * e)) & 0xFFFFu);
-                    const double b = bf16_bits_to_f64((hi_w[w] >> (16 * e)) & 0xFFFFu);
-                    double c, s;
-                    if (LONG) {
-                        const double2 t = cs_sn[2 * w + e][threadIdx.x];
-                        c = t.x;
-                        s = t.y;
-                    } else {
-                        c = cs[2 * w + e];
-                        s = sn[2 * w + e];
+                            for (int e = 0; e < 2; ++e) {
+                                const double a = bf16_bits_to_f64((lw[w] >> (16 * e)) & 0xFFFFu);
+                                const double b = bf16_bits_to_f64((hw[w] >> (16 * e)) & 0xFFFFu);
+                                const double2 cs = sm.cs64[buf][t * HALF + (2 * w + e) * TPV + v];
+                                ra[e] = __double2float_rn(__dsub_rn(__dmul_rn(a, cs.x), __dmul_rn(b, cs.y)));
+                                rb[e] = __double2float_rn(__dadd_rn(__dmul_rn(b, cs.x), __dmul_rn(a, cs.y)));
+                            }
+                            ol[w] = pack_bf16x2(ra[0], ra[1]);
+                            oh[w] = pack_bf16x2(rb[0], rb[1]);
+                        }
                     }
-                    ra[e] = __dsub_rn(__dmul_rn(a, c), __dmul_rn(b, s));
-                    rb[e] = __dadd_rn(__dmul_rn(b, c), __dmul_rn(a, s));
+                    out_lo = make_uint4(ol[0], ol[1], ol[2], ol[3]);
+                    out_hi = make_uint4(oh[0], oh[1], oh[2], oh[3]);
+                } else {
+                    dst = p.v_out + (tok0 * p.Hv + (u - nqk)) * D;
                 }
-                out_lo[w] = f64x2_to_bf16x2_bits(ra[0], ra[1]);
-                out_hi[w] = f64x2_to_bf16x2_bits(rb[0], rb[1]);
+                st_stream(dst + i0, out_lo);
+                st_stream(dst + i0 + HALF, out_hi);
             }
-            st_stream(dst + i0, make_uint4(out_lo[0], out_lo[1], out_lo[2], out_lo[3]));
-            st_stream(dst + i0 + HALF, make_uint4(out_hi[0], out_hi[1], out_hi[2], out_hi[3]));
+            ring = ring + 1 == kRopeRing ? 0 : ring + 1;
         }
     }
 }
 
-cudaError_t launch_rope(const RopeParams& p, int head_dim, cudaStream_t stream) {
-    if (p.n_tokens <= 0 || p.Hq + p.Hkv == 0) return cudaSuccess;
-    const int slots_per_cta = kRopeThreads / (head_dim / 16);
-    const int64_t resident = static_cast<int64_t>(kNumSms) * kRopeCtasPerSm;  // CTAs the GPU holds at once
-    RopeParams q = p;
-    // short ranges: split a token's heads until the launch has about two CTAs per SM
-    q.head_split = 1;
-    while (q.head_split < 32 && q.head_split * 2 <= p.Hq + p.Hkv && p.n_tokens * q.head_split < 2 * kNumSms * slots_per_cta)
-        q.head_split *= 2;
-    const int64_t groups = (p.n_tokens * q.head_split + slots_per_cta - 1) / slots_per_cta;
-    const int64_t cap = 2 * resident;  // CTAs stride over the remaining groups
-    const unsigned grid = static_cast<unsigned>(groups < cap ? groups : cap);
-    const int mode = !q.pos3 ? 0 : ((q.sec_end0 | q.sec_end1) & 7) == 0 ? 1 : 2;
-    const bool long_range = q.head_split == 1 && groups >= resident;  // at least one full round of resident CTAs
-#define PEVLM_ROPE_LAUNCH(D_, M_)                                                                   \
-    do {                                                                                            \
-        if (long_range) rope_kernel<D_, M_, true><<<grid, kRopeThreads, 0, stream>>>(q);            \
-        else rope_kernel<D_, M_, false><<<grid, kRopeThreads, 0, stream>>>(q);                      \
-    } while (0)
-    if (head_dim == 128) {
-        if (mode == 0) PEVLM_ROPE_LAUNCH(128, 0);
-        else if (mode == 1) PEVLM_ROPE_LAUNCH(128, 1);
-        else PEVLM_ROPE_LAUNCH(128, 2);
-    } else {
-        if (mode == 0) PEVLM_ROPE_LAUNCH(64, 0);
-        else if (mode == 1) PEVLM_ROPE_LAUNCH(64, 1);
-        else PEVLM_ROPE_LAUNCH(64, 2);
-    }
-#undef PEVLM_ROPE_LAUNCH
-    return cudaGetLastError();
+cudaError_t launch_rope(const RopeParams& params, int head_dim, cudaStream_t stream) {
+    if (params.n_tokens <= 0 || params.Hq + params.Hkv + params.Hv == 0) return cudaSuccess;
+    RopeParams p = params;
+    // Groups as large as leaves every resident CTA four of them (the shares of the CTAs differ by one group), at least
+    // one token.
+    const int64_t resident = static_cast<int64_t>(kNumSms) * kRopeCtasPerSm;
+    p.group = kRopeTokens;
+    while (p.group > 1 && p.n_tokens < 4 * resident * p.group) p.group /= 2;
+    p.div_hq = make_divisor(p.Hq);
+    p.div_hkv = make_divisor(p.Hkv);
+    const int64_t groups = (p.n_tokens + p.group - 1) / p.group;
+    const unsigned grid = static_cast<unsigned>(groups < resident ? groups : resident);
+    return head_dim == 128 ? launch_chained(rope_kernel<128>, grid, kRopeThreads, sizeof(RopeSmem<128>), stream, p)
+                           : launch_chained(rope_kernel<64>, grid, kRopeThreads, sizeof(RopeSmem<64>), stream, p);
 }
 
 }  // namespace pevlm
