@@ -309,9 +309,6 @@ static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, 
     rc = check_device();
     if (rc != PEVLM_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "workspace memset");
-
     const int d = s->head_dim;
     const int64_t q_rows = blocks_only ? block_rows : nv;   // rows of q, o, lse
     const int64_t kv_rows = blocks_only ? cache_rows : nv;  // rows of k, v
@@ -379,7 +376,8 @@ static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, 
         if ((rc = make_tmap(&m.v, vb + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
         p.o = static_cast<__nv_bfloat16*>(o) + qoff;
         p.lse = lse ? lse + static_cast<int64_t>(b) * p.Hq * q_rows : nullptr;
-        e = launch_attn(p, d, m, st);
+        p.clear_status = b == 0;
+        cudaError_t e = launch_attn(p, d, m, st);
         if (e != cudaSuccess) return cuda_fail(e, "prefill attention launch");
     }
     return PEVLM_OK;
@@ -407,9 +405,6 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
     rc = check_device();
     if (rc != PEVLM_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(workspace, 0, kStatusBytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "workspace memset");
-
     const int d = s->head_dim;
     const int64_t nv = n_video(s);
     const int64_t L = nv + s->query_len;
@@ -444,7 +439,8 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
         if ((rc = make_tmap(&maps.k, static_cast<const __nv_bfloat16*>(k_cache) + koff, L, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
         if ((rc = make_tmap(&maps.v, static_cast<const __nv_bfloat16*>(v_cache) + koff, L, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
         maps.q_tail_block = maps.q; maps.q_tail_sink = maps.q; maps.k_sink = maps.k; maps.v_sink = maps.v;
-        e = launch_attn(p, d, maps, st);
+        p.clear_status = b == 0;
+        cudaError_t e = launch_attn(p, d, maps, st);
         if (e != cudaSuccess) return cuda_fail(e, "question attention launch");
         MergeParams m;
         m.Q = p.Q; m.Hq = p.Hq; m.d = d; m.n_splits = p.n_splits;

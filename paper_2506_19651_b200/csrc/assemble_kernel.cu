@@ -2,6 +2,7 @@
 // copy of up to four segments (K video, K question, V video, V question) into the two
 // contiguous caches, one launch.  Pure HBM traffic: reads and writes each byte once.
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace pevlm {
 
@@ -21,6 +22,8 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
 }
 
 __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __grid_constant__ CopySegments s) {
+    grid_wait();
+    grid_launch_dependents();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kCopyThreads * kCopyUnroll;
     for (int64_t base = static_cast<int64_t>(blockIdx.x) * kCopyThreads * kCopyUnroll + threadIdx.x; base < s.total;
          base += stride) {
@@ -55,8 +58,7 @@ cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream) {
     int64_t ctas = (s.total + per_cta - 1) / per_cta;
     const int64_t cap = 148 * 16;  // a few waves of the 148 SMs; the loop strides over the rest
     if (ctas > cap) ctas = cap;
-    copy_segments_kernel<<<static_cast<unsigned>(ctas), kCopyThreads, 0, stream>>>(s);
-    return cudaGetLastError();
+    return launch_chained(copy_segments_kernel, static_cast<unsigned>(ctas), kCopyThreads, 0, stream, s);
 }
 
 }  // namespace pevlm

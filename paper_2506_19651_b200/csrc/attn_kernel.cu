@@ -315,6 +315,14 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
     cluster_sync_all();  // also: the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
+    grid_wait();  // nothing above touches global memory
+    grid_launch_dependents();
+    // The status word of the previous call on this workspace is cleared by the launch's first block, long before any wait
+    // of this launch can have run out.
+    if (p.clear_status && blockIdx.x == 0 && tid == 0) {
+        p.hdr->detail = 0;
+        *reinterpret_cast<volatile int32_t*>(&p.hdr->status) = 0;
+    }
 
 #ifdef PEVLM_TRACE
     __shared__ unsigned s_waits[16][kTraceIds];
@@ -351,7 +359,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
             if (lane == 0) {
                 int w = static_cast<int>(blockIdx.x >> 1);
                 int published = 0, asked = 0;
-                if (*reinterpret_cast<volatile int32_t*>(&p.hdr->status) != 0) w = -1;
+                // After a timeout the clusters that are still to be launched do nothing (those of the first wave may find
+                // an older call's status, so they do not look).
+                if (w >= kNumSms / 2 && *reinterpret_cast<volatile int32_t*>(&p.hdr->status) != 0) w = -1;
                 while (true) {
                     const int slot = published % kItems;
                     if (published >= kItems) wait_asleep(bars.item_free[slot], (published / kItems - 1) & 1, kWaitItemFree);
@@ -730,12 +740,7 @@ cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cu
     const size_t smem = attn_smem_bytes(head_dim);
     // one cluster per work item; those that run take the rest from the hardware's queue
     const unsigned grid = 2u * static_cast<unsigned>(p.n_items);
-    auto go = [&](auto kernel) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        kernel<<<grid, kAttnThreads, smem, stream>>>(p, m.q, m.q_tail_block, m.q_tail_sink, m.k_sink, m.v_sink, m.k, m.v);
-        return cudaGetLastError();
-    };
+    auto go = [&](auto kernel) { return launch_chained(kernel, grid, kAttnThreads, smem, stream, p, m.q, m.q_tail_block, m.q_tail_sink, m.k_sink, m.v_sink, m.k, m.v); };
     if (p.mode == 0) return head_dim == 128 ? go(attn_kernel<128, 0>) : go(attn_kernel<64, 0>);
     return head_dim == 128 ? go(attn_kernel<128, 1>) : go(attn_kernel<64, 1>);
 }

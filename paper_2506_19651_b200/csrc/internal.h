@@ -102,6 +102,7 @@ struct AttnParams {
     float* part_o;          // mode 1: [n_splits, Q, Hq, d] fp32
     float* part_lse;        // mode 1: [n_splits, Q, Hq]
     WorkspaceHeader* hdr;
+    int32_t clear_status;   // 1 in the first launch of a call
 };
 
 struct MergeParams {

@@ -14,6 +14,8 @@ constexpr int kMergeMaxParts = 160;  // >= the largest split count (one split pe
 // Many rows (a prefill-sized question block): one thread per (row, 4 output columns), the splits one after
 // another; tens of thousands of threads hide the latency of the dependent loads.
 __global__ void merge_kernel(const __grid_constant__ MergeParams p) {
+    grid_wait();
+    grid_launch_dependents();
     const int vec_per_row = p.d / 4;
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t rows = static_cast<int64_t>(p.Q) * p.Hq;
@@ -54,6 +56,8 @@ __global__ void merge_kernel(const __grid_constant__ MergeParams p) {
 // chunk issued before the first is used.
 __global__ void __launch_bounds__(kMergeThreads) merge_rows_kernel(const __grid_constant__ MergeParams p) {
     __shared__ float weights[kMergeThreads / 32][kMergeMaxParts];
+    grid_wait();
+    grid_launch_dependents();
     const int lane = threadIdx.x & 31;
     float* w = weights[threadIdx.x >> 5];
     const int64_t row = static_cast<int64_t>(blockIdx.x) * (kMergeThreads / 32) + (threadIdx.x >> 5);
@@ -118,12 +122,11 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream) {
     const int rows_per_cta = kMergeThreads / 32;
     if (rows <= static_cast<int64_t>(kNumSms) * rows_per_cta && p.n_splits <= kMergeMaxParts) {
         // at most one CTA per SM of warp-per-row work: the latency-oriented form
-        merge_rows_kernel<<<static_cast<unsigned>((rows + rows_per_cta - 1) / rows_per_cta), kMergeThreads, 0, stream>>>(p);
-    } else {
-        const int64_t n = rows * (p.d / 4);
-        merge_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(p);
+        return launch_chained(merge_rows_kernel, static_cast<unsigned>((rows + rows_per_cta - 1) / rows_per_cta), kMergeThreads, 0,
+                              stream, p);
     }
-    return cudaGetLastError();
+    const int64_t n = rows * (p.d / 4);
+    return launch_chained(merge_kernel, static_cast<unsigned>((n + kMergeThreads - 1) / kMergeThreads), kMergeThreads, 0, stream, p);
 }
 
 }  // namespace pevlm
