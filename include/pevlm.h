@@ -75,7 +75,7 @@ typedef struct {
 
 typedef enum {
     PEVLM_WS_PREFILL = 0, /* workspace of pevlm_parallel_prefill_attn */
-    PEVLM_WS_QUERY = 1    /* workspace of pevlm_query_attn */
+    PEVLM_WS_QUERY = 1    /* workspace of pevlm_query_attn and of the question in pevlm_layer_forward */
 } pevlm_workspace_kind_t;
 
 /*
@@ -91,6 +91,15 @@ typedef enum {
 int pevlm_rope_qk(const pevlm_shape_t* shape, const void* q_in, const void* k_in, void* q_out,
                   void* k_out, int64_t first_token, int64_t n_tokens, const int32_t* pos_ids,
                   void* stream);
+
+/*
+ * pevlm_rope_qk and, in the same launch, the copy of the same tokens' V rows: v_in [n_tokens, Hkv, d] to v_out (for
+ * instance the slot of these tokens in the V cache); a NULL pair skips that tensor as it does for Q and K, of which one
+ * must be given.  batch applies to all six tensors.
+ */
+int pevlm_rope_qkv(const pevlm_shape_t* shape, const void* q_in, const void* k_in, const void* v_in, void* q_out,
+                   void* k_out, void* v_out, int64_t first_token, int64_t n_tokens, const int32_t* pos_ids,
+                   void* stream);
 
 /*
  * Multimodal RoPE: the model family the paper evaluates encodes temporal and spatial coordinates in its
@@ -171,7 +180,7 @@ int pevlm_query_attn(const pevlm_shape_t* shape, const void* q_question, const v
  * arguments, results and errors as pevlm_query_attn, minus the workspace: the split-KV partials
  * go to a fixed array of PEVLM_NOALLOC_SCRATCH_BYTES that is part of the library image, so
  * every GPU that loads the library holds that much device memory until the process exits.
- *   - Shapes whose pevlm_workspace_bytes(shape, PEVLM_WS_QUERY) exceeds that size are rejected
+ *   - Shapes whose partials exceed that size are rejected
  *     with PEVLM_EWORKSPACE before any launch (text via pevlm_last_cuda_error).
  *   - The call itself performs no cudaMalloc / cudaFree and uses no allocating routine.
  *   - The first call on each device resolves the array's device address
@@ -187,6 +196,22 @@ int pevlm_query_attn(const pevlm_shape_t* shape, const void* q_question, const v
 #define PEVLM_NOALLOC_SCRATCH_BYTES (32u << 20)
 int pevlm_query_attn_noalloc(const pevlm_shape_t* shape, const void* q_question, const void* k_cache,
                              const void* v_cache, void* o, float* lse, void* stream);
+
+/*
+ * The whole pass of one layer over one sequence [Sec. 3.2; Eq. 3-5], from un-roped q [L, Hq, d], k, v [L, Hkv, d]: RoPE at
+ * global positions with K and V written to the caches, the prefill attention of the video rows (or full causal) and the
+ * question attention.  The same results as pevlm_rope_qk, pevlm_assemble_kv, pevlm_parallel_prefill_attn and
+ * pevlm_query_attn in that order (the question's key splits differ, so its sums may differ in their last bits), in three
+ * launches: the work items of both attention steps share one, so that neither leaves SMs idle.
+ *   q_video [S+N*B, Hq, d], q_question [Q, Hq, d]: roped copies (scratch); k_cache, v_cache [L, Hkv, d], o_*, lse_*: written.
+ *   last_len > 0: the last of the num_blocks blocks has only that many tokens (<= block_len), L and S+N*B accordingly.
+ * batch must be 1.  Pointers of an empty part (no video rows, no question) may be NULL.  Workspaces as for the two attention
+ * calls; ws_query must have pevlm_workspace_bytes(shape, PEVLM_WS_QUERY) bytes.
+ */
+int pevlm_layer_forward(const pevlm_shape_t* shape, int32_t last_len, const void* q, const void* k, const void* v,
+                        void* q_video, void* q_question, void* k_cache, void* v_cache, void* o_video, float* lse_video,
+                        void* o_question, float* lse_question, void* ws_prefill, size_t ws_prefill_bytes,
+                        void* ws_query, size_t ws_query_bytes, void* stream);
 
 /* Bytes of workspace the given call needs for this shape (0 if the shape is invalid). */
 size_t pevlm_workspace_bytes(const pevlm_shape_t* shape, int which /* pevlm_workspace_kind_t */);

@@ -21,7 +21,7 @@ WS_PREFILL, WS_QUERY = 0, 1
 
 NOALLOC_SCRATCH_BYTES = 32 << 20
 
-EXPORTS = ["pevlm_rope_qk", "pevlm_rope_qk_mrope", "pevlm_parallel_prefill_attn", "pevlm_block_attn", "pevlm_assemble_kv", "pevlm_query_attn",
+EXPORTS = ["pevlm_rope_qk", "pevlm_rope_qkv", "pevlm_layer_forward", "pevlm_rope_qk_mrope", "pevlm_parallel_prefill_attn", "pevlm_block_attn", "pevlm_assemble_kv", "pevlm_query_attn",
            "pevlm_query_attn_noalloc",
            "pevlm_workspace_bytes", "pevlm_read_status", "pevlm_selftest_wait_expiry", "pevlm_tile_stats", "pevlm_strerror",
            "pevlm_last_cuda_error"]
@@ -67,6 +67,10 @@ def lib():
         l = C.CDLL(LIB_PATH)
         vp, sp = C.c_void_p, C.POINTER(Shape)
         l.pevlm_rope_qk.argtypes = [sp, vp, vp, vp, vp, C.c_int64, C.c_int64, vp, vp]
+        l.pevlm_rope_qkv.argtypes = [sp, vp, vp, vp, vp, vp, vp, C.c_int64, C.c_int64, vp, vp]
+        l.pevlm_rope_qkv.restype = C.c_int
+        l.pevlm_layer_forward.argtypes = [sp, C.c_int32] + [vp] * 11 + [vp, C.c_size_t, vp, C.c_size_t, vp]
+        l.pevlm_layer_forward.restype = C.c_int
         l.pevlm_rope_qk_mrope.argtypes = [sp, vp, vp, vp, vp, C.c_int64, vp, C.POINTER(C.c_int32), vp]
         l.pevlm_rope_qk_mrope.restype = C.c_int
         l.pevlm_parallel_prefill_attn.argtypes = [sp, vp, vp, vp, vp, vp, vp, C.c_size_t, vp]
@@ -93,12 +97,23 @@ def lib():
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = None
 
 
 def _stream():
-    import torch
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """Handle of torch's current stream on the current device (the raw accessor costs a third of building a Stream object)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        else:
+            _raw_stream = lambda: raw(torch.cuda.current_device())
+    return _raw_stream()
 
 
 def _check(rc, where):
@@ -115,6 +130,19 @@ def pevlm_rope_qk(shape: Shape, q_in, k_in, q_out, k_out, first_token: int, n_to
                                first_token, n_tokens, _ptr(pos_ids), _stream()), "pevlm_rope_qk")
 
 
+def pevlm_rope_qkv(shape: Shape, q_in, k_in, v_in, q_out, k_out, v_out, first_token: int, n_tokens: int, pos_ids=None):
+    _check(lib().pevlm_rope_qkv(C.byref(shape), _ptr(q_in), _ptr(k_in), _ptr(v_in), _ptr(q_out), _ptr(k_out), _ptr(v_out),
+                                first_token, n_tokens, _ptr(pos_ids), _stream()), "pevlm_rope_qkv")
+
+
+def pevlm_layer_forward(shape: Shape, q, k, v, q_video, q_question, k_cache, v_cache, o_video, lse_video, o_question,
+                        lse_question, ws_prefill, ws_query, last_len: int = 0):
+    _check(lib().pevlm_layer_forward(C.byref(shape), last_len, _ptr(q), _ptr(k), _ptr(v), _ptr(q_video), _ptr(q_question),
+                                     _ptr(k_cache), _ptr(v_cache), _ptr(o_video), _ptr(lse_video), _ptr(o_question),
+                                     _ptr(lse_question), _ptr(ws_prefill), ws_prefill.nbytes, _ptr(ws_query),
+                                     ws_query.nbytes, _stream()), "pevlm_layer_forward")
+
+
 def pevlm_rope_qk_mrope(shape: Shape, q_in, k_in, q_out, k_out, n_tokens: int, pos_ids3, sections):
     sec = (C.c_int32 * 3)(*sections)
     _check(lib().pevlm_rope_qk_mrope(C.byref(shape), _ptr(q_in), _ptr(k_in), _ptr(q_out), _ptr(k_out),
@@ -123,14 +151,14 @@ def pevlm_rope_qk_mrope(shape: Shape, q_in, k_in, q_out, k_out, n_tokens: int, p
 
 def pevlm_parallel_prefill_attn(shape: Shape, q, k, v, o, lse, workspace):
     _check(lib().pevlm_parallel_prefill_attn(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
-                                             _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                             _ptr(workspace), workspace.nbytes,
                                              _stream()), "pevlm_parallel_prefill_attn")
 
 
 def pevlm_block_attn(shape: Shape, q_blocks, k_cache, v_cache, first_key_row: int, cache_rows: int, o, lse, workspace):
     _check(lib().pevlm_block_attn(C.byref(shape), _ptr(q_blocks), _ptr(k_cache), _ptr(v_cache), first_key_row,
                                   cache_rows, _ptr(o), _ptr(lse), _ptr(workspace),
-                                  workspace.numel() * workspace.element_size(), _stream()), "pevlm_block_attn")
+                                  workspace.nbytes, _stream()), "pevlm_block_attn")
 
 
 def pevlm_assemble_kv(shape: Shape, k_video, v_video, k_question, v_question, k_cache, v_cache):
@@ -140,7 +168,7 @@ def pevlm_assemble_kv(shape: Shape, k_video, v_video, k_question, v_question, k_
 
 def pevlm_query_attn(shape: Shape, q_question, k_cache, v_cache, o, lse, workspace):
     _check(lib().pevlm_query_attn(C.byref(shape), _ptr(q_question), _ptr(k_cache), _ptr(v_cache), _ptr(o),
-                                  _ptr(lse), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                  _ptr(lse), _ptr(workspace), workspace.nbytes,
                                   _stream()), "pevlm_query_attn")
 
 
@@ -152,7 +180,7 @@ def pevlm_query_attn_noalloc(shape: Shape, q_question, k_cache, v_cache, o, lse)
 
 
 def pevlm_selftest_wait_expiry(workspace, limit_ns: int):
-    _check(lib().pevlm_selftest_wait_expiry(_ptr(workspace), workspace.numel() * workspace.element_size(),
+    _check(lib().pevlm_selftest_wait_expiry(_ptr(workspace), workspace.nbytes,
                                             limit_ns, _stream()), "pevlm_selftest_wait_expiry")
 
 

@@ -1,6 +1,7 @@
 // C ABI of the library: argument checking, TMA tensor-map encoding and kernel launches.
 // Everything here runs on the host; no device memory is allocated and nothing synchronises
 // except pevlm_read_status.
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -41,18 +42,23 @@ static int check_shape(const pevlm_shape_t* s) {
     return PEVLM_OK;
 }
 
-static int64_t n_video(const pevlm_shape_t* s) {
-    return static_cast<int64_t>(s->sink_len) + static_cast<int64_t>(s->num_blocks) * s->block_len;
+// Video tokens; last_len > 0: the last of the blocks has that many tokens.
+static int64_t n_video(const pevlm_shape_t* s, int last_len = 0) {
+    return static_cast<int64_t>(s->sink_len) + static_cast<int64_t>(s->num_blocks) * s->block_len - (last_len > 0 ? s->block_len - last_len : 0);
 }
 
+// What a device is does not change: looked up once for each.
 static int check_device() {
+    static std::atomic<uint64_t> good{0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+    if (dev < 64 && (good.load(std::memory_order_relaxed) >> dev & 1)) return PEVLM_OK;
     int major = 0;
     e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
     if (major != 10) return PEVLM_EUNSUPPORTED;
+    if (dev < 64) good.fetch_or(1ull << dev, std::memory_order_relaxed);
     return PEVLM_OK;
 }
 
@@ -61,14 +67,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 static EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
+    static const EncodeTiledFn fn = [] {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
+        const bool found = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
+                           q == cudaDriverEntryPointSuccess;
+        return found ? reinterpret_cast<EncodeTiledFn>(p) : nullptr;
+    }();
     return fn;
 }
 
@@ -129,10 +134,10 @@ struct QueryPlan {
     int tok_per_tile, q_tiles, total_kv_tiles, n_splits, tiles_per_split;
 };
 
-static QueryPlan plan_query(const pevlm_shape_t* s) {
+static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false, int last_len = 0) {
     QueryPlan q;
     const int G = s->num_q_heads / s->num_kv_heads;
-    const int64_t L = n_video(s) + s->query_len;
+    const int64_t L = n_video(s, last_len) + s->query_len;
     q.tok_per_tile = kTile / G;
     q.q_tiles = (s->query_len + q.tok_per_tile - 1) / q.tok_per_tile;
     q.total_kv_tiles = static_cast<int>((L + kTile - 1) / kTile);
@@ -141,6 +146,13 @@ static QueryPlan plan_query(const pevlm_shape_t* s) {
     const int pairs = (q.q_tiles + 1) / 2;
     const int groups = s->num_kv_heads * (pairs > 0 ? pairs : 1);
     int want = kNumSms / 2 / groups;
+    if (beside_prefill) {
+        // in one launch with the prefill items, which fill in behind them: enough items for every pair of CTAs, none
+        // longer than 64 key tiles (a prefill item of the 50K-token stream has 25), none shorter than 4
+        const int per_pair = static_cast<int>((static_cast<int64_t>(groups) * q.total_kv_tiles + kNumSms / 2 - 1) / (kNumSms / 2));
+        const int tiles = per_pair < 4 ? 4 : per_pair > 64 ? 64 : per_pair;
+        want = (q.total_kv_tiles + tiles - 1) / tiles;
+    }
     if (want < 1) want = 1;
     if (want > q.total_kv_tiles) want = q.total_kv_tiles;
     q.tiles_per_split = (q.total_kv_tiles + want - 1) / want;
@@ -151,6 +163,12 @@ static QueryPlan plan_query(const pevlm_shape_t* s) {
 static size_t query_partial_floats(const pevlm_shape_t* s, const QueryPlan& q) {
     return static_cast<size_t>(q.n_splits) * s->query_len * s->num_q_heads * (s->head_dim + 1);
 }
+
+// Bytes of the question attention's workspace: the status header and the partials of every sequence.
+static size_t query_bytes(const pevlm_shape_t* s, const QueryPlan& q) {
+    return kStatusBytes + static_cast<size_t>(s->batch) * ((query_partial_floats(s, q) * sizeof(float) + 255) / 256 * 256);
+}
+size_t query_workspace_bytes(const pevlm_shape_t* s) { return query_bytes(s, plan_query(s)); }
 
 // Host-side argument checks of the question attention, shared by its two entry points.
 int check_query_args(const pevlm_shape_t* s, const void* q_question, const void* k_cache, const void* v_cache,
@@ -188,21 +206,54 @@ size_t pevlm_workspace_bytes(const pevlm_shape_t* s, int which) {
     if (check_shape(s) != PEVLM_OK) return 0;
     if (which == PEVLM_WS_PREFILL) return kStatusBytes;
     if (which == PEVLM_WS_QUERY) {
-        const QueryPlan q = plan_query(s);
-        return kStatusBytes + static_cast<size_t>(s->batch) * ((query_partial_floats(s, q) * sizeof(float) + 255) / 256 * 256);
+        // pevlm_query_attn, and pevlm_layer_forward with a last block of any length: the most splits that plan_query
+        // can choose for no more key tiles than these
+        QueryPlan q = plan_query(s);
+        const size_t alone = query_bytes(s, q);
+        const int groups = s->num_kv_heads * (q.q_tiles > 1 ? (q.q_tiles + 1) / 2 : 1);
+        const int by_length = (q.total_kv_tiles + 63) / 64, by_pairs = (kNumSms / 2 + groups - 1) / groups;
+        q.n_splits = by_length > by_pairs ? by_length : by_pairs;
+        if (q.n_splits > q.total_kv_tiles) q.n_splits = q.total_kv_tiles;
+        const size_t beside = query_bytes(s, q);
+        return alone > beside ? alone : beside;
     }
     return 0;
 }
 
-static int rope_common(const pevlm_shape_t* s, const void* q_in, const void* k_in, void* q_out, void* k_out,
-                       int64_t first_token, int64_t n_tokens, const int32_t* pos_ids, const int32_t* pos3,
-                       const int32_t* sections, void* stream) {
+// theta^(-2i/d) in fp64; the last ones asked for by this thread are kept (64 calls of pow cost as much as a launch).
+static const double* inverse_frequencies(float theta, int d) {
+    static thread_local float of_theta = 0.f;
+    static thread_local int of_d = 0;
+    static thread_local double f[64];
+    if (theta != of_theta || d != of_d) {
+        for (int i = 0; i < 64; ++i) f[i] = i < d / 2 ? pow(static_cast<double>(theta), -2.0 * i / d) : 0.0;
+        of_theta = theta;
+        of_d = d;
+    }
+    return f;
+}
+
+// Sequences of one launch: the most (at least one) whose rows can be counted in 30 bits.
+static int launch_batch(int batch, int64_t rows) {
+    const int64_t most = rows > 0 ? (1ll << 30) / rows : batch;
+    const int64_t n = most < 1 ? 1 : most < 32768 ? most : 32768;
+    return static_cast<int>(n < batch ? n : batch);
+}
+
+// RoPE of q and k (NULL pairs skipped) and a copy of v's rows (NULL = none).  q rows of tokens from `split` on go to
+// q_out2 (counted from its first row).
+static int rope_common(const pevlm_shape_t* s, const void* q_in, const void* k_in, const void* v_in, void* q_out, void* q_out2,
+                       int64_t split, void* k_out, void* v_out, int64_t first_token, int64_t n_tokens, const int32_t* pos_ids,
+                       const int32_t* pos3, const int32_t* sections, void* stream) {
     int rc = check_shape(s);
     if (rc != PEVLM_OK) return rc;
     if (n_tokens < 0 || first_token < 0 || first_token + n_tokens > (1ll << 31)) return PEVLM_EINVAL;
-    if ((q_in == nullptr) != (q_out == nullptr) || (k_in == nullptr) != (k_out == nullptr)) return PEVLM_EINVAL;
+    if ((q_in == nullptr) != (q_out == nullptr) || (k_in == nullptr) != (k_out == nullptr) || (v_in == nullptr) != (v_out == nullptr))
+        return PEVLM_EINVAL;
     if (!q_in && !k_in) return PEVLM_EINVAL;
-    if (!aligned16(q_in) || !aligned16(k_in) || !aligned16(q_out) || !aligned16(k_out)) return PEVLM_EALIGN;
+    if (!aligned16(q_in) || !aligned16(k_in) || !aligned16(v_in) || !aligned16(q_out) || !aligned16(q_out2) || !aligned16(k_out) ||
+        !aligned16(v_out))
+        return PEVLM_EALIGN;
     if (pos_ids && (reinterpret_cast<uintptr_t>(pos_ids) & 3u)) return PEVLM_EALIGN;
     if (pos3 && (reinterpret_cast<uintptr_t>(pos3) & 3u)) return PEVLM_EALIGN;
     const int d = s->head_dim;
@@ -212,28 +263,31 @@ static int rope_common(const pevlm_shape_t* s, const void* q_in, const void* k_i
     }
     if (n_tokens == 0) return PEVLM_OK;
     RopeParams p;
-    for (int i = 0; i < d / 2; ++i) p.inv_freq[i] = pow(static_cast<double>(s->rope_theta), -2.0 * i / d);
-    for (int i = d / 2; i < 64; ++i) p.inv_freq[i] = 0.0;
+    memcpy(p.inv_freq, inverse_frequencies(s->rope_theta, d), sizeof(p.inv_freq));
     p.first_token = first_token;
-    p.n_tokens = n_tokens;
+    p.seq_len = static_cast<int32_t>(n_tokens < INT32_MAX ? n_tokens : INT32_MAX);
     p.Hq = q_in ? s->num_q_heads : 0;
     p.Hkv = k_in ? s->num_kv_heads : 0;
-    p.split_token = n_tokens;
-    p.q_out2 = nullptr;
-    p.v_in = nullptr;
-    p.v_out = nullptr;
-    p.Hv = 0;
+    p.Hv = v_in ? s->num_kv_heads : 0;
     p.sec_end0 = sections ? sections[0] : 0;
     p.sec_end1 = sections ? sections[0] + sections[1] : 0;
-    for (int b = 0; b < s->batch; ++b) {
-        const int64_t qo = static_cast<int64_t>(b) * n_tokens * s->num_q_heads * d;
-        const int64_t ko = static_cast<int64_t>(b) * n_tokens * s->num_kv_heads * d;
-        p.q_in = q_in ? static_cast<const __nv_bfloat16*>(q_in) + qo : nullptr;
-        p.q_out = q_out ? static_cast<__nv_bfloat16*>(q_out) + qo : nullptr;
-        p.k_in = k_in ? static_cast<const __nv_bfloat16*>(k_in) + ko : nullptr;
-        p.k_out = k_out ? static_cast<__nv_bfloat16*>(k_out) + ko : nullptr;
-        p.pos_ids = pos_ids ? pos_ids + static_cast<int64_t>(b) * n_tokens : nullptr;
-        p.pos3 = pos3 ? pos3 + static_cast<int64_t>(b) * 3 * n_tokens : nullptr;
+    const int step = launch_batch(s->batch, n_tokens);
+    for (int b = 0; b < s->batch; b += step) {
+        const int64_t t0 = static_cast<int64_t>(b) * n_tokens;
+        const int64_t qo = t0 * s->num_q_heads * d, ko = t0 * s->num_kv_heads * d;
+        auto at = [](const void* base, int64_t off) { return base ? static_cast<const __nv_bfloat16*>(base) + off : nullptr; };
+        p.n_tokens = n_tokens * (s->batch - b < step ? s->batch - b : step);
+        p.q_in = at(q_in, qo);
+        p.q_out = const_cast<__nv_bfloat16*>(at(q_out, qo));
+        p.split_token = q_out2 ? split : p.n_tokens;
+        // the kernel counts rows from the first token
+        p.q_out2 = q_out2 ? static_cast<__nv_bfloat16*>(q_out2) - split * s->num_q_heads * d : nullptr;
+        p.k_in = at(k_in, ko);
+        p.k_out = const_cast<__nv_bfloat16*>(at(k_out, ko));
+        p.v_in = at(v_in, ko);
+        p.v_out = const_cast<__nv_bfloat16*>(at(v_out, ko));
+        p.pos_ids = pos_ids ? pos_ids + t0 : nullptr;
+        p.pos3 = pos3 ? pos3 + 3 * t0 : nullptr;
         cudaError_t e = launch_rope(p, d, static_cast<cudaStream_t>(stream));
         if (e != cudaSuccess) return cuda_fail(e, "rope launch");
     }
@@ -242,13 +296,18 @@ static int rope_common(const pevlm_shape_t* s, const void* q_in, const void* k_i
 
 int pevlm_rope_qk(const pevlm_shape_t* s, const void* q_in, const void* k_in, void* q_out, void* k_out,
                   int64_t first_token, int64_t n_tokens, const int32_t* pos_ids, void* stream) {
-    return rope_common(s, q_in, k_in, q_out, k_out, first_token, n_tokens, pos_ids, nullptr, nullptr, stream);
+    return rope_common(s, q_in, k_in, nullptr, q_out, nullptr, 0, k_out, nullptr, first_token, n_tokens, pos_ids, nullptr, nullptr, stream);
 }
 
 int pevlm_rope_qk_mrope(const pevlm_shape_t* s, const void* q_in, const void* k_in, void* q_out, void* k_out,
                         int64_t n_tokens, const int32_t* pos_ids3, const int32_t* sections, void* stream) {
     if (!pos_ids3 || !sections) return PEVLM_EINVAL;
-    return rope_common(s, q_in, k_in, q_out, k_out, 0, n_tokens, nullptr, pos_ids3, sections, stream);
+    return rope_common(s, q_in, k_in, nullptr, q_out, nullptr, 0, k_out, nullptr, 0, n_tokens, nullptr, pos_ids3, sections, stream);
+}
+
+int pevlm_rope_qkv(const pevlm_shape_t* s, const void* q_in, const void* k_in, const void* v_in, void* q_out, void* k_out, void* v_out,
+                   int64_t first_token, int64_t n_tokens, const int32_t* pos_ids, void* stream) {
+    return rope_common(s, q_in, k_in, v_in, q_out, nullptr, 0, k_out, v_out, first_token, n_tokens, pos_ids, nullptr, nullptr, stream);
 }
 
 int pevlm_assemble_kv(const pevlm_shape_t* s, const void* k_video, const void* v_video, const void* k_question,
@@ -263,17 +322,20 @@ int pevlm_assemble_kv(const pevlm_shape_t* s, const void* k_video, const void* v
     const int64_t nv = n_video(s);
     const int64_t row_vec = static_cast<int64_t>(s->num_kv_heads) * s->head_dim * 2 / 16;  // 16-byte vectors per token
     const int64_t L = nv + s->query_len;
-    for (int b = 0; b < s->batch; ++b) {
-        CopySegments seg;
-        const void* srcs[4] = {k_video, k_question, v_video, v_question};
-        void* dsts[4] = {k_cache, k_cache, v_cache, v_cache};
-        const int64_t rows[4] = {nv, s->query_len, nv, s->query_len};
-        const int64_t dst_row0[4] = {0, nv, 0, nv};
+    CopySegments seg;
+    const void* srcs[4] = {k_video, k_question, v_video, v_question};
+    void* dsts[4] = {k_cache, k_cache, v_cache, v_cache};
+    const int64_t rows[4] = {nv, s->query_len, nv, s->query_len};
+    const int64_t dst_row0[4] = {0, nv, 0, nv};
+    seg.dst_stride = L * row_vec;
+    for (int b = 0; b < s->batch; b += 32768) {
+        seg.batch = s->batch - b < 32768 ? s->batch - b : 32768;
         seg.total = 0;
         for (int i = 0; i < 4; ++i) {
             const int64_t n = srcs[i] ? rows[i] * row_vec : 0;
             seg.n_vec[i] = n;
-            seg.src[i] = srcs[i] ? static_cast<const uint4*>(srcs[i]) + static_cast<int64_t>(b) * rows[i] * row_vec : nullptr;
+            seg.src_stride[i] = n;
+            seg.src[i] = srcs[i] ? static_cast<const uint4*>(srcs[i]) + b * n : nullptr;
             seg.dst[i] = dsts[i] ? static_cast<uint4*>(dsts[i]) + (static_cast<int64_t>(b) * L + dst_row0[i]) * row_vec : nullptr;
             seg.total += n;
         }
@@ -283,55 +345,44 @@ int pevlm_assemble_kv(const pevlm_shape_t* s, const void* k_video, const void* v
     return PEVLM_OK;
 }
 
-// Prefill attention launches.  blocks_only = false: the whole video stream [sink | N blocks] (or full causal).
-// blocks_only = true: N blocks whose K/V sit at rows [first_key_row, first_key_row + N*B) of a cache of cache_rows
-// rows whose first S rows are the sink; q / o / lse cover the N*B block rows only and the sink rows are not computed.
-static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, const void* v, void* o, float* lse,
-                          void* workspace, size_t workspace_bytes, void* stream, bool blocks_only,
-                          int64_t first_key_row, int64_t cache_rows) {
-    int rc = check_shape(s);
-    if (rc != PEVLM_OK) return rc;
-    if (!q || !k || !v || !o) return PEVLM_EINVAL;
-    // the output rows are written with 32-byte vector stores
-    if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned32(o) || !aligned16(lse)) return PEVLM_EALIGN;
-    if (!workspace || workspace_bytes < pevlm_workspace_bytes(s, PEVLM_WS_PREFILL)) return PEVLM_EWORKSPACE;
-    if (!aligned256(workspace)) return PEVLM_EALIGN;
-    const int64_t nv = n_video(s);
-    const int64_t block_rows = static_cast<int64_t>(s->num_blocks) * s->block_len;
-    if (blocks_only) {
-        if (s->mask_mode != PEVLM_MASK_PEVLM) return PEVLM_EINVAL;
-        if (first_key_row < s->sink_len || first_key_row + block_rows > cache_rows || cache_rows > (1ll << 30))
-            return PEVLM_EINVAL;
-        if (block_rows == 0) return PEVLM_OK;
-    } else if (nv == 0) {
-        return PEVLM_OK;
-    }
-    rc = check_device();
-    if (rc != PEVLM_OK) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int d = s->head_dim;
-    const int64_t q_rows = blocks_only ? block_rows : nv;   // rows of q, o, lse
-    const int64_t kv_rows = blocks_only ? cache_rows : nv;  // rows of k, v
+// ---- parameters of an attention launch
+static AttnParams common_params(const pevlm_shape_t* s, int last_len = 0) {
     AttnParams p;
     memset(&p, 0, sizeof(p));
-    p.mode = 0;
+    p.n_video = static_cast<int>(n_video(s, last_len));
+    p.Q = s->query_len;
+    p.L = p.n_video + s->query_len;
+    p.Hq = s->num_q_heads; p.Hkv = s->num_kv_heads; p.G = p.Hq / p.Hkv;
+    p.scale = resolve_scale(s);
+    p.scale_log2 = p.scale * 1.4426950408889634f;
+    p.wait_limit_ns = kDefaultWaitLimitNs;
+    return p;
+}
+
+// Prefill rows.  blocks_only = false: the whole video stream [sink | N blocks] (or full causal).  blocks_only = true: N
+// blocks whose K/V sit at rows [first_key_row, first_key_row + N*B) of a cache of cache_rows rows whose first S rows are
+// the sink; q / o / lse cover the N*B block rows only and the sink rows are not computed.
+static void add_prefill(AttnParams& p, const pevlm_shape_t* s, bool blocks_only, int64_t first_key_row, int64_t cache_rows, int last_len = 0) {
+    const int64_t nv = p.n_video;
+    p.mode |= 1;
     if (s->mask_mode == PEVLM_MASK_FULL_CAUSAL) {
         p.S = 0; p.B = static_cast<int>(nv); p.N = 1;
     } else {
-        p.S = s->sink_len; p.B = s->num_blocks > 0 ? s->block_len : 0; p.N = s->num_blocks;
+        p.S = s->sink_len; p.B = s->num_blocks > 0 ? s->block_len : 0; p.N = s->num_blocks - (last_len > 0 ? 1 : 0);
+        p.last_len = last_len;
     }
-    p.n_video = static_cast<int>(nv);
     p.blk_key0 = blocks_only ? static_cast<int>(first_key_row) : p.S;
     p.blk_q0 = blocks_only ? 0 : p.S;
-    p.q_rows = static_cast<int>(q_rows);
-    p.Q = s->query_len;
-    p.L = static_cast<int>(nv + s->query_len);
-    p.Hq = s->num_q_heads; p.Hkv = s->num_kv_heads; p.G = p.Hq / p.Hkv;
+    p.q_rows = static_cast<int>(blocks_only ? static_cast<int64_t>(s->num_blocks) * s->block_len : nv);
+    p.kv_rows = static_cast<int>(blocks_only ? cache_rows : nv);
+    p.lse_stride = p.q_rows;
     p.tiles_sink = (p.S + kTile - 1) / kTile;
     p.tiles_block = p.N > 0 ? (p.B + kTile - 1) / kTile : 0;
-    const SegPlan pb = plan_segment(p.N > 0 ? p.B : 0, p.G), ps = plan_segment(blocks_only ? 0 : p.S, p.G);
+    const SegPlan pb = plan_segment(p.N > 0 ? p.B : 0, p.G), ps = plan_segment(blocks_only ? 0 : p.S, p.G), pl = plan_segment(p.last_len, p.G);
     p.pairs_block = pb.pairs;
     p.pairs_sink = ps.pairs;
+    p.pairs_last = pl.pairs;
+    p.tail_rows_last = pl.tail_rows; p.tail_heads_last = pl.tail_heads; p.tail_tiles_last = pl.tail_tiles;
     p.tail_rows_block = pb.tail_rows; p.tail_heads_block = pb.tail_heads; p.tail_tiles_block = pb.tail_tiles;
     p.tail_rows_sink = ps.tail_rows; p.tail_heads_sink = ps.tail_heads; p.tail_tiles_sink = ps.tail_tiles;
     // How many pairs of one (block, kv head) are handed out together (decode_item): the whole list keeps the CTAs
@@ -344,40 +395,112 @@ static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, 
     p.pair_chunk = p.pairs_block > 0 ? (want_pc < p.pairs_block ? want_pc : p.pairs_block) : 1;
     const int n_chunks = p.pairs_block > 0 ? (p.pairs_block + p.pair_chunk - 1) / p.pair_chunk : 0;
     p.items_block = p.N * p.Hkv * p.pair_chunk * n_chunks;
-    p.n_items = p.items_block + p.Hkv * p.pairs_sink;
+    p.items_last = p.Hkv * p.pairs_last;
+    p.n_items += p.items_block + p.items_last + p.Hkv * p.pairs_sink;
     p.div_per_chunk = make_divisor(p.N * p.Hkv * p.pair_chunk);
     p.div_pair_chunk = make_divisor(p.pair_chunk);
     p.div_hkv = make_divisor(p.Hkv);
     p.div_pairs_sink = make_divisor(p.pairs_sink);
+    p.div_pairs_last = make_divisor(p.pairs_last);
     p.div_g = make_divisor(p.G);
-    p.scale = resolve_scale(s);
-    p.scale_log2 = p.scale * 1.4426950408889634f;
-    p.wait_limit_ns = kDefaultWaitLimitNs;
+}
+
+static void add_question(AttnParams& p, const QueryPlan& qp) {
+    p.mode |= 2;
+    p.tok_per_tile = qp.tok_per_tile;
+    p.q_tiles = qp.q_tiles;
+    p.n_splits = qp.n_splits;
+    p.tiles_per_split = qp.tiles_per_split;
+    p.items_question = p.Hkv * ((p.q_tiles + 1) / 2) * p.n_splits;
+    p.n_items += p.items_question;
+    p.div_splits = make_divisor(p.n_splits);
+    p.div_q_pairs = make_divisor((p.q_tiles + 1) / 2);
+}
+
+// Tensor maps over the rows of p.batch sequences.  Between two sequences of a batch a ragged last key tile brings in rows
+// of the next range instead of zeros; they are masked, and finite like every input.  (Block ranges, whose cache may hold
+// anything elsewhere, are launched one sequence at a time.)
+static int prefill_maps(AttnMaps& m, const AttnParams& p, int d, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v) {
+    int rc;
+    const int64_t q_rows = static_cast<int64_t>(p.batch) * p.q_rows, before = static_cast<int64_t>(p.batch - 1) * p.kv_rows;
+    if ((rc = make_tmap(&m.q, q, q_rows, p.Hq, d, 1, kTile)) != PEVLM_OK) return rc;
+    m.q_tail_block = m.q;
+    m.q_tail_sink = m.q;
+    m.q_tail_last = m.q;
+    if (p.tail_tiles_last > 0 && (rc = make_tmap(&m.q_tail_last, q, q_rows, p.Hq, d, p.tail_heads_last, p.tail_rows_last)) != PEVLM_OK) return rc;
+    if (p.tail_tiles_block > 0 && (rc = make_tmap(&m.q_tail_block, q, q_rows, p.Hq, d, p.tail_heads_block, p.tail_rows_block)) != PEVLM_OK) return rc;
+    if (p.tail_tiles_sink > 0) {
+        if (p.tail_tiles_block > 0 && p.tail_heads_sink == p.tail_heads_block && p.tail_rows_sink == p.tail_rows_block) m.q_tail_sink = m.q_tail_block;
+        else if ((rc = make_tmap(&m.q_tail_sink, q, q_rows, p.Hq, d, p.tail_heads_sink, p.tail_rows_sink)) != PEVLM_OK) return rc;
+    }
+    // K and V: one map over the sink rows [0, S) and one over the block rows, so that the ragged last key
+    // tile of either range reads zeros past its end (a map needs at least one row; an empty range is never read)
+    const int64_t blk_off = static_cast<int64_t>(p.blk_key0) * p.Hkv * d, block_rows = static_cast<int64_t>(p.N) * p.B + p.last_len;
+    const int64_t sink_rows = before + (p.S > 0 ? p.S : 1), blk_rows = before + (block_rows > 0 ? block_rows : 1);
+    if ((rc = make_tmap(&m.k_sink, k, sink_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.v_sink, v, sink_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.k, k + blk_off, blk_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+    return make_tmap(&m.v, v + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2);
+}
+
+static int question_maps(AttnMaps& m, const AttnParams& p, int d, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v) {
+    int rc;
+    const int64_t rows = static_cast<int64_t>(p.batch) * p.L;
+    if ((rc = make_tmap(&m.q_question, q, static_cast<int64_t>(p.batch) * p.Q, p.Hq, d, p.G, p.tok_per_tile)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.k_cache, k, rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+    return make_tmap(&m.v_cache, v, rows, p.Hkv, d, 1, kTile, d / 2);
+}
+
+static int merge_question(const AttnParams& p, int d, __nv_bfloat16* o, float* lse, cudaStream_t st) {
+    MergeParams m;
+    m.batch = p.batch; m.Q = p.Q; m.Hq = p.Hq; m.d = d; m.n_splits = p.n_splits;
+    m.part_o = p.part_o; m.part_lse = p.part_lse;
+    m.o = o;
+    m.lse = lse;
+    const cudaError_t e = launch_merge(m, st);
+    return e == cudaSuccess ? PEVLM_OK : cuda_fail(e, "merge launch");
+}
+
+static const __nv_bfloat16* rows_of(const void* base, int64_t rows, int heads, int d) {
+    return static_cast<const __nv_bfloat16*>(base) + rows * heads * d;
+}
+
+static int prefill_common(const pevlm_shape_t* s, const void* q, const void* k, const void* v, void* o, float* lse,
+                          void* workspace, size_t workspace_bytes, void* stream, bool blocks_only,
+                          int64_t first_key_row, int64_t cache_rows) {
+    int rc = check_shape(s);
+    if (rc != PEVLM_OK) return rc;
+    if (!q || !k || !v || !o) return PEVLM_EINVAL;
+    // the output rows are written with 32-byte vector stores
+    if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned32(o) || !aligned16(lse)) return PEVLM_EALIGN;
+    if (!workspace || workspace_bytes < pevlm_workspace_bytes(s, PEVLM_WS_PREFILL)) return PEVLM_EWORKSPACE;
+    if (!aligned256(workspace)) return PEVLM_EALIGN;
+    const int64_t block_rows = static_cast<int64_t>(s->num_blocks) * s->block_len;
+    if (blocks_only) {
+        if (s->mask_mode != PEVLM_MASK_PEVLM) return PEVLM_EINVAL;
+        if (first_key_row < s->sink_len || first_key_row + block_rows > cache_rows || cache_rows > (1ll << 30))
+            return PEVLM_EINVAL;
+        if (block_rows == 0) return PEVLM_OK;
+    } else if (n_video(s) == 0) {
+        return PEVLM_OK;
+    }
+    rc = check_device();
+    if (rc != PEVLM_OK) return rc;
+    const int d = s->head_dim;
+    AttnParams p = common_params(s);
+    add_prefill(p, s, blocks_only, first_key_row, cache_rows);
+    p.div_items = make_divisor(p.n_items);
     p.hdr = static_cast<WorkspaceHeader*>(workspace);
-    const int64_t block_rows_launch = static_cast<int64_t>(p.N) * p.B;  // full causal: the whole stream as one block
-    for (int b = 0; b < s->batch; ++b) {
-        const int64_t qoff = static_cast<int64_t>(b) * q_rows * p.Hq * d, koff = static_cast<int64_t>(b) * kv_rows * p.Hkv * d;
+    const int step = blocks_only ? 1 : launch_batch(s->batch, p.kv_rows > p.n_items ? p.kv_rows : p.n_items);
+    for (int b = 0; b < s->batch; b += step) {
+        p.batch = s->batch - b < step ? s->batch - b : step;
+        p.keep_status = b > 0;
+        const int64_t q0 = static_cast<int64_t>(b) * p.q_rows, k0 = static_cast<int64_t>(b) * p.kv_rows;
         AttnMaps m;
-        const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q) + qoff;
-        if ((rc = make_tmap(&m.q, qb, q_rows, p.Hq, d, 1, kTile)) != PEVLM_OK) return rc;
-        m.q_tail_block = m.q;
-        m.q_tail_sink = m.q;
-        if (pb.tail_tiles > 0 && (rc = make_tmap(&m.q_tail_block, qb, q_rows, p.Hq, d, pb.tail_heads, pb.tail_rows)) != PEVLM_OK) return rc;
-        if (ps.tail_tiles > 0 && (rc = make_tmap(&m.q_tail_sink, qb, q_rows, p.Hq, d, ps.tail_heads, ps.tail_rows)) != PEVLM_OK) return rc;
-        // K and V: one map over the sink rows [0, S) and one over the block rows, so that the ragged last key
-        // tile of either range reads zeros past its end (a map needs at least one row; an empty range is never read)
-        const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k) + koff;
-        const __nv_bfloat16* vb = static_cast<const __nv_bfloat16*>(v) + koff;
-        const int64_t blk_off = static_cast<int64_t>(p.blk_key0) * p.Hkv * d;
-        const int64_t sink_rows = p.S > 0 ? p.S : 1, blk_rows = block_rows_launch > 0 ? block_rows_launch : 1;
-        if ((rc = make_tmap(&m.k_sink, kb, sink_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&m.v_sink, vb, sink_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&m.k, kb + blk_off, blk_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&m.v, vb + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
-        p.o = static_cast<__nv_bfloat16*>(o) + qoff;
-        p.lse = lse ? lse + static_cast<int64_t>(b) * p.Hq * q_rows : nullptr;
-        p.clear_status = b == 0;
-        cudaError_t e = launch_attn(p, d, m, st);
+        if ((rc = prefill_maps(m, p, d, rows_of(q, q0, p.Hq, d), rows_of(k, k0, p.Hkv, d), rows_of(v, k0, p.Hkv, d))) != PEVLM_OK) return rc;
+        p.o = const_cast<__nv_bfloat16*>(rows_of(o, q0, p.Hq, d));
+        p.lse = lse ? lse + static_cast<int64_t>(p.Hq) * q0 : nullptr;
+        const cudaError_t e = launch_attn(p, d, m, static_cast<cudaStream_t>(stream));
         if (e != cudaSuccess) return cuda_fail(e, "prefill attention launch");
     }
     return PEVLM_OK;
@@ -399,58 +522,85 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
                      float* lse, void* workspace, size_t workspace_bytes, void* stream) {
     int rc = check_query_args(s, q_question, k_cache, v_cache, o, lse);
     if (rc != PEVLM_OK) return rc;
-    if (!workspace || workspace_bytes < pevlm_workspace_bytes(s, PEVLM_WS_QUERY)) return PEVLM_EWORKSPACE;
+    if (!workspace || workspace_bytes < query_workspace_bytes(s)) return PEVLM_EWORKSPACE;
     if (!aligned256(workspace)) return PEVLM_EALIGN;
     if (s->query_len == 0) return PEVLM_OK;
     rc = check_device();
     if (rc != PEVLM_OK) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int d = s->head_dim;
-    const int64_t nv = n_video(s);
-    const int64_t L = nv + s->query_len;
     const QueryPlan qp = plan_query(s);
-    AttnParams p;
-    memset(&p, 0, sizeof(p));
-    p.mode = 1;
-    p.n_video = static_cast<int>(nv);
-    p.Q = s->query_len;
-    p.L = static_cast<int>(L);
-    p.Hq = s->num_q_heads; p.Hkv = s->num_kv_heads; p.G = p.Hq / p.Hkv;
-    p.tok_per_tile = qp.tok_per_tile;
-    p.q_tiles = qp.q_tiles;
-    p.n_splits = qp.n_splits;
-    p.tiles_per_split = qp.tiles_per_split;
-    p.n_items = p.Hkv * ((p.q_tiles + 1) / 2) * p.n_splits;
-    p.div_splits = make_divisor(p.n_splits);
-    p.div_q_pairs = make_divisor((p.q_tiles + 1) / 2);
-    p.scale = resolve_scale(s);
-    p.scale_log2 = p.scale * 1.4426950408889634f;
-    p.wait_limit_ns = kDefaultWaitLimitNs;
+    AttnParams p = common_params(s);
+    add_question(p, qp);
+    p.div_items = make_divisor(p.n_items);
     p.hdr = static_cast<WorkspaceHeader*>(workspace);
-    const size_t part_floats = query_partial_floats(s, qp);
-    const size_t part_stride = (part_floats * sizeof(float) + 255) / 256 * 256;
-    for (int b = 0; b < s->batch; ++b) {
-        float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + kStatusBytes + b * part_stride);
-        p.part_o = part;
-        p.part_lse = part + static_cast<size_t>(p.n_splits) * p.Q * p.Hq * d;
-        const int64_t qoff = static_cast<int64_t>(b) * p.Q * p.Hq * d, koff = static_cast<int64_t>(b) * L * p.Hkv * d;
-        AttnMaps maps;
-        if ((rc = make_tmap(&maps.q, static_cast<const __nv_bfloat16*>(q_question) + qoff, p.Q, p.Hq, d, p.G, p.tok_per_tile)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&maps.k, static_cast<const __nv_bfloat16*>(k_cache) + koff, L, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-        if ((rc = make_tmap(&maps.v, static_cast<const __nv_bfloat16*>(v_cache) + koff, L, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
-        maps.q_tail_block = maps.q; maps.q_tail_sink = maps.q; maps.k_sink = maps.k; maps.v_sink = maps.v;
-        p.clear_status = b == 0;
-        cudaError_t e = launch_attn(p, d, maps, st);
+    const int step = launch_batch(s->batch, p.L > p.n_items ? p.L : p.n_items);
+    const size_t seq_floats = static_cast<size_t>(p.n_splits) * p.Q * p.Hq;
+    for (int b = 0; b < s->batch; b += step) {
+        p.batch = s->batch - b < step ? s->batch - b : step;
+        p.keep_status = b > 0;
+        p.part_o = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + kStatusBytes);
+        p.part_lse = p.part_o + seq_floats * d * p.batch;
+        const int64_t q0 = static_cast<int64_t>(b) * p.Q, k0 = static_cast<int64_t>(b) * p.L;
+        AttnMaps m;
+        if ((rc = question_maps(m, p, d, rows_of(q_question, q0, p.Hq, d), rows_of(k_cache, k0, p.Hkv, d), rows_of(v_cache, k0, p.Hkv, d))) != PEVLM_OK) return rc;
+        const cudaError_t e = launch_attn(p, d, m, static_cast<cudaStream_t>(stream));
         if (e != cudaSuccess) return cuda_fail(e, "question attention launch");
-        MergeParams m;
-        m.Q = p.Q; m.Hq = p.Hq; m.d = d; m.n_splits = p.n_splits;
-        m.part_o = p.part_o; m.part_lse = p.part_lse;
-        m.o = static_cast<__nv_bfloat16*>(o) + qoff;
-        m.lse = lse ? lse + static_cast<int64_t>(b) * p.Hq * p.Q : nullptr;
-        e = launch_merge(m, st);
-        if (e != cudaSuccess) return cuda_fail(e, "merge launch");
+        rc = merge_question(p, d, const_cast<__nv_bfloat16*>(rows_of(o, q0, p.Hq, d)), lse ? lse + p.Hq * q0 : nullptr,
+                            static_cast<cudaStream_t>(stream));
+        if (rc != PEVLM_OK) return rc;
     }
     return PEVLM_OK;
+}
+
+int pevlm_layer_forward(const pevlm_shape_t* s, int32_t last_len, const void* q, const void* k, const void* v, void* q_video, void* q_question,
+                        void* k_cache, void* v_cache, void* o_video, float* lse_video, void* o_question, float* lse_question,
+                        void* ws_prefill, size_t ws_prefill_bytes, void* ws_query, size_t ws_query_bytes, void* stream) {
+    int rc = check_shape(s);
+    if (rc != PEVLM_OK) return rc;
+    if (s->batch != 1) return PEVLM_EUNSUPPORTED;
+    if (last_len < 0 || (last_len > 0 && (s->num_blocks < 1 || last_len > s->block_len))) return PEVLM_EINVAL;
+    if (last_len == s->block_len) last_len = 0;
+    const int64_t nv = n_video(s, last_len);
+    const int Q = s->query_len, d = s->head_dim, Hq = s->num_q_heads;
+    if (!q || !k || !v || !k_cache || !v_cache) return PEVLM_EINVAL;
+    if (nv > 0 && (!q_video || !o_video)) return PEVLM_EINVAL;
+    if (Q > 0 && (!q_question || !o_question)) return PEVLM_EINVAL;
+    if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(q_video) || !aligned16(q_question) || !aligned16(k_cache) ||
+        !aligned16(v_cache) || !aligned32(o_video) || !aligned16(lse_video) || !aligned32(o_question) || !aligned16(lse_question))
+        return PEVLM_EALIGN;
+    const QueryPlan qp = plan_query(s, true, last_len);
+    if (nv > 0 && (!ws_prefill || ws_prefill_bytes < pevlm_workspace_bytes(s, PEVLM_WS_PREFILL))) return PEVLM_EWORKSPACE;
+    if (Q > 0 && (!ws_query || ws_query_bytes < query_bytes(s, qp))) return PEVLM_EWORKSPACE;
+    if (!aligned256(ws_prefill) || !aligned256(ws_query)) return PEVLM_EALIGN;
+    rc = check_device();
+    if (rc != PEVLM_OK) return rc;
+    // every token's Q and K roped, K and V into the cache
+    rc = nv > 0 ? rope_common(s, q, k, v, q_video, Q > 0 ? q_question : nullptr, nv, k_cache, v_cache, 0, nv + Q, nullptr, nullptr, nullptr, stream)
+                : rope_common(s, q, k, v, q_question, nullptr, 0, k_cache, v_cache, 0, Q, nullptr, nullptr, nullptr, stream);
+    if (rc != PEVLM_OK) return rc;
+    AttnParams p = common_params(s, last_len);
+    AttnMaps m;
+    p.batch = 1;
+    if (nv > 0) {
+        add_prefill(p, s, false, 0, 0, last_len);
+        rc = prefill_maps(m, p, d, static_cast<const __nv_bfloat16*>(q_video), static_cast<const __nv_bfloat16*>(k_cache), static_cast<const __nv_bfloat16*>(v_cache));
+        if (rc != PEVLM_OK) return rc;
+        p.o = static_cast<__nv_bfloat16*>(o_video);
+        p.lse = lse_video;
+        p.hdr = static_cast<WorkspaceHeader*>(ws_prefill);
+    }
+    if (Q > 0) {
+        add_question(p, qp);
+        rc = question_maps(m, p, d, static_cast<const __nv_bfloat16*>(q_question), static_cast<const __nv_bfloat16*>(k_cache), static_cast<const __nv_bfloat16*>(v_cache));
+        if (rc != PEVLM_OK) return rc;
+        p.hdr_question = static_cast<WorkspaceHeader*>(ws_query);
+        if (nv == 0) p.hdr = p.hdr_question;
+        p.part_o = reinterpret_cast<float*>(static_cast<uint8_t*>(ws_query) + kStatusBytes);
+        p.part_lse = p.part_o + static_cast<size_t>(p.n_splits) * Q * Hq * d;
+    }
+    const cudaError_t e = launch_attn(p, d, m, static_cast<cudaStream_t>(stream));
+    if (e != cudaSuccess) return cuda_fail(e, "attention launch");
+    return Q > 0 ? merge_question(p, d, static_cast<__nv_bfloat16*>(o_question), lse_question, static_cast<cudaStream_t>(stream)) : PEVLM_OK;
 }
 
 int pevlm_selftest_wait_expiry(void* workspace, size_t workspace_bytes, int64_t limit_ns, void* stream) {

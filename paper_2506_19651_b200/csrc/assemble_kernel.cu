@@ -21,9 +21,14 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
                  : "memory");
 }
 
-__global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __grid_constant__ CopySegments s) {
+__global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(CopySegments s) {
     grid_wait();
     grid_launch_dependents();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // the sequence of this row of CTAs
+        s.src[k] += static_cast<int64_t>(blockIdx.y) * s.src_stride[k];
+        s.dst[k] += static_cast<int64_t>(blockIdx.y) * s.dst_stride;
+    }
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kCopyThreads * kCopyUnroll;
     for (int64_t base = static_cast<int64_t>(blockIdx.x) * kCopyThreads * kCopyUnroll + threadIdx.x; base < s.total;
          base += stride) {
@@ -58,7 +63,7 @@ cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream) {
     int64_t ctas = (s.total + per_cta - 1) / per_cta;
     const int64_t cap = 148 * 16;  // a few waves of the 148 SMs; the loop strides over the rest
     if (ctas > cap) ctas = cap;
-    return launch_chained(copy_segments_kernel, static_cast<unsigned>(ctas), kCopyThreads, 0, stream, s);
+    return launch_chained(copy_segments_kernel, dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(s.batch)), kCopyThreads, 0, stream, s);
 }
 
 }  // namespace pevlm

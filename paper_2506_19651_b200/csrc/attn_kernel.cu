@@ -73,7 +73,7 @@ struct AttnSmem {
     static constexpr int kTotal = kV + kRing * kVBytes;
 };
 
-size_t attn_smem_bytes(int head_dim) {
+static size_t attn_smem_bytes(int head_dim) {
     return 1024 + (head_dim == 128 ? AttnSmem<128>::kTotal : AttnSmem<64>::kTotal);
 }
 
@@ -89,10 +89,11 @@ struct QSlot {
 };
 // Key tiles of an item: first the na tiles of the shared range [0, a_end) (the sink), then the tiles of the own
 // range, nt tiles in all (what the longer of the two query tiles needs; the other one masks its surplus tile).
-// The own range is fetched through the block tensor map at row b_coord0 of that map, or, for the sink's own items,
-// through the sink map (own_map = 1).  n_a, n_b: MMA columns of tile na - 1 and of the last tile; the others have 128.
+// The own range is fetched at row b_coord0 of the block tensor map (own_map = 0), for the sink's own items of the sink map
+// (1), for question items of the map of the whole cache (2).  seq: sequence of the batch, k_row0: its first row in the
+// sink and block maps (b_coord0 includes it).  n_a, n_b: MMA columns of tile na - 1 and of the last tile; the others have 128.
 struct WorkItem {
-    int kv_head, a_end, na, nt, n_a, n_b, split, b_coord0, own_map;
+    int kv_head, a_end, na, nt, n_a, n_b, split, b_coord0, own_map, seq, k_row0;
     QSlot s[2];
 };
 
@@ -108,11 +109,21 @@ extern "C" int pevlm_debug_waits(unsigned* host_out) {
 
 __device__ __forceinline__ int cdiv(int a, int b) { return (a + b - 1) / b; }
 
+// MODE: bit 0 = the launch has prefill items, bit 1 = it has question items (handed out first: they are the longest).
+// Items of a sequence follow one another, w counts over the whole batch.
 template <int MODE>
 __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem& it) {
     it.split = 0;
+    it.seq = 0;
+    if (p.batch > 1) {
+        it.seq = quotient(w, p.div_items);
+        w -= it.seq * p.n_items;
+    }
+    const bool question = MODE == 2 || (MODE == 3 && w < p.items_question);
+    if (MODE == 3) w -= question ? 0 : p.items_question;
+    it.k_row0 = it.seq * p.kv_rows;
     int own_keys = 0;  // keys of the own range that the longer query tile sees
-    if (MODE == 0) {
+    if (!question) {
         int seg_q0, seg_len, tiles, pi, g, tail_rows, tail_heads, tail_tiles, qmap_tail;
         if (w < p.items_block) {
             // Order of the items: the pair list of a (block, kv head), heaviest first, is cut into chunks of
@@ -132,10 +143,23 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             tail_rows = p.tail_rows_block; tail_heads = p.tail_heads_block; tail_tiles = p.tail_tiles_block;
             qmap_tail = 1;
             it.a_end = p.S;
-            it.b_coord0 = blk * p.B;
+            it.b_coord0 = it.k_row0 + blk * p.B;
+            it.own_map = 0;
+        } else if (w < p.items_block + p.items_last) {
+            // a shorter last block: its pairs, behind those of the full blocks
+            const int w2 = w - p.items_block;
+            g = quotient(w2, p.div_pairs_last);
+            pi = w2 - g * p.pairs_last;
+            seg_q0 = p.blk_q0 + p.N * p.B;
+            seg_len = p.last_len;
+            tiles = cdiv(p.last_len, kTile);
+            tail_rows = p.tail_rows_last; tail_heads = p.tail_heads_last; tail_tiles = p.tail_tiles_last;
+            qmap_tail = 4;
+            it.a_end = p.S;
+            it.b_coord0 = it.k_row0 + p.N * p.B;
             it.own_map = 0;
         } else {
-            const int w2 = w - p.items_block;
+            const int w2 = w - p.items_block - p.items_last;
             g = quotient(w2, p.div_pairs_sink);
             pi = w2 - g * p.pairs_sink;
             seg_q0 = 0;
@@ -144,7 +168,7 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             tail_rows = p.tail_rows_sink; tail_heads = p.tail_heads_sink; tail_tiles = p.tail_tiles_sink;
             qmap_tail = 2;
             it.a_end = 0;
-            it.b_coord0 = 0;
+            it.b_coord0 = it.k_row0;
             it.own_map = 1;
         }
         it.kv_head = g;
@@ -177,7 +201,7 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
                 s.qmap = 0;
                 s.box_rows = kTile;
             }
-            s.q_tok0 = seg_q0 + qt * kTile;
+            s.q_tok0 = it.seq * p.q_rows + seg_q0 + qt * kTile;
             s.limit0 = qt * kTile;
             s.end = min(qt * kTile + kTile, seg_len);
             if (s.valid) own_keys = max(own_keys, s.end);
@@ -191,8 +215,8 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
         it.kv_head = g;
         it.a_end = 0;
         const int split_lo = it.split * p.tiles_per_split * kTile;
-        it.b_coord0 = split_lo;
-        it.own_map = 0;
+        it.b_coord0 = it.seq * p.L + split_lo;
+        it.own_map = 2;
 #pragma unroll 1
         for (int x = 0; x < 2; ++x) {
             const int qt = 2 * pi + x;
@@ -200,12 +224,12 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             s.valid = qt < p.q_tiles;
             const int tok0 = qt * p.tok_per_tile;
             const int ntok = max(0, min(p.tok_per_tile, p.Q - tok0));
-            s.q_tok0 = tok0;
+            s.q_tok0 = it.seq * p.Q + tok0;
             s.q_head0 = g * p.G;
             s.row_div = p.G;
             s.ntok = ntok;
             s.nheads = p.G;
-            s.qmap = 0;
+            s.qmap = 3;
             s.box_rows = p.G * p.tok_per_tile;
             s.limit0 = p.n_video + tok0 - split_lo;
             // keys past the last row's limit are never visible; a split that lies past it altogether still takes
@@ -235,10 +259,7 @@ __device__ __forceinline__ void pass_on(int what, int wg, int quarter) {
 
 template <int D, int MODE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kAttnThreads, 1)
-attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tmap_q,
-            const __grid_constant__ CUtensorMap tmap_q_tail_block, const __grid_constant__ CUtensorMap tmap_q_tail_sink,
-            const __grid_constant__ CUtensorMap tmap_k_sink, const __grid_constant__ CUtensorMap tmap_v_sink,
-            const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v) {
+attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMaps maps) {
     using L = AttnSmem<D>;
     constexpr int NP = L::kPanels;
     extern __shared__ uint8_t smem_raw[];
@@ -266,7 +287,8 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
     __shared__ int s_item[kItems];       // 1 = a work item, -1 = no more work
     __shared__ WorkItem s_decoded[kItems];
     __shared__ float s_max[2][kTile];
-    __shared__ float2 s_sums[kSums][2][kTile];  // (row sum, reference maximum) of each warpgroup's tiles
+    __shared__ float2 s_sums[kSums][2][kTile];  // (row sum, reference maximum) of the even and of the odd tiles:
+                                              // added in this order, whichever warpgroup had them
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
@@ -299,13 +321,18 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
         mbar_init(smem_u32(&bars.clc), 1);
         mbar_init(smem_u32(&bars.clc_read), 1);
         fence_mbar_init();
-        tma_prefetch_desc(&tmap_q);
-        tma_prefetch_desc(&tmap_q_tail_block);
-        tma_prefetch_desc(&tmap_q_tail_sink);
-        tma_prefetch_desc(&tmap_k_sink);
-        tma_prefetch_desc(&tmap_v_sink);
-        tma_prefetch_desc(&tmap_k);
-        tma_prefetch_desc(&tmap_v);
+        if (MODE & 1) {
+            tma_prefetch_desc(&maps.q);
+            tma_prefetch_desc(&maps.k_sink);
+            tma_prefetch_desc(&maps.v_sink);
+            tma_prefetch_desc(&maps.k);
+            tma_prefetch_desc(&maps.v);
+        }
+        if (MODE & 2) {
+            tma_prefetch_desc(&maps.q_question);
+            tma_prefetch_desc(&maps.k_cache);
+            tma_prefetch_desc(&maps.v_cache);
+        }
     }
     if (warp == 12) {
         __syncwarp();
@@ -319,9 +346,10 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
     grid_launch_dependents();
     // The status word of the previous call on this workspace is cleared by the launch's first block, long before any wait
     // of this launch can have run out.
-    if (p.clear_status && blockIdx.x == 0 && tid == 0) {
+    if (blockIdx.x == 0 && tid == 0 && !p.keep_status) {
         p.hdr->detail = 0;
         *reinterpret_cast<volatile int32_t*>(&p.hdr->status) = 0;
+        if (MODE == 3) p.hdr_question->status = p.hdr_question->detail = 0;
     }
 
 #ifdef PEVLM_TRACE
@@ -396,13 +424,13 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
             // --------------------------------------------------------- TMA producer: K(s), then V(s - kQkAhead)
             if (lane == 0) {
                 struct Cursor {
-                    int k, j, nt, na, kv_head, b_coord0, own_map;
+                    int k, j, nt, na, kv_head, b_coord0, own_map, k_row0;
                 };
                 auto enter = [&](Cursor& c) {  // the cursor's item; false: no more work
                     if (!item_ready(c.k)) return false;
                     const WorkItem& it = s_decoded[c.k % kItems];
                     c.j = 0; c.nt = it.nt; c.na = it.na;
-                    c.kv_head = it.kv_head; c.b_coord0 = it.b_coord0; c.own_map = it.own_map;
+                    c.kv_head = it.kv_head; c.b_coord0 = it.b_coord0; c.own_map = it.own_map; c.k_row0 = it.k_row0;
                     return true;
                 };
                 Cursor kc{}, vc{};
@@ -424,7 +452,8 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
                                                       static_cast<uint32_t>(NP * 128 * ((it.s[0].valid ? it.s[0].box_rows : 0) +
                                                                                         (it.s[1].valid ? it.s[1].box_rows : 0))));
                             if (q.valid) {
-                                const CUtensorMap* qmap = q.qmap == 0 ? &tmap_q : q.qmap == 1 ? &tmap_q_tail_block : &tmap_q_tail_sink;
+                                const CUtensorMap* qmap = MODE == 2 || (MODE == 3 && q.qmap == 3) ? &maps.q_question
+                                                        : q.qmap == 0 ? &maps.q : q.qmap == 1 ? &maps.q_tail_block : q.qmap == 2 ? &maps.q_tail_sink : &maps.q_tail_last;
                                 const uint32_t bar = map_to_cta(smem_u32(&bars.q_full[qb]), 0);
                                 for (int h = 0; h < NP; ++h)
                                     tma_load_3d_pair(smem_base + L::kQ + qb * L::kQBytes + h * L::kQPanelBytes, qmap, h * 64,
@@ -437,9 +466,10 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
                     if (!k_end) {
                         const int j = kc.j++;
                         if (rank == 0 && j == max(0, kc.nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
-                        const CUtensorMap* map = (j < kc.na || kc.own_map != 0) ? &tmap_k_sink : &tmap_k;
+                        const CUtensorMap* map = MODE == 2 || (MODE == 3 && kc.own_map == 2) ? &maps.k_cache
+                                                 : (j < kc.na || kc.own_map == 1) ? &maps.k_sink : &maps.k;
                         const int n = j == kc.na - 1 ? n_a : j == kc.nt - 1 ? n_b : kTile;  // this CTA's keys: half of them
-                        const int row = (j < kc.na ? j * kTile : kc.b_coord0 + (j - kc.na) * kTile) + static_cast<int>(rank) * (n >> 1);
+                        const int row = (j < kc.na ? kc.k_row0 + j * kTile : kc.b_coord0 + (j - kc.na) * kTile) + static_cast<int>(rank) * (n >> 1);
                         const uint32_t slot = tiles % kRing;
                         if (tiles >= kRing) wait_s_full(tiles - kRing, kWaitKvFree);
                         if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[slot]), 2 * L::kKBytes);
@@ -456,8 +486,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
                             item_release(vc.k);
                         }
                         const int j = vc.j++;
-                        const CUtensorMap* map = (j < vc.na || vc.own_map != 0) ? &tmap_v_sink : &tmap_v;
-                        const int row = j < vc.na ? j * kTile : vc.b_coord0 + (j - vc.na) * kTile;
+                        const CUtensorMap* map = MODE == 2 || (MODE == 3 && vc.own_map == 2) ? &maps.v_cache
+                                                 : (j < vc.na || vc.own_map == 1) ? &maps.v_sink : &maps.v;
+                        const int row = j < vc.na ? vc.k_row0 + j * kTile : vc.b_coord0 + (j - vc.na) * kTile;
                         const uint32_t slot = u % kRing;
                         if (u >= kRing) wait_pv_done(u - kRing, kWaitKvFree);
                         if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[slot]), 2 * L::kVBytes);
@@ -543,7 +574,8 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
             const bool row_ok = qs.valid && (row_tok < qs.ntok) && (row_head < qs.nheads);
             const int tok = qs.q_tok0 + row_tok;
             const int head = qs.q_head0 + row_head;
-            const int split = it.split;
+            const int split = it.split, seq = it.seq;
+            const bool question = MODE == 2 || (MODE == 3 && it.own_map == 2);
             __syncwarp();
             if (lane == 0) item_release(k);
             wait_asleep(bars.sums_full[k % kSums], (k / kSums) & 1, kWaitSum);
@@ -557,8 +589,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
             tc_fence_after_sync();
             // 32 columns at a time, in a loop that stays one; 32 bytes per store: every lane writes whole sectors of
             // its own row
-            const size_t r = MODE == 0 ? static_cast<size_t>(tok) * p.Hq + head
-                                       : (static_cast<size_t>(split) * p.Q + tok) * p.Hq + head;
+            // (tok counts over the batch; the partials are ordered sequence, split, token, head)
+            const size_t r = !question ? static_cast<size_t>(tok) * p.Hq + head
+                                       : (static_cast<size_t>(seq * (p.n_splits - 1) + split) * p.Q + tok) * p.Hq + head;
 #pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t o[32];
@@ -569,7 +602,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(o_free_bar);
                 }
-                if (MODE == 0) {
+                if (!question) {
                     uint32_t wd[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e)
@@ -586,8 +619,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
                     for (int v = 0; v < 4; ++v) st_global_v8(p.part_o + r * D + c * 32 + v * 8, *reinterpret_cast<uint32_t(*)[8]>(&o[8 * v]));
                 }
             }
-            if (row_ok && MODE == 0 && p.lse) st_global_stream_f32(p.lse + static_cast<size_t>(head) * p.q_rows + tok, lse_val);
-            if (row_ok && MODE == 1) st_global_stream_f32(p.part_lse + r, lse_val);
+            if (row_ok && !question && p.lse)
+                st_global_stream_f32(p.lse + static_cast<size_t>(seq * p.Hq + head) * p.lse_stride + (tok - seq * p.q_rows), lse_val);
+            if (row_ok && question) st_global_stream_f32(p.part_lse + r, lse_val);
         }
     } else {
         // ------------------------------------------------------------- softmax, every other key tile
@@ -613,8 +647,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
             if (lane == 0) item_release(k);
             float m_own = -INFINITY;  // reference maximum (raw score units) this warpgroup's row sum is scaled by
             float l_run = 0.f;
+            const int first = static_cast<int>((t0 ^ static_cast<uint32_t>(wg)) & 1u);  // this warpgroup has the even or the odd tiles
 #pragma unroll 1
-            for (int j = static_cast<int>((t0 ^ static_cast<uint32_t>(wg)) & 1u); j < nt; j += 2) {
+            for (int j = first; j < nt; j += 2) {
                 const uint32_t t = t0 + j;
                 // keys of this tile that the row sees, and that every row of the query tile sees
                 const int max_col = j < na ? a_end - j * kTile : my_limit + 1 - (j - na) * kTile;
@@ -708,7 +743,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
 #endif
             }
             t0 += nt;
-            s_sums[k % kSums][wg][row] = make_float2(l_run, m_own);
+            s_sums[k % kSums][first][row] = make_float2(l_run, m_own);
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bars.sums_full[k % kSums]));
         }
@@ -731,18 +766,22 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtens
         __syncwarp();
         tmem_dealloc_pair(tmem_base, 512);
     }
-    if (tid == 0 && abort_flag != 0 && atomicCAS(&p.hdr->status, 0, PEVLM_ETIMEOUT) == 0)
-        p.hdr->detail = abort_flag * 1000000 + blockIdx.x;
+    if (tid == 0 && abort_flag != 0) {
+        const int detail = abort_flag * 1000000 + blockIdx.x;
+        if (atomicCAS(&p.hdr->status, 0, PEVLM_ETIMEOUT) == 0) p.hdr->detail = detail;
+        if (MODE == 3 && atomicCAS(&p.hdr_question->status, 0, PEVLM_ETIMEOUT) == 0) p.hdr_question->detail = detail;
+    }
 }
 
 cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cudaStream_t stream) {
-    if (p.n_items <= 0) return cudaSuccess;
+    const int64_t items = static_cast<int64_t>(p.n_items) * p.batch;
+    if (items <= 0) return cudaSuccess;
     const size_t smem = attn_smem_bytes(head_dim);
     // one cluster per work item; those that run take the rest from the hardware's queue
-    const unsigned grid = 2u * static_cast<unsigned>(p.n_items);
-    auto go = [&](auto kernel) { return launch_chained(kernel, grid, kAttnThreads, smem, stream, p, m.q, m.q_tail_block, m.q_tail_sink, m.k_sink, m.v_sink, m.k, m.v); };
-    if (p.mode == 0) return head_dim == 128 ? go(attn_kernel<128, 0>) : go(attn_kernel<64, 0>);
-    return head_dim == 128 ? go(attn_kernel<128, 1>) : go(attn_kernel<64, 1>);
+    const unsigned grid = 2u * static_cast<unsigned>(items);
+    auto go = [&](auto kernel) { return launch_chained(kernel, grid, kAttnThreads, smem, stream, p, m); };
+    if (head_dim == 128) return p.mode == 1 ? go(attn_kernel<128, 1>) : p.mode == 2 ? go(attn_kernel<128, 2>) : go(attn_kernel<128, 3>);
+    return p.mode == 1 ? go(attn_kernel<64, 1>) : p.mode == 2 ? go(attn_kernel<64, 2>) : go(attn_kernel<64, 3>);
 }
 
 }  // namespace pevlm

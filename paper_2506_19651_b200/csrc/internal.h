@@ -45,7 +45,7 @@ __device__ __forceinline__ int quotient(int a, const Divisor& b) {
 // global memory.  All kernels ask for the same split of the SM's memory (as much shared memory as there is), because an
 // SM has to run empty before it can change the split.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned threads, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
                                   const Args&... args) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
@@ -57,7 +57,7 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsi
     chained.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     chained.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t config{};
-    config.gridDim = dim3(grid);
+    config.gridDim = grid;
     config.blockDim = dim3(threads);
     config.dynamicSmemBytes = smem;
     config.stream = stream;
@@ -67,15 +67,18 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsi
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// What one launch of the attention kernel does.  mode 0: prefill rows (sink + blocks, or
-// full causal); mode 1: question rows against the assembled cache, split over keys.
+// What one launch of the attention kernel does, bit 0 of mode: prefill rows (sink + blocks, or full causal); bit 1:
+// question rows against the assembled cache, split over keys.
 struct AttnParams {
     int32_t mode;
+    int32_t batch;          // sequences, each with n_items work items
     int32_t S, B, N;        // prefill geometry (full causal: S = 0, B = n_video, N = 1)
     int32_t n_video;        // S + N*B
-    int32_t blk_key0;       // mode 0: K/V row of the first context block (S, or the cache row of a block range)
-    int32_t blk_q0;         // mode 0: row of q / o where the first context block starts (S, or 0 for a block range)
-    int32_t q_rows;         // mode 0: rows of q / o = row stride of lse
+    int32_t blk_key0;       // prefill: K/V row of the first context block (S, or the cache row of a block range)
+    int32_t blk_q0;         // prefill: row of q / o where the first context block starts (S, or 0 for a block range)
+    int32_t q_rows;         // prefill: rows of q / o of a sequence
+    int32_t kv_rows;        // prefill: rows of k / v of a sequence
+    int32_t lse_stride;     // prefill: row stride of lse
     int32_t Q, L;           // question length, total length
     int32_t Hq, Hkv, G;
     int32_t tiles_sink;     // ceil(S / 128)
@@ -84,33 +87,39 @@ struct AttnParams {
     int32_t pairs_sink;     // ceil(G * tiles_sink / 2) query-tile pairs per kv head
     int32_t pair_chunk;     // pairs of one (block, kv head) handed out together (see decode_item)
     int32_t items_block;    // work items over the context blocks, padded: N * Hkv * pair_chunk * chunks
-    int32_t n_items;        // all work items of the launch
+    int32_t last_len;       // tokens of one more, shorter context block behind the N full ones (0 = none)
+    int32_t pairs_last;     // query-tile pairs of it per kv head
+    int32_t items_last;     // Hkv * pairs_last
+    int32_t items_question; // question work items
+    int32_t n_items;        // all work items of a sequence
     // ragged last query tile of a segment (len % 128 rows): the tails of tail_heads q heads of one kv
     // group are packed into one 128-row tile, tail_tiles such tiles per (segment, kv head); 0 = no packing
     int32_t tail_rows_block, tail_heads_block, tail_tiles_block;
     int32_t tail_rows_sink, tail_heads_sink, tail_tiles_sink;
-    int32_t tok_per_tile;   // mode 1: question tokens per query tile = 128 / G
-    int32_t q_tiles;        // mode 1: ceil(Q / tok_per_tile)
-    int32_t n_splits;       // mode 1
-    int32_t tiles_per_split;// mode 1
-    Divisor div_per_chunk, div_pair_chunk, div_hkv, div_pairs_sink, div_g, div_splits, div_q_pairs;  // decode_item
+    int32_t tail_rows_last, tail_heads_last, tail_tiles_last;
+    int32_t tok_per_tile;   // question: tokens per query tile = 128 / G
+    int32_t q_tiles;        // question: ceil(Q / tok_per_tile)
+    int32_t n_splits;       // question
+    int32_t tiles_per_split;// question
+    Divisor div_items, div_per_chunk, div_pair_chunk, div_hkv, div_pairs_sink, div_pairs_last, div_g, div_splits, div_q_pairs;  // decode_item
     uint32_t wait_limit_ns; // longest a single device-side wait may last before the launch reports PEVLM_ETIMEOUT
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
-    __nv_bfloat16* o;       // mode 0: [n_video, Hq, d]
-    float* lse;             // mode 0: [Hq, n_video] or NULL
-    float* part_o;          // mode 1: [n_splits, Q, Hq, d] fp32
-    float* part_lse;        // mode 1: [n_splits, Q, Hq]
+    __nv_bfloat16* o;       // prefill: [batch * q_rows, Hq, d]
+    float* lse;             // prefill: [batch, Hq, lse_stride] or NULL
+    float* part_o;          // question: [batch, n_splits, Q, Hq, d] fp32
+    float* part_lse;        // question: [batch, n_splits, Q, Hq]
     WorkspaceHeader* hdr;
-    int32_t clear_status;   // 1 in the first launch of a call
+    WorkspaceHeader* hdr_question;  // mode 3: header of the question's workspace
+    int32_t keep_status;    // a later launch of the same call
 };
 
 struct MergeParams {
-    int32_t Q, Hq, d, n_splits;
+    int32_t batch, Q, Hq, d, n_splits;
     const float* part_o;
     const float* part_lse;
-    __nv_bfloat16* o;  // [Q, Hq, d]
-    float* lse;        // [Hq, Q] or NULL
+    __nv_bfloat16* o;  // [batch, Q, Hq, d]
+    float* lse;        // [batch, Hq, Q] or NULL
 };
 
 struct RopeParams {
@@ -129,10 +138,12 @@ struct RopeParams {
     const __nv_bfloat16* v_in;  // rows copied along: Hv heads of v_in to v_out (0 = none)
     __nv_bfloat16* v_out;
     int32_t Hv;
+    int32_t seq_len;  // tokens of a sequence, n_tokens = batch * seq_len (pos_ids [batch, seq_len], pos3 [batch, 3, seq_len])
+    Divisor div_seq;
     int32_t group;  // tokens per CTA (this and the divisors are set by launch_rope)
     Divisor div_hq, div_hkv;
     // multimodal RoPE: pos3 != NULL selects it; rotary pair i takes its position from component 0 for
-    // i < sec_end0, component 1 for i < sec_end1, else component 2; pos3 is [3, n_tokens]
+    // i < sec_end0, component 1 for i < sec_end1, else component 2
     const int32_t* pos3;
     int32_t sec_end0, sec_end1;
 };
@@ -142,6 +153,8 @@ struct CopySegments {
     uint4* dst[4];
     int64_t n_vec[4];  // 16-byte vectors per segment
     int64_t total;
+    int64_t src_stride[4], dst_stride;  // vectors from one sequence to the next
+    int32_t batch;
 };
 
 cudaError_t launch_rope(const RopeParams& p, int head_dim, cudaStream_t stream);
@@ -149,18 +162,19 @@ cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream);
 // Tensor maps of one attention launch.  q: [rows, Hq, d] with a 128-token box; q_tail_*: the same tensor with the
 // box of a packed ragged tail (heads x tail rows).  K and V each have two maps so that a ragged last key tile
 // reads zeros past the end of its range instead of a neighbour's rows: *_sink covers cache rows [0, S), k / v
-// cover the context blocks of the call (base at the first block's row) or, for the question attention, the cache.
+// cover the context blocks of the call (base at the first block's row).  q_question, k_cache, v_cache: the question rows
+// (box: one kv group's heads x the tokens of a tile) and the whole cache.
 struct AttnMaps {
-    CUtensorMap q, q_tail_block, q_tail_sink, k_sink, v_sink, k, v;
+    CUtensorMap q, q_tail_block, q_tail_sink, q_tail_last, k_sink, v_sink, k, v, q_question, k_cache, v_cache;
 };
 cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cudaStream_t stream);
 cudaError_t launch_wait_selftest(WorkspaceHeader* hdr, uint32_t limit_ns, cudaStream_t stream);
 // device address of the built-in scratch array of pevlm_query_attn_noalloc on the current device
 int noalloc_scratch_for_current_device(void** out);
+size_t query_workspace_bytes(const pevlm_shape_t* s);  // of pevlm_query_attn
 int check_query_args(const pevlm_shape_t* s, const void* q_question, const void* k_cache, const void* v_cache,
                      const void* o, const float* lse);
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream);
-size_t attn_smem_bytes(int head_dim);
 // error reporting shared by the host-side translation units: both record a text that
 // pevlm_last_cuda_error returns on the calling thread
 int cuda_fail(cudaError_t e, const char* what);      // returns PEVLM_ECUDA

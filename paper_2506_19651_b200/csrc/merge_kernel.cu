@@ -13,7 +13,7 @@ constexpr int kMergeMaxParts = 160;  // >= the largest split count (one split pe
 
 // Many rows (a prefill-sized question block): one thread per (row, 4 output columns), the splits one after
 // another; tens of thousands of threads hide the latency of the dependent loads.
-__global__ void merge_kernel(const __grid_constant__ MergeParams p) {
+__global__ void merge_kernel(MergeParams p) {
     grid_wait();
     grid_launch_dependents();
     const int vec_per_row = p.d / 4;
@@ -23,6 +23,11 @@ __global__ void merge_kernel(const __grid_constant__ MergeParams p) {
     const int64_t row = idx / vec_per_row;  // = tok * Hq + head
     const int v = static_cast<int>(idx % vec_per_row);
     const int n = p.n_splits;
+    const int64_t seq = blockIdx.y;
+    p.part_o += seq * n * rows * p.d;
+    p.part_lse += seq * n * rows;
+    p.o += seq * rows * p.d;
+    if (p.lse) p.lse += seq * rows;
     float m = -INFINITY;
     for (int s = 0; s < n; ++s) m = fmaxf(m, p.part_lse[s * rows + row]);
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -54,7 +59,7 @@ __global__ void merge_kernel(const __grid_constant__ MergeParams p) {
 // (lane l takes splits l, l + 32, ...) are requested together; the lanes reduce the maximum and the sum, leave
 // the normalised weights in shared memory, and the partial rows follow in chunks of kMergeChunk, all loads of a
 // chunk issued before the first is used.
-__global__ void __launch_bounds__(kMergeThreads) merge_rows_kernel(const __grid_constant__ MergeParams p) {
+__global__ void __launch_bounds__(kMergeThreads) merge_rows_kernel(MergeParams p) {
     __shared__ float weights[kMergeThreads / 32][kMergeMaxParts];
     grid_wait();
     grid_launch_dependents();
@@ -64,6 +69,11 @@ __global__ void __launch_bounds__(kMergeThreads) merge_rows_kernel(const __grid_
     const int64_t rows = static_cast<int64_t>(p.Q) * p.Hq;
     if (row >= rows) return;
     const int n = p.n_splits;
+    const int64_t seq = blockIdx.y;
+    p.part_o += seq * n * rows * p.d;
+    p.part_lse += seq * n * rows;
+    p.o += seq * rows * p.d;
+    if (p.lse) p.lse += seq * rows;
     const bool col_ok = lane * 4 < p.d;
     auto load_chunk = [&](int s0, float4 (&o)[kMergeChunk]) {
 #pragma unroll
@@ -120,13 +130,15 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream) {
     const int64_t rows = static_cast<int64_t>(p.Q) * p.Hq;
     if (rows <= 0) return cudaSuccess;
     const int rows_per_cta = kMergeThreads / 32;
-    if (rows <= static_cast<int64_t>(kNumSms) * rows_per_cta && p.n_splits <= kMergeMaxParts) {
+    const unsigned batch = static_cast<unsigned>(p.batch);
+    if (rows * batch <= static_cast<int64_t>(kNumSms) * rows_per_cta && p.n_splits <= kMergeMaxParts) {
         // at most one CTA per SM of warp-per-row work: the latency-oriented form
-        return launch_chained(merge_rows_kernel, static_cast<unsigned>((rows + rows_per_cta - 1) / rows_per_cta), kMergeThreads, 0,
-                              stream, p);
+        return launch_chained(merge_rows_kernel, dim3(static_cast<unsigned>((rows + rows_per_cta - 1) / rows_per_cta), batch),
+                              kMergeThreads, 0, stream, p);
     }
     const int64_t n = rows * (p.d / 4);
-    return launch_chained(merge_kernel, static_cast<unsigned>((n + kMergeThreads - 1) / kMergeThreads), kMergeThreads, 0, stream, p);
+    return launch_chained(merge_kernel, dim3(static_cast<unsigned>((n + kMergeThreads - 1) / kMergeThreads), batch), kMergeThreads, 0,
+                          stream, p);
 }
 
 }  // namespace pevlm

@@ -49,7 +49,7 @@ extern "C" int pevlm_query_attn_noalloc(const pevlm_shape_t* shape, const void* 
     // pointer by the same checks as the workspace entry point, then a shape beyond the array.
     const int bad = pevlm::check_query_args(shape, q_question, k_cache, v_cache, o, lse);
     if (bad != PEVLM_OK) return bad;
-    const size_t need = pevlm_workspace_bytes(shape, PEVLM_WS_QUERY);
+    const size_t need = pevlm::query_workspace_bytes(shape);
     if (need > kScratchBytes) {
         char text[160];
         snprintf(text, sizeof(text), "pevlm_query_attn_noalloc: this shape needs %zu scratch bytes, the built-in array holds %zu",

@@ -92,9 +92,11 @@ __global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(cons
             const int t = a / HALF, i = a % HALF;
             const int64_t tok = tok0 + t;
             // one position per token, or, multimodal, the component that the rotary pair's section picks
-            const int64_t pos = p.pos3 ? p.pos3[(i < p.sec_end0 ? 0 : i < p.sec_end1 ? 1 : 2) * p.n_tokens + tok]
+            const int64_t seq = p.n_tokens == p.seq_len ? 0 : quotient(static_cast<int>(tok), p.div_seq);
+            const int comp = i < p.sec_end0 ? 0 : i < p.sec_end1 ? 1 : 2;
+            const int64_t pos = p.pos3 ? p.pos3[(2 * seq + comp) * p.seq_len + tok]
                               : p.pos_ids ? p.pos_ids[tok]
-                                          : p.first_token + tok;
+                                          : p.first_token + tok - seq * p.seq_len;
             double sn, cn;
             sincos(__dmul_rn(static_cast<double>(pos), p.inv_freq[i]), &sn, &cn);
             const int e = i % 8, w = i / 8;
@@ -196,6 +198,7 @@ cudaError_t launch_rope(const RopeParams& params, int head_dim, cudaStream_t str
     while (p.group > 1 && p.n_tokens < 4 * resident * p.group) p.group /= 2;
     p.div_hq = make_divisor(p.Hq);
     p.div_hkv = make_divisor(p.Hkv);
+    p.div_seq = make_divisor(p.seq_len);
     const int64_t groups = (p.n_tokens + p.group - 1) / p.group;
     const unsigned grid = static_cast<unsigned>(groups < resident ? groups : resident);
     return head_dim == 128 ? launch_chained(rope_kernel<128>, grid, kRopeThreads, sizeof(RopeSmem<128>), stream, p)

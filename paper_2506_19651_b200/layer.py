@@ -36,16 +36,23 @@ class LayerBuffers:
         self.ws_query = alloc((pb.pevlm_workspace_bytes(s, pb.WS_QUERY),), torch.uint8, zero=True)
 
 
-KERNELS_PER_PASS = 7  # rope, V copy, prefill attention, rope, V copy, question attention, merge
+KERNELS_PER_PASS = 3          # rope and V copy, attention of video and question rows, merge
+KERNELS_PER_PASS_BY_CALL = 7  # with `mark`: rope, V copy, prefill attention, rope, V copy, question attention, merge
 
 
 def layer_forward(buf: LayerBuffers, q, k, v, mark=None):
     """q [L,Hq,d], k, v [L,Hkv,d]: un-roped bf16 device tensors of the whole stream.
     Leaves O/LSE of the video rows and of the question rows in `buf`.  `mark(name)`, if
-    given, is called before the first call and after each C-ABI call (for event timing)."""
+    given, is called before the first call and after each C-ABI call (for event timing); without it the pass is one
+    call (pevlm_layer_forward)."""
     s = buf.shape
     nv, Q = s.n_video, s.query_len
-    mark = mark or (lambda name: None)
+    if mark is None:
+        if s.batch == 1:
+            pb.pevlm_layer_forward(s, q, k, v, buf.q_video, buf.q_question, buf.k_cache, buf.v_cache, buf.o_video,
+                                   buf.lse_video, buf.o_question, buf.lse_question, buf.ws_prefill, buf.ws_query)
+            return buf
+        mark = lambda name: None
     mark("start")
     if nv > 0:
         # K goes straight into its cache slot; Q is roped into a scratch copy
@@ -73,45 +80,34 @@ def ragged_layer_forward(q, k, v, S, B, N, B_last, Q, theta, scale=0.0, alloc=No
     remainder as one shorter block).  q [L,Hq,d], k, v [L,Hkv,d] un-roped device tensors of the whole
     stream, L = S + (N-1)*B + B_last + Q.  Returns (o_video, lse_video, o_question, lse_question, workspaces).
 
-    The uniform prefix runs through pevlm_parallel_prefill_attn, the last block through pevlm_block_attn
-    against the same cache, the question through pevlm_query_attn; positions are the global ones.
+    One call (pevlm_layer_forward with the length of the last block); positions are the global ones.
     `alloc(shape, dtype, zero)` replaces torch.empty / torch.zeros (see LayerBuffers).
     """
     import torch
     Hq, Hkv, d = q.shape[1], k.shape[1], q.shape[2]
-    nv_full = S + (N - 1) * B
-    nv = nv_full + B_last
+    nv = S + (N - 1) * B + B_last
     L = nv + Q
     assert N >= 1 and 1 <= B_last <= B and q.shape[0] == L
     dev, bf, f32 = q.device, torch.bfloat16, torch.float32
-    s_all = pb.make_shape(nv, 1, 0, Q, Hq, Hkv, d, theta=theta, scale=scale)          # [video | question]
-    s_full = pb.make_shape(S, B, N - 1, 0, Hq, Hkv, d, theta=theta, scale=scale)      # uniform prefix
-    s_last = pb.make_shape(S, B_last, 1, 0, Hq, Hkv, d, theta=theta, scale=scale)     # the shorter last block
+    s = pb.make_shape(S, B, N, Q, Hq, Hkv, d, theta=theta, scale=scale)
     if alloc is None:
         def alloc(shp, dtype, zero=False):
-            return (torch.zeros if zero else torch.empty)(shp, dtype=dtype, device=dev)
+            return torch.empty(shp, dtype=dtype, device=dev)
     q_roped = alloc((L, Hq, d), bf)
     k_cache = alloc((L, Hkv, d), bf)
     v_cache = alloc((L, Hkv, d), bf)
     o_video = alloc((nv, Hq, d), bf)
     lse_video = alloc((Hq, nv), f32)
-    lse_last = alloc((Hq, B_last), f32)
     o_question = alloc((max(Q, 1), Hq, d), bf)
     lse_question = alloc((Hq, max(Q, 1)), f32)
-    ws = [alloc((pb.pevlm_workspace_bytes(s, which),), torch.uint8, zero=True)
-          for s, which in ((s_full, pb.WS_PREFILL), (s_last, pb.WS_PREFILL), (s_all, pb.WS_QUERY))]
-    pb.pevlm_rope_qk(s_all, q, k, q_roped, k_cache, 0, L)
-    pb.pevlm_assemble_kv(s_all, None, v[:nv], None, v[nv:] if Q > 0 else None, k_cache, v_cache)
-    lse_full = alloc((Hq, max(nv_full, 1)), f32)
-    if nv_full > 0:
-        pb.pevlm_parallel_prefill_attn(s_full, q_roped[:nv_full], k_cache[:nv_full], v_cache[:nv_full],
-                                       o_video[:nv_full], lse_full, ws[0])
-        lse_video[:, :nv_full] = lse_full
-    pb.pevlm_block_attn(s_last, q_roped[nv_full:nv], k_cache, v_cache, nv_full, L, o_video[nv_full:nv], lse_last, ws[1])
-    lse_video[:, nv_full:] = lse_last
-    if Q > 0:
-        pb.pevlm_query_attn(s_all, q_roped[nv:], k_cache, v_cache, o_question, lse_question, ws[2])
-    return o_video, lse_video, o_question, lse_question, ws
+    # the launch writes the status words; a part that is not launched has none to write
+    ws_prefill = alloc((pb.pevlm_workspace_bytes(s, pb.WS_PREFILL),), torch.uint8)
+    ws_query = alloc((pb.pevlm_workspace_bytes(s, pb.WS_QUERY),), torch.uint8, zero=Q == 0)
+    if Q == 0:
+        ws_query[:256].zero_()
+    pb.pevlm_layer_forward(s, q, k, v, q_roped, q_roped[nv:], k_cache, v_cache, o_video, lse_video, o_question, lse_question,
+                           ws_prefill, ws_query, last_len=B_last)
+    return o_video, lse_video, o_question, lse_question, [ws_prefill, ws_query]
 
 
 class StreamingWindow:
@@ -149,9 +145,8 @@ class StreamingWindow:
         S = self.S
         o = torch.empty((S, self.Hq, self.d), dtype=self._bf, device=self._dev)
         lse = torch.empty((self.Hq, S), dtype=self._f32, device=self._dev)
-        pb.pevlm_rope_qk(self.s_sink, q, k, self.q_buf[:S], self.k_cache[:S], 0, S)
-        pb.pevlm_assemble_kv(self.s_sink, None, v, None, None, self.k_cache, self.v_cache)
-        pb.pevlm_parallel_prefill_attn(self.s_sink, self.q_buf[:S], self.k_cache[:S], self.v_cache[:S], o, lse, self.ws_sink)
+        pb.pevlm_rope_qkv(self.s_sink, q, k, v, self.q_buf, self.k_cache, self.v_cache, 0, S)
+        pb.pevlm_parallel_prefill_attn(self.s_sink, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_sink)
         return o, lse
 
     def append_block(self, q, k, v):
@@ -162,10 +157,8 @@ class StreamingWindow:
         row0 = S + (t % self.W) * B
         o = torch.empty((B, self.Hq, self.d), dtype=self._bf, device=self._dev)
         lse = torch.empty((self.Hq, B), dtype=self._f32, device=self._dev)
-        pb.pevlm_rope_qk(self.s_block, q, k, self.q_buf[:B], self.k_cache[row0:row0 + B], S + t * B, B)
-        # the V rows go to cache rows [row0, row0 + B): the copy call with those rows as its trailing segment
-        pb.pevlm_assemble_kv(self._shape(row0, 1, 0, B), None, None, None, v, self.k_cache, self.v_cache)
-        pb.pevlm_block_attn(self.s_block, self.q_buf[:B], self.k_cache, self.v_cache, row0, self.rows, o, lse, self.ws_block)
+        pb.pevlm_rope_qkv(self.s_block, q, k, v, self.q_buf, self.k_cache[row0:], self.v_cache[row0:], S + t * B, B)
+        pb.pevlm_block_attn(self.s_block, self.q_buf, self.k_cache, self.v_cache, row0, self.rows, o, lse, self.ws_block)
         self.blocks_seen = t + 1
         return o, lse
 
@@ -179,7 +172,6 @@ class StreamingWindow:
         s = self._shape(nv, 1, 0, Qn)
         o = torch.empty((Qn, self.Hq, self.d), dtype=self._bf, device=self._dev)
         lse = torch.empty((self.Hq, Qn), dtype=self._f32, device=self._dev)
-        pb.pevlm_rope_qk(s, q, k, self.q_buf[:Qn], self.k_cache[nv:nv + Qn], self.S + self.blocks_seen * self.B, Qn)
-        pb.pevlm_assemble_kv(s, None, None, None, v, self.k_cache, self.v_cache)
-        pb.pevlm_query_attn(s, self.q_buf[:Qn], self.k_cache[:nv + Qn], self.v_cache[:nv + Qn], o, lse, self.ws_query)
+        pb.pevlm_rope_qkv(s, q, k, v, self.q_buf, self.k_cache[nv:], self.v_cache[nv:], self.S + self.blocks_seen * self.B, Qn)
+        pb.pevlm_query_attn(s, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_query)
         return o, lse
