@@ -132,6 +132,7 @@ static SegPlan plan_segment(int len, int G) {
 // ---- question-attention decomposition (shared by the launch, the workspace size and the stats)
 struct QueryPlan {
     int tok_per_tile, q_tiles, total_kv_tiles, n_splits, tiles_per_split;
+    int pieces, pieces_per_split;  // decode kernel (at most kDecodeRows rows per kv head): 16-key pieces; 0 = tile kernel
 };
 
 static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false, int last_len = 0) {
@@ -155,6 +156,18 @@ static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false,
     }
     if (want < 1) want = 1;
     if (want > q.total_kv_tiles) want = q.total_kv_tiles;
+    q.pieces = q.pieces_per_split = 0;
+    if (!beside_prefill && s->query_len * G <= kDecodeRows) {
+        // one CTA for every SM, no range shorter than the eight pieces its warps take at a time
+        q.pieces = static_cast<int>((L + 15) / 16);
+        int64_t splits = kNumSms / (static_cast<int64_t>(s->num_kv_heads) * s->batch);
+        if (splits > (q.pieces + 7) / 8) splits = (q.pieces + 7) / 8;
+        if (splits < 1) splits = 1;
+        q.pieces_per_split = static_cast<int>((q.pieces + splits - 1) / splits);
+        q.tiles_per_split = 0;
+        q.n_splits = (q.pieces + q.pieces_per_split - 1) / q.pieces_per_split;
+        return q;
+    }
     q.tiles_per_split = (q.total_kv_tiles + want - 1) / want;
     q.n_splits = (q.total_kv_tiles + q.tiles_per_split - 1) / q.tiles_per_split;
     return q;
@@ -518,6 +531,32 @@ int pevlm_block_attn(const pevlm_shape_t* s, const void* q_blocks, const void* k
                           first_key_row, cache_rows);
 }
 
+static int decode(const pevlm_shape_t* s, const QueryPlan& qp, const void* q, const void* k, const void* v, void* o, float* lse,
+                  void* workspace, cudaStream_t st) {
+    const int d = s->head_dim;
+    AttnParams a = common_params(s);
+    a.n_splits = qp.n_splits;
+    DecodeParams p;
+    p.Q = a.Q; p.L = a.L; p.n_video = a.n_video; p.Hq = a.Hq; p.Hkv = a.Hkv; p.G = a.G;
+    p.pieces = qp.pieces; p.pieces_per_split = qp.pieces_per_split; p.n_splits = qp.n_splits;
+    p.scale = a.scale; p.scale_log2 = a.scale_log2;
+    p.hdr = static_cast<WorkspaceHeader*>(workspace);
+    for (int b = 0; b < s->batch; b += 32768) {
+        a.batch = p.batch = s->batch - b < 32768 ? s->batch - b : 32768;
+        a.part_o = p.part_o = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + kStatusBytes);
+        a.part_lse = p.part_lse = p.part_o + static_cast<size_t>(p.batch) * p.n_splits * p.Q * p.Hq * d;
+        const int64_t q0 = static_cast<int64_t>(b) * p.Q, k0 = static_cast<int64_t>(b) * p.L;
+        p.q = rows_of(q, q0, p.Hq, d);
+        p.k = rows_of(k, k0, p.Hkv, d);
+        p.v = rows_of(v, k0, p.Hkv, d);
+        const cudaError_t e = launch_decode(p, d, st);
+        if (e != cudaSuccess) return cuda_fail(e, "decode launch");
+        const int rc = merge_question(a, d, const_cast<__nv_bfloat16*>(rows_of(o, q0, p.Hq, d)), lse ? lse + p.Hq * q0 : nullptr, st);
+        if (rc != PEVLM_OK) return rc;
+    }
+    return PEVLM_OK;
+}
+
 int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void* k_cache, const void* v_cache, void* o,
                      float* lse, void* workspace, size_t workspace_bytes, void* stream) {
     int rc = check_query_args(s, q_question, k_cache, v_cache, o, lse);
@@ -529,6 +568,7 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
     if (rc != PEVLM_OK) return rc;
     const int d = s->head_dim;
     const QueryPlan qp = plan_query(s);
+    if (qp.pieces > 0) return decode(s, qp, q_question, k_cache, v_cache, o, lse, workspace, static_cast<cudaStream_t>(stream));
     AttnParams p = common_params(s);
     add_question(p, qp);
     p.div_items = make_divisor(p.n_items);
@@ -676,6 +716,13 @@ int pevlm_tile_stats(const pevlm_shape_t* s, int which, int64_t* tiles, double* 
         cols *= s->num_kv_heads;
     } else if (which == PEVLM_WS_QUERY) {
         const QueryPlan qp = plan_query(s);
+        if (qp.pieces > 0) {  // decode kernel: 16 or 32 rows against 16 keys at a time, counted in key tiles of 128
+            n_tiles = (qp.pieces + 7) / 8 * static_cast<int64_t>(s->num_kv_heads);
+            *tiles = n_tiles * s->batch;
+            const int rows = s->query_len * (s->num_q_heads / s->num_kv_heads);
+            *flops = 4.0 * d * (rows > 16 ? 32 : 16) * 16.0 * qp.pieces * s->num_kv_heads * s->batch;
+            return PEVLM_OK;
+        }
         for (int qt = 0; qt < qp.q_tiles; ++qt) {
             const int tok0 = qt * qp.tok_per_tile;
             const int ntok = s->query_len - tok0 < qp.tok_per_tile ? s->query_len - tok0 : qp.tok_per_tile;

@@ -114,6 +114,23 @@ struct AttnParams {
     int32_t keep_status;    // a later launch of the same call
 };
 
+constexpr int kDecodeRows = 32;  // most rows (question tokens x heads of a kv group) of the decode kernel
+
+// Question attention of a few rows, see decode_kernel.cu.
+struct DecodeParams {
+    const __nv_bfloat16* q;  // [batch, Q, Hq, d]
+    const __nv_bfloat16* k;  // [batch, L, Hkv, d]
+    const __nv_bfloat16* v;
+    float* part_o;           // [batch, n_splits, Q, Hq, d]
+    float* part_lse;         // [batch, n_splits, Q, Hq]
+    WorkspaceHeader* hdr;
+    int32_t batch, Q, L, n_video, Hq, Hkv, G;
+    int32_t pieces;            // ceil(L / 16)
+    int32_t pieces_per_split;
+    int32_t n_splits;
+    float scale, scale_log2;
+};
+
 struct MergeParams {
     int32_t batch, Q, Hq, d, n_splits;
     const float* part_o;
@@ -174,6 +191,7 @@ int noalloc_scratch_for_current_device(void** out);
 size_t query_workspace_bytes(const pevlm_shape_t* s);  // of pevlm_query_attn
 int check_query_args(const pevlm_shape_t* s, const void* q_question, const void* k_cache, const void* v_cache,
                      const void* o, const float* lse);
+cudaError_t launch_decode(const DecodeParams& p, int head_dim, cudaStream_t stream);
 cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream);
 // error reporting shared by the host-side translation units: both record a text that
 // pevlm_last_cuda_error returns on the calling thread
