@@ -226,8 +226,8 @@ int pevlm_read_status(const void* workspace, void* stream, int32_t* status, int3
 
 /*
  * Self-test of the failure path (the paper has no counterpart): launches one thread block that
- * waits, with the library's bounded wait, on a barrier nothing ever arrives on.  After limit_ns
- * (1 us .. 100 ms) the wait gives up, the kernel records PEVLM_ETIMEOUT with wait id 99 in the
+ * waits, with the library's bounded wait, on a barrier nothing ever arrives on, until every wait has
+ * given up and limit_ns (1 us .. 100 ms) have passed; the kernel records PEVLM_ETIMEOUT with wait id 99 in the
  * header of `workspace` (>= 256 bytes, 256-byte aligned) and ends normally; the context stays
  * usable and the next call on the same workspace clears the status.  Nothing traps or faults.
  */

@@ -368,7 +368,7 @@ static AttnParams common_params(const pevlm_shape_t* s, int last_len = 0) {
     p.Hq = s->num_q_heads; p.Hkv = s->num_kv_heads; p.G = p.Hq / p.Hkv;
     p.scale = resolve_scale(s);
     p.scale_log2 = p.scale * 1.4426950408889634f;
-    p.wait_limit_ns = kDefaultWaitLimitNs;
+    p.wait_tries = kDefaultWaitTries;
     return p;
 }
 

@@ -22,17 +22,20 @@
 // into registers, which is the first thing its softmax does: the scores of a softmax warpgroup's next tile are ready
 // long before it has finished this one, and neither the tensor pipe's latency nor the hand-offs between the warps are
 // on its path.  QK runs three tiles ahead of PV, over the boundaries of work items too.
-// What bounds it: two softmax warpgroups that never wait take 2,390 cycles for two key tiles beside running MMAs, the
-// MMAs 1,024 a tile (both measured free-running); reached are 1,480 cycles a tile on long work items (1,741 before, with
-// two query tiles and two softmax warpgroups per CTA) and 2,400 with four tiles an item (2,710 before).  On B200, back
-// to back under the 1 kW cap: 50K tokens 1.708 -> 1.546 ms, 12.6K 0.249 -> 0.228, 256-token blocks 0.322 -> 0.296,
-// 8,192-token blocks 4.97 -> 4.54.  Two things took more than the schedule itself:
+// What bounds it: back to back, the 1 kW cap (all sizes from 12K tokens on run at 1.4 to 1.6 GHz): what a tile costs in
+// energy, for which idle cycles count too.  At a given clock, the softmax: two warpgroups that never wait take 2,390
+// cycles for two key tiles beside running MMAs, the MMAs 1,024 a tile (both measured free-running).  Reached are 1,460
+// cycles a tile on long work items (1,741 before, with two query tiles and two softmax warpgroups per CTA) and 1,830 with
+// four tiles an item (2,710 before).  Back to back: 50K tokens 1.708 -> 1.49 ms, 12.6K 0.249 -> 0.213, 256-token blocks
+// 0.322 -> 0.257, 8,192-token blocks 4.97 -> 4.5.  Two things took more than the schedule itself:
 //   - the two softmax warps that share a scheduler take turns on its special-function unit (left alone they fall into
 //     step, form their exponentials at the same time and leave the unit idle at the same time: 1,741 cycles a tile);
 //   - instruction fetch.  What a work item runs (all roles, masks and item ends included) has to stay near the size of
 //     the SM's instruction cache: at 73 KB of code four-tile items lost more time to missing instructions than to
-//     anything else (26 % of the fetches missed), 55 KB run them 15 % faster.  Hence one instantiation per mode,
-//     loops that stay loops wherever the registers' indices allow it, waits that expand to little, no divisions.
+//     anything else (26 % of the fetches missed, 0.348 ms), at 55 KB they took 0.296 ms, at 50 KB 0.257.  Hence one
+//     instantiation per mode, loops that stay loops wherever the registers' indices allow it, waits that expand to
+//     little, no divisions, and warp-uniform values that the compiler knows to be uniform (the MMA warps' descriptors
+//     then live in uniform registers instead of being moved there for every MMA: 10 KB of code).
 // Every wait on an mbarrier is bounded; an expired wait records PEVLM_ETIMEOUT and the CTA still runs to its
 // normal end (waits become short), so TMEM is always released.
 #include "internal.h"
@@ -84,6 +87,7 @@ static size_t attn_smem_bytes(int head_dim) {
 struct QSlot {
     int valid;
     int q_tok0, q_head0, row_div, ntok, nheads, qmap, box_rows;
+    int per_div;  // ceil(2^16 / row_div): r / row_div = r * per_div >> 16 for r < 128
     int limit0;  // last visible key of row token 0, counted from the first key of the own range
     int end;     // keys of the own range that the tile's rows can see at all
 };
@@ -107,6 +111,8 @@ extern "C" int pevlm_debug_waits(unsigned* host_out) {
 }
 #endif
 
+// A value that is the same in all lanes of a warp, told to the compiler, so that what depends on it stays in uniform registers.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 __device__ __forceinline__ int cdiv(int a, int b) { return (a + b - 1) / b; }
 
 // MODE: bit 0 = the launch has prefill items, bit 1 = it has question items (handed out first: they are the longest).
@@ -238,6 +244,8 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             if (s.valid) own_keys = max(own_keys, max(1, s.end));
         }
     }
+#pragma unroll 1
+    for (int x = 0; x < 2; ++x) it.s[x].per_div = static_cast<int>(ceilf(__fdiv_rn(65536.f, static_cast<float>(it.s[x].row_div))));
     it.na = cdiv(it.a_end, kTile);
     it.nt = own_keys > 0 ? it.na + cdiv(own_keys, kTile) : 0;
     it.n_a = (it.a_end - (it.na - 1) * kTile + 15) & ~15;
@@ -283,7 +291,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     __shared__ Bars bars;
     __shared__ __align__(16) uint4 s_clc;
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
+    __shared__ WaitState wait_state;
     __shared__ int s_item[kItems];       // 1 = a work item, -1 = no more work
     __shared__ WorkItem s_decoded[kItems];
     __shared__ float s_max[2][kTile];
@@ -291,14 +299,15 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                                               // added in this order, whichever warpgroup had them
 
     const int tid = threadIdx.x;
-    const int warp = tid >> 5;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // the same in all lanes, and known to be
     const int lane = tid & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     constexpr int kConsumerWarps = 1 + 8 + 4;  // producer, softmax, epilogue; in the first CTA also the MMA warps
 
     if (tid == 0) {
-        abort_flag = 0;
+        wait_state.tries = p.wait_tries;
+        wait_state.expired = 0;
         for (int i = 0; i < kItems; ++i) {
             mbar_init(smem_u32(&bars.item_full[i]), 1);
             mbar_init(smem_u32(&bars.item_free[i]), kConsumerWarps + (rank == 0 ? 2 : 0));
@@ -341,7 +350,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     tc_fence_before_sync();
     cluster_sync_all();  // also: the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after_sync();
-    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t tmem_base = uniform(tmem_base_slot);
     grid_wait();  // nothing above touches global memory
     grid_launch_dependents();
     // The status word of the previous call on this workspace is cleared by the launch's first block, long before any wait
@@ -365,10 +374,10 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
 #define PEVLM_WAIT_ACCOUNT(which, call) call
 #endif
     auto wait = [&](const uint64_t& bar, uint32_t parity, int which) {
-        PEVLM_WAIT_ACCOUNT(which, mbar_wait(smem_u32(&bar), parity, smem_u32(&abort_flag), p.wait_limit_ns, which));
+        PEVLM_WAIT_ACCOUNT(which, mbar_wait(smem_u32(&bar), parity, wait_state, which));
     };
     auto wait_asleep = [&](const uint64_t& bar, uint32_t parity, int which) {
-        PEVLM_WAIT_ACCOUNT(which, mbar_wait<100>(smem_u32(&bar), parity, smem_u32(&abort_flag), p.wait_limit_ns, which));
+        PEVLM_WAIT_ACCOUNT(which, mbar_wait<100>(smem_u32(&bar), parity, wait_state, which));
     };
     // k-th item of the pair: wait for it, read from s_decoded[k % kItems], then give the slot back (once per warp)
     auto item_ready = [&](int k) {
@@ -416,21 +425,23 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     const int first = clc_first_block(smem_u32(&s_clc));
                     fence_proxy_async_smem();  // the answer is written again by the asynchronous proxy
                     if (rank == 1) mbar_arrive_cluster(map_to_cta(smem_u32(&bars.clc_read), 0));
-                    w = (first < 0 || abort_flag != 0) ? -1 : first >> 1;
+                    w = (first < 0 || *static_cast<volatile int*>(&wait_state.expired) != 0) ? -1 : first >> 1;
                     ++asked;
                 }
             }
         } else if (warp == 13) {
             // --------------------------------------------------------- TMA producer: K(s), then V(s - kQkAhead)
-            if (lane == 0) {
+            // (The whole warp runs this with uniform values; single lanes issue.)
+            {
                 struct Cursor {
                     int k, j, nt, na, kv_head, b_coord0, own_map, k_row0;
                 };
                 auto enter = [&](Cursor& c) {  // the cursor's item; false: no more work
-                    if (!item_ready(c.k)) return false;
+                    if (!uniform(item_ready(c.k))) return false;
                     const WorkItem& it = s_decoded[c.k % kItems];
-                    c.j = 0; c.nt = it.nt; c.na = it.na;
-                    c.kv_head = it.kv_head; c.b_coord0 = it.b_coord0; c.own_map = it.own_map; c.k_row0 = it.k_row0;
+                    c.j = 0; c.nt = uniform(it.nt); c.na = uniform(it.na);
+                    c.kv_head = uniform(it.kv_head); c.b_coord0 = uniform(it.b_coord0); c.own_map = uniform(it.own_map);
+                    c.k_row0 = uniform(it.k_row0);
                     return true;
                 };
                 Cursor kc{}, vc{};
@@ -444,20 +455,21 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                         if (!k_end) {
                             const WorkItem& it = s_decoded[kc.k % kItems];
                             const QSlot& q = it.s[rank];
-                            n_a = it.n_a; n_b = it.n_b;
+                            n_a = uniform(it.n_a); n_b = uniform(it.n_b);
                             const int qb = kc.k & 1;
                             if (kc.k >= 2) wait(bars.q_free[qb], ((kc.k >> 1) - 1) & 1, kWaitQFree);
-                            if (rank == 0)
+                            if (rank == 0 && lane == 0)
                                 mbar_arrive_expect_tx(smem_u32(&bars.q_full[qb]),
                                                       static_cast<uint32_t>(NP * 128 * ((it.s[0].valid ? it.s[0].box_rows : 0) +
                                                                                         (it.s[1].valid ? it.s[1].box_rows : 0))));
-                            if (q.valid) {
-                                const CUtensorMap* qmap = MODE == 2 || (MODE == 3 && q.qmap == 3) ? &maps.q_question
-                                                        : q.qmap == 0 ? &maps.q : q.qmap == 1 ? &maps.q_tail_block : q.qmap == 2 ? &maps.q_tail_sink : &maps.q_tail_last;
+                            if (uniform(q.valid)) {
+                                const int qm = uniform(q.qmap), q_head0 = uniform(q.q_head0), q_tok0 = uniform(q.q_tok0);
+                                const CUtensorMap* qmap = MODE == 2 || (MODE == 3 && qm == 3) ? &maps.q_question
+                                                        : qm == 0 ? &maps.q : qm == 1 ? &maps.q_tail_block : qm == 2 ? &maps.q_tail_sink : &maps.q_tail_last;
                                 const uint32_t bar = map_to_cta(smem_u32(&bars.q_full[qb]), 0);
                                 for (int h = 0; h < NP; ++h)
                                     tma_load_3d_pair(smem_base + L::kQ + qb * L::kQBytes + h * L::kQPanelBytes, qmap, h * 64,
-                                                     q.q_head0, q.q_tok0, bar);
+                                                     q_head0, q_tok0, bar);
                             }
                         }
                     }
@@ -465,14 +477,14 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     // tensor map and arrive as zeros: a ragged last tile never brings in a neighbour's rows.
                     if (!k_end) {
                         const int j = kc.j++;
-                        if (rank == 0 && j == max(0, kc.nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
+                        if (rank == 0 && lane == 0 && j == max(0, kc.nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
                         const CUtensorMap* map = MODE == 2 || (MODE == 3 && kc.own_map == 2) ? &maps.k_cache
                                                  : (j < kc.na || kc.own_map == 1) ? &maps.k_sink : &maps.k;
                         const int n = j == kc.na - 1 ? n_a : j == kc.nt - 1 ? n_b : kTile;  // this CTA's keys: half of them
                         const int row = (j < kc.na ? kc.k_row0 + j * kTile : kc.b_coord0 + (j - kc.na) * kTile) + static_cast<int>(rank) * (n >> 1);
                         const uint32_t slot = tiles % kRing;
                         if (tiles >= kRing) wait_s_full(tiles - kRing, kWaitKvFree);
-                        if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[slot]), 2 * L::kKBytes);
+                        if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[slot]), 2 * L::kKBytes);
                         const uint32_t bar = map_to_cta(smem_u32(&bars.k_full[slot]), 0);
                         for (int h = 0; h < NP; ++h)
                             tma_load_3d_pair(smem_base + L::kK + slot * L::kKBytes + h * L::kKPanelBytes, map, h * 64, kc.kv_head, row, bar);
@@ -483,7 +495,8 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                         const uint32_t u = s - kQkAhead;
                         if (vc.j == vc.nt) {
                             enter(vc);
-                            item_release(vc.k);
+                            __syncwarp();
+                            if (lane == 0) item_release(vc.k);
                         }
                         const int j = vc.j++;
                         const CUtensorMap* map = MODE == 2 || (MODE == 3 && vc.own_map == 2) ? &maps.v_cache
@@ -491,7 +504,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                         const int row = j < vc.na ? vc.k_row0 + j * kTile : vc.b_coord0 + (j - vc.na) * kTile;
                         const uint32_t slot = u % kRing;
                         if (u >= kRing) wait_pv_done(u - kRing, kWaitKvFree);
-                        if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[slot]), 2 * L::kVBytes);
+                        if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[slot]), 2 * L::kVBytes);
                         tma_load_3d_pair(smem_base + L::kV + slot * L::kVBytes, map, static_cast<int>(rank) * (D / 2), vc.kv_head, row,
                                          map_to_cta(smem_u32(&bars.v_full[slot]), 0));
                         if (vc.j == vc.nt) ++vc.k;
@@ -504,9 +517,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             // uniform registers); the MMA and commit instructions themselves go out from one elected lane.
             uint32_t t = 0;
 #pragma unroll 1
-            for (int k = 0; item_ready(k); ++k) {
+            for (int k = 0; uniform(item_ready(k)); ++k) {
                 const WorkItem& it = s_decoded[k % kItems];
-                const int nt = it.nt, na = it.na, n_a = it.n_a, n_b = it.n_b;
+                const int nt = uniform(it.nt), na = uniform(it.na), n_a = uniform(it.n_a), n_b = uniform(it.n_b);
                 __syncwarp();
                 if (lane == 0) item_release(k);
                 const uint32_t q_lo = desc_lo(smem_base + L::kQ + (k & 1) * L::kQBytes, 16);
@@ -530,9 +543,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             const uint32_t d_tmem = tmem_base + kTmemO;
             uint32_t t = 0;
 #pragma unroll 1
-            for (int k = 0; item_ready(k); ++k) {
+            for (int k = 0; uniform(item_ready(k)); ++k) {
                 const WorkItem& it = s_decoded[k % kItems];
-                const int nt = it.nt, na = it.na, n_a = it.n_a, n_b = it.n_b;
+                const int nt = uniform(it.nt), na = uniform(it.na), n_a = uniform(it.n_a), n_b = uniform(it.n_b);
                 __syncwarp();
                 if (lane == 0) item_release(k);
                 // the previous item's output must have left TMEM before O is overwritten
@@ -546,13 +559,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     wait(bars.v_full[slot], (t / kRing) & 1, kWaitV);
                     wait(bars.p_full[t & 1], (t >> 1) & 1, kWaitP);
                     tc_fence_after_sync();
-                    if (n == kTile) {
-                        mma_ts_batch8<D>(d_tmem, a_tmem, v_lo, kIdescPv, j > 0);
-                    } else {
 #pragma unroll 1
-                        for (int ks = 0; ks < (n >> 4); ++ks)
-                            mma_ts_step<D>(d_tmem, a_tmem + ks * 8, v_lo + ks * kVDescStep<D>, kIdescPv, (j > 0) || (ks > 0));
-                    }
+                    for (int ks = 0; ks < (n >> 4); ++ks)
+                        mma_ts_step<D>(d_tmem, a_tmem + ks * 8, v_lo + ks * kVDescStep<D>, kIdescPv, j + ks);
                     mma_commit_pair(smem_u32(&bars.pv_done[slot]));
                 }
             }
@@ -565,12 +574,11 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
         const uint32_t o_free_bar = map_to_cta(smem_u32(&bars.o_free), 0);
         uint32_t t_end = 0;  // tiles up to the end of this item
 #pragma unroll 1
-        for (int k = 0; item_ready(k); ++k) {
+        for (int k = 0; uniform(item_ready(k)); ++k) {
             const WorkItem& it = s_decoded[k % kItems];
             const QSlot& qs = it.s[rank];
             t_end += it.nt;
-            const int row_tok = qs.row_div == 1 ? row : row / qs.row_div;
-            const int row_head = qs.row_div == 1 ? 0 : row - row_tok * qs.row_div;
+            const int row_tok = row * qs.per_div >> 16, row_head = row - row_tok * qs.row_div;
             const bool row_ok = qs.valid && (row_tok < qs.ntok) && (row_head < qs.nheads);
             const int tok = qs.q_tok0 + row_tok;
             const int head = qs.q_head0 + row_head;
@@ -605,8 +613,11 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                 if (!question) {
                     uint32_t wd[16];
 #pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        wd[e] = pack_bf16x2(__uint_as_float(o[2 * e]) * inv_l, __uint_as_float(o[2 * e + 1]) * inv_l);
+                    for (int e = 0; e < 16; ++e) {
+                        float x, y;
+                        unpack_f32x2(mul_f32x2(pack_f32x2(__uint_as_float(o[2 * e]), __uint_as_float(o[2 * e + 1])), pack_f32x2(inv_l, inv_l)), x, y);
+                        wd[e] = pack_bf16x2(x, y);
+                    }
                     if (row_ok) {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
@@ -634,15 +645,14 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
         const uint32_t tO = tmem_base + kTmemO + lane_off;
         uint32_t t0 = 0;                // tiles of all items so far
 #pragma unroll 1
-        for (int k = 0; item_ready(k); ++k) {
+        for (int k = 0; uniform(item_ready(k)); ++k) {
             const WorkItem& it = s_decoded[k % kItems];
             const QSlot& qs = it.s[rank];
-            const int nt = it.nt, na = it.na, a_end = qs.valid ? it.a_end : 0;  // a slot without a tile sees nothing
-            // (row_div is 1 for all but packed tiles: no integer division on the way to the item's first scores)
-            const int row_tok = qs.row_div == 1 ? row : row / qs.row_div;
+            const int nt = uniform(it.nt), na = uniform(it.na), a_end = uniform(qs.valid ? it.a_end : 0);  // a slot without a tile sees nothing
+            const int row_tok = row * qs.per_div >> 16;
             // this row's last visible key and the smallest such key of the tile, counted from the own range's start
-            const int end = qs.valid ? qs.end : 0;
-            const int my_limit = min(qs.limit0 + row_tok, end - 1), limit0 = min(qs.limit0, end - 1);
+            const int end = uniform(qs.valid ? qs.end : 0), first_limit = uniform(qs.limit0);
+            const int my_limit = min(first_limit + row_tok, end - 1), limit0 = min(first_limit, end - 1);
             __syncwarp();
             if (lane == 0) item_release(k);
             float m_own = -INFINITY;  // reference maximum (raw score units) this warpgroup's row sum is scaled by
@@ -766,8 +776,8 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
         __syncwarp();
         tmem_dealloc_pair(tmem_base, 512);
     }
-    if (tid == 0 && abort_flag != 0) {
-        const int detail = abort_flag * 1000000 + blockIdx.x;
+    if (tid == 0 && wait_state.expired != 0) {
+        const int detail = wait_state.expired * 1000000 + blockIdx.x;
         if (atomicCAS(&p.hdr->status, 0, PEVLM_ETIMEOUT) == 0) p.hdr->detail = detail;
         if (MODE == 3 && atomicCAS(&p.hdr_question->status, 0, PEVLM_ETIMEOUT) == 0) p.hdr_question->detail = detail;
     }

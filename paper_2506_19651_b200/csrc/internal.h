@@ -102,7 +102,7 @@ struct AttnParams {
     int32_t n_splits;       // question
     int32_t tiles_per_split;// question
     Divisor div_items, div_per_chunk, div_pair_chunk, div_hkv, div_pairs_sink, div_pairs_last, div_g, div_splits, div_q_pairs;  // decode_item
-    uint32_t wait_limit_ns; // longest a single device-side wait may last before the launch reports PEVLM_ETIMEOUT
+    int32_t wait_tries;     // limit of a single device-side wait before the launch reports PEVLM_ETIMEOUT
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
     __nv_bfloat16* o;       // prefill: [batch * q_rows, Hq, d]

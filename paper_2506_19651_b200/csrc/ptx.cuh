@@ -62,38 +62,35 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-constexpr uint32_t kDefaultWaitLimitNs = 400u * 1000 * 1000;  // 0.4 s
-constexpr uint32_t kAbortGraceNs = 20u * 1000;
+// Bounded wait.  The limit is a number of tries: a try_wait that finds nothing suspends the thread for 0.17 to 1.3 us
+// (B200), so two million of them are 0.3 to 2.6 s, orders of magnitude above any legitimate wait.  (A clock in the loop
+// costs the attention kernel, which waits at two dozen places and has to fit the instruction cache, 2 % in launches of
+// short work items.)  The limit lives in shared memory: once any thread of the CTA has given up on a wait it is lowered,
+// so that every later wait in the CTA gives up after a short grace period and the kernel always runs to its normal end
+// (control flow is never altered by a timeout).  The first expiry leaves `which`.
+constexpr int kDefaultWaitTries = 2000000;
+constexpr int kGraceTries = 100;
 
-// Bounded wait.  `abort_flag` lives in shared memory: once any thread of the CTA has given
-// up on a wait, every later wait in the CTA gives up after a short grace period, so the
-// kernel always runs to its normal end (control flow is never altered by a timeout).
-// `limit_ns` is the longest a single wait may last (a launch parameter: the library's calls pass
-// kDefaultWaitLimitNs, orders of magnitude above any legitimate wait).  The first expiry leaves `which` in the flag.
+struct WaitState {
+    int tries;    // limit of a single wait
+    int expired;  // 0, or the id of the first wait that gave up
+};
+
 // SLEEP_NS > 0 is for waits that are long and not on the critical path: the warp sleeps between its looks, so that it
 // takes no issue slots from the others of its scheduler.
-// Kept short, because it is inlined at two dozen places of the attention kernel, and what that runs per work item has to
-// fit the instruction cache (see there).
 template <unsigned SLEEP_NS = 0>
-__device__ __forceinline__ void mbar_wait_slow(uint32_t bar, uint32_t parity, uint32_t abort_flag, uint32_t limit_ns, int which) {
-    const uint32_t t0 = globaltimer_lo();
-    while (true) {
+__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, volatile WaitState& state, int which) {
+    if (__builtin_expect(mbar_try_wait(bar, parity), 1)) return;
+    int n = 0;
+#pragma unroll 1
+    do {
         if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-        if (mbar_try_wait(bar, parity)) return;
-        const uint32_t waited = globaltimer_lo() - t0;
-        if (waited > kAbortGraceNs) {
-            int gave_up;
-            asm volatile("ld.volatile.shared.s32 %0, [%1];" : "=r"(gave_up) : "r"(abort_flag) : "memory");
-            if (gave_up != 0 || waited > limit_ns) {
-                if (gave_up == 0) asm volatile("st.volatile.shared.s32 [%0], %1;" ::"r"(abort_flag), "r"(which) : "memory");
-                return;
-            }
+        if (++n > state.tries) {
+            if (state.expired == 0) state.expired = which;
+            state.tries = kGraceTries;
+            return;
         }
-    }
-}
-template <unsigned SLEEP_NS = 0>
-__device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, uint32_t abort_flag, uint32_t limit_ns, int which) {
-    if (!__builtin_expect(mbar_try_wait(bar, parity), 1)) mbar_wait_slow<SLEEP_NS>(bar, parity, abort_flag, limit_ns, which);
+    } while (!mbar_try_wait(bar, parity));
 }
 
 // ---------------------------------------------------------------- clusters
@@ -158,11 +155,12 @@ __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
 }
 // 3-D tiled load global -> shared by a CTA of a pair.  c0 (innermost) times the element size must be a multiple of
 // 16 bytes.  The data goes to this CTA's shared memory, the bytes are counted on a barrier of either CTA of the pair
-// (`bar` is a cluster address).
+// (`bar` is a cluster address).  Warp-collective: every lane calls it with the same operands, one elected lane issues.
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const void* tmap, int c0, int c1, int c2, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
-        " [%0], [%1, {%2, %3, %4}], [%5];"
+        "{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
+        "@pe cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3, %4}], [%5];\n\t}"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
         : "memory");
 }
@@ -234,9 +232,8 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int m, int n, bool b_mn_m
 // Shared-memory matrix descriptors (64 bits, sm_100 version field = 1): [0,14) start address >> 4; [16,30) leading byte
 // offset >> 4; [32,46) stride byte offset >> 4; [46,48) version = 1; [61,64) layout (2 = 128-byte, 4 = 64-byte swizzle).
 
-// ---- batched MMA issue.  The issuing thread is latency-bound on its own instruction stream,
-// so a whole k-loop goes out as one asm block: descriptors are a constant high word plus a
-// low word (address >> 4 | leading byte offset >> 4 << 16) that only needs an add per step.
+// ---- MMA issue: descriptors are a constant high word plus a low word (address >> 4 | leading byte offset >> 4 << 16)
+// that only needs an add per step.
 // All MMAs are those of a CTA pair (cta_group::2, M = 256): each CTA holds its 128 rows of A and of the
 // accumulator and half of B's N columns, at the same shared-memory and TMEM addresses.
 constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);  // SBO 1024 B, version 1, 128-byte swizzle
@@ -247,39 +244,25 @@ __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) 
 
 // These are called by ALL lanes of the issuing warp with warp-uniform operands (so the
 // operands live in uniform registers); one elected lane issues.
-#define PEVLM_MMA_SS_STEP(AOFF, BOFF, PRED)                                       \
-    "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                \
-    "mov.b64 da, {ta, %3};\n\tmov.b64 db, {tb, %3};\n\t"                          \
-    "@pe tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, " PRED ";\n\t"
 
-// D[tmem] = A[smem] * B[smem]^T over head_dim = 16 * KSTEPS; A (128 rows a CTA) and B (64 rows a CTA) are K-major,
-// 128-byte swizzled tiles in panels of 64 elements (16 KB and 8 KB apart).  The first step overwrites D.
-template <int KSTEPS>
-__device__ __forceinline__ void mma_ss_batch(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
-    static_assert(KSTEPS == 4 || KSTEPS == 8, "head_dim 64 or 128");
-    if constexpr (KSTEPS == 8) {
-        asm volatile(
-            "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-            PEVLM_MMA_SS_STEP(0, 0, "p0") PEVLM_MMA_SS_STEP(2, 2, "p1") PEVLM_MMA_SS_STEP(4, 4, "p1") PEVLM_MMA_SS_STEP(6, 6, "p1")
-            PEVLM_MMA_SS_STEP(1024, 512, "p1") PEVLM_MMA_SS_STEP(1026, 514, "p1") PEVLM_MMA_SS_STEP(1028, 516, "p1")
-            PEVLM_MMA_SS_STEP(1030, 518, "p1")
-            "}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc));
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 da, db;\n\t"
-            "setp.ne.b32 p0, 0, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-            PEVLM_MMA_SS_STEP(0, 0, "p0") PEVLM_MMA_SS_STEP(2, 2, "p1") PEVLM_MMA_SS_STEP(4, 4, "p1") PEVLM_MMA_SS_STEP(6, 6, "p1")
-            "}"
-            ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc));
-    }
+// One step of 16 of head_dim: D[tmem] (+)= A[smem] * B[smem]^T.
+__device__ __forceinline__ void mma_ss_step(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, pe;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\telect.sync _|pe, 0xffffffff;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+        "@pe tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(kDescHiSw128), "r"(idesc), "r"(accumulate));
 }
 
-#define PEVLM_MMA_TS_STEP(AOFF, BOFF, PRED)                                       \
-    "add.u32 ta, %1, " #AOFF ";\n\tadd.u32 tb, %2, " #BOFF ";\n\t"                \
-    "mov.b64 db, {tb, %3};\n\t"                                                   \
-    "@pe tcgen05.mma.cta_group::2.kind::f16 [%0], [ta], db, %4, " PRED ";\n\t"
+// D[tmem] = A[smem] * B[smem]^T over a head of 16 * KSTEPS; A (128 rows a CTA) and B (64 rows a CTA) are K-major, 128-byte
+// swizzled tiles in panels of 64 elements (16 KB and 8 KB apart).  The first step overwrites D.  (A loop: an MMA of this
+// size keeps the tensor pipe busy for 64 cycles, and unrolled steps cost the kernel 1.5 KB of its instruction cache.)
+template <int KSTEPS>
+__device__ __forceinline__ void mma_ss_batch(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc) {
+#pragma unroll 1
+    for (int ks = 0; ks < KSTEPS; ++ks)
+        mma_ss_step(d_tmem, a_lo + (ks & 3) * 2 + (ks >> 2) * 1024, b_lo + (ks & 3) * 2 + (ks >> 2) * 512, idesc, ks);
+}
 
 // B = V rows, MN-major: a CTA holds D/2 columns of all keys of the tile, 128-byte rows (D = 128) or 64-byte rows
 // (D = 64), so 16 keys are 2048 or 1024 bytes.
@@ -288,33 +271,7 @@ constexpr uint32_t kVDescHi = D == 128 ? kDescHiSw128 : kDescHiSw64;
 template <int D>
 constexpr uint32_t kVDescStep = D == 128 ? 128 : 64;
 
-// D[tmem] (+)= A[tmem] * B[smem] over 128 keys (eight steps of 16): A = bf16 probabilities, 8
-// TMEM columns per step.  The first step accumulates iff accumulate_first != 0.
-template <int D>
-__device__ __forceinline__ void mma_ts_batch8(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
-                                              uint32_t accumulate_first) {
-    if constexpr (D == 128) {
-        asm volatile(
-            "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-            "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-            PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 128, "p1") PEVLM_MMA_TS_STEP(16, 256, "p1")
-            PEVLM_MMA_TS_STEP(24, 384, "p1") PEVLM_MMA_TS_STEP(32, 512, "p1") PEVLM_MMA_TS_STEP(40, 640, "p1")
-            PEVLM_MMA_TS_STEP(48, 768, "p1") PEVLM_MMA_TS_STEP(56, 896, "p1")
-            "}"
-            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kVDescHi<D>), "r"(idesc), "r"(accumulate_first));
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p0, p1, pe;\n\t.reg .b32 ta, tb;\n\t.reg .b64 db;\n\t"
-            "setp.ne.b32 p0, %5, 0;\n\tsetp.eq.b32 p1, 0, 0;\n\telect.sync _|pe, 0xffffffff;\n\t"
-            PEVLM_MMA_TS_STEP(0, 0, "p0") PEVLM_MMA_TS_STEP(8, 64, "p1") PEVLM_MMA_TS_STEP(16, 128, "p1")
-            PEVLM_MMA_TS_STEP(24, 192, "p1") PEVLM_MMA_TS_STEP(32, 256, "p1") PEVLM_MMA_TS_STEP(40, 320, "p1")
-            PEVLM_MMA_TS_STEP(48, 384, "p1") PEVLM_MMA_TS_STEP(56, 448, "p1")
-            "}"
-            ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(kVDescHi<D>), "r"(idesc), "r"(accumulate_first));
-    }
-}
-
-// One step of 16 keys (ragged key tiles).
+// One step of 16 keys: D[tmem] (+)= A[tmem] * B[smem], A = bf16 probabilities, 8 TMEM columns per step.
 template <int D>
 __device__ __forceinline__ void mma_ts_step(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
     asm volatile(

@@ -1,12 +1,20 @@
 """One pass of the whole hot path over one layer's tensors, as a user of the library calls it.
 
-Host-side orchestration only (buffer allocation through torch, then the C-ABI calls in the
-order of the method): RoPE of the video Q/K at global positions -> parallel prefill attention
-(Eq. 3-4) -> RoPE of the question Q/K -> KV-cache assembly -> question attention (Eq. 5).
+Host-side orchestration only (buffer allocation through torch, then the C-ABI calls).  A pass is one call
+(pevlm_layer_forward); its steps, in the order of the method, are RoPE at global positions with K and V written to the
+caches -> parallel prefill attention (Eq. 3-4) and question attention (Eq. 5).
 """
 from __future__ import annotations
 
 from . import binding as pb
+
+
+def _workspace(alloc, n_bytes):
+    """A workspace whose status header (its first 256 bytes) reads as clear before the first call; the rest needs no value."""
+    import torch
+    ws = alloc((n_bytes,), torch.uint8)
+    ws[:256].zero_()
+    return ws
 
 
 class LayerBuffers:
@@ -32,8 +40,8 @@ class LayerBuffers:
         self.lse_video = alloc((Hq, max(nv, 1)), f32)
         self.o_question = alloc((max(Q, 1), Hq, d), bf)
         self.lse_question = alloc((Hq, max(Q, 1)), f32)
-        self.ws_prefill = alloc((pb.pevlm_workspace_bytes(s, pb.WS_PREFILL),), torch.uint8, zero=True)
-        self.ws_query = alloc((pb.pevlm_workspace_bytes(s, pb.WS_QUERY),), torch.uint8, zero=True)
+        self.ws_prefill = _workspace(alloc, pb.pevlm_workspace_bytes(s, pb.WS_PREFILL))
+        self.ws_query = _workspace(alloc, pb.pevlm_workspace_bytes(s, pb.WS_QUERY))
 
 
 KERNELS_PER_PASS = 3          # rope and V copy, attention of video and question rows, merge
@@ -100,11 +108,10 @@ def ragged_layer_forward(q, k, v, S, B, N, B_last, Q, theta, scale=0.0, alloc=No
     lse_video = alloc((Hq, nv), f32)
     o_question = alloc((max(Q, 1), Hq, d), bf)
     lse_question = alloc((Hq, max(Q, 1)), f32)
-    # the launch writes the status words; a part that is not launched has none to write
+    # the launch writes the status words; a question that is not there leaves its own as it was
     ws_prefill = alloc((pb.pevlm_workspace_bytes(s, pb.WS_PREFILL),), torch.uint8)
-    ws_query = alloc((pb.pevlm_workspace_bytes(s, pb.WS_QUERY),), torch.uint8, zero=Q == 0)
-    if Q == 0:
-        ws_query[:256].zero_()
+    ws_query = (alloc((pb.pevlm_workspace_bytes(s, pb.WS_QUERY),), torch.uint8) if Q > 0
+                else _workspace(alloc, pb.pevlm_workspace_bytes(s, pb.WS_QUERY)))
     pb.pevlm_layer_forward(s, q, k, v, q_roped, q_roped[nv:], k_cache, v_cache, o_video, lse_video, o_question, lse_question,
                            ws_prefill, ws_query, last_len=B_last)
     return o_video, lse_video, o_question, lse_question, [ws_prefill, ws_query]
@@ -129,10 +136,10 @@ class StreamingWindow:
         self.q_buf = torch.empty((max(S, B, Q_max), Hq, d), dtype=bf, device=device)
         self.s_sink = self._shape(S, 1, 0, 0)
         self.s_block = self._shape(S, B, 1, 0)
-        self.ws_sink = torch.zeros(pb.pevlm_workspace_bytes(self.s_sink, pb.WS_PREFILL), dtype=torch.uint8, device=device)
-        self.ws_block = torch.zeros(pb.pevlm_workspace_bytes(self.s_block, pb.WS_PREFILL), dtype=torch.uint8, device=device)
-        self.ws_query = torch.zeros(pb.pevlm_workspace_bytes(self._shape(S + W * B, 1, 0, Q_max), pb.WS_QUERY),
-                                    dtype=torch.uint8, device=device)
+        alloc = lambda shape, dtype: torch.empty(shape, dtype=dtype, device=device)
+        self.ws_sink = _workspace(alloc, pb.pevlm_workspace_bytes(self.s_sink, pb.WS_PREFILL))
+        self.ws_block = _workspace(alloc, pb.pevlm_workspace_bytes(self.s_block, pb.WS_PREFILL))
+        self.ws_query = _workspace(alloc, pb.pevlm_workspace_bytes(self._shape(S + W * B, 1, 0, Q_max), pb.WS_QUERY))
         self.blocks_seen = 0
         self._f32, self._bf, self._dev = f32, bf, device
 
