@@ -378,44 +378,43 @@ static AttnParams common_params(const pevlm_shape_t* s, int last_len = 0) {
 static void add_prefill(AttnParams& p, const pevlm_shape_t* s, bool blocks_only, int64_t first_key_row, int64_t cache_rows, int last_len = 0) {
     const int64_t nv = p.n_video;
     p.mode |= 1;
+    int S = s->sink_len, B = s->num_blocks > 0 ? s->block_len : 0, N = s->num_blocks - (last_len > 0 ? 1 : 0);
     if (s->mask_mode == PEVLM_MASK_FULL_CAUSAL) {
-        p.S = 0; p.B = static_cast<int>(nv); p.N = 1;
-    } else {
-        p.S = s->sink_len; p.B = s->num_blocks > 0 ? s->block_len : 0; p.N = s->num_blocks - (last_len > 0 ? 1 : 0);
-        p.last_len = last_len;
+        S = 0; B = static_cast<int>(nv); N = 1;
+        last_len = 0;
     }
-    p.blk_key0 = blocks_only ? static_cast<int>(first_key_row) : p.S;
-    p.blk_q0 = blocks_only ? 0 : p.S;
+    p.sink_len = S;
+    p.block_rows = N * B + last_len;
+    p.blk_key0 = blocks_only ? static_cast<int>(first_key_row) : S;
+    const int blk_q0 = blocks_only ? 0 : S;
     p.q_rows = static_cast<int>(blocks_only ? static_cast<int64_t>(s->num_blocks) * s->block_len : nv);
     p.kv_rows = static_cast<int>(blocks_only ? cache_rows : nv);
     p.lse_stride = p.q_rows;
-    p.tiles_sink = (p.S + kTile - 1) / kTile;
-    p.tiles_block = p.N > 0 ? (p.B + kTile - 1) / kTile : 0;
-    const SegPlan pb = plan_segment(p.N > 0 ? p.B : 0, p.G), ps = plan_segment(blocks_only ? 0 : p.S, p.G), pl = plan_segment(p.last_len, p.G);
-    p.pairs_block = pb.pairs;
-    p.pairs_sink = ps.pairs;
-    p.pairs_last = pl.pairs;
-    p.tail_rows_last = pl.tail_rows; p.tail_heads_last = pl.tail_heads; p.tail_tiles_last = pl.tail_tiles;
-    p.tail_rows_block = pb.tail_rows; p.tail_heads_block = pb.tail_heads; p.tail_tiles_block = pb.tail_tiles;
-    p.tail_rows_sink = ps.tail_rows; p.tail_heads_sink = ps.tail_heads; p.tail_tiles_sink = ps.tail_tiles;
-    // How many pairs of one (block, kv head) are handed out together (decode_item): the whole list keeps the CTAs
-    // that run at the same time on few K/V tiles (best for long blocks); short blocks (at most 4 query tiles)
-    // run faster when pairs of equal length are handed out together across all blocks, and a launch with few
-    // items per SM balances best with single pairs, heaviest first.  Thresholds from measurements on B200.
-    int want_pc = p.pairs_block;
-    if (p.tiles_block <= 4) want_pc = p.G / 2 > 0 ? p.G / 2 : 1;
-    else if (static_cast<int64_t>(p.N) * p.Hkv * p.pairs_block < 16 * kNumSms) want_pc = 1;
-    p.pair_chunk = p.pairs_block > 0 ? (want_pc < p.pairs_block ? want_pc : p.pairs_block) : 1;
-    const int n_chunks = p.pairs_block > 0 ? (p.pairs_block + p.pair_chunk - 1) / p.pair_chunk : 0;
-    p.items_block = p.N * p.Hkv * p.pair_chunk * n_chunks;
-    p.items_last = p.Hkv * p.pairs_last;
-    p.n_items += p.items_block + p.items_last + p.Hkv * p.pairs_sink;
-    p.div_per_chunk = make_divisor(p.N * p.Hkv * p.pair_chunk);
-    p.div_pair_chunk = make_divisor(p.pair_chunk);
     p.div_hkv = make_divisor(p.Hkv);
-    p.div_pairs_sink = make_divisor(p.pairs_sink);
-    p.div_pairs_last = make_divisor(p.pairs_last);
     p.div_g = make_divisor(p.G);
+    auto fill = [&](Segment& g, int n, int len, int q0, int key0, int a_end, int own_map, bool blocks) {
+        const SegPlan sp = plan_segment(n > 0 ? len : 0, p.G);
+        g.len = len; g.q0 = q0; g.key0 = key0; g.a_end = a_end; g.own_map = own_map;
+        g.full_tiles = sp.full_tiles; g.entries = sp.entries;
+        g.tail_rows = sp.tail_rows; g.tail_heads = sp.tail_heads; g.tail_tiles = sp.tail_tiles;
+        // How many pairs of one (block, kv head) are handed out together (decode_item): the whole list keeps the CTAs
+        // that run at the same time on few K/V tiles (best for long blocks); short blocks (at most 4 query tiles)
+        // run faster when pairs of equal length are handed out together across all blocks, and a launch with few
+        // items per SM balances best with single pairs, heaviest first.  Thresholds from measurements on B200.
+        int want_pc = sp.pairs;
+        if (blocks && sp.tiles <= 4) want_pc = p.G / 2 > 0 ? p.G / 2 : 1;
+        else if (blocks && static_cast<int64_t>(n) * p.Hkv * sp.pairs < 16 * kNumSms) want_pc = 1;
+        g.pair_chunk = sp.pairs > 0 ? (want_pc < sp.pairs ? want_pc : sp.pairs) : 1;
+        const int n_chunks = sp.pairs > 0 ? (sp.pairs + g.pair_chunk - 1) / g.pair_chunk : 0;
+        g.per_chunk = n * p.Hkv * g.pair_chunk;
+        g.items = g.per_chunk * n_chunks;
+        g.div_per_chunk = make_divisor(g.per_chunk);
+        g.div_pair_chunk = make_divisor(g.pair_chunk);
+        p.n_items += g.items;
+    };
+    fill(p.seg[0], N, B, blk_q0, 0, S, 0, true);
+    fill(p.seg[1], last_len > 0, last_len, blk_q0 + N * B, N * B, S, 0, false);
+    fill(p.seg[2], S > 0 && !blocks_only, S, 0, 0, 0, 1, false);
 }
 
 static void add_question(AttnParams& p, const QueryPlan& qp) {
@@ -436,32 +435,26 @@ static void add_question(AttnParams& p, const QueryPlan& qp) {
 static int prefill_maps(AttnMaps& m, const AttnParams& p, int d, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v) {
     int rc;
     const int64_t q_rows = static_cast<int64_t>(p.batch) * p.q_rows, before = static_cast<int64_t>(p.batch - 1) * p.kv_rows;
-    if ((rc = make_tmap(&m.q, q, q_rows, p.Hq, d, 1, kTile)) != PEVLM_OK) return rc;
-    m.q_tail_block = m.q;
-    m.q_tail_sink = m.q;
-    m.q_tail_last = m.q;
-    if (p.tail_tiles_last > 0 && (rc = make_tmap(&m.q_tail_last, q, q_rows, p.Hq, d, p.tail_heads_last, p.tail_rows_last)) != PEVLM_OK) return rc;
-    if (p.tail_tiles_block > 0 && (rc = make_tmap(&m.q_tail_block, q, q_rows, p.Hq, d, p.tail_heads_block, p.tail_rows_block)) != PEVLM_OK) return rc;
-    if (p.tail_tiles_sink > 0) {
-        if (p.tail_tiles_block > 0 && p.tail_heads_sink == p.tail_heads_block && p.tail_rows_sink == p.tail_rows_block) m.q_tail_sink = m.q_tail_block;
-        else if ((rc = make_tmap(&m.q_tail_sink, q, q_rows, p.Hq, d, p.tail_heads_sink, p.tail_rows_sink)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.q[0], q, q_rows, p.Hq, d, 1, kTile)) != PEVLM_OK) return rc;
+    for (int i = 0; i < 3; ++i) {
+        const Segment& g = p.seg[i];
+        if (g.items > 0 && g.tail_tiles > 0 && (rc = make_tmap(&m.q[1 + i], q, q_rows, p.Hq, d, g.tail_heads, g.tail_rows)) != PEVLM_OK) return rc;
     }
-    // K and V: one map over the sink rows [0, S) and one over the block rows, so that the ragged last key
-    // tile of either range reads zeros past its end (a map needs at least one row; an empty range is never read)
-    const int64_t blk_off = static_cast<int64_t>(p.blk_key0) * p.Hkv * d, block_rows = static_cast<int64_t>(p.N) * p.B + p.last_len;
-    const int64_t sink_rows = before + (p.S > 0 ? p.S : 1), blk_rows = before + (block_rows > 0 ? block_rows : 1);
-    if ((rc = make_tmap(&m.k_sink, k, sink_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-    if ((rc = make_tmap(&m.v_sink, v, sink_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
-    if ((rc = make_tmap(&m.k, k + blk_off, blk_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-    return make_tmap(&m.v, v + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2);
+    // (a map needs at least one row; an empty range is never read)
+    const int64_t blk_off = static_cast<int64_t>(p.blk_key0) * p.Hkv * d;
+    const int64_t sink_rows = before + (p.sink_len > 0 ? p.sink_len : 1), blk_rows = before + (p.block_rows > 0 ? p.block_rows : 1);
+    if ((rc = make_tmap(&m.k[0], k + blk_off, blk_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.v[0], v + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.k[1], k, sink_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+    return make_tmap(&m.v[1], v, sink_rows, p.Hkv, d, 1, kTile, d / 2);
 }
 
 static int question_maps(AttnMaps& m, const AttnParams& p, int d, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v) {
     int rc;
     const int64_t rows = static_cast<int64_t>(p.batch) * p.L;
-    if ((rc = make_tmap(&m.q_question, q, static_cast<int64_t>(p.batch) * p.Q, p.Hq, d, p.G, p.tok_per_tile)) != PEVLM_OK) return rc;
-    if ((rc = make_tmap(&m.k_cache, k, rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-    return make_tmap(&m.v_cache, v, rows, p.Hkv, d, 1, kTile, d / 2);
+    if ((rc = make_tmap(&m.q[4], q, static_cast<int64_t>(p.batch) * p.Q, p.Hq, d, p.G, p.tok_per_tile)) != PEVLM_OK) return rc;
+    if ((rc = make_tmap(&m.k[2], k, rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
+    return make_tmap(&m.v[2], v, rows, p.Hkv, d, 1, kTile, d / 2);
 }
 
 static int merge_question(const AttnParams& p, int d, __nv_bfloat16* o, float* lse, cudaStream_t st) {

@@ -130,86 +130,44 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
     it.k_row0 = it.seq * p.kv_rows;
     int own_keys = 0;  // keys of the own range that the longer query tile sees
     if (!question) {
-        int seg_q0, seg_len, tiles, pi, g, tail_rows, tail_heads, tail_tiles, qmap_tail;
-        if (w < p.items_block) {
-            // Order of the items: the pair list of a (block, kv head), heaviest first, is cut into chunks of
-            // pair_chunk pairs; chunk-major, then (block, kv head), then the pairs of the chunk.  CTAs that run
-            // at the same time then share few K/V tiles' worth of L2 traffic, and the launch ends on the
-            // lightest chunk of every (block, kv head) rather than on the last block's whole list.  A pair
-            // index past the end of the list (padding of the last chunk) is an empty item.
-            const int per_chunk = p.N * p.Hkv * p.pair_chunk;
-            const int chunk = quotient(w, p.div_per_chunk), r = w - chunk * per_chunk;
-            const int combo = quotient(r, p.div_pair_chunk);
-            pi = chunk * p.pair_chunk + r - combo * p.pair_chunk;
-            const int blk = quotient(combo, p.div_hkv);
-            g = combo - blk * p.Hkv;
-            seg_q0 = p.blk_q0 + blk * p.B;       // the block's rows in q / o
-            seg_len = p.B;
-            tiles = p.tiles_block;
-            tail_rows = p.tail_rows_block; tail_heads = p.tail_heads_block; tail_tiles = p.tail_tiles_block;
-            qmap_tail = 1;
-            it.a_end = p.S;
-            it.b_coord0 = it.k_row0 + blk * p.B;
-            it.own_map = 0;
-        } else if (w < p.items_block + p.items_last) {
-            // a shorter last block: its pairs, behind those of the full blocks
-            const int w2 = w - p.items_block;
-            g = quotient(w2, p.div_pairs_last);
-            pi = w2 - g * p.pairs_last;
-            seg_q0 = p.blk_q0 + p.N * p.B;
-            seg_len = p.last_len;
-            tiles = cdiv(p.last_len, kTile);
-            tail_rows = p.tail_rows_last; tail_heads = p.tail_heads_last; tail_tiles = p.tail_tiles_last;
-            qmap_tail = 4;
-            it.a_end = p.S;
-            it.b_coord0 = it.k_row0 + p.N * p.B;
-            it.own_map = 0;
-        } else {
-            const int w2 = w - p.items_block - p.items_last;
-            g = quotient(w2, p.div_pairs_sink);
-            pi = w2 - g * p.pairs_sink;
-            seg_q0 = 0;
-            seg_len = p.S;
-            tiles = p.tiles_sink;
-            tail_rows = p.tail_rows_sink; tail_heads = p.tail_heads_sink; tail_tiles = p.tail_tiles_sink;
-            qmap_tail = 2;
-            it.a_end = 0;
-            it.b_coord0 = it.k_row0;
-            it.own_map = 1;
-        }
+        // Which kind of segment: the full blocks, a shorter last block, the sink.
+        int kind = 0;
+#pragma unroll 1
+        while (kind < 2 && w >= p.seg[kind].items) w -= p.seg[kind++].items;
+        const Segment& sg = p.seg[kind];
+        // Order of the items: the pair list of a (block, kv head), heaviest first, is cut into chunks of
+        // pair_chunk pairs; chunk-major, then (block, kv head), then the pairs of the chunk.  CTAs that run
+        // at the same time then share few K/V tiles' worth of L2 traffic, and the launch ends on the
+        // lightest chunk of every (block, kv head) rather than on the last block's whole list.  A pair
+        // index past the end of the list (padding of the last chunk) is an empty item.
+        const int chunk = quotient(w, sg.div_per_chunk), r = w - chunk * sg.per_chunk;
+        const int combo = quotient(r, sg.div_pair_chunk);
+        const int pi = chunk * sg.pair_chunk + r - combo * sg.pair_chunk;
+        const int blk = quotient(combo, p.div_hkv), g = combo - blk * p.Hkv;
         it.kv_head = g;
+        it.a_end = sg.a_end;
+        it.b_coord0 = it.k_row0 + sg.key0 + blk * sg.len;
+        it.own_map = sg.own_map;
         // entries of this (segment, kv head), heaviest first: the packed tail tiles (last tile position of
         // the segment, tail_heads q heads each), then (tile position, q head) for the full positions
-        const int full_tiles = tiles - (tail_tiles > 0 ? 1 : 0);
-        const int entries = tail_tiles + p.G * full_tiles;
 #pragma unroll 1
         for (int x = 0; x < 2; ++x) {
             const int e = 2 * pi + x;
             QSlot& s = it.s[x];
-            s.valid = e < entries;
-            int qt;
-            if (e < tail_tiles) {
-                qt = tiles - 1;
-                s.q_head0 = g * p.G + e * tail_heads;
-                s.row_div = tail_heads;
-                s.ntok = tail_rows;
-                s.nheads = min(tail_heads, p.G - e * tail_heads);
-                s.qmap = qmap_tail;
-                s.box_rows = tail_heads * tail_rows;
-            } else {
-                const int e2 = e - tail_tiles;
-                const int up = quotient(e2, p.div_g);
-                qt = full_tiles - 1 - up;
-                s.q_head0 = g * p.G + e2 - up * p.G;
-                s.row_div = 1;
-                s.ntok = min(kTile, seg_len - qt * kTile);
-                s.nheads = 1;
-                s.qmap = 0;
-                s.box_rows = kTile;
-            }
-            s.q_tok0 = it.seq * p.q_rows + seg_q0 + qt * kTile;
+            s.valid = e < sg.entries;
+            const bool tail = e < sg.tail_tiles;
+            const int e2 = e - sg.tail_tiles, up = quotient(max(e2, 0), p.div_g);
+            const int qt = tail ? sg.full_tiles : sg.full_tiles - 1 - up;
+            const int head = tail ? e * sg.tail_heads : e2 - up * p.G;
+            s.q_head0 = g * p.G + head;
+            s.row_div = tail ? sg.tail_heads : 1;
+            s.ntok = tail ? sg.tail_rows : min(kTile, sg.len - qt * kTile);
+            s.nheads = tail ? min(sg.tail_heads, p.G - head) : 1;
+            s.qmap = tail ? 1 + kind : 0;
+            s.box_rows = tail ? sg.tail_heads * sg.tail_rows : kTile;
+            s.q_tok0 = it.seq * p.q_rows + sg.q0 + blk * sg.len + qt * kTile;
             s.limit0 = qt * kTile;
-            s.end = min(qt * kTile + kTile, seg_len);
+            s.end = min(qt * kTile + kTile, sg.len);
             if (s.valid) own_keys = max(own_keys, s.end);
         }
     } else {
@@ -235,7 +193,7 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             s.row_div = p.G;
             s.ntok = ntok;
             s.nheads = p.G;
-            s.qmap = 3;
+            s.qmap = 4;
             s.box_rows = p.G * p.tok_per_tile;
             s.limit0 = p.n_video + tok0 - split_lo;
             // keys past the last row's limit are never visible; a split that lies past it altogether still takes
@@ -331,16 +289,17 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
         mbar_init(smem_u32(&bars.clc_read), 1);
         fence_mbar_init();
         if (MODE & 1) {
-            tma_prefetch_desc(&maps.q);
-            tma_prefetch_desc(&maps.k_sink);
-            tma_prefetch_desc(&maps.v_sink);
-            tma_prefetch_desc(&maps.k);
-            tma_prefetch_desc(&maps.v);
+            tma_prefetch_desc(&maps.q[0]);
+#pragma unroll 1
+            for (int i = 0; i < 2; ++i) {
+                tma_prefetch_desc(&maps.k[i]);
+                tma_prefetch_desc(&maps.v[i]);
+            }
         }
         if (MODE & 2) {
-            tma_prefetch_desc(&maps.q_question);
-            tma_prefetch_desc(&maps.k_cache);
-            tma_prefetch_desc(&maps.v_cache);
+            tma_prefetch_desc(&maps.q[4]);
+            tma_prefetch_desc(&maps.k[2]);
+            tma_prefetch_desc(&maps.v[2]);
         }
     }
     if (warp == 12) {
@@ -433,82 +392,74 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             // --------------------------------------------------------- TMA producer: K(s), then V(s - kQkAhead)
             // (The whole warp runs this with uniform values; single lanes issue.)
             {
-                struct Cursor {
-                    int k, j, nt, na, kv_head, b_coord0, own_map, k_row0;
-                };
-                auto enter = [&](Cursor& c) {  // the cursor's item; false: no more work
-                    if (!uniform(item_ready(c.k))) return false;
-                    const WorkItem& it = s_decoded[c.k % kItems];
-                    c.j = 0; c.nt = uniform(it.nt); c.na = uniform(it.na);
-                    c.kv_head = uniform(it.kv_head); c.b_coord0 = uniform(it.b_coord0); c.own_map = uniform(it.own_map);
-                    c.k_row0 = uniform(it.k_row0);
-                    return true;
-                };
-                Cursor kc{}, vc{};
-                int n_a = 0, n_b = 0;
-                bool k_end = false;
+                // The K cursor's item, and where V has to come from: the rows of the last kQkAhead K tiles (base row of the
+                // tile, kv head and map), the V tile of a step being that of kQkAhead steps ago.
+                int k = -1, j = 0, nt = 0, na = 0, n_a = 0, n_b = 0, kv_head = 0, b_coord0 = 0, own_map = 0, k_row0 = 0;
+                int v_row[kQkAhead], v_from[kQkAhead];
                 uint32_t tiles = 0;  // K tiles loaded so far
+                bool more = true;
 #pragma unroll 1
-                for (uint32_t s = 0; !k_end || s < tiles + kQkAhead; ++s) {
-                    if (!k_end && kc.j == kc.nt) {
-                        k_end = !enter(kc);
-                        if (!k_end) {
-                            const WorkItem& it = s_decoded[kc.k % kItems];
+                for (uint32_t s = 0; more || s < tiles + kQkAhead; ++s) {
+                    if (more && j == nt) {
+                        more = uniform(item_ready(++k));
+                        if (more) {
+                            const WorkItem& it = s_decoded[k % kItems];
                             const QSlot& q = it.s[rank];
-                            n_a = uniform(it.n_a); n_b = uniform(it.n_b);
-                            const int qb = kc.k & 1;
-                            if (kc.k >= 2) wait(bars.q_free[qb], ((kc.k >> 1) - 1) & 1, kWaitQFree);
-                            if (rank == 0 && lane == 0)
-                                mbar_arrive_expect_tx(smem_u32(&bars.q_full[qb]),
-                                                      static_cast<uint32_t>(NP * 128 * ((it.s[0].valid ? it.s[0].box_rows : 0) +
-                                                                                        (it.s[1].valid ? it.s[1].box_rows : 0))));
-                            if (uniform(q.valid)) {
-                                const int qm = uniform(q.qmap), q_head0 = uniform(q.q_head0), q_tok0 = uniform(q.q_tok0);
-                                const CUtensorMap* qmap = MODE == 2 || (MODE == 3 && qm == 3) ? &maps.q_question
-                                                        : qm == 0 ? &maps.q : qm == 1 ? &maps.q_tail_block : qm == 2 ? &maps.q_tail_sink : &maps.q_tail_last;
+                            j = 0;
+                            nt = uniform(it.nt); na = uniform(it.na); n_a = uniform(it.n_a); n_b = uniform(it.n_b);
+                            kv_head = uniform(it.kv_head); b_coord0 = uniform(it.b_coord0); own_map = uniform(it.own_map);
+                            k_row0 = uniform(it.k_row0);
+                            const int qm = uniform(q.qmap), q_head0 = uniform(q.q_head0), q_tok0 = uniform(q.q_tok0);
+                            const int valid = uniform(q.valid);
+                            const int rows = uniform((it.s[0].valid ? it.s[0].box_rows : 0) + (it.s[1].valid ? it.s[1].box_rows : 0));
+                            __syncwarp();
+                            if (lane == 0) item_release(k);
+                            const int qb = k & 1;
+                            if (k >= 2) wait(bars.q_free[qb], ((k >> 1) - 1) & 1, kWaitQFree);
+                            if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.q_full[qb]), static_cast<uint32_t>(NP * 128 * rows));
+                            if (valid) {
                                 const uint32_t bar = map_to_cta(smem_u32(&bars.q_full[qb]), 0);
+#pragma unroll 1
                                 for (int h = 0; h < NP; ++h)
-                                    tma_load_3d_pair(smem_base + L::kQ + qb * L::kQBytes + h * L::kQPanelBytes, qmap, h * 64,
-                                                     q_head0, q_tok0, bar);
+                                    tma_load_3d_pair(smem_base + L::kQ + qb * L::kQBytes + h * L::kQPanelBytes, &maps.q[MODE == 2 ? 4 : qm],
+                                                     h * 64, q_head0, q_tok0, bar);
                             }
                         }
                     }
                     // Rows past the end of the sink, and past the end of the block range, are outside their
                     // tensor map and arrive as zeros: a ragged last tile never brings in a neighbour's rows.
-                    if (!k_end) {
-                        const int j = kc.j++;
-                        if (rank == 0 && lane == 0 && j == max(0, kc.nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
-                        const CUtensorMap* map = MODE == 2 || (MODE == 3 && kc.own_map == 2) ? &maps.k_cache
-                                                 : (j < kc.na || kc.own_map == 1) ? &maps.k_sink : &maps.k;
-                        const int n = j == kc.na - 1 ? n_a : j == kc.nt - 1 ? n_b : kTile;  // this CTA's keys: half of them
-                        const int row = (j < kc.na ? kc.k_row0 + j * kTile : kc.b_coord0 + (j - kc.na) * kTile) + static_cast<int>(rank) * (n >> 1);
+                    int row = 0, from = 0;
+                    if (more) {
+                        if (rank == 0 && lane == 0 && j == max(0, nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
+                        const int map = MODE == 2 ? 2 : j < na ? 1 : own_map;
+                        const int n = j == na - 1 ? n_a : j == nt - 1 ? n_b : kTile;  // this CTA's keys: half of them
+                        row = j < na ? k_row0 + j * kTile : b_coord0 + (j - na) * kTile;
+                        from = kv_head * 4 + map;
                         const uint32_t slot = tiles % kRing;
                         if (tiles >= kRing) wait_s_full(tiles - kRing, kWaitKvFree);
                         if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.k_full[slot]), 2 * L::kKBytes);
                         const uint32_t bar = map_to_cta(smem_u32(&bars.k_full[slot]), 0);
+#pragma unroll 1
                         for (int h = 0; h < NP; ++h)
-                            tma_load_3d_pair(smem_base + L::kK + slot * L::kKBytes + h * L::kKPanelBytes, map, h * 64, kc.kv_head, row, bar);
+                            tma_load_3d_pair(smem_base + L::kK + slot * L::kKBytes + h * L::kKPanelBytes, &maps.k[map], h * 64, kv_head,
+                                             row + static_cast<int>(rank) * (n >> 1), bar);
+                        ++j;
                         ++tiles;
-                        if (kc.j == kc.nt) ++kc.k;
                     }
                     if (s >= kQkAhead && s - kQkAhead < tiles) {
-                        const uint32_t u = s - kQkAhead;
-                        if (vc.j == vc.nt) {
-                            enter(vc);
-                            __syncwarp();
-                            if (lane == 0) item_release(vc.k);
-                        }
-                        const int j = vc.j++;
-                        const CUtensorMap* map = MODE == 2 || (MODE == 3 && vc.own_map == 2) ? &maps.v_cache
-                                                 : (j < vc.na || vc.own_map == 1) ? &maps.v_sink : &maps.v;
-                        const int row = j < vc.na ? vc.k_row0 + j * kTile : vc.b_coord0 + (j - vc.na) * kTile;
-                        const uint32_t slot = u % kRing;
+                        const uint32_t u = s - kQkAhead, slot = u % kRing;
                         if (u >= kRing) wait_pv_done(u - kRing, kWaitKvFree);
                         if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[slot]), 2 * L::kVBytes);
-                        tma_load_3d_pair(smem_base + L::kV + slot * L::kVBytes, map, static_cast<int>(rank) * (D / 2), vc.kv_head, row,
-                                         map_to_cta(smem_u32(&bars.v_full[slot]), 0));
-                        if (vc.j == vc.nt) ++vc.k;
+                        tma_load_3d_pair(smem_base + L::kV + slot * L::kVBytes, &maps.v[v_from[0] & 3], static_cast<int>(rank) * (D / 2),
+                                         v_from[0] >> 2, v_row[0], map_to_cta(smem_u32(&bars.v_full[slot]), 0));
                     }
+#pragma unroll
+                    for (int i = 0; i < kQkAhead - 1; ++i) {
+                        v_row[i] = v_row[i + 1];
+                        v_from[i] = v_from[i + 1];
+                    }
+                    v_row[kQkAhead - 1] = row;
+                    v_from[kQkAhead - 1] = from;
                 }
             }
         } else if (rank == 0 && warp == 12) {

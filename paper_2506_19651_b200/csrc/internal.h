@@ -67,41 +67,46 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, unsigned
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// One kind of prefill segment (full context blocks, a shorter last block, the sink) and its work items.
+struct Segment {
+    int32_t items;       // work items, padded: (per_chunk =) blocks * Hkv * pair_chunk, times chunks
+    int32_t len;         // tokens of a segment
+    int32_t q0;          // row of q / o where the first one starts
+    int32_t key0;        // row where the first one starts in the tensor map of its keys
+    int32_t a_end;       // keys of the shared range (the sink) that its rows see
+    int32_t own_map;     // which K / V map its own keys are in: 0 blocks, 1 sink
+    int32_t full_tiles;  // query tile positions without the packed tail
+    int32_t entries;     // query tiles of one (segment, kv head): tail_tiles + G * full_tiles
+    // ragged last query tile (len % 128 rows): the tails of tail_heads q heads of one kv group are packed into one
+    // 128-row tile, tail_tiles such tiles per (segment, kv head); 0 = no packing
+    int32_t tail_rows, tail_heads, tail_tiles;
+    int32_t pair_chunk;  // pairs of one (segment, kv head) handed out together (see decode_item)
+    int32_t per_chunk;
+    Divisor div_per_chunk, div_pair_chunk;
+};
+
 // What one launch of the attention kernel does, bit 0 of mode: prefill rows (sink + blocks, or full causal); bit 1:
 // question rows against the assembled cache, split over keys.
 struct AttnParams {
     int32_t mode;
     int32_t batch;          // sequences, each with n_items work items
-    int32_t S, B, N;        // prefill geometry (full causal: S = 0, B = n_video, N = 1)
-    int32_t n_video;        // S + N*B
-    int32_t blk_key0;       // prefill: K/V row of the first context block (S, or the cache row of a block range)
-    int32_t blk_q0;         // prefill: row of q / o where the first context block starts (S, or 0 for a block range)
+    Segment seg[3];         // prefill: full blocks (full causal: the whole stream as one), shorter last block, sink
+    int32_t n_video;        // S + N*B (+ the last block)
+    int32_t sink_len;       // prefill (host only): S,
+    int32_t block_rows;     // rows of all blocks
+    int32_t blk_key0;       // and K/V row of the first block (S, or the cache row of a block range)
     int32_t q_rows;         // prefill: rows of q / o of a sequence
     int32_t kv_rows;        // prefill: rows of k / v of a sequence
     int32_t lse_stride;     // prefill: row stride of lse
     int32_t Q, L;           // question length, total length
     int32_t Hq, Hkv, G;
-    int32_t tiles_sink;     // ceil(S / 128)
-    int32_t tiles_block;    // ceil(B / 128)
-    int32_t pairs_block;    // ceil(G * tiles_block / 2) query-tile pairs per (block, kv head)
-    int32_t pairs_sink;     // ceil(G * tiles_sink / 2) query-tile pairs per kv head
-    int32_t pair_chunk;     // pairs of one (block, kv head) handed out together (see decode_item)
-    int32_t items_block;    // work items over the context blocks, padded: N * Hkv * pair_chunk * chunks
-    int32_t last_len;       // tokens of one more, shorter context block behind the N full ones (0 = none)
-    int32_t pairs_last;     // query-tile pairs of it per kv head
-    int32_t items_last;     // Hkv * pairs_last
     int32_t items_question; // question work items
     int32_t n_items;        // all work items of a sequence
-    // ragged last query tile of a segment (len % 128 rows): the tails of tail_heads q heads of one kv
-    // group are packed into one 128-row tile, tail_tiles such tiles per (segment, kv head); 0 = no packing
-    int32_t tail_rows_block, tail_heads_block, tail_tiles_block;
-    int32_t tail_rows_sink, tail_heads_sink, tail_tiles_sink;
-    int32_t tail_rows_last, tail_heads_last, tail_tiles_last;
     int32_t tok_per_tile;   // question: tokens per query tile = 128 / G
     int32_t q_tiles;        // question: ceil(Q / tok_per_tile)
     int32_t n_splits;       // question
     int32_t tiles_per_split;// question
-    Divisor div_items, div_per_chunk, div_pair_chunk, div_hkv, div_pairs_sink, div_pairs_last, div_g, div_splits, div_q_pairs;  // decode_item
+    Divisor div_items, div_hkv, div_g, div_splits, div_q_pairs;  // decode_item
     int32_t wait_tries;     // limit of a single device-side wait before the launch reports PEVLM_ETIMEOUT
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
@@ -176,13 +181,13 @@ struct CopySegments {
 
 cudaError_t launch_rope(const RopeParams& p, int head_dim, cudaStream_t stream);
 cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream);
-// Tensor maps of one attention launch.  q: [rows, Hq, d] with a 128-token box; q_tail_*: the same tensor with the
-// box of a packed ragged tail (heads x tail rows).  K and V each have two maps so that a ragged last key tile
-// reads zeros past the end of its range instead of a neighbour's rows: *_sink covers cache rows [0, S), k / v
-// cover the context blocks of the call (base at the first block's row).  q_question, k_cache, v_cache: the question rows
-// (box: one kv group's heads x the tokens of a tile) and the whole cache.
+// Tensor maps of one attention launch.
+//   q[0]: [rows, Hq, d] with a 128-token box; q[1 + kind]: the same tensor with the box of the segment kind's packed ragged
+//   tail (heads x tail rows); q[4]: the question rows (box: one kv group's heads x the tokens of a tile)
+//   k, v[0]: the context blocks of the call (base at the first block's row); [1]: the sink, rows [0, S), so that a ragged
+//   last key tile of either range reads zeros past its end instead of a neighbour's rows; [2]: the whole cache
 struct AttnMaps {
-    CUtensorMap q, q_tail_block, q_tail_sink, q_tail_last, k_sink, v_sink, k, v, q_question, k_cache, v_cache;
+    CUtensorMap q[5], k[3], v[3];
 };
 cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cudaStream_t stream);
 cudaError_t launch_wait_selftest(WorkspaceHeader* hdr, uint32_t limit_ns, cudaStream_t stream);
