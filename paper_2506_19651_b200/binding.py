@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the C ABI of libpevlm.so (include/pevlm.h), same names.
+"""Thin binding over the C ABI of libpevlm.so (include/pevlm.h), same names: the calls that launch work go through the
+_pevlm_call module (csrc/pycall.c), the others through ctypes.
 
 Argument marshalling only: every step of the path runs in the library's CUDA kernels.
 Tensors are torch CUDA tensors (torch is used for device memory and streams); a call
@@ -100,6 +101,22 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+_calls = None
+
+
+def _native():
+    """The module with the library's calls.  A missing library raises as in lib()."""
+    global _calls
+    if _calls is None:
+        lib()
+        try:
+            from . import _pevlm_call
+        except ImportError as e:
+            raise RuntimeError("_pevlm_call is missing: build it with `python -m paper_2506_19651_b200.build`") from e
+        _calls = _pevlm_call
+    return _calls
+
+
 _raw_stream = None
 
 
@@ -112,7 +129,10 @@ def _stream():
         if raw is None:
             _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
         else:
-            _raw_stream = lambda: raw(torch.cuda.current_device())
+            device = torch.cuda.current_device   # also initialises CUDA where nothing has yet
+            device()
+            device = getattr(torch._C, "_cuda_getDevice", device)
+            _raw_stream = lambda: raw(device())
     return _raw_stream()
 
 
@@ -125,58 +145,53 @@ def pevlm_workspace_bytes(shape: Shape, which: int) -> int:
     return int(lib().pevlm_workspace_bytes(C.byref(shape), which))
 
 
+# A tensor argument may also be None where the C call takes NULL, or a device address.
+
 def pevlm_rope_qk(shape: Shape, q_in, k_in, q_out, k_out, first_token: int, n_tokens: int, pos_ids=None):
-    _check(lib().pevlm_rope_qk(C.byref(shape), _ptr(q_in), _ptr(k_in), _ptr(q_out), _ptr(k_out),
-                               first_token, n_tokens, _ptr(pos_ids), _stream()), "pevlm_rope_qk")
+    _check(_native().rope_qk(C.addressof(shape), q_in, k_in, q_out, k_out, first_token, n_tokens, pos_ids, _stream()), "pevlm_rope_qk")
 
 
 def pevlm_rope_qkv(shape: Shape, q_in, k_in, v_in, q_out, k_out, v_out, first_token: int, n_tokens: int, pos_ids=None):
-    _check(lib().pevlm_rope_qkv(C.byref(shape), _ptr(q_in), _ptr(k_in), _ptr(v_in), _ptr(q_out), _ptr(k_out), _ptr(v_out),
-                                first_token, n_tokens, _ptr(pos_ids), _stream()), "pevlm_rope_qkv")
+    _check(_native().rope_qkv(C.addressof(shape), q_in, k_in, v_in, q_out, k_out, v_out, first_token, n_tokens, pos_ids, _stream()),
+           "pevlm_rope_qkv")
 
 
 def pevlm_layer_forward(shape: Shape, q, k, v, q_video, q_question, k_cache, v_cache, o_video, lse_video, o_question,
                         lse_question, ws_prefill, ws_query, last_len: int = 0):
-    _check(lib().pevlm_layer_forward(C.byref(shape), last_len, _ptr(q), _ptr(k), _ptr(v), _ptr(q_video), _ptr(q_question),
-                                     _ptr(k_cache), _ptr(v_cache), _ptr(o_video), _ptr(lse_video), _ptr(o_question),
-                                     _ptr(lse_question), _ptr(ws_prefill), ws_prefill.nbytes, _ptr(ws_query),
-                                     ws_query.nbytes, _stream()), "pevlm_layer_forward")
+    _check(_native().layer_forward(C.addressof(shape), last_len, q, k, v, q_video, q_question, k_cache, v_cache, o_video, lse_video,
+                                   o_question, lse_question, ws_prefill, ws_prefill.nbytes, ws_query, ws_query.nbytes, _stream()),
+           "pevlm_layer_forward")
 
 
 def pevlm_rope_qk_mrope(shape: Shape, q_in, k_in, q_out, k_out, n_tokens: int, pos_ids3, sections):
-    sec = (C.c_int32 * 3)(*sections)
-    _check(lib().pevlm_rope_qk_mrope(C.byref(shape), _ptr(q_in), _ptr(k_in), _ptr(q_out), _ptr(k_out),
-                                     n_tokens, _ptr(pos_ids3), sec, _stream()), "pevlm_rope_qk_mrope")
+    _check(_native().rope_qk_mrope(C.addressof(shape), q_in, k_in, q_out, k_out, n_tokens, pos_ids3, *sections, _stream()),
+           "pevlm_rope_qk_mrope")
 
 
 def pevlm_parallel_prefill_attn(shape: Shape, q, k, v, o, lse, workspace):
-    _check(lib().pevlm_parallel_prefill_attn(C.byref(shape), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
-                                             _ptr(workspace), workspace.nbytes,
-                                             _stream()), "pevlm_parallel_prefill_attn")
+    _check(_native().parallel_prefill_attn(C.addressof(shape), q, k, v, o, lse, workspace, workspace.nbytes, _stream()),
+           "pevlm_parallel_prefill_attn")
 
 
 def pevlm_block_attn(shape: Shape, q_blocks, k_cache, v_cache, first_key_row: int, cache_rows: int, o, lse, workspace):
-    _check(lib().pevlm_block_attn(C.byref(shape), _ptr(q_blocks), _ptr(k_cache), _ptr(v_cache), first_key_row,
-                                  cache_rows, _ptr(o), _ptr(lse), _ptr(workspace),
-                                  workspace.nbytes, _stream()), "pevlm_block_attn")
+    _check(_native().block_attn(C.addressof(shape), q_blocks, k_cache, v_cache, first_key_row, cache_rows, o, lse, workspace,
+                                workspace.nbytes, _stream()), "pevlm_block_attn")
 
 
 def pevlm_assemble_kv(shape: Shape, k_video, v_video, k_question, v_question, k_cache, v_cache):
-    _check(lib().pevlm_assemble_kv(C.byref(shape), _ptr(k_video), _ptr(v_video), _ptr(k_question),
-                                   _ptr(v_question), _ptr(k_cache), _ptr(v_cache), _stream()), "pevlm_assemble_kv")
+    _check(_native().assemble_kv(C.addressof(shape), k_video, v_video, k_question, v_question, k_cache, v_cache, _stream()),
+           "pevlm_assemble_kv")
 
 
 def pevlm_query_attn(shape: Shape, q_question, k_cache, v_cache, o, lse, workspace):
-    _check(lib().pevlm_query_attn(C.byref(shape), _ptr(q_question), _ptr(k_cache), _ptr(v_cache), _ptr(o),
-                                  _ptr(lse), _ptr(workspace), workspace.nbytes,
-                                  _stream()), "pevlm_query_attn")
+    _check(_native().query_attn(C.addressof(shape), q_question, k_cache, v_cache, o, lse, workspace, workspace.nbytes, _stream()),
+           "pevlm_query_attn")
 
 
 def pevlm_query_attn_noalloc(shape: Shape, q_question, k_cache, v_cache, o, lse):
     """Question attention for callers that cannot allocate device memory: no workspace argument,
     the partials go to the library's built-in scratch array (see include/pevlm.h for its limits)."""
-    _check(lib().pevlm_query_attn_noalloc(C.byref(shape), _ptr(q_question), _ptr(k_cache), _ptr(v_cache), _ptr(o),
-                                          _ptr(lse), _stream()), "pevlm_query_attn_noalloc")
+    _check(_native().query_attn_noalloc(C.addressof(shape), q_question, k_cache, v_cache, o, lse, _stream()), "pevlm_query_attn_noalloc")
 
 
 def pevlm_selftest_wait_expiry(workspace, limit_ns: int):

@@ -1,4 +1,5 @@
-"""Build the CUDA library in-tree: paper_2506_19651_b200/libpevlm.so (sm_100a only).
+"""Build the CUDA library in-tree: paper_2506_19651_b200/libpevlm.so (sm_100a only), and the module through which Python
+calls it (_pevlm_call, linked against the library next to it).
 
     python -m paper_2506_19651_b200.build [--force]
 
@@ -10,12 +11,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 _DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_DIR, "csrc")
 LIB = os.path.join(_DIR, "libpevlm.so")
+CALL = os.path.join(_DIR, "_pevlm_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["api.cu", "rope_kernel.cu", "assemble_kernel.cu", "attn_kernel.cu", "decode_kernel.cu", "merge_kernel.cu", "query_noalloc.cu", "selftest.cu"]
-HEADERS = ["internal.h", "ptx.cuh", os.path.join("..", "..", "include", "pevlm.h")]
+HEADERS = ["internal.h", "ptx.cuh", "pycall.c", os.path.join("..", "..", "include", "pevlm.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-cudart", "static"]
 
@@ -28,9 +31,9 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALL))
     deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -59,6 +62,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     link = [_nvcc(), "-shared", *NVCC_FLAGS[:2], "-cudart", "static", "-o", tmp, *objs]
     subprocess.run(link, check=True)
     os.replace(tmp, LIB)
+    tmp = CALL + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CC", "gcc"), "-shared", "-fPIC", "-O2", "-Wall", "-I", sysconfig.get_paths()["include"],
+                    os.path.join(CSRC, "pycall.c"), "-o", tmp, "-L", _DIR, "-l:libpevlm.so", "-Wl,-rpath,$ORIGIN"], check=True)
+    os.replace(tmp, CALL)
     return LIB
 
 

@@ -63,7 +63,7 @@ cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream) {
     int64_t ctas = (s.total + per_cta - 1) / per_cta;
     const int64_t cap = 148 * 16;  // a few waves of the 148 SMs; the loop strides over the rest
     if (ctas > cap) ctas = cap;
-    return launch_chained(copy_segments_kernel, dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(s.batch)), kCopyThreads, 0, stream, s);
+    return launch_chained<copy_segments_kernel>(dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(s.batch)), kCopyThreads, 0, stream, s);
 }
 
 }  // namespace pevlm

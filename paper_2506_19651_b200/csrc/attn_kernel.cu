@@ -740,9 +740,10 @@ cudaError_t launch_attn(const AttnParams& p, int head_dim, const AttnMaps& m, cu
     const size_t smem = attn_smem_bytes(head_dim);
     // one cluster per work item; those that run take the rest from the hardware's queue
     const unsigned grid = 2u * static_cast<unsigned>(items);
-    auto go = [&](auto kernel) { return launch_chained(kernel, grid, kAttnThreads, smem, stream, p, m); };
-    if (head_dim == 128) return p.mode == 1 ? go(attn_kernel<128, 1>) : p.mode == 2 ? go(attn_kernel<128, 2>) : go(attn_kernel<128, 3>);
-    return p.mode == 1 ? go(attn_kernel<64, 1>) : p.mode == 2 ? go(attn_kernel<64, 2>) : go(attn_kernel<64, 3>);
+#define PEVLM_GO(D_, M_) launch_chained<attn_kernel<D_, M_>>(grid, kAttnThreads, smem, stream, p, m)
+    if (head_dim == 128) return p.mode == 1 ? PEVLM_GO(128, 1) : p.mode == 2 ? PEVLM_GO(128, 2) : PEVLM_GO(128, 3);
+    return p.mode == 1 ? PEVLM_GO(64, 1) : p.mode == 2 ? PEVLM_GO(64, 2) : PEVLM_GO(64, 3);
+#undef PEVLM_GO
 }
 
 }  // namespace pevlm

@@ -231,10 +231,10 @@ cudaError_t launch_decode(const DecodeParams& p, int head_dim, cudaStream_t stre
     const dim3 grid(static_cast<unsigned>(p.n_splits), static_cast<unsigned>(p.Hkv), static_cast<unsigned>(p.batch));
     const bool two = p.Q * p.G > 16;
     if (head_dim == 128)
-        return two ? launch_chained(decode_kernel<128, 2>, grid, kDecodeThreads, DecodeSmem<128, 2>::kTotal, stream, p)
-                   : launch_chained(decode_kernel<128, 1>, grid, kDecodeThreads, DecodeSmem<128, 1>::kTotal, stream, p);
-    return two ? launch_chained(decode_kernel<64, 2>, grid, kDecodeThreads, DecodeSmem<64, 2>::kTotal, stream, p)
-               : launch_chained(decode_kernel<64, 1>, grid, kDecodeThreads, DecodeSmem<64, 1>::kTotal, stream, p);
+        return two ? launch_chained<decode_kernel<128, 2>>(grid, kDecodeThreads, DecodeSmem<128, 2>::kTotal, stream, p)
+                   : launch_chained<decode_kernel<128, 1>>(grid, kDecodeThreads, DecodeSmem<128, 1>::kTotal, stream, p);
+    return two ? launch_chained<decode_kernel<64, 2>>(grid, kDecodeThreads, DecodeSmem<64, 2>::kTotal, stream, p)
+               : launch_chained<decode_kernel<64, 1>>(grid, kDecodeThreads, DecodeSmem<64, 1>::kTotal, stream, p);
 }
 
 }  // namespace pevlm

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/pevlm.h"
 
 namespace pevlm {
@@ -44,14 +46,19 @@ __device__ __forceinline__ int quotient(int a, const Divisor& b) {
 // in the stream still runs, so that its launch costs nothing; every kernel therefore calls grid_wait() before it touches
 // global memory.  All kernels ask for the same split of the SM's memory (as much shared memory as there is), because an
 // SM has to run empty before it can change the split.
-template <typename... Params, typename... Args>
-inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
-                                  const Args&... args) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+template <auto Kernel, typename... Args>
+inline cudaError_t launch_chained(dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, const Args&... args) {
+    // attributes of a kernel: once on each device (smem is the same in every launch of a kernel)
+    static std::atomic<uint64_t> prepared{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (dev >= 64 || !(prepared.load(std::memory_order_acquire) >> dev & 1)) {
+        e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+        if (e == cudaSuccess && smem > 48 * 1024)
+            e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
+        if (dev < 64) prepared.fetch_or(1ull << dev, std::memory_order_release);
     }
     cudaLaunchAttribute chained;
     chained.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -63,7 +70,7 @@ inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, unsigned
     config.stream = stream;
     config.attrs = &chained;
     config.numAttrs = 1;
-    e = cudaLaunchKernelEx(&config, kernel, args...);
+    e = cudaLaunchKernelEx(&config, Kernel, args...);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

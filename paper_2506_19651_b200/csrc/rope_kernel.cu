@@ -201,8 +201,8 @@ cudaError_t launch_rope(const RopeParams& params, int head_dim, cudaStream_t str
     p.div_seq = make_divisor(p.seq_len);
     const int64_t groups = (p.n_tokens + p.group - 1) / p.group;
     const unsigned grid = static_cast<unsigned>(groups < resident ? groups : resident);
-    return head_dim == 128 ? launch_chained(rope_kernel<128>, grid, kRopeThreads, sizeof(RopeSmem<128>), stream, p)
-                           : launch_chained(rope_kernel<64>, grid, kRopeThreads, sizeof(RopeSmem<64>), stream, p);
+    return head_dim == 128 ? launch_chained<rope_kernel<128>>(grid, kRopeThreads, sizeof(RopeSmem<128>), stream, p)
+                           : launch_chained<rope_kernel<64>>(grid, kRopeThreads, sizeof(RopeSmem<64>), stream, p);
 }
 
 }  // namespace pevlm

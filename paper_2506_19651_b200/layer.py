@@ -146,6 +146,10 @@ class StreamingWindow:
     def _shape(self, S, B, N, Q):
         return pb.make_shape(S, B, N, Q, self.Hq, self.Hkv, self.d, theta=self.theta, scale=self.scale)
 
+    def _row(self, cache, row):
+        """Address of a cache row (what cache[row:] would point to, without building the view)."""
+        return cache.data_ptr() + row * self.Hkv * self.d * 2
+
     def set_sink(self, q, k, v):
         """Encode the sink (Eq. 3).  Returns (o [S,Hq,d], lse [Hq,S])."""
         import torch
@@ -164,7 +168,7 @@ class StreamingWindow:
         row0 = S + (t % self.W) * B
         o = torch.empty((B, self.Hq, self.d), dtype=self._bf, device=self._dev)
         lse = torch.empty((self.Hq, B), dtype=self._f32, device=self._dev)
-        pb.pevlm_rope_qkv(self.s_block, q, k, v, self.q_buf, self.k_cache[row0:], self.v_cache[row0:], S + t * B, B)
+        pb.pevlm_rope_qkv(self.s_block, q, k, v, self.q_buf, self._row(self.k_cache, row0), self._row(self.v_cache, row0), S + t * B, B)
         pb.pevlm_block_attn(self.s_block, self.q_buf, self.k_cache, self.v_cache, row0, self.rows, o, lse, self.ws_block)
         self.blocks_seen = t + 1
         return o, lse
@@ -179,6 +183,7 @@ class StreamingWindow:
         s = self._shape(nv, 1, 0, Qn)
         o = torch.empty((Qn, self.Hq, self.d), dtype=self._bf, device=self._dev)
         lse = torch.empty((self.Hq, Qn), dtype=self._f32, device=self._dev)
-        pb.pevlm_rope_qkv(s, q, k, v, self.q_buf, self.k_cache[nv:], self.v_cache[nv:], self.S + self.blocks_seen * self.B, Qn)
+        pb.pevlm_rope_qkv(s, q, k, v, self.q_buf, self._row(self.k_cache, nv), self._row(self.v_cache, nv),
+                          self.S + self.blocks_seen * self.B, Qn)
         pb.pevlm_query_attn(s, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_query)
         return o, lse
