@@ -20,6 +20,7 @@ namespace pevlm {
 constexpr int kDecodeThreads = 256;
 constexpr int kDecodeWarps = kDecodeThreads / 32;
 constexpr int kPiece = 16;  // keys a warp takes at a time
+constexpr int kEarlyPieces = 8;  // of a warp, fetched into L2 ahead (50K keys: a step takes 27.2 us with 0, 26.7 with 4, 26.4 with 8)
 
 // MT: 16-row tiles
 template <int D, int MT>
@@ -62,13 +63,25 @@ __global__ void __launch_bounds__(kDecodeThreads, 1) decode_kernel(const __grid_
     const int piece0 = split * p.pieces_per_split;
     const int pieces = min(p.pieces_per_split, p.pieces - piece0);
     const int mine = pieces > warp ? (pieces - warp + kDecodeWarps - 1) / kDecodeWarps : 0;  // pieces of this warp
+    const int64_t row_stride = static_cast<int64_t>(p.Hkv) * D;
+    const __nv_bfloat16* k = p.k + seq * p.L * row_stride + g * D;
+    const __nv_bfloat16* v = p.v + seq * p.L * row_stride + g * D;
+    // While the kernels before this one finish (a decode step's RoPE and copy of one token leave nearly all SMs idle), the
+    // first pieces are brought into L2: that reads nothing, so what those kernels still write is seen all the same.
+    for (int n = 0; n < min(mine, kEarlyPieces); ++n) {
+        const int key0 = (piece0 + warp + n * kDecodeWarps) * kPiece;
+        constexpr int kLines = D * 2 / 128;  // lines of a row
+        for (int i = lane; i < kPiece * kLines; i += 32) {
+            const int64_t key = min(key0 + i / kLines, p.L - 1);
+            const int64_t off = key * row_stride + i % kLines * 64;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(k + off));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(v + off));
+        }
+    }
     grid_wait();
     grid_launch_dependents();
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) p.hdr->status = p.hdr->detail = 0;
 
-    const int64_t row_stride = static_cast<int64_t>(p.Hkv) * D;
-    const __nv_bfloat16* k = p.k + seq * p.L * row_stride + g * D;
-    const __nv_bfloat16* v = p.v + seq * p.L * row_stride + g * D;
     auto fetch = [&](int n) {  // the warp's n-th piece
         if (n < mine) {
             const int key0 = (piece0 + warp + n * kDecodeWarps) * kPiece;
