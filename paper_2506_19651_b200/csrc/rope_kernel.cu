@@ -3,7 +3,7 @@
 // fused multiply-add in the rotation, so every fp64 operation rounds exactly once), then one rounding fp64 -> fp32 ->
 // bf16 (round to nearest even).
 //
-// The CTAs share the tokens out in groups of up to 8 neighbours.  A CTA evaluates a group's angles once (fp64 sincos)
+// The CTAs share the tokens out in groups of up to 4 neighbours.  A CTA evaluates a group's angles once (fp64 sincos)
 // into shared memory, one group ahead, and its threads walk over the group's head vectors of Q and K: d/16 threads a
 // vector, 16 bytes of either half each; the vectors of a group are one contiguous range per tensor.  What bounds it: DRAM
 // traffic.  Two things used to stand in the way (numbers for B200, 28/4 heads of 128):
@@ -25,8 +25,11 @@ namespace pevlm {
 
 constexpr int kRopeThreads = 256;
 constexpr int kRopeCtasPerSm = 3;
-constexpr int kRopeTokens = 8;   // most tokens of a group
-constexpr int kRopeRing = 6;     // vectors a thread has in flight
+// Most tokens of a group, and vectors a thread has in flight: with V copied along, 50K tokens of 28/4 heads take 171 us with
+// groups of 8 and a ring of 6, 151 with 4 and 6, 150 with 4 and 5, 164 with 2 and 6; two CTAs per SM with longer rings are
+// faster at 32/8 heads only (130 against 148 us for 33K tokens), slower everywhere else.
+constexpr int kRopeTokens = 4;
+constexpr int kRopeRing = 5;
 
 // 16-byte accesses that do not allocate in L1 (every byte is touched once)
 __device__ __forceinline__ void fetch16(uint32_t dst, const __nv_bfloat16* src) {
