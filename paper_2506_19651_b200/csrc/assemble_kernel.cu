@@ -22,8 +22,8 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
 }
 
 __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(CopySegments s) {
-    grid_wait();
     grid_launch_dependents();
+    grid_wait();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {  // the sequence of this row of CTAs
         s.src[k] += static_cast<int64_t>(blockIdx.y) * s.src_stride[k];

@@ -310,15 +310,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     cluster_sync_all();  // also: the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after_sync();
     const uint32_t tmem_base = uniform(tmem_base_slot);
-    grid_wait();  // nothing above touches global memory
+    // The roles that touch global memory (producer, epilogue, scheduler) call grid_wait() themselves, so that the first item
+    // is decoded while the kernels before this one finish.
     grid_launch_dependents();
-    // The status word of the previous call on this workspace is cleared by the launch's first block, long before any wait
-    // of this launch can have run out.
-    if (blockIdx.x == 0 && tid == 0 && !p.keep_status) {
-        p.hdr->detail = 0;
-        *reinterpret_cast<volatile int32_t*>(&p.hdr->status) = 0;
-        if (MODE == 3) p.hdr_question->status = p.hdr_question->detail = 0;
-    }
 
 #ifdef PEVLM_TRACE
     __shared__ unsigned s_waits[16][kTraceIds];
@@ -357,7 +351,10 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                 int published = 0, asked = 0;
                 // After a timeout the clusters that are still to be launched do nothing (those of the first wave may find
                 // an older call's status, so they do not look).
-                if (w >= kNumSms / 2 && *reinterpret_cast<volatile int32_t*>(&p.hdr->status) != 0) w = -1;
+                if (w >= kNumSms / 2) {
+                    grid_wait();
+                    if (*reinterpret_cast<volatile int32_t*>(&p.hdr->status) != 0) w = -1;
+                }
                 while (true) {
                     const int slot = published % kItems;
                     if (published >= kItems) wait_asleep(bars.item_free[slot], (published / kItems - 1) & 1, kWaitItemFree);
@@ -391,6 +388,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
         } else if (warp == 13) {
             // --------------------------------------------------------- TMA producer: K(s), then V(s - kQkAhead)
             // (The whole warp runs this with uniform values; single lanes issue.)
+            grid_wait();
             {
                 // The K cursor's item, and where V has to come from: the rows of the last kQkAhead K tiles (base row of the
                 // tile, kv head and map), the V tile of a step being that of kQkAhead steps ago.
@@ -520,6 +518,14 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     } else if (warp >= 8) {
         // ------------------------------------------------------------- epilogue
         reg_dealloc<96>();
+        grid_wait();
+        // The status word of the previous call on this workspace is cleared by the launch's first block, long before any
+        // wait of this launch can have run out.
+        if (blockIdx.x == 0 && tid == 256 && !p.keep_status) {
+            p.hdr->detail = 0;
+            *reinterpret_cast<volatile int32_t*>(&p.hdr->status) = 0;
+            if (MODE == 3) p.hdr_question->status = p.hdr_question->detail = 0;
+        }
         const int row = tid & 127;
         const uint32_t tO = tmem_base + kTmemO + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const uint32_t o_free_bar = map_to_cta(smem_u32(&bars.o_free), 0);

@@ -133,8 +133,8 @@ __global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(cons
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    grid_wait();
     grid_launch_dependents();
+    grid_wait();
 #pragma unroll 1
     for (int i = 0; i < kRopeRing - 1; ++i) fetch();
     int buf = 0, ring = 0;
