@@ -310,8 +310,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     cluster_sync_all();  // also: the other CTA's barriers are initialised before anything arrives on them
     tc_fence_after_sync();
     const uint32_t tmem_base = uniform(tmem_base_slot);
-    // The roles that touch global memory (producer, epilogue, scheduler) call grid_wait() themselves, so that the first item
-    // is decoded while the kernels before this one finish.
+    // Every role reads its first item while the kernels before this one finish and then calls grid_wait(), before it touches
+    // global memory or waits for what others fetch from there: the kernels before do not count towards the limit of a wait,
+    // however many they are.  (All of them waiting before the first item is decoded: 0.45 us a launch.)
     grid_launch_dependents();
 
 #ifdef PEVLM_TRACE
@@ -368,6 +369,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                         mbar_arrive(smem_u32(&bars.item_full[slot]));  // release: the decoded item is visible
                         if (w < 0) break;
                         ++published;
+                        if (published == 1) grid_wait();
                         // the next item is claimed when the loads of this one near their end, so that a pair never
                         // sits on work another one could take
                         if (rank == 0) wait_asleep(bars.go, (published - 1) & 1, kWaitGo);
@@ -388,7 +390,6 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
         } else if (warp == 13) {
             // --------------------------------------------------------- TMA producer: K(s), then V(s - kQkAhead)
             // (The whole warp runs this with uniform values; single lanes issue.)
-            grid_wait();
             {
                 // The K cursor's item, and where V has to come from: the rows of the last kQkAhead K tiles (base row of the
                 // tile, kv head and map), the V tile of a step being that of kQkAhead steps ago.
@@ -412,6 +413,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                             const int rows = uniform((it.s[0].valid ? it.s[0].box_rows : 0) + (it.s[1].valid ? it.s[1].box_rows : 0));
                             __syncwarp();
                             if (lane == 0) item_release(k);
+                            if (k == 0) grid_wait();
                             const int qb = k & 1;
                             if (k >= 2) wait(bars.q_free[qb], ((k >> 1) - 1) & 1, kWaitQFree);
                             if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.q_full[qb]), static_cast<uint32_t>(NP * 128 * rows));
@@ -472,6 +474,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                 __syncwarp();
                 if (lane == 0) item_release(k);
                 const uint32_t q_lo = desc_lo(smem_base + L::kQ + (k & 1) * L::kQBytes, 16);
+                if (k == 0) grid_wait();
                 wait(bars.q_full[k & 1], (k >> 1) & 1, kWaitQ);
 #pragma unroll 1
                 for (int j = 0; j < nt; ++j, ++t) {
@@ -499,6 +502,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                 if (lane == 0) item_release(k);
                 // the previous item's output must have left TMEM before O is overwritten
                 if (k > 0) wait(bars.o_free, (k - 1) & 1, kWaitOFree);
+                else grid_wait();
 #pragma unroll 1
                 for (int j = 0; j < nt; ++j, ++t) {
                     const int n = j == na - 1 ? n_a : j == nt - 1 ? n_b : kTile;
@@ -612,6 +616,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             const int my_limit = min(first_limit + row_tok, end - 1), limit0 = min(first_limit, end - 1);
             __syncwarp();
             if (lane == 0) item_release(k);
+            if (k == 0) grid_wait();
             float m_own = -INFINITY;  // reference maximum (raw score units) this warpgroup's row sum is scaled by
             float l_run = 0.f;
             const int first = static_cast<int>((t0 ^ static_cast<uint32_t>(wg)) & 1u);  // this warpgroup has the even or the odd tiles
