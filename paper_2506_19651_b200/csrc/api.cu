@@ -135,6 +135,32 @@ struct QueryPlan {
     int pieces, pieces_per_split;  // decode kernel (at most kDecodeRows rows per kv head): 16-key pieces; 0 = tile kernel
 };
 
+// Key tiles of the prefill work items (each a pair of query tiles): of the longest one, and of all together, with two
+// for the start and the end of each item.
+struct PrefillSize {
+    int longest;
+    int64_t all;
+};
+
+static PrefillSize prefill_size(const pevlm_shape_t* s, int last_len) {
+    const int G = s->num_q_heads / s->num_kv_heads;
+    PrefillSize r{0, 0};
+    auto add = [&](int64_t segments, int64_t shared, int64_t len) {
+        if (segments <= 0 || len <= 0) return;
+        const int64_t a = (shared + kTile - 1) / kTile, n = (len + kTile - 1) / kTile;
+        r.all += segments * s->num_kv_heads * ((G * (n * a + n * (n + 1) / 2) + 1) / 2 + 2 * plan_segment(static_cast<int>(len), G).pairs);
+        if (a + n > r.longest) r.longest = static_cast<int>(a + n);
+    };
+    if (s->mask_mode == PEVLM_MASK_FULL_CAUSAL) {
+        add(1, 0, n_video(s, last_len));
+    } else {
+        add(1, 0, s->sink_len);
+        add(s->num_blocks - (last_len > 0 ? 1 : 0), s->sink_len, s->block_len);
+        add(last_len > 0 ? 1 : 0, s->sink_len, last_len);
+    }
+    return r;
+}
+
 static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false, int last_len = 0) {
     QueryPlan q;
     const int G = s->num_q_heads / s->num_kv_heads;
@@ -147,13 +173,26 @@ static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false,
     const int pairs = (q.q_tiles + 1) / 2;
     const int groups = s->num_kv_heads * (pairs > 0 ? pairs : 1);
     int want = kNumSms / 2 / groups;
+    // Keys up to `whole` tiles are not split, and there is nothing to merge.  Measured, whole against split: alone, 4/2 heads
+    // and 50 tokens, 4 tiles 6.9 / 7.7 us, 5 tiles 7.7 / 7.8, 6 tiles 8.6 / 8.2; 28/4 heads and 60 tokens, whose merge is one of many
+    // rows, 8 tiles 10.3 / 12.7.  Behind prefill items: 5 tiles more than the longest of them 16.6 / 17.5, 7 more 18.2 / 18.6,
+    // 9 more 21.0 / 19.2; 200 tokens of 28/4 heads, 8 more 22.0 / 25.3.
+    const bool many_rows = static_cast<int64_t>(s->batch) * s->query_len * s->num_q_heads > kMergeRows;
+    int whole = many_rows ? 8 : 5;
     if (beside_prefill) {
-        // in one launch with the prefill items, which fill in behind them: enough items for every pair of CTAs, none
-        // longer than 64 key tiles (a prefill item of the 50K-token stream has 25), none shorter than 4
-        const int per_pair = static_cast<int>((static_cast<int64_t>(groups) * q.total_kv_tiles + kNumSms / 2 - 1) / (kNumSms / 2));
-        const int tiles = per_pair < 4 ? 4 : per_pair > 64 ? 64 : per_pair;
+        // In one launch with the prefill items, which fill in behind them.  Enough items for every pair of CTAs, none
+        // longer than 64 key tiles, none shorter than 4; but where the question is the smaller part of the launch, an item
+        // may take as long as the launch takes anyway, since it starts first: as a rule no split at all (12.6K tokens
+        // 282 -> 277 us, 74K 2,222 -> 2,191; 1.8K tokens 35.2 -> 29.4).
+        const PrefillSize pre = prefill_size(s, last_len);
+        const int64_t own = static_cast<int64_t>(groups) * q.total_kv_tiles, most = (own + pre.all) / (kNumSms / 2);
+        const int per_pair = static_cast<int>((own + kNumSms / 2 - 1) / (kNumSms / 2));
+        int tiles = per_pair < 4 ? 4 : per_pair > 64 ? 64 : per_pair;
+        if (own <= pre.all && most > tiles) tiles = most < q.total_kv_tiles ? static_cast<int>(most) : q.total_kv_tiles;
         want = (q.total_kv_tiles + tiles - 1) / tiles;
+        whole = pre.longest + (many_rows ? 9 : 7);
     }
+    if (q.total_kv_tiles <= whole) want = 1;
     if (want < 1) want = 1;
     if (want > q.total_kv_tiles) want = q.total_kv_tiles;
     q.pieces = q.pieces_per_split = 0;
@@ -389,7 +428,6 @@ static void add_prefill(AttnParams& p, const pevlm_shape_t* s, bool blocks_only,
     const int blk_q0 = blocks_only ? 0 : S;
     p.q_rows = static_cast<int>(blocks_only ? static_cast<int64_t>(s->num_blocks) * s->block_len : nv);
     p.kv_rows = static_cast<int>(blocks_only ? cache_rows : nv);
-    p.lse_stride = p.q_rows;
     p.div_hkv = make_divisor(p.Hkv);
     p.div_g = make_divisor(p.G);
     auto fill = [&](Segment& g, int n, int len, int q0, int key0, int a_end, int own_map, bool blocks) {
@@ -576,10 +614,11 @@ int pevlm_query_attn(const pevlm_shape_t* s, const void* q_question, const void*
         const int64_t q0 = static_cast<int64_t>(b) * p.Q, k0 = static_cast<int64_t>(b) * p.L;
         AttnMaps m;
         if ((rc = question_maps(m, p, d, rows_of(q_question, q0, p.Hq, d), rows_of(k_cache, k0, p.Hkv, d), rows_of(v_cache, k0, p.Hkv, d))) != PEVLM_OK) return rc;
+        p.o_question = const_cast<__nv_bfloat16*>(rows_of(o, q0, p.Hq, d));
+        p.lse_question = lse ? lse + p.Hq * q0 : nullptr;
         const cudaError_t e = launch_attn(p, d, m, static_cast<cudaStream_t>(stream));
         if (e != cudaSuccess) return cuda_fail(e, "question attention launch");
-        rc = merge_question(p, d, const_cast<__nv_bfloat16*>(rows_of(o, q0, p.Hq, d)), lse ? lse + p.Hq * q0 : nullptr,
-                            static_cast<cudaStream_t>(stream));
+        if (p.n_splits > 1) rc = merge_question(p, d, p.o_question, p.lse_question, static_cast<cudaStream_t>(stream));
         if (rc != PEVLM_OK) return rc;
     }
     return PEVLM_OK;
@@ -626,6 +665,8 @@ int pevlm_layer_forward(const pevlm_shape_t* s, int32_t last_len, const void* q,
         add_question(p, qp);
         rc = question_maps(m, p, d, static_cast<const __nv_bfloat16*>(q_question), static_cast<const __nv_bfloat16*>(k_cache), static_cast<const __nv_bfloat16*>(v_cache));
         if (rc != PEVLM_OK) return rc;
+        p.o_question = static_cast<__nv_bfloat16*>(o_question);
+        p.lse_question = lse_question;
         p.hdr_question = static_cast<WorkspaceHeader*>(ws_query);
         if (nv == 0) p.hdr = p.hdr_question;
         p.part_o = reinterpret_cast<float*>(static_cast<uint8_t*>(ws_query) + kStatusBytes);
@@ -633,7 +674,7 @@ int pevlm_layer_forward(const pevlm_shape_t* s, int32_t last_len, const void* q,
     }
     const cudaError_t e = launch_attn(p, d, m, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(e, "attention launch");
-    return Q > 0 ? merge_question(p, d, static_cast<__nv_bfloat16*>(o_question), lse_question, static_cast<cudaStream_t>(stream)) : PEVLM_OK;
+    return Q > 0 && p.n_splits > 1 ? merge_question(p, d, p.o_question, p.lse_question, static_cast<cudaStream_t>(stream)) : PEVLM_OK;
 }
 
 int pevlm_selftest_wait_expiry(void* workspace, size_t workspace_bytes, int64_t limit_ns, void* stream) {

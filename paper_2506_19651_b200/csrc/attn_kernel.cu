@@ -545,6 +545,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             const int head = qs.q_head0 + row_head;
             const int split = it.split, seq = it.seq;
             const bool question = MODE == 2 || (MODE == 3 && it.own_map == 2);
+            const bool partial = question && p.n_splits > 1;  // left to the merge
             __syncwarp();
             if (lane == 0) item_release(k);
             wait_asleep(bars.sums_full[k % kSums], (k / kSums) & 1, kWaitSum);
@@ -559,8 +560,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             // 32 columns at a time, in a loop that stays one; 32 bytes per store: every lane writes whole sectors of
             // its own row
             // (tok counts over the batch; the partials are ordered sequence, split, token, head)
-            const size_t r = !question ? static_cast<size_t>(tok) * p.Hq + head
-                                       : (static_cast<size_t>(seq * (p.n_splits - 1) + split) * p.Q + tok) * p.Hq + head;
+            const size_t r = !partial ? static_cast<size_t>(tok) * p.Hq + head
+                                      : (static_cast<size_t>(seq * (p.n_splits - 1) + split) * p.Q + tok) * p.Hq + head;
+            __nv_bfloat16* const out = question ? p.o_question : p.o;
 #pragma unroll 1
             for (int c = 0; c < D / 32; ++c) {
                 uint32_t o[32];
@@ -571,7 +573,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(o_free_bar);
                 }
-                if (!question) {
+                if (!partial) {
                     uint32_t wd[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) {
@@ -582,7 +584,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     if (row_ok) {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
-                            st_global_v8(p.o + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]));
+                            st_global_v8(out + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]));
                     }
                 } else if (row_ok) {
 #pragma unroll
@@ -591,9 +593,10 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     for (int v = 0; v < 4; ++v) st_global_v8(p.part_o + r * D + c * 32 + v * 8, *reinterpret_cast<uint32_t(*)[8]>(&o[8 * v]));
                 }
             }
-            if (row_ok && !question && p.lse)
-                st_global_stream_f32(p.lse + static_cast<size_t>(seq * p.Hq + head) * p.lse_stride + (tok - seq * p.q_rows), lse_val);
-            if (row_ok && question) st_global_stream_f32(p.part_lse + r, lse_val);
+            float* const lse = partial ? p.part_lse : question ? p.lse_question : p.lse;
+            const int rows = question ? p.Q : p.q_rows;  // of a sequence
+            const size_t at = partial ? r : static_cast<size_t>(seq * p.Hq + head) * rows + (tok - seq * rows);
+            if (row_ok && lse) st_global_stream_f32(lse + at, lse_val);
         }
     } else {
         // ------------------------------------------------------------- softmax, every other key tile

@@ -104,9 +104,8 @@ struct AttnParams {
     int32_t sink_len;       // prefill (host only): S,
     int32_t block_rows;     // rows of all blocks
     int32_t blk_key0;       // and K/V row of the first block (S, or the cache row of a block range)
-    int32_t q_rows;         // prefill: rows of q / o of a sequence
+    int32_t q_rows;         // prefill: rows of q / o (and columns of lse) of a sequence
     int32_t kv_rows;        // prefill: rows of k / v of a sequence
-    int32_t lse_stride;     // prefill: row stride of lse
     int32_t Q, L;           // question length, total length
     int32_t Hq, Hkv, G;
     int32_t items_question; // question work items
@@ -120,14 +119,17 @@ struct AttnParams {
     float scale;            // softmax scale
     float scale_log2;       // scale * log2(e)
     __nv_bfloat16* o;       // prefill: [batch * q_rows, Hq, d]
-    float* lse;             // prefill: [batch, Hq, lse_stride] or NULL
-    float* part_o;          // question: [batch, n_splits, Q, Hq, d] fp32
-    float* part_lse;        // question: [batch, n_splits, Q, Hq]
+    float* lse;             // prefill: [batch, Hq, q_rows] or NULL
+    __nv_bfloat16* o_question;  // question, n_splits = 1: [batch, Q, Hq, d]
+    float* lse_question;        // and [batch, Hq, Q] or NULL
+    float* part_o;          // question, n_splits > 1: [batch, n_splits, Q, Hq, d] fp32
+    float* part_lse;        // and [batch, n_splits, Q, Hq]
     WorkspaceHeader* hdr;
     WorkspaceHeader* hdr_question;  // mode 3: header of the question's workspace
     int32_t keep_status;    // a later launch of the same call
 };
 
+constexpr int kMergeRows = 8 * kNumSms;  // most rows of the merge that takes a CTA for each (as many as are resident)
 constexpr int kDecodeRows = 32;  // most rows (question tokens x heads of a kv group) of the decode kernel
 
 // Question attention of a few rows, see decode_kernel.cu.

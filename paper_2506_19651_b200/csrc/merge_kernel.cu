@@ -133,8 +133,8 @@ cudaError_t launch_merge(const MergeParams& p, cudaStream_t stream) {
     const int64_t rows = static_cast<int64_t>(p.Q) * p.Hq;
     if (rows <= 0) return cudaSuccess;
     const unsigned batch = static_cast<unsigned>(p.batch);
-    // up to eight CTAs per SM (as many as are resident): the latency-oriented form
-    if (rows * batch <= static_cast<int64_t>(kNumSms) * 8 && p.n_splits <= kMergeMaxParts)
+    // few rows: the latency-oriented form
+    if (rows * batch <= kMergeRows && p.n_splits <= kMergeMaxParts)
         return launch_chained<merge_rows_kernel>(dim3(static_cast<unsigned>(rows), batch), kMergeThreads, 0, stream, p);
     const int64_t n = rows * (p.d / 4);
     return launch_chained<merge_kernel>(dim3(static_cast<unsigned>((n + kMergeThreads - 1) / kMergeThreads), batch), kMergeThreads, 0,

@@ -44,7 +44,7 @@ class LayerBuffers:
         self.ws_query = _workspace(alloc, pb.pevlm_workspace_bytes(s, pb.WS_QUERY))
 
 
-KERNELS_PER_PASS = 3          # rope and V copy, attention of video and question rows, merge
+KERNELS_PER_PASS = 2          # rope and V copy, attention of video and question rows; a merge too where the question's keys are split
 KERNELS_PER_PASS_BY_CALL = 7  # with `mark`: rope, V copy, prefill attention, rope, V copy, question attention, merge
 
 
