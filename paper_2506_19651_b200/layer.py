@@ -96,11 +96,12 @@ def ragged_layer_forward(q, k, v, S, B, N, B_last, Q, theta, scale=0.0, alloc=No
     nv = S + (N - 1) * B + B_last
     L = nv + Q
     assert N >= 1 and 1 <= B_last <= B and q.shape[0] == L
-    dev, bf, f32 = q.device, torch.bfloat16, torch.float32
+    bf, f32 = torch.bfloat16, torch.float32
     s = pb.make_shape(S, B, N, Q, Hq, Hkv, d, theta=theta, scale=scale)
     if alloc is None:
+        # (new_empty takes type and device from the tensor: half of torch.empty's time on the host)
         def alloc(shp, dtype, zero=False):
-            return torch.empty(shp, dtype=dtype, device=dev)
+            return q.new_empty(shp) if dtype is q.dtype else q.new_empty(shp, dtype=dtype)
     q_roped = alloc((L, Hq, d), bf)
     k_cache = alloc((L, Hkv, d), bf)
     v_cache = alloc((L, Hkv, d), bf)
@@ -141,7 +142,11 @@ class StreamingWindow:
         self.ws_block = _workspace(alloc, pb.pevlm_workspace_bytes(self.s_block, pb.WS_PREFILL))
         self.ws_query = _workspace(alloc, pb.pevlm_workspace_bytes(self._shape(S + W * B, 1, 0, Q_max), pb.WS_QUERY))
         self.blocks_seen = 0
-        self._f32, self._bf, self._dev = f32, bf, device
+        self._f32 = torch.empty((0,), dtype=f32, device=device)
+
+    def _outputs(self, n):
+        """o [n,Hq,d] and lse [Hq,n] (new_empty, which takes type and device from a tensor, costs the host half of torch.empty)."""
+        return self.k_cache.new_empty((n, self.Hq, self.d)), self._f32.new_empty((self.Hq, n))
 
     def _shape(self, S, B, N, Q):
         return pb.make_shape(S, B, N, Q, self.Hq, self.Hkv, self.d, theta=self.theta, scale=self.scale)
@@ -152,22 +157,18 @@ class StreamingWindow:
 
     def set_sink(self, q, k, v):
         """Encode the sink (Eq. 3).  Returns (o [S,Hq,d], lse [Hq,S])."""
-        import torch
         S = self.S
-        o = torch.empty((S, self.Hq, self.d), dtype=self._bf, device=self._dev)
-        lse = torch.empty((self.Hq, S), dtype=self._f32, device=self._dev)
+        o, lse = self._outputs(S)
         pb.pevlm_rope_qkv(self.s_sink, q, k, v, self.q_buf, self.k_cache, self.v_cache, 0, S)
         pb.pevlm_parallel_prefill_attn(self.s_sink, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_sink)
         return o, lse
 
     def append_block(self, q, k, v):
         """Encode the next block of the stream into the slot of the oldest one.  Returns (o [B,Hq,d], lse [Hq,B])."""
-        import torch
         S, B = self.S, self.B
         t = self.blocks_seen
         row0 = S + (t % self.W) * B
-        o = torch.empty((B, self.Hq, self.d), dtype=self._bf, device=self._dev)
-        lse = torch.empty((self.Hq, B), dtype=self._f32, device=self._dev)
+        o, lse = self._outputs(B)
         pb.pevlm_rope_qkv(self.s_block, q, k, v, self.q_buf, self._row(self.k_cache, row0), self._row(self.v_cache, row0), S + t * B, B)
         pb.pevlm_block_attn(self.s_block, self.q_buf, self.k_cache, self.v_cache, row0, self.rows, o, lse, self.ws_block)
         self.blocks_seen = t + 1
@@ -176,13 +177,11 @@ class StreamingWindow:
     def ask(self, q, k, v):
         """Question of Qn <= Q_max tokens at the positions that follow the stream so far, against the sink
         and the blocks in the window (Eq. 5).  Returns (o [Qn,Hq,d], lse [Hq,Qn])."""
-        import torch
         Qn = q.shape[0]
         held = min(self.blocks_seen, self.W)
         nv = self.S + held * self.B
         s = self._shape(nv, 1, 0, Qn)
-        o = torch.empty((Qn, self.Hq, self.d), dtype=self._bf, device=self._dev)
-        lse = torch.empty((self.Hq, Qn), dtype=self._f32, device=self._dev)
+        o, lse = self._outputs(Qn)
         pb.pevlm_rope_qkv(s, q, k, v, self.q_buf, self._row(self.k_cache, nv), self._row(self.v_cache, nv),
                           self.S + self.blocks_seen * self.B, Qn)
         pb.pevlm_query_attn(s, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_query)
