@@ -83,7 +83,7 @@ static size_t attn_smem_bytes(int head_dim) {
 // One query tile.  Row r of the tile is token q_tok0 + r / row_div, head q_head0 + r % row_div; it
 // exists iff r / row_div < ntok and r % row_div < nheads.  Full prefill tiles have row_div = 1; the
 // ragged last tile of a segment packs the tails of several q heads of the kv group (row_div heads,
-// ntok = the tail's rows); question tiles pack all G heads of the group.
+// ntok = the tail's rows, or some of them and all heads); question tiles pack all G heads of the group.
 struct QSlot {
     int valid;
     int q_tok0, q_head0, row_div, ntok, nheads, qmap, box_rows;
@@ -149,7 +149,7 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
         it.b_coord0 = it.k_row0 + sg.key0 + blk * sg.len;
         it.own_map = sg.own_map;
         // entries of this (segment, kv head), heaviest first: the packed tail tiles (last tile position of
-        // the segment, tail_heads q heads each), then (tile position, q head) for the full positions
+        // the segment), then (tile position, q head) for the full positions
 #pragma unroll 1
         for (int x = 0; x < 2; ++x) {
             const int e = 2 * pi + x;
@@ -158,16 +158,18 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
             const bool tail = e < sg.tail_tiles;
             const int e2 = e - sg.tail_tiles, up = quotient(max(e2, 0), p.div_g);
             const int qt = tail ? sg.full_tiles : sg.full_tiles - 1 - up;
-            const int head = tail ? e * sg.tail_heads : e2 - up * p.G;
+            const int n = tail ? e : e2 - up * p.G;  // of the tiles at this position
+            const QTile& form = sg.form[tail];
+            const int head = n * form.head_step, tok = qt * kTile + n * form.tok_step;
             s.q_head0 = g * p.G + head;
-            s.row_div = tail ? sg.tail_heads : 1;
-            s.ntok = tail ? sg.tail_rows : min(kTile, sg.len - qt * kTile);
-            s.nheads = tail ? min(sg.tail_heads, p.G - head) : 1;
+            s.row_div = form.heads;
+            s.ntok = min(form.toks, sg.len - tok);
+            s.nheads = min(form.heads, p.G - head);
             s.qmap = tail ? 1 + kind : 0;
-            s.box_rows = tail ? sg.tail_heads * sg.tail_rows : kTile;
-            s.q_tok0 = it.seq * p.q_rows + sg.q0 + blk * sg.len + qt * kTile;
-            s.limit0 = qt * kTile;
-            s.end = min(qt * kTile + kTile, sg.len);
+            s.box_rows = form.box_rows;
+            s.q_tok0 = it.seq * p.q_rows + sg.q0 + blk * sg.len + tok;
+            s.limit0 = tok;
+            s.end = tok + s.ntok;
             if (s.valid) own_keys = max(own_keys, s.end);
         }
     } else {

@@ -76,6 +76,12 @@ inline cudaError_t launch_chained(dim3 grid, unsigned threads, size_t smem, cuda
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// How the query tiles of one position of a segment follow one another: `toks` tokens of `heads` q heads of one kv group
+// each (a full position: 128 of one), the next tile head_step heads or tok_step tokens on.
+struct QTile {
+    int32_t heads, toks, head_step, tok_step, box_rows;
+};
+
 // One kind of prefill segment (full context blocks, a shorter last block, the sink) and its work items.
 struct Segment {
     int32_t items;       // work items, padded: (per_chunk =) blocks * Hkv * pair_chunk, times chunks
@@ -86,9 +92,8 @@ struct Segment {
     int32_t own_map;     // which K / V map its own keys are in: 0 blocks, 1 sink
     int32_t full_tiles;  // query tile positions without the packed tail
     int32_t entries;     // query tiles of one (segment, kv head): tail_tiles + G * full_tiles
-    // ragged last query tile (len % 128 rows): the tails of tail_heads q heads of one kv group are packed into one
-    // 128-row tile, tail_tiles such tiles per (segment, kv head); 0 = no packing
-    int32_t tail_rows, tail_heads, tail_tiles;
+    int32_t tail_tiles;  // tiles of a ragged last position (len % 128 rows) whose rows are packed; 0 = no packing
+    QTile form[2];       // of a full position, of a packed tail
     int32_t pair_chunk;  // pairs of one (segment, kv head) handed out together (see decode_item)
     int32_t per_chunk;
     Divisor div_per_chunk, div_pair_chunk;
