@@ -164,7 +164,8 @@ int pevlm_assemble_kv(const pevlm_shape_t* shape, const void* k_video, const voi
  * range; partials are merged by their log-sum-exp.
  *   q_question [Q, Hq, d] roped; k_cache, v_cache [L, Hkv, d]
  *   o [Q, Hq, d] bf16, lse [Hq, Q] fp32 (may be NULL)
- * workspace: >= pevlm_workspace_bytes(shape, PEVLM_WS_QUERY) bytes, 256-byte aligned.
+ * workspace: >= pevlm_workspace_bytes(shape, PEVLM_WS_QUERY) bytes, 256-byte aligned; those of a shape are enough for shorter
+ * questions and caches too.
  */
 int pevlm_query_attn(const pevlm_shape_t* shape, const void* q_question, const void* k_cache,
                      const void* v_cache, void* o, float* lse, void* workspace,
@@ -201,7 +202,7 @@ int pevlm_query_attn_noalloc(const pevlm_shape_t* shape, const void* q_question,
  * The whole pass of one layer over one sequence [Sec. 3.2; Eq. 3-5], from un-roped q [L, Hq, d], k, v [L, Hkv, d]: RoPE at
  * global positions with K and V written to the caches, the prefill attention of the video rows (or full causal) and the
  * question attention.  The same results as pevlm_rope_qk, pevlm_assemble_kv, pevlm_parallel_prefill_attn and
- * pevlm_query_attn in that order (the question's key splits differ, so its sums may differ in their last bits), in three
+ * pevlm_query_attn in that order (the question's key splits differ, so its sums may differ in their last bits), in two or three
  * launches: the work items of both attention steps share one, so that neither leaves SMs idle.
  *   q_video [S+N*B, Hq, d], q_question [Q, Hq, d]: roped copies (scratch); k_cache, v_cache [L, Hkv, d], o_*, lse_*: written.
  *   last_len > 0: the last of the num_blocks blocks has only that many tokens (<= block_len), L and S+N*B accordingly.

@@ -268,16 +268,23 @@ size_t pevlm_workspace_bytes(const pevlm_shape_t* s, int which) {
     if (check_shape(s) != PEVLM_OK) return 0;
     if (which == PEVLM_WS_PREFILL) return kStatusBytes;
     if (which == PEVLM_WS_QUERY) {
-        // pevlm_query_attn, and pevlm_layer_forward with a last block of any length: the most splits that plan_query
-        // can choose for no more key tiles than these
-        QueryPlan q = plan_query(s);
-        const size_t alone = query_bytes(s, q);
-        const int groups = s->num_kv_heads * (q.q_tiles > 1 ? (q.q_tiles + 1) / 2 : 1);
-        const int by_length = (q.total_kv_tiles + 63) / 64, by_pairs = (kNumSms / 2 + groups - 1) / groups;
-        q.n_splits = by_length > by_pairs ? by_length : by_pairs;
-        if (q.n_splits > q.total_kv_tiles) q.n_splits = q.total_kv_tiles;
-        const size_t beside = query_bytes(s, q);
-        return alone > beside ? alone : beside;
+        // The most partial rows that plan_query can ask for: pevlm_layer_forward with a last block of any length,
+        // pevlm_query_attn with this question and cache or shorter ones (a window that is still filling; neither the
+        // splits nor splits times rows grow steadily with the lengths).
+        const QueryPlan q = plan_query(s);
+        const int G = s->num_q_heads / s->num_kv_heads, Q = s->query_len, T = q.total_kv_tiles;
+        auto at_most = [](int64_t a, int64_t b) { return a < b ? a : b; };
+        auto at_least = [](int64_t a, int64_t b) { return a > b ? a : b; };
+        int64_t rows = at_most((T + 63) / 64, T) * Q;
+        for (int pairs = 1; pairs == 1 || pairs <= (q.q_tiles + 1) / 2; ++pairs) {
+            const int groups = s->num_kv_heads * pairs;
+            rows = at_least(rows, at_most((kNumSms / 2 + groups - 1) / groups, T) * at_most(Q, 2ll * q.tok_per_tile * pairs));
+        }
+        const int64_t pieces = (n_video(s) + Q + 15) / 16;
+        const int64_t decode_splits = at_least(1, at_most(kNumSms / (static_cast<int64_t>(s->num_kv_heads) * s->batch), (pieces + 7) / 8));
+        rows = at_least(rows, decode_splits * at_most(Q, kDecodeRows / G));
+        const size_t seq = static_cast<size_t>(rows) * s->num_q_heads * (s->head_dim + 1) * sizeof(float);
+        return kStatusBytes + static_cast<size_t>(s->batch) * ((seq + 255) / 256 * 256);
     }
     return 0;
 }
