@@ -8,12 +8,9 @@
 // vector, 16 bytes of either half each; the vectors of a group are one contiguous range per tensor.  What bounds it: DRAM
 // traffic.  Two things used to stand in the way (numbers for B200, 28/4 heads of 128):
 //   - the fp64 <-> fp32 conversion unit (16 values per clock and SM, 70 % busy at 50K tokens).  The rotation therefore
-//     runs in fp32, with the sine and cosine rounded to fp32, and takes its result only where it cannot differ: with
-//     |cos|, |sin| <= 1 and fp32 rounding (2^-24 relative, half an ulp) of the cosine, the sine, the product b s and the
-//     sum, the error of a c - b s is below 3 * 2^-25 (|a| + |b|) * 1.01 < E = 2^-23 (|a| + |b|), and the rounding to
-//     fp32 and to bf16 is monotone, so if r - E and r + E round to the same bf16, the fp64 value does too.  The remaining
-//     quarter of E covers the rounding of r -+ E itself.  Where they differ (about one head vector of a warp in
-//     sixteen) the thread repeats its eight pairs in fp64;
+//     runs in fp32, with the sine and cosine rounded to fp32, and takes its result r only where it cannot differ: where
+//     r - E and r + E, E = 2^-23 (|a| + |b|), round to the same bf16 (see rotate2 for why that is enough).  Elsewhere
+//     (about one head vector of a warp in sixteen) the thread repeats its eight pairs in fp64;
 //   - the bytes in flight, above all in ranges that do not fill the GPU many times over (12.5K tokens took 73 us where
 //     50K took 148).  The loads go through a ring in shared memory, kRopeRing vectors ahead, over the ends of groups
 //     too, which costs no registers.  A thread reads only what it has fetched itself, so the ring needs no barrier.
@@ -45,14 +42,32 @@ __device__ __forceinline__ double bf16_bits_to_f64(uint32_t bits16) {
 }
 
 // Two rotation pairs (a0, b0), (a1, b1), packed as bf16 words: outputs of both halves, and whether any of the four could
-// round differently from the exact value.  cs = (cos0, cos1, sin0, sin1).
-__device__ __forceinline__ uint32_t rotate2(uint32_t a, uint32_t b, const float4& cs, uint32_t& out_a, uint32_t& out_b) {
+// round differently from the exact value.  cs = (cos0, cos1, sin0, sin1).  least: the smallest |a| + |b| - 1 as bits, so
+// that zero counts as the largest.
+//
+// Why r = fl(a C - fl(b S)) may be taken where lo = fl(r - E) and hi = fl(r + E) round to the same bf16.  Let x be the
+// fp64 result and t = fl(x), M = |a| + |b| in [2^k, 2^(k+1)), u = 2^(k-23) (fp32's spacing there); E >= u, as fl(M) >= 2^k.
+// Rounding is monotone, so lo <= t <= hi is enough.  |x - r| is at most 2^-25 M (C and S, of magnitude <= 1) + half a
+// spacing at b S + half a spacing at r, and fp64's own 2^-51 M.
+//   - r >= 2^k (magnitudes), M >= 1.34 * 2^k: at most 2^-25 M + u <= 3.99 * 2^-25 M < E (fl(M) is off by 2^-24 M).
+//   - r >= 2^k, M < 1.34 * 2^k: at most 1.34 u, so t is less than 2 u off.  Both lie on the grid of u: t is r or its
+//     neighbour, and lo and hi reach the neighbours.  (t below 2^k: then everything is within 4 u of 2^k, which is
+//     itself a bf16, and rounds to it.)  This is the one case where |x - r| does exceed E, by up to a third.
+//   - r < 2^k: half a spacing at r is u / 4, in all at most 2^-25 M + 3/4 u <= 3.98 * 2^-25 M < E from M = 1.01 * 2^k on, and
+//     below that at most 1.003 u with t and r on the grid of u / 2 (or finer, with smaller terms): t is at most u off, as above.
+// The second output is the same with a and b exchanged.  M >= 2^-126 is needed: below, the spacing stays 2^-149, E is less than
+// that and t may be r's neighbour unnoticed (5 of 10^7 outputs differed).  Such pairs, both subnormal and not both zero, count
+// as unsure; M = 0 gives an exact zero (with the sign checked by lo and hi).  (The check is
+// nine instructions: 12.6K tokens 267.7 -> 268.8 us a layer, 50K tokens 1,741 -> 1,744.)
+__device__ __forceinline__ uint32_t rotate2(uint32_t a, uint32_t b, const float4& cs, uint32_t& out_a, uint32_t& out_b, uint32_t& least) {
     const float a0 = __uint_as_float(a << 16), a1 = __uint_as_float(a & 0xffff0000u);
     const float b0 = __uint_as_float(b << 16), b1 = __uint_as_float(b & 0xffff0000u);
     const uint64_t A = pack_f32x2(a0, a1), B = pack_f32x2(b0, b1);
     const uint64_t C = pack_f32x2(cs.x, cs.y), S = pack_f32x2(cs.z, cs.w), nS = pack_f32x2(-cs.z, -cs.w);
     const uint64_t ra = fma_f32x2(A, C, mul_f32x2(B, nS)), rb = fma_f32x2(B, C, mul_f32x2(A, S));
-    const uint64_t m = pack_f32x2(fabsf(a0) + fabsf(b0), fabsf(a1) + fabsf(b1));
+    const float m0 = fabsf(a0) + fabsf(b0), m1 = fabsf(a1) + fabsf(b1);
+    least = __viaddmin_u32(__float_as_uint(m0), ~0u, __viaddmin_u32(__float_as_uint(m1), ~0u, least));
+    const uint64_t m = pack_f32x2(m0, m1);
     const float e = 1.0f / 8388608.0f;  // 2^-23
     const uint64_t up = pack_f32x2(e, e), down = pack_f32x2(-e, -e);
     float x0, x1, y0, y1;
@@ -167,11 +182,11 @@ __global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(cons
                     if (is_q) dst = (tok0 + t < p.split_token ? p.q_out : p.q_out2) + (tok0 * p.Hq + u) * D;
                     else dst = p.k_out + (tok0 * p.Hkv + (u - nq)) * D;
                     const uint32_t lw[4] = {lo.x, lo.y, lo.z, lo.w}, hw[4] = {hi.x, hi.y, hi.z, hi.w};
-                    uint32_t ol[4], oh[4], unsure = 0;
+                    uint32_t ol[4], oh[4], unsure = 0, least = ~0u;
 #pragma unroll
                     for (int w = 0; w < 4; ++w)
-                        unsure |= rotate2(lw[w], hw[w], sm.cs32[buf][t * (HALF / 2) + w * TPV + v], ol[w], oh[w]);
-                    if (__builtin_expect(unsure != 0, 0)) {
+                        unsure |= rotate2(lw[w], hw[w], sm.cs32[buf][t * (HALF / 2) + w * TPV + v], ol[w], oh[w], least);
+                    if (__builtin_expect(unsure != 0 || least < 0x007fffffu, 0)) {
 #pragma unroll
                         for (int w = 0; w < 4; ++w) {
                             float ra[2], rb[2];
