@@ -9,11 +9,14 @@ namespace pevlm {
 constexpr int kCopyThreads = 256;
 constexpr int kCopyUnroll = 4;
 
+// Read from L2, not through the non-coherent path: this kernel may be on the GPU while the one that writes its sources still
+// runs (launch_chained), and what an SM's L1 holds of a buffer may be from an earlier copy out of it.
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p));
+                 : "l"(p)
+                 : "memory");
     return v;
 }
 __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
