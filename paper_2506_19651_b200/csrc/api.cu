@@ -78,20 +78,21 @@ static EncodeTiledFn encode_fn() {
 }
 
 // Tensor map over a [tokens, heads, d] bf16 tensor (d contiguous) with a box of box_elems (64 or 32) elements x
-// box_heads x box_tokens and the swizzle of the box's row (128 or 64 bytes) that the MMA descriptors expect.
-// Rows past the end of the tensor read as zero.
+// box_heads x box_tokens and the swizzle of the box's row (128 or 64 bytes) that the MMA descriptors expect; with
+// batch > 0 over that many such tensors, seq_tokens rows apart, as a fourth dimension.  Rows past the end of the tensor read as zero.
 static int make_tmap(CUtensorMap* m, const void* base, int64_t tokens, int heads, int d, int box_heads, int box_tokens,
-                     int box_elems = 64) {
+                     int box_elems = 64, int batch = 0, int64_t seq_tokens = 0) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) {
         snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled entry point not found");
         return PEVLM_ECUDA;
     }
-    cuuint64_t dims[3] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(heads), static_cast<cuuint64_t>(tokens)};
-    cuuint64_t strides[2] = {static_cast<cuuint64_t>(d) * 2, static_cast<cuuint64_t>(d) * 2 * heads};
-    cuuint32_t box[3] = {static_cast<cuuint32_t>(box_elems), static_cast<cuuint32_t>(box_heads), static_cast<cuuint32_t>(box_tokens)};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+    const cuuint64_t row = static_cast<cuuint64_t>(d) * 2 * heads;
+    cuuint64_t dims[4] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(heads), static_cast<cuuint64_t>(tokens), static_cast<cuuint64_t>(batch)};
+    cuuint64_t strides[3] = {static_cast<cuuint64_t>(d) * 2, row, row * static_cast<cuuint64_t>(batch > 1 ? seq_tokens : 1)};
+    cuuint32_t box[4] = {static_cast<cuuint32_t>(box_elems), static_cast<cuuint32_t>(box_heads), static_cast<cuuint32_t>(box_tokens), 1};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, batch > 0 ? 4 : 3, const_cast<void*>(base), dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE,
                      box_elems == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -486,32 +487,30 @@ static void add_question(AttnParams& p, const QueryPlan& qp) {
     p.div_q_pairs = make_divisor((p.q_tiles + 1) / 2);
 }
 
-// Tensor maps over the rows of p.batch sequences.  Between two sequences of a batch a ragged last key tile brings in rows
-// of the next range instead of zeros; they are masked, and finite like every input.  (Block ranges, whose cache may hold
-// anything elsewhere, are launched one sequence at a time.)
+// K and V of one range of each of p.batch sequences: `rows` rows from the base on, the sequences seq_rows apart.  (A map needs at
+// least one row; an empty range is never read.)
+static int kv_maps(AttnMaps& m, int i, const AttnParams& p, int d, const __nv_bfloat16* k, const __nv_bfloat16* v, int64_t rows, int64_t seq_rows) {
+    const int64_t n = rows > 0 ? rows : 1;
+    const int rc = make_tmap(&m.k[i], k, n, p.Hkv, d, 1, kTile / 2, 64, p.batch, seq_rows);
+    return rc != PEVLM_OK ? rc : make_tmap(&m.v[i], v, n, p.Hkv, d, 1, kTile, d / 2, p.batch, seq_rows);
+}
+
 static int prefill_maps(AttnMaps& m, const AttnParams& p, int d, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v) {
     int rc;
-    const int64_t q_rows = static_cast<int64_t>(p.batch) * p.q_rows, before = static_cast<int64_t>(p.batch - 1) * p.kv_rows;
+    const int64_t q_rows = static_cast<int64_t>(p.batch) * p.q_rows;
     if ((rc = make_tmap(&m.q[0], q, q_rows, p.Hq, d, 1, kTile)) != PEVLM_OK) return rc;
     for (int i = 0; i < 3; ++i) {
         const Segment& g = p.seg[i];
         if (g.items > 0 && g.tail_tiles > 0 && (rc = make_tmap(&m.q[1 + i], q, q_rows, p.Hq, d, g.form[1].heads, g.form[1].toks)) != PEVLM_OK) return rc;
     }
-    // (a map needs at least one row; an empty range is never read)
     const int64_t blk_off = static_cast<int64_t>(p.blk_key0) * p.Hkv * d;
-    const int64_t sink_rows = before + (p.sink_len > 0 ? p.sink_len : 1), blk_rows = before + (p.block_rows > 0 ? p.block_rows : 1);
-    if ((rc = make_tmap(&m.k[0], k + blk_off, blk_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-    if ((rc = make_tmap(&m.v[0], v + blk_off, blk_rows, p.Hkv, d, 1, kTile, d / 2)) != PEVLM_OK) return rc;
-    if ((rc = make_tmap(&m.k[1], k, sink_rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-    return make_tmap(&m.v[1], v, sink_rows, p.Hkv, d, 1, kTile, d / 2);
+    if ((rc = kv_maps(m, 0, p, d, k + blk_off, v + blk_off, p.block_rows, p.kv_rows)) != PEVLM_OK) return rc;
+    return kv_maps(m, 1, p, d, k, v, p.sink_len, p.kv_rows);
 }
 
 static int question_maps(AttnMaps& m, const AttnParams& p, int d, const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v) {
-    int rc;
-    const int64_t rows = static_cast<int64_t>(p.batch) * p.L;
-    if ((rc = make_tmap(&m.q[4], q, static_cast<int64_t>(p.batch) * p.Q, p.Hq, d, p.G, p.tok_per_tile)) != PEVLM_OK) return rc;
-    if ((rc = make_tmap(&m.k[2], k, rows, p.Hkv, d, 1, kTile / 2)) != PEVLM_OK) return rc;
-    return make_tmap(&m.v[2], v, rows, p.Hkv, d, 1, kTile, d / 2);
+    const int rc = make_tmap(&m.q[4], q, static_cast<int64_t>(p.batch) * p.Q, p.Hq, d, p.G, p.tok_per_tile);
+    return rc != PEVLM_OK ? rc : kv_maps(m, 2, p, d, k, v, p.L, p.L);
 }
 
 static int merge_question(const AttnParams& p, int d, __nv_bfloat16* o, float* lse, cudaStream_t st) {

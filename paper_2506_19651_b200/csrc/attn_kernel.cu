@@ -94,10 +94,10 @@ struct QSlot {
 // Key tiles of an item: first the na tiles of the shared range [0, a_end) (the sink), then the tiles of the own
 // range, nt tiles in all (what the longer of the two query tiles needs; the other one masks its surplus tile).
 // The own range is fetched at row b_coord0 of the block tensor map (own_map = 0), for the sink's own items of the sink map
-// (1), for question items of the map of the whole cache (2).  seq: sequence of the batch, k_row0: its first row in the
-// sink and block maps (b_coord0 includes it).  n_a, n_b: MMA columns of tile na - 1 and of the last tile; the others have 128.
+// (1), for question items of the map of the whole cache (2).  seq: sequence of the batch, a dimension of those maps of its own.
+// n_a, n_b: MMA columns of tile na - 1 and of the last tile; the others have 128.
 struct WorkItem {
-    int kv_head, a_end, na, nt, n_a, n_b, split, b_coord0, own_map, seq, k_row0;
+    int kv_head, a_end, na, nt, n_a, n_b, split, b_coord0, own_map, seq;
     QSlot s[2];
 };
 
@@ -127,7 +127,6 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
     }
     const bool question = MODE == 2 || (MODE == 3 && w < p.items_question);
     if (MODE == 3) w -= question ? 0 : p.items_question;
-    it.k_row0 = it.seq * p.kv_rows;
     int own_keys = 0;  // keys of the own range that the longer query tile sees
     if (!question) {
         // Which kind of segment: the full blocks, a shorter last block, the sink.
@@ -146,7 +145,7 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
         const int blk = quotient(combo, p.div_hkv), g = combo - blk * p.Hkv;
         it.kv_head = g;
         it.a_end = sg.a_end;
-        it.b_coord0 = it.k_row0 + sg.key0 + blk * sg.len;
+        it.b_coord0 = sg.key0 + blk * sg.len;
         it.own_map = sg.own_map;
         // entries of this (segment, kv head), heaviest first: the packed tail tiles (last tile position of
         // the segment), then (tile position, q head) for the full positions
@@ -181,7 +180,7 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
         it.kv_head = g;
         it.a_end = 0;
         const int split_lo = it.split * p.tiles_per_split * kTile;
-        it.b_coord0 = it.seq * p.L + split_lo;
+        it.b_coord0 = split_lo;
         it.own_map = 2;
 #pragma unroll 1
         for (int x = 0; x < 2; ++x) {
@@ -394,9 +393,9 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
             // (The whole warp runs this with uniform values; single lanes issue.)
             {
                 // The K cursor's item, and where V has to come from: the rows of the last kQkAhead K tiles (base row of the
-                // tile, kv head and map), the V tile of a step being that of kQkAhead steps ago.
-                int k = -1, j = 0, nt = 0, na = 0, n_a = 0, n_b = 0, kv_head = 0, b_coord0 = 0, own_map = 0, k_row0 = 0;
-                int v_row[kQkAhead], v_from[kQkAhead];
+                // tile, kv head and map, sequence), the V tile of a step being that of kQkAhead steps ago.
+                int k = -1, j = 0, nt = 0, na = 0, n_a = 0, n_b = 0, kv_head = 0, b_coord0 = 0, own_map = 0, seq = 0;
+                int v_row[kQkAhead], v_from[kQkAhead], v_seq[kQkAhead];
                 uint32_t tiles = 0;  // K tiles loaded so far
                 bool more = true;
 #pragma unroll 1
@@ -409,7 +408,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                             j = 0;
                             nt = uniform(it.nt); na = uniform(it.na); n_a = uniform(it.n_a); n_b = uniform(it.n_b);
                             kv_head = uniform(it.kv_head); b_coord0 = uniform(it.b_coord0); own_map = uniform(it.own_map);
-                            k_row0 = uniform(it.k_row0);
+                            seq = uniform(it.seq);
                             const int qm = uniform(q.qmap), q_head0 = uniform(q.q_head0), q_tok0 = uniform(q.q_tok0);
                             const int valid = uniform(q.valid);
                             const int rows = uniform((it.s[0].valid ? it.s[0].box_rows : 0) + (it.s[1].valid ? it.s[1].box_rows : 0));
@@ -428,14 +427,15 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                             }
                         }
                     }
-                    // Rows past the end of the sink, and past the end of the block range, are outside their
-                    // tensor map and arrive as zeros: a ragged last tile never brings in a neighbour's rows.
+                    // Rows past the end of the sink, and past the end of the block range, are outside their tensor map, in
+                    // every sequence of a batch, and arrive as zeros: a ragged last tile brings in no rows of the range or
+                    // the sequence behind it, whatever those hold (a probability of 0 times a NaN in V would be one).
                     int row = 0, from = 0;
                     if (more) {
                         if (rank == 0 && lane == 0 && j == max(0, nt - kClaimAhead)) mbar_arrive(smem_u32(&bars.go));
                         const int map = MODE == 2 ? 2 : j < na ? 1 : own_map;
                         const int n = j == na - 1 ? n_a : j == nt - 1 ? n_b : kTile;  // this CTA's keys: half of them
-                        row = j < na ? k_row0 + j * kTile : b_coord0 + (j - na) * kTile;
+                        row = j < na ? j * kTile : b_coord0 + (j - na) * kTile;
                         from = kv_head * 4 + map;
                         const uint32_t slot = tiles % kRing;
                         if (tiles >= kRing) wait_s_full(tiles - kRing, kWaitKvFree);
@@ -443,8 +443,8 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                         const uint32_t bar = map_to_cta(smem_u32(&bars.k_full[slot]), 0);
 #pragma unroll 1
                         for (int h = 0; h < NP; ++h)
-                            tma_load_3d_pair(smem_base + L::kK + slot * L::kKBytes + h * L::kKPanelBytes, &maps.k[map], h * 64, kv_head,
-                                             row + static_cast<int>(rank) * (n >> 1), bar);
+                            tma_load_4d_pair(smem_base + L::kK + slot * L::kKBytes + h * L::kKPanelBytes, &maps.k[map], h * 64, kv_head,
+                                             row + static_cast<int>(rank) * (n >> 1), seq, bar);
                         ++j;
                         ++tiles;
                     }
@@ -452,16 +452,18 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                         const uint32_t u = s - kQkAhead, slot = u % kRing;
                         if (u >= kRing) wait_pv_done(u - kRing, kWaitKvFree);
                         if (rank == 0 && lane == 0) mbar_arrive_expect_tx(smem_u32(&bars.v_full[slot]), 2 * L::kVBytes);
-                        tma_load_3d_pair(smem_base + L::kV + slot * L::kVBytes, &maps.v[v_from[0] & 3], static_cast<int>(rank) * (D / 2),
-                                         v_from[0] >> 2, v_row[0], map_to_cta(smem_u32(&bars.v_full[slot]), 0));
+                        tma_load_4d_pair(smem_base + L::kV + slot * L::kVBytes, &maps.v[v_from[0] & 3], static_cast<int>(rank) * (D / 2),
+                                         v_from[0] >> 2, v_row[0], v_seq[0], map_to_cta(smem_u32(&bars.v_full[slot]), 0));
                     }
 #pragma unroll
                     for (int i = 0; i < kQkAhead - 1; ++i) {
                         v_row[i] = v_row[i + 1];
                         v_from[i] = v_from[i + 1];
+                        v_seq[i] = v_seq[i + 1];
                     }
                     v_row[kQkAhead - 1] = row;
                     v_from[kQkAhead - 1] = from;
+                    v_seq[kQkAhead - 1] = seq;
                 }
             }
         } else if (rank == 0 && warp == 12) {

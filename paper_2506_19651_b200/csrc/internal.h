@@ -110,7 +110,7 @@ struct AttnParams {
     int32_t block_rows;     // rows of all blocks
     int32_t blk_key0;       // and K/V row of the first block (S, or the cache row of a block range)
     int32_t q_rows;         // prefill: rows of q / o (and columns of lse) of a sequence
-    int32_t kv_rows;        // prefill: rows of k / v of a sequence
+    int32_t kv_rows;        // prefill (host only): rows of k / v of a sequence
     int32_t Q, L;           // question length, total length
     int32_t Hq, Hkv, G;
     int32_t items_question; // question work items
@@ -201,7 +201,8 @@ cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream);
 //   q[0]: [rows, Hq, d] with a 128-token box; q[1 + kind]: the same tensor with the box of the segment kind's packed ragged
 //   tail (heads x tail rows); q[4]: the question rows (box: one kv group's heads x the tokens of a tile)
 //   k, v[0]: the context blocks of the call (base at the first block's row); [1]: the sink, rows [0, S), so that a ragged
-//   last key tile of either range reads zeros past its end instead of a neighbour's rows; [2]: the whole cache
+//   last key tile of either range reads zeros past its end instead of a neighbour's rows; [2]: the whole cache.  The
+//   sequences of a batch are the maps' last dimension, so that the end of the range is the end of the map in each of them
 struct AttnMaps {
     CUtensorMap q[5], k[3], v[3];
 };
