@@ -48,6 +48,7 @@ constexpr int kRing = 4;      // K tiles and V tiles in flight
 constexpr int kQkAhead = 3;   // tiles by which QK runs ahead of PV
 constexpr int kItems = 8;     // decoded work items in flight
 constexpr int kSums = 8;      // items whose row sums may be in flight between softmax and epilogue
+constexpr unsigned kNoMore = 1u << 31;
 constexpr int kClaimAhead = 6;  // tiles before the end of an item's loads at which the next item is claimed
 // pair of exponentials (of 64) after which a softmax warp passes the turn on: the rest overlaps the other warp's start
 // (measured: 16 to 40 within 1 % of each other, 52 and later 4 % slower)
@@ -213,8 +214,9 @@ __device__ __forceinline__ void decode_item(const AttnParams& p, int w, WorkItem
 
 // Between the two softmax warps that share a scheduler (warp `quarter` of each warpgroup), hardware barriers of 64
 // threads, one id per direction, all sixteen in use (the kernel has no __syncthreads: the cluster barrier stands at its
-// start and end).  Both warps go through the same tiles whatever happens, so every pass meets its wait; what the passing
-// warp wrote to shared memory before is seen after the wait.  kPassMax: the row maxima of a tile; kPassTurn: the turn on
+// start and end).  These have no limit: both warps go through the same tiles whatever happens, a timeout included, because
+// they see the same work items (item_ready), so every pass meets its wait.  What the passing warp wrote to shared memory
+// before is seen after the wait.  kPassMax: the row maxima of a tile; kPassTurn: the turn on
 // the scheduler's special-function unit.
 constexpr int kPassMax = 0, kPassTurn = 8;
 __device__ __forceinline__ void pass_wait(int what, int wg, int quarter) {
@@ -251,7 +253,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     __shared__ __align__(16) uint4 s_clc;
     __shared__ uint32_t tmem_base_slot;
     __shared__ WaitState wait_state;
-    __shared__ int s_item[kItems];       // 1 = a work item, -1 = no more work
+    __shared__ unsigned s_published;     // work items so far; kNoMore added: there will be no others
     __shared__ WorkItem s_decoded[kItems];
     __shared__ float s_max[2][kTile];
     __shared__ float2 s_sums[kSums][2][kTile];  // (row sum, reference maximum) of the even and of the odd tiles:
@@ -267,6 +269,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     if (tid == 0) {
         wait_state.tries = p.wait_tries;
         wait_state.expired = 0;
+        s_published = 0;
         for (int i = 0; i < kItems; ++i) {
             mbar_init(smem_u32(&bars.item_full[i]), 1);
             mbar_init(smem_u32(&bars.item_free[i]), kConsumerWarps + (rank == 0 ? 2 : 0));
@@ -334,10 +337,14 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     auto wait_asleep = [&](const uint64_t& bar, uint32_t parity, int which) {
         PEVLM_WAIT_ACCOUNT(which, mbar_wait<100>(smem_u32(&bar), parity, wait_state, which));
     };
-    // k-th item of the pair: wait for it, read from s_decoded[k % kItems], then give the slot back (once per warp)
+    // k-th item of the pair: wait for it, read from s_decoded[k % kItems], then give the slot back (once per warp).
+    // Whether there is a k-th item has the same answer in every warp, a timeout included: it is decided in one word, where
+    // the scheduler counts item k in before it lets anyone have it and a wait that runs out says that there are no more,
+    // whichever comes first.  (Warps that disagreed would wait for one another in pass_wait, without a limit.)
     auto item_ready = [&](int k) {
         wait(bars.item_full[k % kItems], (k / kItems) & 1, kWaitItem);
-        return s_item[k % kItems] > 0;
+        if (static_cast<int>(*static_cast<volatile unsigned*>(&s_published) & ~kNoMore) > k) return true;
+        return static_cast<int>(atomicOr(&s_published, kNoMore) & ~kNoMore) > k;
     };
     auto item_release = [&](int k) { mbar_arrive(smem_u32(&bars.item_free[k % kItems])); };
     auto wait_s_full = [&](uint32_t t, int which) { wait(bars.s_full[t % kRing], (t / kRing) & 1, which); };
@@ -359,15 +366,20 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                 }
                 while (true) {
                     const int slot = published % kItems;
-                    if (published >= kItems) wait_asleep(bars.item_free[slot], (published / kItems - 1) & 1, kWaitItemFree);
+                    if (published >= kItems) {
+                        wait_asleep(bars.item_free[slot], (published / kItems - 1) & 1, kWaitItemFree);
+                        if (!mbar_try_wait(smem_u32(&bars.item_free[slot]), (published / kItems - 1) & 1)) w = -2;  // may still be read
+                    }
                     bool some = false;
                     if (w >= 0) {
                         decode_item<MODE>(p, w, s_decoded[slot]);
                         some = s_decoded[slot].nt > 0;  // padding of the item list is skipped
                     }
                     if (w < 0 || some) {
-                        s_item[slot] = w < 0 ? -1 : 1;
-                        mbar_arrive(smem_u32(&bars.item_full[slot]));  // release: the decoded item is visible
+                        __threadfence_block();
+                        if (w < 0) atomicOr(&s_published, kNoMore);
+                        else if (atomicCAS(&s_published, published, published + 1) != static_cast<unsigned>(published)) w = -1;
+                        if (w != -2) mbar_arrive(smem_u32(&bars.item_full[slot]));  // release: the decoded item is visible
                         if (w < 0) break;
                         ++published;
                         if (published == 1) grid_wait();
