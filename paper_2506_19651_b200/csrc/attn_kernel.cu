@@ -37,7 +37,8 @@
 //     little, no divisions, and warp-uniform values that the compiler knows to be uniform (the MMA warps' descriptors
 //     then live in uniform registers instead of being moved there for every MMA: 10 KB of code).
 // Every wait on an mbarrier is bounded; an expired wait records PEVLM_ETIMEOUT and the CTA still runs to its
-// normal end (waits become short), so TMEM is always released.
+// normal end (waits become short) and stays until what is in flight has landed, so TMEM is always released and nothing
+// writes to shared memory that has a new owner.
 #include "internal.h"
 #include "ptx.cuh"
 
@@ -48,6 +49,7 @@ constexpr int kRing = 4;      // K tiles and V tiles in flight
 constexpr int kQkAhead = 3;   // tiles by which QK runs ahead of PV
 constexpr int kItems = 8;     // decoded work items in flight
 constexpr int kSums = 8;      // items whose row sums may be in flight between softmax and epilogue
+constexpr int kDrainUs = 64;
 constexpr unsigned kNoMore = 1u << 31;
 constexpr int kClaimAhead = 6;  // tiles before the end of an item's loads at which the next item is claimed
 // pair of exponentials (of 64) after which a softmax warp passes the turn on: the rest overlaps the other warp's start
@@ -750,6 +752,12 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
     if (blockIdx.x < 2)
         for (int i = lane; i < kTraceIds; i += 32) g_waits[blockIdx.x][warp][i] = s_waits[warp][i];
 #endif
+    // A wait that ran out may have left loads, MMAs or an answer of the hardware queue on their way into this pair's memory.
+    // They take microseconds; the pair stays until they have had tens of them.
+    if (*static_cast<volatile int*>(&wait_state.expired) != 0) {
+#pragma unroll 1
+        for (int i = 0; i < kDrainUs; ++i) __nanosleep(1000);
+    }
     tc_fence_before_sync();
     __syncwarp();
     cluster_sync_all();  // neither CTA leaves, or frees TMEM, while the other may still reach it
