@@ -17,14 +17,20 @@ def _workspace(alloc, n_bytes):
     return ws
 
 
+def _one_sequence(shape):
+    if shape.batch != 1:
+        raise ValueError(f"a layer pass is over one sequence, not a batch of {shape.batch}: its buffers hold the rows of one")
+
+
 class LayerBuffers:
-    """Device buffers of one layer pass, allocated once and reused across steps."""
+    """Device buffers of one layer pass over one sequence, allocated once and reused across steps."""
 
     def __init__(self, shape: pb.Shape, device="cuda", alloc=None):
         """`alloc(shape, dtype, zero)` replaces torch.empty / torch.zeros (the tests pass an allocator that puts
         guard bytes around every buffer)."""
         import torch
         s = shape
+        _one_sequence(s)
         nv, Q, L = s.n_video, s.query_len, s.L
         Hq, Hkv, d = s.num_q_heads, s.num_kv_heads, s.head_dim
         bf, f32 = torch.bfloat16, torch.float32
@@ -55,12 +61,11 @@ def layer_forward(buf: LayerBuffers, q, k, v, mark=None):
     call (pevlm_layer_forward)."""
     s = buf.shape
     nv, Q = s.n_video, s.query_len
+    _one_sequence(s)
     if mark is None:
-        if s.batch == 1:
-            pb.pevlm_layer_forward(s, q, k, v, buf.q_video, buf.q_question, buf.k_cache, buf.v_cache, buf.o_video,
-                                   buf.lse_video, buf.o_question, buf.lse_question, buf.ws_prefill, buf.ws_query)
-            return buf
-        mark = lambda name: None
+        pb.pevlm_layer_forward(s, q, k, v, buf.q_video, buf.q_question, buf.k_cache, buf.v_cache, buf.o_video,
+                               buf.lse_video, buf.o_question, buf.lse_question, buf.ws_prefill, buf.ws_query)
+        return buf
     mark("start")
     if nv > 0:
         # K goes straight into its cache slot; Q is roped into a scratch copy
