@@ -160,9 +160,17 @@ class StreamingWindow:
         """Address of a cache row (what cache[row:] would point to, without building the view)."""
         return cache.data_ptr() + row * self.Hkv * self.d * 2
 
+    @staticmethod
+    def _has_rows(n, *tensors):
+        """The calls get addresses only: that there are n rows behind them is seen to here."""
+        for t in tensors:
+            if t.shape[0] < n:
+                raise ValueError(f"{t.shape[0]} rows where {n} are read")
+
     def set_sink(self, q, k, v):
         """Encode the sink (Eq. 3).  Returns (o [S,Hq,d], lse [Hq,S])."""
         S = self.S
+        self._has_rows(S, q, k, v)
         o, lse = self._outputs(S)
         pb.pevlm_rope_qkv(self.s_sink, q, k, v, self.q_buf, self.k_cache, self.v_cache, 0, S)
         pb.pevlm_parallel_prefill_attn(self.s_sink, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_sink)
@@ -171,6 +179,7 @@ class StreamingWindow:
     def append_block(self, q, k, v):
         """Encode the next block of the stream into the slot of the oldest one.  Returns (o [B,Hq,d], lse [Hq,B])."""
         S, B = self.S, self.B
+        self._has_rows(B, q, k, v)
         t = self.blocks_seen
         row0 = S + (t % self.W) * B
         o, lse = self._outputs(B)
@@ -185,6 +194,10 @@ class StreamingWindow:
         Qn = q.shape[0]
         held = min(self.blocks_seen, self.W)
         nv = self.S + held * self.B
+        self._has_rows(Qn, k, v)
+        room = min(self.rows - nv, self.q_buf.shape[0])  # more than Q_max while the window fills
+        if Qn > room:
+            raise ValueError(f"a question of {Qn} rows where {room} fit")
         s = self._shape(nv, 1, 0, Qn)
         o, lse = self._outputs(Qn)
         pb.pevlm_rope_qkv(s, q, k, v, self.q_buf, self._row(self.k_cache, nv), self._row(self.v_cache, nv),

@@ -31,3 +31,32 @@ def test_layer_pass_is_one_sequence(no_calls, mark):
     with pytest.raises(ValueError, match="one sequence"):
         layer.layer_forward(buf, t, t, t, mark=mark)
     assert not no_calls
+
+
+def test_streaming_window_takes_only_rows_that_fit(no_calls):
+    import torch
+    S, B, W, Q_max = 8, 16, 2, 4
+    win = layer.StreamingWindow(S, B, W, Q_max, 4, 2, 64, 1e4, device="cpu")
+    rows = lambda n: [torch.zeros(n, h, 64, dtype=torch.bfloat16) for h in (4, 2, 2)]
+    short = lambda n, i: [t[:-1] if j == i else t for j, t in enumerate(rows(n))]
+    for i in range(3):
+        with pytest.raises(ValueError, match="rows"):
+            win.set_sink(*short(S, i))
+        with pytest.raises(ValueError, match="rows"):
+            win.append_block(*short(B, i))
+        if i:
+            with pytest.raises(ValueError, match="rows"):
+                win.ask(*short(3, i))
+    assert not no_calls and win.blocks_seen == 0
+    win.set_sink(*rows(S))
+    win.append_block(*rows(B))
+    win.ask(*rows(B))  # one block of two: the question has the other's room too
+    win.append_block(*rows(B))
+    win.ask(*rows(Q_max))
+    no_calls.clear()
+    for n in (Q_max + 1, B + 1):  # past the end of the caches; of the roped question too
+        with pytest.raises(ValueError, match="rows"):
+            win.ask(*rows(n))
+    assert not no_calls
+    win.append_block(*rows(B + 5))  # rows past the block's are not looked at
+    assert no_calls and win.blocks_seen == 3
