@@ -10,8 +10,9 @@
 
 static PyObject* g_data_ptr; /* interned "data_ptr" */
 
+/* Both do nothing once an argument was bad: its exception is pending. */
 static void* as_pointer(PyObject* o, int* bad) {
-    if (o == Py_None) return NULL;
+    if (*bad || o == Py_None) return NULL;
     if (PyLong_Check(o)) {
         void* p = PyLong_AsVoidPtr(o);
         if (!p && PyErr_Occurred()) *bad = 1;
@@ -29,6 +30,7 @@ static void* as_pointer(PyObject* o, int* bad) {
 }
 
 static int64_t as_int(PyObject* o, int* bad) {
+    if (*bad) return 0;
     const long long v = PyLong_AsLongLong(o);
     if (v == -1 && PyErr_Occurred()) *bad = 1;
     return v;
