@@ -164,6 +164,9 @@ def pevlm_layer_forward(shape: Shape, q, k, v, q_video, q_question, k_cache, v_c
 
 
 def pevlm_rope_qk_mrope(shape: Shape, q_in, k_in, q_out, k_out, n_tokens: int, pos_ids3, sections):
+    """sections: pairs per position component; components that are not given have none."""
+    sections = tuple(sections)
+    sections += (0,) * (3 - len(sections))
     _check(_native().rope_qk_mrope(C.addressof(shape), q_in, k_in, q_out, k_out, n_tokens, pos_ids3, *sections, _stream()),
            "pevlm_rope_qk_mrope")
 

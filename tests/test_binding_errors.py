@@ -58,3 +58,17 @@ def test_an_exception_of_a_tensor_comes_through(s):
     t = Tensor()
     with pytest.raises(RuntimeError, match="storage is gone"):
         pb.pevlm_rope_qk(s, Gone(), t, t, t, 0, 4)
+
+
+def test_fewer_than_three_sections(s):
+    # those that are not given are empty, as in a C array; the alignment of q_in is looked at before their sum
+    t = Tensor()
+    for sections, code in (((32,), pb.PEVLM_EALIGN), ([8, 24], pb.PEVLM_EALIGN), ((), pb.PEVLM_EALIGN)):
+        with pytest.raises(pb.PevlmError) as e:
+            pb.pevlm_rope_qk_mrope(s, Tensor(4098), t, t, t, 4, t, sections)
+        assert e.value.code == code
+    with pytest.raises(pb.PevlmError) as e:
+        pb.pevlm_rope_qk_mrope(s, t, t, t, t, 4, t, (8, 23))
+    assert e.value.code == pb.PEVLM_EINVAL
+    with pytest.raises((TypeError, IndexError)):
+        pb.pevlm_rope_qk_mrope(s, t, t, t, t, 4, t, (8, 12, 12, 0))
