@@ -136,6 +136,12 @@ def _stream():
     return _raw_stream()
 
 
+def _address(shape):
+    if not isinstance(shape, Shape):
+        raise C.ArgumentError(f"expected a Shape, got {type(shape).__name__}")
+    return C.addressof(shape)
+
+
 def _check(rc, where):
     if rc != PEVLM_OK:
         raise PevlmError(rc, where)
@@ -148,17 +154,17 @@ def pevlm_workspace_bytes(shape: Shape, which: int) -> int:
 # A tensor argument may also be None where the C call takes NULL, or a device address.
 
 def pevlm_rope_qk(shape: Shape, q_in, k_in, q_out, k_out, first_token: int, n_tokens: int, pos_ids=None):
-    _check(_native().rope_qk(C.addressof(shape), q_in, k_in, q_out, k_out, first_token, n_tokens, pos_ids, _stream()), "pevlm_rope_qk")
+    _check(_native().rope_qk(_address(shape), q_in, k_in, q_out, k_out, first_token, n_tokens, pos_ids, _stream()), "pevlm_rope_qk")
 
 
 def pevlm_rope_qkv(shape: Shape, q_in, k_in, v_in, q_out, k_out, v_out, first_token: int, n_tokens: int, pos_ids=None):
-    _check(_native().rope_qkv(C.addressof(shape), q_in, k_in, v_in, q_out, k_out, v_out, first_token, n_tokens, pos_ids, _stream()),
+    _check(_native().rope_qkv(_address(shape), q_in, k_in, v_in, q_out, k_out, v_out, first_token, n_tokens, pos_ids, _stream()),
            "pevlm_rope_qkv")
 
 
 def pevlm_layer_forward(shape: Shape, q, k, v, q_video, q_question, k_cache, v_cache, o_video, lse_video, o_question,
                         lse_question, ws_prefill, ws_query, last_len: int = 0):
-    _check(_native().layer_forward(C.addressof(shape), last_len, q, k, v, q_video, q_question, k_cache, v_cache, o_video, lse_video,
+    _check(_native().layer_forward(_address(shape), last_len, q, k, v, q_video, q_question, k_cache, v_cache, o_video, lse_video,
                                    o_question, lse_question, ws_prefill, ws_prefill.nbytes, ws_query, ws_query.nbytes, _stream()),
            "pevlm_layer_forward")
 
@@ -167,34 +173,34 @@ def pevlm_rope_qk_mrope(shape: Shape, q_in, k_in, q_out, k_out, n_tokens: int, p
     """sections: pairs per position component; components that are not given have none."""
     sections = tuple(sections)
     sections += (0,) * (3 - len(sections))
-    _check(_native().rope_qk_mrope(C.addressof(shape), q_in, k_in, q_out, k_out, n_tokens, pos_ids3, *sections, _stream()),
+    _check(_native().rope_qk_mrope(_address(shape), q_in, k_in, q_out, k_out, n_tokens, pos_ids3, *sections, _stream()),
            "pevlm_rope_qk_mrope")
 
 
 def pevlm_parallel_prefill_attn(shape: Shape, q, k, v, o, lse, workspace):
-    _check(_native().parallel_prefill_attn(C.addressof(shape), q, k, v, o, lse, workspace, workspace.nbytes, _stream()),
+    _check(_native().parallel_prefill_attn(_address(shape), q, k, v, o, lse, workspace, workspace.nbytes, _stream()),
            "pevlm_parallel_prefill_attn")
 
 
 def pevlm_block_attn(shape: Shape, q_blocks, k_cache, v_cache, first_key_row: int, cache_rows: int, o, lse, workspace):
-    _check(_native().block_attn(C.addressof(shape), q_blocks, k_cache, v_cache, first_key_row, cache_rows, o, lse, workspace,
+    _check(_native().block_attn(_address(shape), q_blocks, k_cache, v_cache, first_key_row, cache_rows, o, lse, workspace,
                                 workspace.nbytes, _stream()), "pevlm_block_attn")
 
 
 def pevlm_assemble_kv(shape: Shape, k_video, v_video, k_question, v_question, k_cache, v_cache):
-    _check(_native().assemble_kv(C.addressof(shape), k_video, v_video, k_question, v_question, k_cache, v_cache, _stream()),
+    _check(_native().assemble_kv(_address(shape), k_video, v_video, k_question, v_question, k_cache, v_cache, _stream()),
            "pevlm_assemble_kv")
 
 
 def pevlm_query_attn(shape: Shape, q_question, k_cache, v_cache, o, lse, workspace):
-    _check(_native().query_attn(C.addressof(shape), q_question, k_cache, v_cache, o, lse, workspace, workspace.nbytes, _stream()),
+    _check(_native().query_attn(_address(shape), q_question, k_cache, v_cache, o, lse, workspace, workspace.nbytes, _stream()),
            "pevlm_query_attn")
 
 
 def pevlm_query_attn_noalloc(shape: Shape, q_question, k_cache, v_cache, o, lse):
     """Question attention for callers that cannot allocate device memory: no workspace argument,
     the partials go to the library's built-in scratch array (see include/pevlm.h for its limits)."""
-    _check(_native().query_attn_noalloc(C.addressof(shape), q_question, k_cache, v_cache, o, lse, _stream()), "pevlm_query_attn_noalloc")
+    _check(_native().query_attn_noalloc(_address(shape), q_question, k_cache, v_cache, o, lse, _stream()), "pevlm_query_attn_noalloc")
 
 
 def pevlm_selftest_wait_expiry(workspace, limit_ns: int):

@@ -72,3 +72,18 @@ def test_fewer_than_three_sections(s):
     assert e.value.code == pb.PEVLM_EINVAL
     with pytest.raises((TypeError, IndexError)):
         pb.pevlm_rope_qk_mrope(s, t, t, t, t, 4, t, (8, 12, 12, 0))
+
+
+def test_a_shape_is_a_shape(s):
+    class Other(C.Structure):
+        _fields_ = [("batch", C.c_int32)]
+
+    class Mine(pb.Shape):
+        pass
+    for f, args in calls(s):
+        for bad in (Other(1), C.c_int32(1), C.pointer(s), None, 4096):  # what ctypes refuses for a pevlm_shape_t*
+            with pytest.raises((C.ArgumentError, TypeError)):
+                f(bad, *args)
+        with pytest.raises(pb.PevlmError) as e:
+            f(Mine(*(getattr(s, n) for n, _ in pb.Shape._fields_)), *args)
+        assert e.value.code == pb.PEVLM_EALIGN
