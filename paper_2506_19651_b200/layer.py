@@ -91,7 +91,8 @@ def ragged_layer_forward(q, k, v, S, B, N, B_last, Q, theta, scale=0.0, alloc=No
     """Layer pass over a video whose length is not a multiple of the block length: N context blocks, the
     first N-1 of B tokens, the last one of B_last < B tokens (the uniform partition of Sec. 3.2.1 with the
     remainder as one shorter block).  q [L,Hq,d], k, v [L,Hkv,d] un-roped device tensors of the whole
-    stream, L = S + (N-1)*B + B_last + Q.  Returns (o_video, lse_video, o_question, lse_question, workspaces).
+    stream, L = S + (N-1)*B + B_last + Q.  Returns (o_video, lse_video, o_question, lse_question, workspaces), the workspaces
+    (for pevlm_read_status) being those of sink and full blocks, of the last block and of the question; the first two are one.
 
     One call (pevlm_layer_forward with the length of the last block); positions are the global ones.
     `alloc(shape, dtype, zero)` replaces torch.empty / torch.zeros (see LayerBuffers).
@@ -120,7 +121,7 @@ def ragged_layer_forward(q, k, v, S, B, N, B_last, Q, theta, scale=0.0, alloc=No
                 else _workspace(alloc, pb.pevlm_workspace_bytes(s, pb.WS_QUERY)))
     pb.pevlm_layer_forward(s, q, k, v, q_roped, q_roped[nv:], k_cache, v_cache, o_video, lse_video, o_question, lse_question,
                            ws_prefill, ws_query, last_len=B_last)
-    return o_video, lse_video, o_question, lse_question, [ws_prefill, ws_query]
+    return o_video, lse_video, o_question, lse_question, [ws_prefill, ws_prefill, ws_query]
 
 
 class StreamingWindow:

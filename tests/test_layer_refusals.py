@@ -1,4 +1,4 @@
-"""What layer.py refuses on the host, before anything is launched (no device is needed to see it)."""
+"""What layer.py refuses on the host, before anything is launched, and what it returns (no device is needed to see it)."""
 import pytest
 
 from paper_2506_19651_b200 import binding as pb
@@ -60,3 +60,14 @@ def test_streaming_window_takes_only_rows_that_fit(no_calls):
     assert not no_calls
     win.append_block(*rows(B + 5))  # rows past the block's are not looked at
     assert no_calls and win.blocks_seen == 3
+
+
+@pytest.mark.parametrize("Q", [0, 5])
+def test_ragged_pass_names_a_workspace_for_each_part(no_calls, Q):
+    import torch
+    L = 8 + 16 + 7 + Q
+    t = [torch.zeros(L, h, 64, dtype=torch.bfloat16) for h in (4, 2, 2)]
+    full, last, question = layer.ragged_layer_forward(*t, 8, 16, 2, 7, Q, 1e4)[4]  # of the full blocks, the last one, the question
+    shape = pb.make_shape(8, 16, 2, Q, 4, 2, 64)
+    assert full.numel() == last.numel() == pb.pevlm_workspace_bytes(shape, pb.WS_PREFILL)
+    assert question.numel() == pb.pevlm_workspace_bytes(shape, pb.WS_QUERY)
