@@ -172,6 +172,12 @@ static PrefillSize prefill_size(const pevlm_shape_t* s, int last_len) {
     return r;
 }
 
+// Most key splits of a question beside a prefill part: a question long enough to be many waves of items by itself gains
+// nothing from more of them, and its partials (an fp32 row for each row and split) would outgrow its cache: 256K tokens of
+// 28/4 heads against 1M keys asked for 485 GB of workspace with splits of 64 key tiles.
+constexpr int kMostQuestionItems = 16 * (kNumSms / 2);
+static int most_splits(int groups) { return groups < kMostQuestionItems ? kMostQuestionItems / groups : 1; }
+
 static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false, int last_len = 0) {
     QueryPlan q;
     const int G = s->num_q_heads / s->num_kv_heads;
@@ -201,6 +207,7 @@ static QueryPlan plan_query(const pevlm_shape_t* s, bool beside_prefill = false,
         int tiles = per_pair < 4 ? 4 : per_pair > 64 ? 64 : per_pair;
         if (own <= pre.all && most > tiles) tiles = most < q.total_kv_tiles ? static_cast<int>(most) : q.total_kv_tiles;
         want = (q.total_kv_tiles + tiles - 1) / tiles;
+        if (want > most_splits(groups)) want = most_splits(groups);
         whole = pre.longest + (many_rows ? 9 : 7);
     }
     if (q.total_kv_tiles <= whole) want = 1;
@@ -276,10 +283,11 @@ size_t pevlm_workspace_bytes(const pevlm_shape_t* s, int which) {
         const int G = s->num_q_heads / s->num_kv_heads, Q = s->query_len, T = q.total_kv_tiles;
         auto at_most = [](int64_t a, int64_t b) { return a < b ? a : b; };
         auto at_least = [](int64_t a, int64_t b) { return a > b ? a : b; };
-        int64_t rows = at_most((T + 63) / 64, T) * Q;
+        int64_t rows = 0;
         for (int pairs = 1; pairs == 1 || pairs <= (q.q_tiles + 1) / 2; ++pairs) {
             const int groups = s->num_kv_heads * pairs;
-            rows = at_least(rows, at_most((kNumSms / 2 + groups - 1) / groups, T) * at_most(Q, 2ll * q.tok_per_tile * pairs));
+            const int64_t splits = at_least((kNumSms / 2 + groups - 1) / groups, at_most((T + 63) / 64, most_splits(groups)));
+            rows = at_least(rows, at_most(splits, T) * at_most(Q, 2ll * q.tok_per_tile * pairs));
         }
         const int64_t pieces = (n_video(s) + Q + 15) / 16;
         const int64_t decode_splits = at_least(1, at_most(kNumSms / (static_cast<int64_t>(s->num_kv_heads) * s->batch), (pieces + 7) / 8));
