@@ -43,8 +43,8 @@ __device__ __forceinline__ int quotient(int a, const Divisor& b) {
 #endif
 
 // Launch of one of the library's kernels behind another.  The kernel may be brought onto the GPU while the one before it
-// in the stream still runs, so that its launch costs nothing; every kernel therefore calls grid_wait() before it touches
-// global memory.  Most let the next kernel come before their own wait; the decode kernel and the merge only after it,
+// in the stream still runs, so that its launch costs nothing; every kernel therefore calls grid_wait() before it reads or writes
+// global memory (the decode kernel prefetches keys into L2 before, which reads nothing into registers or shared memory).  Most let the next kernel come before their own wait; the decode kernel and the merge only after it,
 // because the launches behind them would otherwise arrive two steps early and hold the SMs that the step needs whole
 // (a decode step 25.2 us so, 27.4 with all of them early, 26.5 with none).  All kernels ask for the same split of the SM's memory (as much shared memory as there is), because an
 // SM has to run empty before it can change the split.

@@ -9,7 +9,10 @@ namespace pevlm {
 
 constexpr int kMergeThreads = 256;
 constexpr int kMergeChunk = 8;       // partial rows of a warp whose loads are in flight together
-constexpr int kMergeMaxParts = 160;  // >= the largest split count (one split per SM at most)
+// most splits of the form for few rows (its weights are an array in shared memory).  The tile kernel alone and the decode kernel
+// make 148 at most; beside a prefill part there can be more (one kv head, 1,024 question tokens, 1.3M keys: 161), which
+// launch_merge gives to the other form
+constexpr int kMergeMaxParts = 160;
 
 // Many rows (a prefill-sized question block): one thread per (row, 4 output columns), the splits one after
 // another; tens of thousands of threads hide the latency of the dependent loads.

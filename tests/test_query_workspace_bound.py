@@ -26,15 +26,17 @@ def test_bounded_and_enough(Hq, Hkv, d, S, B, Q, L):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("S,B,N,Q,Hq,Hkv,d", [(1024, 1024, 31, 8192, 8, 8, 64), (300, 1000, 33, 3001, 12, 6, 128)])
-def test_few_splits_of_a_long_question(S, B, N, Q, Hq, Hkv, d):
+@pytest.mark.parametrize("S,B,N,Q,Hq,Hkv,d", [
+    (1024, 1024, 31, 8192, 8, 8, 64), (300, 1000, 33, 3001, 12, 6, 128),
+    (0, 128, 10240, 1024, 1, 1, 64)])  # 161 splits, more than the merge of few rows has room for
+def test_splits_of_a_long_question(S, B, N, Q, Hq, Hkv, d):
     import torch
     from paper_2506_19651_b200.layer import LayerBuffers, layer_forward
     s = pb.make_shape(S, B, N, Q, Hq, Hkv, d, theta=1e6)
     g = torch.Generator(device="cuda").manual_seed(2)
     q, k, v = (torch.randn(s.L, h, d, generator=g, device="cuda").bfloat16() for h in (Hq, Hkv, Hkv))
     one = layer_forward(LayerBuffers(s), q, k, v)
-    many = layer_forward(LayerBuffers(s), q, k, v, mark=lambda name: None)  # the question's keys in one piece
+    many = layer_forward(LayerBuffers(s), q, k, v, mark=lambda name: None)  # one piece, or 18
     torch.cuda.synchronize()
     assert pb.pevlm_read_status(one.ws_query)[0] == 0
     assert (one.lse_question - many.lse_question).abs().max() <= 1e-5  # fp32 sums in another order
