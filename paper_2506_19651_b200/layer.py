@@ -50,10 +50,6 @@ class LayerBuffers:
         self.ws_query = _workspace(alloc, pb.pevlm_workspace_bytes(s, pb.WS_QUERY))
 
 
-KERNELS_PER_PASS = 2          # rope and V copy, attention of video and question rows; a merge too where the question's keys are split
-KERNELS_PER_PASS_BY_CALL = 7  # with `mark`: rope, V copy, prefill attention, rope, V copy, question attention, merge
-
-
 def layer_forward(buf: LayerBuffers, q, k, v, mark=None):
     """q [L,Hq,d], k, v [L,Hkv,d]: un-roped bf16 device tensors of the whole stream.
     Leaves O/LSE of the video rows and of the question rows in `buf`.  `mark(name)`, if
