@@ -276,7 +276,7 @@ size_t pevlm_workspace_bytes(const pevlm_shape_t* s, int which) {
     if (check_shape(s) != PEVLM_OK) return 0;
     if (which == PEVLM_WS_PREFILL) return kStatusBytes;
     if (which == PEVLM_WS_QUERY) {
-        // The most partial rows that plan_query can ask for: pevlm_layer_forward with a last block of any length,
+        // The most partial rows that plan_query can ask for: pevlm_layer_forward (of one sequence) with a last block of any length,
         // pevlm_query_attn with this question and cache or shorter ones (a window that is still filling; neither the
         // splits nor splits times rows grow steadily with the lengths).
         const QueryPlan q = plan_query(s);
@@ -286,7 +286,8 @@ size_t pevlm_workspace_bytes(const pevlm_shape_t* s, int which) {
         int64_t rows = 0;
         for (int pairs = 1; pairs == 1 || pairs <= (q.q_tiles + 1) / 2; ++pairs) {
             const int groups = s->num_kv_heads * pairs;
-            const int64_t splits = at_least((kNumSms / 2 + groups - 1) / groups, at_most((T + 63) / 64, most_splits(groups)));
+            int64_t splits = (kNumSms / 2 + groups - 1) / groups;
+            if (s->batch == 1) splits = at_least(splits, at_most((T + 63) / 64, most_splits(groups)));
             rows = at_least(rows, at_most(splits, T) * at_most(Q, 2ll * q.tok_per_tile * pairs));
         }
         const int64_t pieces = (n_video(s) + Q + 15) / 16;

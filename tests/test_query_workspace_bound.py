@@ -42,3 +42,13 @@ def test_splits_of_a_long_question(S, B, N, Q, Hq, Hkv, d):
     assert (one.lse_question - many.lse_question).abs().max() <= 1e-5  # fp32 sums in another order
     a, b = one.o_question.float(), many.o_question.float()
     assert ((a - b).abs() <= 2.0 ** -7 * b.abs() + 2e-3).all()
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,Q,L,batch", [(56, 8, 128, 2148, 62932, 40), (16, 2, 128, 2683, 105810, 3), (256, 16, 128, 105, 49171, 5)])
+def test_a_batch_needs_no_room_for_the_one_call_pass(Hq, Hkv, d, Q, L, batch):
+    # pevlm_layer_forward takes one sequence; the question attention of a batch alone has at most 74 items of 256 rows a sequence
+    s = pb.make_shape(L - Q, 1, 0, Q, Hq, Hkv, d, batch=batch)
+    n = pb.pevlm_workspace_bytes(s, pb.WS_QUERY)
+    assert n <= 256 + batch * (256 + (Q * Hq + 74 * 256) * (d + 1) * 4)
+    p, ws = C.c_void_p(4096), C.c_void_p(4096 + 16)
+    assert pb.lib().pevlm_query_attn(C.byref(s), p, p, p, p, None, ws, n, None) == pb.PEVLM_EALIGN
