@@ -66,15 +66,28 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+template <typename Fn>
+static Fn driver_entry(const char* name) {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool found = cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+    return found ? reinterpret_cast<Fn>(p) : nullptr;
+}
+
 static EncodeTiledFn encode_fn() {
-    static const EncodeTiledFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const bool found = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-                           q == cudaDriverEntryPointSuccess;
-        return found ? reinterpret_cast<EncodeTiledFn>(p) : nullptr;
-    }();
+    static const EncodeTiledFn fn = driver_entry<EncodeTiledFn>("cuTensorMapEncodeTiled");
     return fn;
+}
+
+uint64_t context_id() {
+    typedef CUresult (*CurrentFn)(CUcontext*);
+    typedef CUresult (*IdFn)(CUcontext, unsigned long long*);
+    static const CurrentFn current = driver_entry<CurrentFn>("cuCtxGetCurrent");
+    static const IdFn id_of = driver_entry<IdFn>("cuCtxGetId");
+    CUcontext c = nullptr;
+    unsigned long long id = 0;
+    if (!current || !id_of || current(&c) != CUDA_SUCCESS || !c || id_of(c, &id) != CUDA_SUCCESS) return 0;
+    return id + 1;
 }
 
 // Tensor map over a [tokens, heads, d] bf16 tensor (d contiguous) with a box of box_elems (64 or 32) elements x

@@ -42,6 +42,9 @@ __device__ __forceinline__ int quotient(int a, const Divisor& b) {
 }
 #endif
 
+// The calling thread's context: a number that no other context of the process ever has; 0 if it has none yet (or if the driver does not say).
+uint64_t context_id();
+
 // Launch of one of the library's kernels behind another.  The kernel may be brought onto the GPU while the one before it
 // in the stream still runs, so that its launch costs nothing; every kernel therefore calls grid_wait() before it reads or writes
 // global memory (the decode kernel prefetches keys into L2 before, which reads nothing into registers or shared memory).  Most let the next kernel come before their own wait; the decode kernel and the merge only after it,
@@ -50,17 +53,18 @@ __device__ __forceinline__ int quotient(int a, const Divisor& b) {
 // SM has to run empty before it can change the split.
 template <auto Kernel, typename... Args>
 inline cudaError_t launch_chained(dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, const Args&... args) {
-    // attributes of a kernel: once on each device (smem is the same in every launch of a kernel)
-    static std::atomic<uint64_t> prepared{0};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 64 || !(prepared.load(std::memory_order_acquire) >> dev & 1)) {
+    // attributes of a kernel: once in each context (a second one on a device, or the one after a reset, has its own; smem
+    // is the same in every launch of a kernel).  Contexts whose ids share a place take turns in it.
+    static std::atomic<uint64_t> prepared[64] = {};
+    const uint64_t context = context_id();
+    std::atomic<uint64_t>& place = prepared[context % 64];
+    cudaError_t e = cudaSuccess;
+    if (context == 0 || place.load(std::memory_order_acquire) != context) {
         e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
         if (e == cudaSuccess && smem > 48 * 1024)
             e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
-        if (dev < 64) prepared.fetch_or(1ull << dev, std::memory_order_release);
+        place.store(context, std::memory_order_release);
     }
     cudaLaunchAttribute chained;
     chained.id = cudaLaunchAttributeProgrammaticStreamSerialization;
