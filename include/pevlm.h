@@ -26,7 +26,7 @@
  *     memory, never synchronises the device (pevlm_read_status excepted) and never frees
  *     anything.  Calls are asynchronous on `stream`.  No state is kept between calls, with
  *     one exception: pevlm_query_attn_noalloc owns a fixed device array per GPU and
- *     remembers its address (see there).
+ *     remembers its address in each context (see there).
  *   - batch > 1 means `batch` independent sequences of the same shape, stored one after
  *     another (the leading dimension of every tensor, and of the workspace partials).
  *   - Return value: PEVLM_OK (0) or a negative pevlm_status_t.  All argument checking
@@ -184,7 +184,7 @@ int pevlm_query_attn(const pevlm_shape_t* shape, const void* q_question, const v
  *   - Shapes whose partials exceed that size are rejected
  *     with PEVLM_EWORKSPACE before any launch (text via pevlm_last_cuda_error).
  *   - The call itself performs no cudaMalloc / cudaFree and uses no allocating routine.
- *   - The first call on each device resolves the array's device address
+ *   - The first call in each context (one per device, as a rule) resolves the array's device address
  *     (cudaGetSymbolAddress, with that device current); make that first call outside any
  *     stream capture.
  *   - All calls on one device share the one array, which keeps the previous call's contents:

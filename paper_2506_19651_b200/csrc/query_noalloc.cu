@@ -14,32 +14,35 @@
 namespace {
 
 constexpr size_t kScratchBytes = PEVLM_NOALLOC_SCRATCH_BYTES;
-constexpr int kMaxDevices = 64;
+constexpr int kPlaces = 64;
 
 // File-scope device array: every GPU that loads the library holds these bytes until the
 // process exits.  In HOST code this name is only a stand-in for the symbol; the device address
 // comes from cudaGetSymbolAddress below and is what the kernels receive.
 static __device__ __align__(256) unsigned char g_query_scratch[kScratchBytes];
 
+// its address in a context, looked up once in each; contexts whose ids share a place take turns in it
 std::mutex g_setup_mutex;
-void* g_scratch_ptr[kMaxDevices] = {};
+struct {
+    uint64_t context;
+    void* ptr;
+} g_scratch[kPlaces] = {};
 
 }  // namespace
 
-// Once per device, with that device current: resolve the device address of the scratch array.
+// Device address of the scratch array in the calling thread's context.
 int pevlm::noalloc_scratch_for_current_device(void** out) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return pevlm::cuda_fail(e, "cudaGetDevice");
-    if (dev < 0 || dev >= kMaxDevices) return pevlm::fail_with_text(PEVLM_EUNSUPPORTED, "device ordinal beyond 63");
+    const uint64_t context = pevlm::context_id();
     std::lock_guard<std::mutex> lock(g_setup_mutex);
-    if (!g_scratch_ptr[dev]) {
+    auto& place = g_scratch[context % kPlaces];
+    if (context == 0 || place.context != context) {
         void* ptr = nullptr;
-        e = cudaGetSymbolAddress(&ptr, g_query_scratch);
+        const cudaError_t e = cudaGetSymbolAddress(&ptr, g_query_scratch);
         if (e != cudaSuccess) return pevlm::cuda_fail(e, "cudaGetSymbolAddress(no-alloc scratch)");
-        g_scratch_ptr[dev] = ptr;
+        place.context = context;
+        place.ptr = ptr;
     }
-    *out = g_scratch_ptr[dev];
+    *out = place.ptr;
     return PEVLM_OK;
 }
 

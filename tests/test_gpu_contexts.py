@@ -1,4 +1,5 @@
-"""The library in a second context on the same device, in a process of its own: kernel attributes belong to a context."""
+"""The library in a second context on the same device, in a process of its own: kernel attributes and the addresses of device
+arrays belong to a context."""
 import subprocess
 import sys
 import os
@@ -28,7 +29,11 @@ def run():
         s.sink_len = n - 400 - Q
         s.query_len = Q
         ok(lib.pevlm_query_attn(b, q, k, v, oq, None, ws, 1 << 23, None))
+    ok(lib.pevlm_query_attn_noalloc(b, q, k, v, oq, None, None))  # partials in the context's own copy of the built-in array
     ok(cu.cuCtxSynchronize())
+    status = C.c_int32(1)
+    ok(lib.pevlm_read_status(None, None, C.byref(status), None))
+    assert status.value == 0
     got = (C.c_uint16 * (8 * 128 * 700))()
     ok(cu.cuMemcpyDtoH_v2(got, o, C.c_size_t(2 * len(got))))
     assert set(got) == {one}  # averages of ones
