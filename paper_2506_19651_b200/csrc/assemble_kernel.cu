@@ -10,8 +10,7 @@ constexpr int kCopyThreads = 256;
 constexpr int kCopyUnroll = 4;
 
 // An ordinary load, not one through the non-coherent path (.nc): this kernel may be on the GPU while the one that writes its
-// sources still runs (launch_chained), and grid_wait() orders ordinary accesses only.  (Past L1 altogether, ld.global.cg,
-// copies of 8,000 rows of 4 heads of 128 take 10.8 us instead of 13.1, of 50,000 rows 55.0 instead of 51.9.)
+// sources still runs (launch_chained), and grid_wait() orders ordinary accesses only.
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 v;
     asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -25,14 +24,13 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
                  : "memory");
 }
 
-__global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(CopySegments s) {
+// The segments are indexed where they are, in the parameters: a copy of them that the thread changes (to the sequence's own
+// addresses) ends up in local memory, with a load from it before every access.  K and V of 15,360 tokens of 4 heads of 128
+// 7.1 us (21.0 with such a copy), of 50,000 tokens 33.4 (53.6) = 6.1 TB/s.
+__global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __grid_constant__ CopySegments s) {
     grid_launch_dependents();
     grid_wait();
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {  // the sequence of this row of CTAs
-        s.src[k] += static_cast<int64_t>(blockIdx.y) * s.src_stride[k];
-        s.dst[k] += static_cast<int64_t>(blockIdx.y) * s.dst_stride;
-    }
+    const int64_t seq = blockIdx.y;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kCopyThreads * kCopyUnroll;
     for (int64_t base = static_cast<int64_t>(blockIdx.x) * kCopyThreads * kCopyUnroll + threadIdx.x; base < s.total;
          base += stride) {
@@ -51,8 +49,8 @@ __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(CopySegment
                         seg = k + 1;
                     }
                 }
-                v[u] = ld_stream(s.src[seg] + i);
-                dst[u] = s.dst[seg] + i;
+                v[u] = ld_stream(s.src[seg] + seq * s.src_stride[seg] + i);
+                dst[u] = s.dst[seg] + seq * s.dst_stride + i;
             }
         }
 #pragma unroll
