@@ -104,20 +104,24 @@ __global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(cons
     // groups of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ... of p.group tokens each
     const int64_t stride = static_cast<int64_t>(gridDim.x) * p.group;
     auto size_of = [&](int64_t tok0) { return static_cast<int>(p.n_tokens - tok0 < p.group ? p.n_tokens - tok0 : p.group); };
+    // The pair that this thread forms angles of: always the same one, so its frequency is read once (the lanes of a warp read
+    // different words of constant memory, one after another).  One position per token, or, multimodal, the component that the
+    // pair's section picks.
+    static_assert(kRopeThreads % HALF == 0, "a thread keeps its pair");
+    const int pair = threadIdx.x % HALF;
+    const double freq = p.inv_freq[pair];
+    const int comp = pair < p.sec_end0 ? 0 : pair < p.sec_end1 ? 1 : 2;
     auto angles = [&](int64_t tok0, int buf) {
         if (tok0 >= p.n_tokens) return;
-        for (int a = threadIdx.x; a < size_of(tok0) * HALF; a += kRopeThreads) {
-            const int t = a / HALF, i = a % HALF;
+        for (int t = threadIdx.x / HALF; t < size_of(tok0); t += kRopeThreads / HALF) {
             const int64_t tok = tok0 + t;
-            // one position per token, or, multimodal, the component that the rotary pair's section picks
             const int64_t seq = p.n_tokens == p.seq_len ? 0 : quotient(static_cast<int>(tok), p.div_seq);
-            const int comp = i < p.sec_end0 ? 0 : i < p.sec_end1 ? 1 : 2;
             const int64_t pos = p.pos3 ? p.pos3[(2 * seq + comp) * p.seq_len + tok]
                               : p.pos_ids ? p.pos_ids[tok]
                                           : p.first_token + tok - seq * p.seq_len;
             double sn, cn;
-            sincos(__dmul_rn(static_cast<double>(pos), p.inv_freq[i]), &sn, &cn);
-            const int e = i % 8, w = i / 8;
+            sincos(__dmul_rn(static_cast<double>(pos), freq), &sn, &cn);
+            const int e = pair % 8, w = pair / 8;
             sm.cs64[buf][t * HALF + e * TPV + w] = make_double2(cn, sn);
             float* f = reinterpret_cast<float*>(&sm.cs32[buf][t * (HALF / 2) + (e / 2) * TPV + w]);
             f[e % 2] = __double2float_rn(cn);
