@@ -12,7 +12,7 @@
 //     r - E and r + E, E = 2^-23 (|a| + |b|), round to the same bf16 (see rotate2 for why that is enough).  Elsewhere
 //     (about one head vector of a warp in sixteen) the thread repeats its eight pairs in fp64;
 //   - the bytes in flight, above all in ranges that do not fill the GPU many times over (12.5K tokens took 73 us where
-//     50K took 148).  The loads go through a ring in shared memory, kRopeRing vectors ahead, over the ends of groups
+//     50K took 148).  The loads go through a ring in shared memory, kRing vectors ahead, over the ends of groups
 //     too, which costs no registers.  A thread reads only what it has fetched itself, so the ring needs no barrier.
 // The V rows of the same tokens can be copied along (V needs no rotation): a third range of vectors.
 #include "internal.h"
@@ -20,13 +20,20 @@
 
 namespace pevlm {
 
-constexpr int kRopeThreads = 256;
-constexpr int kRopeCtasPerSm = 3;
-// Most tokens of a group, and vectors a thread has in flight: with V copied along, 50K tokens of 28/4 heads take 171 us with
-// groups of 8 and a ring of 6, 151 with 4 and 6, 150 with 4 and 5, 164 with 2 and 6; two CTAs per SM with longer rings are
-// faster at 32/8 heads only (130 against 148 us for 33K tokens), slower everywhere else.
-constexpr int kRopeTokens = 4;
-constexpr int kRopeRing = 5;
+// Threads of a CTA, CTAs of an SM, most tokens of a group and vectors a thread has in flight.  With V copied along, 50K tokens of
+// 28/4 heads take 171 us with groups of 8 and a ring of 6, 151 with 4 and 6, 150 with 4 and 5, 164 with 2 and 6; two CTAs per SM
+// with longer rings are faster at 32/8 heads only (130 against 148 us for 33K tokens), slower everywhere else.
+// FEW: calls with few heads (launch_rope).  There is little to rotate for each angle then: the fp64 evaluations, some 240 cycles
+// for a warp on its scheduler, are the larger part, and with groups of four tokens in large CTAs the warps wait for one another's
+// (33K tokens of 8/2 heads of 128 with V 45.7 us, 38.9 in this form; 1/1 heads 26.9, 17.2; rings of 5 and five CTAs 39.5, 17.6; 64
+// registers and eight CTAs 41.7 for 8/2 heads without V where this form takes 36.7).
+template <bool FEW>
+struct RopeForm {
+    static constexpr int kThreads = FEW ? 128 : 256;
+    static constexpr int kCtasPerSm = FEW ? 6 : 3;
+    static constexpr int kTokens = FEW ? 8 : 4;
+    static constexpr int kRing = FEW ? 3 : 5;
+};
 
 // 16-byte accesses that do not allocate in L1 (every byte is touched once)
 __device__ __forceinline__ void fetch16(uint32_t dst, const __nv_bfloat16* src) {
@@ -81,22 +88,24 @@ __device__ __forceinline__ uint32_t rotate2(uint32_t a, uint32_t b, const float4
     return (out_a ^ other_a) | (out_b ^ pack_bf16x2(y0, y1));
 }
 
-template <int D>
+template <int D, bool FEW>
 struct RopeSmem {
+    using F = RopeForm<FEW>;
     static constexpr int kHalf = D / 2;
     // per token: [pair / 2 of the thread][thread of the vector], so that the threads of a vector read 16 contiguous bytes each
-    float4 cs32[2][kRopeTokens * kHalf / 2];   // (cos0, cos1, sin0, sin1) of two pairs
-    double2 cs64[2][kRopeTokens * kHalf];      // (cos, sin), [pair of the thread][thread of the vector]
-    uint4 ring[kRopeRing][2][kRopeThreads];    // [half of the vector][thread]
+    float4 cs32[2][F::kTokens * kHalf / 2];   // (cos0, cos1, sin0, sin1) of two pairs
+    double2 cs64[2][F::kTokens * kHalf];      // (cos, sin), [pair of the thread][thread of the vector]
+    uint4 ring[F::kRing][2][F::kThreads];    // [half of the vector][thread]
 };
 
-template <int D>
-__global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(const __grid_constant__ RopeParams p) {
+template <int D, bool FEW>
+__global__ void __launch_bounds__(RopeForm<FEW>::kThreads, RopeForm<FEW>::kCtasPerSm) rope_kernel(const __grid_constant__ RopeParams p) {
+    constexpr int kRopeThreads = RopeForm<FEW>::kThreads, kRopeRing = RopeForm<FEW>::kRing;
     constexpr int HALF = D / 2;
     constexpr int TPV = HALF / 8;                // threads per head vector: 8 rotation pairs each
     constexpr int SLOTS = kRopeThreads / TPV;    // vectors the CTA has in hand at a time
     extern __shared__ __align__(16) uint8_t raw[];
-    RopeSmem<D>& sm = *reinterpret_cast<RopeSmem<D>*>(raw);
+    RopeSmem<D, FEW>& sm = *reinterpret_cast<RopeSmem<D, FEW>*>(raw);
     const int v = threadIdx.x % TPV, slot = threadIdx.x / TPV;
     const int i0 = v * 8;
     const int heads = p.Hq + p.Hkv + p.Hv;
@@ -219,21 +228,32 @@ __global__ void __launch_bounds__(kRopeThreads, kRopeCtasPerSm) rope_kernel(cons
     }
 }
 
-cudaError_t launch_rope(const RopeParams& params, int head_dim, cudaStream_t stream) {
-    if (params.n_tokens <= 0 || params.Hq + params.Hkv + params.Hv == 0) return cudaSuccess;
+template <int D, bool FEW>
+static cudaError_t launch_form(const RopeParams& params, cudaStream_t stream) {
+    using F = RopeForm<FEW>;
     RopeParams p = params;
-    // Groups as large as leaves every resident CTA four of them (the shares of the CTAs differ by one group), at least
-    // one token.
-    const int64_t resident = static_cast<int64_t>(kNumSms) * kRopeCtasPerSm;
-    p.group = kRopeTokens;
-    while (p.group > 1 && p.n_tokens < 4 * resident * p.group) p.group /= 2;
+    // Groups as large as leaves every resident CTA four (with few heads three) of them (the shares of the CTAs differ by one
+    // group), at least one token; with few heads no smaller than keeps a CTA's threads busy, as long as there is one for every CTA.
+    const int64_t resident = static_cast<int64_t>(kNumSms) * F::kCtasPerSm;
+    p.group = F::kTokens;
+    constexpr int kBusy = FEW ? F::kThreads / (D / 2) : 1;  // tokens whose angles take all threads
+    while (p.group > 1 && p.n_tokens < (FEW ? 3 : 4) * resident * p.group && (p.group > kBusy || p.n_tokens < resident * p.group)) p.group /= 2;
     p.div_hq = make_divisor(p.Hq);
     p.div_hkv = make_divisor(p.Hkv);
     p.div_seq = make_divisor(p.seq_len);
     const int64_t groups = (p.n_tokens + p.group - 1) / p.group;
     const unsigned grid = static_cast<unsigned>(groups < resident ? groups : resident);
-    return head_dim == 128 ? launch_chained<rope_kernel<128>>(grid, kRopeThreads, sizeof(RopeSmem<128>), stream, p)
-                           : launch_chained<rope_kernel<64>>(grid, kRopeThreads, sizeof(RopeSmem<64>), stream, p);
+    return launch_chained<rope_kernel<D, FEW>>(grid, F::kThreads, sizeof(RopeSmem<D, FEW>), stream, p);
+}
+
+cudaError_t launch_rope(const RopeParams& p, int head_dim, cudaStream_t stream) {
+    const int heads = p.Hq + p.Hkv + p.Hv;
+    if (p.n_tokens <= 0 || heads == 0) return cudaSuccess;
+    // The line between the forms, V's heads counted.  The small one against the large one, 12.6K / 33K / 74K tokens: heads of 128, 18 of
+    // them 0.97 / 0.95 / 0.87, 20 0.97 / 0.93 / 0.87, 24 1.04 / 1.06 / 1.02, 28 1.00 / 1.08 / 1.02; heads of 64, 20 of them
+    // 0.92 / 0.81 / 0.77, 24 0.92 / 1.03 / 1.06, 28 0.99 / 0.94 / 0.87.
+    if (head_dim == 128) return heads <= 20 ? launch_form<128, true>(p, stream) : launch_form<128, false>(p, stream);
+    return heads <= 20 ? launch_form<64, true>(p, stream) : launch_form<64, false>(p, stream);
 }
 
 }  // namespace pevlm
