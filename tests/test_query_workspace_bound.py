@@ -52,3 +52,23 @@ def test_a_batch_needs_no_room_for_the_one_call_pass(Hq, Hkv, d, Q, L, batch):
     assert n <= 256 + batch * (256 + (Q * Hq + 74 * 256) * (d + 1) * 4)
     p, ws = C.c_void_p(4096), C.c_void_p(4096 + 16)
     assert pb.lib().pevlm_query_attn(C.byref(s), p, p, p, p, None, ws, n, None) == pb.PEVLM_EALIGN
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,Q,Hq,Hkv,d,batch", [(9000, 356, 28, 4, 128, 1), (8000, 300, 32, 8, 64, 1), (6100, 130, 14, 2, 64, 3)])
+def test_two_waves_of_shorter_items(n, Q, Hq, Hkv, d, batch):
+    import torch
+    s = pb.make_shape(n, 1, 0, Q, Hq, Hkv, d, batch=batch)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    q, k, v = (torch.randn(batch, r, h, d, generator=g, device="cuda").bfloat16() for r, h in ((Q, Hq), (n + Q, Hkv), (n + Q, Hkv)))
+    o, lse = torch.empty_like(q), torch.empty(batch, Hq, Q, device="cuda")
+    size = pb.pevlm_workspace_bytes(s, pb.WS_QUERY)
+    ws = torch.full((size + 256,), 165, dtype=torch.uint8, device="cuda")
+    pb.pevlm_query_attn(s, q, k, v, o, lse, ws[:size])
+    assert pb.pevlm_read_status(ws)[0] == 0 and bool((ws[size:] == 165).all())
+    hidden = torch.arange(n + Q, device="cuda")[None, :] > n + torch.arange(Q, device="cuda")[:, None]
+    for b in range(batch):
+        for h in range(Hq):
+            x = (q[b, :, h].double() @ k[b, :, h * Hkv // Hq].double().T * d ** -0.5).masked_fill(hidden, float("-inf"))
+            assert (lse[b, h] - torch.logsumexp(x, -1)).abs().max() <= 1e-5  # fp32 sums of some thousand terms
+            assert (o[b, :, h].double() - torch.softmax(x, -1) @ v[b, :, h * Hkv // Hq].double()).abs().max() <= 2e-2
