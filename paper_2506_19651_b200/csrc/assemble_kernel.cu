@@ -26,15 +26,17 @@ __device__ __forceinline__ void st_stream(uint4* p, const uint4& v) {
 
 // The segments are indexed where they are, in the parameters: a copy of them that the thread changes (to the sequence's own
 // addresses) ends up in local memory, with a load from it before every access.  K and V of 15,360 tokens of 4 heads of 128
-// 7.1 us (21.0 with such a copy), of 50,000 tokens 33.4 (53.6) = 6.1 TB/s.
+// 6.4 us (20.9 with such a copy), of 50,000 tokens 34.2 (54.2) = 6.0 TB/s.
+// The first addresses are formed before the next kernel may come and before the wait, since they take a chain of reads of the
+// parameters: a decode step, whose copy is one row, 24.97 us; 25.73 with the next kernel let in first, 26.08 with the wait
+// first as well, 25.54 with the next kernel let in after the wait.
 __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __grid_constant__ CopySegments s) {
-    grid_launch_dependents();
-    grid_wait();
     const int64_t seq = blockIdx.y;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * kCopyThreads * kCopyUnroll;
+    bool waited = false;
     for (int64_t base = static_cast<int64_t>(blockIdx.x) * kCopyThreads * kCopyUnroll + threadIdx.x; base < s.total;
          base += stride) {
-        uint4 v[kCopyUnroll];
+        const uint4* src[kCopyUnroll];
         uint4* dst[kCopyUnroll];
 #pragma unroll
         for (int u = 0; u < kCopyUnroll; ++u) {
@@ -49,14 +51,24 @@ __global__ void __launch_bounds__(kCopyThreads) copy_segments_kernel(const __gri
                         seg = k + 1;
                     }
                 }
-                v[u] = ld_stream(s.src[seg] + seq * s.src_stride[seg] + i);
+                src[u] = s.src[seg] + seq * s.src_stride[seg] + i;
                 dst[u] = s.dst[seg] + seq * s.dst_stride + i;
             }
         }
+        if (!waited) {
+            grid_launch_dependents();
+            grid_wait();
+        }
+        waited = true;
+        uint4 v[kCopyUnroll];
+#pragma unroll
+        for (int u = 0; u < kCopyUnroll; ++u)
+            if (dst[u]) v[u] = ld_stream(src[u]);
 #pragma unroll
         for (int u = 0; u < kCopyUnroll; ++u)
             if (dst[u]) st_stream(dst[u], v[u]);
     }
+    if (!waited) grid_wait();
 }
 
 cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream) {
