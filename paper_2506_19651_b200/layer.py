@@ -120,6 +120,12 @@ def ragged_layer_forward(q, k, v, S, B, N, B_last, Q, theta, scale=0.0, alloc=No
     return o_video, lse_video, o_question, lse_question, [ws_prefill, ws_prefill, ws_query]
 
 
+def _need_rows(n, q, k, v):
+    """The calls get addresses only: that there are n rows behind them is seen to here."""
+    if q.shape[0] < n or k.shape[0] < n or v.shape[0] < n:
+        raise ValueError(f"{q.shape[0]}, {k.shape[0]}, {v.shape[0]} rows of q, k, v where {n} are read")
+
+
 class StreamingWindow:
     """A sliding window of W context blocks over a fixed sink (the streaming use the paper names as
     future work, Sec. 5).  The cache is [sink | W block slots | question]; block t of the stream is encoded
@@ -136,7 +142,8 @@ class StreamingWindow:
         bf, f32 = torch.bfloat16, torch.float32
         self.k_cache = torch.zeros((self.rows, Hkv, d), dtype=bf, device=device)
         self.v_cache = torch.zeros((self.rows, Hkv, d), dtype=bf, device=device)
-        self.q_buf = torch.empty((max(S, B, Q_max), Hq, d), dtype=bf, device=device)
+        self.q_rows = max(S, B, Q_max)
+        self.q_buf = torch.empty((self.q_rows, Hq, d), dtype=bf, device=device)
         self.s_sink = self._shape(S, 1, 0, 0)
         self.s_block = self._shape(S, B, 1, 0)
         alloc = lambda shape, dtype: torch.empty(shape, dtype=dtype, device=device)
@@ -157,17 +164,10 @@ class StreamingWindow:
         """Address of a cache row (what cache[row:] would point to, without building the view)."""
         return cache.data_ptr() + row * self.Hkv * self.d * 2
 
-    @staticmethod
-    def _has_rows(n, *tensors):
-        """The calls get addresses only: that there are n rows behind them is seen to here."""
-        for t in tensors:
-            if t.shape[0] < n:
-                raise ValueError(f"{t.shape[0]} rows where {n} are read")
-
     def set_sink(self, q, k, v):
         """Encode the sink (Eq. 3).  Returns (o [S,Hq,d], lse [Hq,S])."""
         S = self.S
-        self._has_rows(S, q, k, v)
+        _need_rows(S, q, k, v)
         o, lse = self._outputs(S)
         pb.pevlm_rope_qkv(self.s_sink, q, k, v, self.q_buf, self.k_cache, self.v_cache, 0, S)
         pb.pevlm_parallel_prefill_attn(self.s_sink, self.q_buf, self.k_cache, self.v_cache, o, lse, self.ws_sink)
@@ -176,7 +176,7 @@ class StreamingWindow:
     def append_block(self, q, k, v):
         """Encode the next block of the stream into the slot of the oldest one.  Returns (o [B,Hq,d], lse [Hq,B])."""
         S, B = self.S, self.B
-        self._has_rows(B, q, k, v)
+        _need_rows(B, q, k, v)
         t = self.blocks_seen
         row0 = S + (t % self.W) * B
         o, lse = self._outputs(B)
@@ -191,9 +191,11 @@ class StreamingWindow:
         Qn = q.shape[0]
         held = min(self.blocks_seen, self.W)
         nv = self.S + held * self.B
-        self._has_rows(Qn, k, v)
-        room = min(self.rows - nv, self.q_buf.shape[0])  # more than Q_max while the window fills
-        if Qn > room:
+        if k.shape[0] < Qn or v.shape[0] < Qn:
+            _need_rows(Qn, q, k, v)
+        room = self.rows - nv  # more than Q_max while the window fills
+        if Qn > room or Qn > self.q_rows:
+            room = min(room, self.q_rows)
             raise ValueError(f"a question of {Qn} rows where {room} fit")
         s = self._shape(nv, 1, 0, Qn)
         o, lse = self._outputs(Qn)
