@@ -59,6 +59,8 @@ def layer_forward(buf: LayerBuffers, q, k, v, mark=None):
     nv, Q = s.n_video, s.query_len
     _one_sequence(s)
     if mark is None:
+        if nv + Q == 0:  # an empty stream is no call's shape
+            return buf
         pb.pevlm_layer_forward(s, q, k, v, buf.q_video, buf.q_question, buf.k_cache, buf.v_cache, buf.o_video,
                                buf.lse_video, buf.o_question, buf.lse_question, buf.ws_prefill, buf.ws_query)
         return buf

@@ -71,3 +71,13 @@ def test_ragged_pass_names_a_workspace_for_each_part(no_calls, Q):
     shape = pb.make_shape(8, 16, 2, Q, 4, 2, 64)
     assert full.numel() == last.numel() == pb.pevlm_workspace_bytes(shape, pb.WS_PREFILL)
     assert question.numel() == pb.pevlm_workspace_bytes(shape, pb.WS_QUERY)
+
+
+def test_nothing_to_do_is_no_error(no_calls):
+    import torch
+    empty = pb.make_shape(0, 16, 0, 0, 4, 2, 64)
+    buf = layer.LayerBuffers(empty, device="cpu")
+    t = torch.zeros(0, 4, 64, dtype=torch.bfloat16)
+    for mark in (None, lambda name: None):
+        assert layer.layer_forward(buf, t, t, t, mark=mark) is buf
+    assert not no_calls
