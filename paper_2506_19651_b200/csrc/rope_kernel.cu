@@ -228,16 +228,42 @@ __global__ void __launch_bounds__(RopeForm<FEW>::kThreads, RopeForm<FEW>::kCtasP
     }
 }
 
+// Tokens of a group.  Calls that are long enough take the most, which costs the least for each token.  In shorter ones the time
+// is the rounds that the resident CTAs take, each of a fixed part (the angles' chain of fp64 operations, the barrier) and one
+// for the vectors: the group with the least of it, a last round that few CTAs have counting from three tenths on.  (Four
+// groups for every CTA, as it was, gave 2,500 tokens groups of one in six rounds.)  RoPE / the whole layer, 28/4 heads of 128: 1,300
+// tokens 6.8 -> 5.5 / 22.0 -> 20.6 us, 2,500 11.7 -> 9.3 / 38.2 -> 36.1, 3,500 15.2 -> 11.7 / 56.6 -> 53.3; 32/8 heads, 3,500 tokens
+// 17.6 -> 14.1 / 67.0 -> 64.0; 14/2 heads, 4,300 tokens 10.0 -> 8.6 / 42.5 -> 40.9; 4/2 heads of 64, 900 tokens 3.0 -> 1.9 / 13.4 -> 11.8.
+// The fixed part is as long as the vectors of 1,600 elements: 0.6 us to 1.25 a token for 28/4 heads, 0.9 to 1.27 for 14/2.  With few
+// heads a CTA forms the angles of kStep tokens at a time, and groups are multiples of that; of one token too where the
+// vectors of kStep take the threads more than one turn (14/2 heads of 64, 300 tokens: 2.0 us, 2.4 in groups of four).
+template <int D, bool FEW>
+static int group_size(int64_t n_tokens, int heads) {
+    using F = RopeForm<FEW>;
+    const int64_t resident = static_cast<int64_t>(kNumSms) * F::kCtasPerSm;
+    if (n_tokens >= (FEW ? 3 : 4) * resident * F::kTokens) return F::kTokens;
+    constexpr int kStep = FEW ? F::kThreads / (D / 2) : 1;
+    int best = 0;
+    int64_t least = 0;
+    for (int g = heads * kStep <= F::kThreads / (D / 16) ? kStep : 1; g <= F::kTokens; g += g < kStep ? kStep - g : kStep) {
+        const int64_t groups = (n_tokens + g - 1) / g, full = groups / resident, rest = groups % resident;
+        int64_t tenths = 10;  // of rounds
+        if (full > 0) tenths = 10 * full + (rest == 0 ? 0 : rest * 5 < resident ? 3 + rest * 30 / resident : 10);
+        const int64_t cost = tenths * (1600 + static_cast<int64_t>(heads) * D * g);
+        if (best == 0 || cost < least) {
+            best = g;
+            least = cost;
+        }
+    }
+    return best;
+}
+
 template <int D, bool FEW>
 static cudaError_t launch_form(const RopeParams& params, cudaStream_t stream) {
     using F = RopeForm<FEW>;
     RopeParams p = params;
-    // Groups as large as leaves every resident CTA four (with few heads three) of them (the shares of the CTAs differ by one
-    // group), at least one token; with few heads no smaller than keeps a CTA's threads busy, as long as there is one for every CTA.
     const int64_t resident = static_cast<int64_t>(kNumSms) * F::kCtasPerSm;
-    p.group = F::kTokens;
-    constexpr int kBusy = FEW ? F::kThreads / (D / 2) : 1;  // tokens whose angles take all threads
-    while (p.group > 1 && p.n_tokens < (FEW ? 3 : 4) * resident * p.group && (p.group > kBusy || p.n_tokens < resident * p.group)) p.group /= 2;
+    p.group = group_size<D, FEW>(p.n_tokens, p.Hq + p.Hkv + p.Hv);
     p.div_hq = make_divisor(p.Hq);
     p.div_hkv = make_divisor(p.Hkv);
     p.div_seq = make_divisor(p.seq_len);
