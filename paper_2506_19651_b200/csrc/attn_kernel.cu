@@ -437,7 +437,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
 #pragma unroll 1
                                 for (int h = 0; h < NP; ++h)
                                     tma_load_3d_pair(smem_base + L::kQ + qb * L::kQBytes + h * L::kQPanelBytes, &maps.q[MODE == 2 ? 4 : qm],
-                                                     h * 64, q_head0, q_tok0, bar);
+                                                     h * 64, q_head0, q_tok0, bar, l2_evict_first());
                             }
                         }
                     }
@@ -602,7 +602,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     if (row_ok) {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
-                            st_global_v8(out + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]));
+                            st_global_v8(out + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]), l2_evict_first());
                     }
                 } else if (row_ok) {
 #pragma unroll

@@ -36,8 +36,8 @@ struct RopeForm {
 };
 
 // 16-byte accesses that do not allocate in L1 (every byte is touched once)
-__device__ __forceinline__ void fetch16(uint32_t dst, const __nv_bfloat16* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+__device__ __forceinline__ void fetch16(uint32_t dst, const __nv_bfloat16* src, uint64_t l2_policy) {
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "l"(l2_policy) : "memory");
 }
 __device__ __forceinline__ void st_stream(__nv_bfloat16* p, const uint4& v) {
     asm volatile("st.global.L1::no_allocate.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(RopeForm<FEW>::kThreads, RopeForm<FEW>::kCtasP
             f[2 + e % 2] = __double2float_rn(sn);
         }
     };
+    const uint64_t once = l2_evict_first();
     // fetch cursor: kRopeRing vectors ahead of the one that is rotated
     int64_t f_tok0 = static_cast<int64_t>(blockIdx.x) * p.group;
     int f_u = slot, f_total = f_tok0 < p.n_tokens ? size_of(f_tok0) * heads : 0, f_ring = 0;
@@ -147,8 +148,8 @@ __global__ void __launch_bounds__(RopeForm<FEW>::kThreads, RopeForm<FEW>::kCtasP
                 const __nv_bfloat16* src = f_u < nq ? p.q_in + (f_tok0 * p.Hq + f_u) * D
                                          : f_u < nqk ? p.k_in + (f_tok0 * p.Hkv + (f_u - nq)) * D
                                                      : p.v_in + (f_tok0 * p.Hv + (f_u - nqk)) * D;
-                fetch16(smem_u32(&sm.ring[f_ring][0][threadIdx.x]), src + i0);
-                fetch16(smem_u32(&sm.ring[f_ring][1][threadIdx.x]), src + i0 + HALF);
+                fetch16(smem_u32(&sm.ring[f_ring][0][threadIdx.x]), src + i0, once);
+                fetch16(smem_u32(&sm.ring[f_ring][1][threadIdx.x]), src + i0 + HALF, once);
             }
             f_u += SLOTS;
             if (f_u - slot >= f_total) {  // the same for all threads: every thread takes the same number of steps
