@@ -602,7 +602,7 @@ attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ AttnMa
                     if (row_ok) {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
-                            st_global_v8(out + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]), l2_evict_first());
+                            st_global_v8(out + r * D + c * 32 + v * 16, *reinterpret_cast<uint32_t(*)[8]>(&wd[8 * v]));
                     }
                 } else if (row_ok) {
 #pragma unroll

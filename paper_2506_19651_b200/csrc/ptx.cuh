@@ -150,10 +150,11 @@ __device__ __forceinline__ void tc_fence_after_sync() {
 }
 
 // ---------------------------------------------------------------- L2
-// Policy for data that the call is done with once it is read or written: such lines leave the L2 before others do.  RoPE's inputs, the
-// attention kernel's Q tiles (read by one item) and its outputs have it; the roped Q, and K and V, which every block reads, are
-// what the L2 is to hold.  Layers back to back: 14/2 heads, 12.8K tokens 144.9 -> 143.6 us, 28/4 heads 12.6K 274 -> 272, 74K 2,175 ->
-// 2,163, 256-token blocks 447 -> 445; the inputs alone change nothing, nor do blocks handed out from the last to the first.
+// Policy for data that nobody reads again: such lines leave the L2 before others do.  RoPE's inputs and the attention kernel's
+// Q tiles have it (a prefill tile is read by one item; a question's by each of its key splits, where it costs nothing: 13 questions of 30
+// to 4,000 tokens against 700 to 50K keys are within 1 % either way).  Not the outputs, which the caller's next kernel reads: with
+// the policy on them too, a layer and a reduction over its output took, 28/4 heads, 5,552 tokens 107.1 us (103.4 without),
+// 6,336 144.7 (140.7), 7,904 177.3 (174.8), 14/2 heads 12.2K 151.6 (148.8); the layers alone are the same within 1 %.
 __device__ __forceinline__ uint64_t l2_evict_first() {
     uint64_t policy;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
@@ -351,11 +352,6 @@ __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
 }
 
 // 32-byte global store (one full sector per lane); the address must be 32-byte aligned.
-__device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&w)[8], uint64_t l2_policy) {
-    asm volatile("st.global.L1::no_allocate.L2::cache_hint.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8}, %9;"
-                 ::"l"(ptr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "l"(l2_policy)
-                 : "memory");
-}
 __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t (&w)[8]) {
     asm volatile("st.global.L1::no_allocate.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  ::"l"(ptr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
