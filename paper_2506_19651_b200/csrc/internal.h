@@ -200,6 +200,8 @@ struct CopySegments {
 };
 
 cudaError_t launch_rope(const RopeParams& p, int head_dim, cudaStream_t stream);
+// tokens of a group of such a call, heads of V counted (not part of the ABI: the tests ask for it)
+extern "C" int pevlm_rope_group_size(int64_t n_tokens, int heads, int head_dim);
 cudaError_t launch_copy_segments(const CopySegments& s, cudaStream_t stream);
 // Tensor maps of one attention launch.
 //   q[0]: [rows, Hq, d] with a 128-token box; q[1 + kind]: the same tensor with the box of the segment kind's packed ragged

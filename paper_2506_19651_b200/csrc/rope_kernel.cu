@@ -3,7 +3,7 @@
 // fused multiply-add in the rotation, so every fp64 operation rounds exactly once), then one rounding fp64 -> fp32 ->
 // bf16 (round to nearest even).
 //
-// The CTAs share the tokens out in groups of up to 4 neighbours.  A CTA evaluates a group's angles once (fp64 sincos)
+// The CTAs share the tokens out in groups of up to 4 neighbours (8 with few heads).  A CTA evaluates a group's angles once (fp64 sincos)
 // into shared memory, one group ahead, and its threads walk over the group's head vectors of Q and K: d/16 threads a
 // vector, 16 bytes of either half each; the vectors of a group are one contiguous range per tensor.  What bounds it: DRAM
 // traffic.  Two things used to stand in the way (numbers for B200, 28/4 heads of 128):
@@ -229,29 +229,33 @@ __global__ void __launch_bounds__(RopeForm<FEW>::kThreads, RopeForm<FEW>::kCtasP
     }
 }
 
-// Tokens of a group.  Calls that are long enough take the most, which costs the least for each token.  In shorter ones the time
-// is the rounds that the resident CTAs take, each of a fixed part (the angles' chain of fp64 operations, the barrier) and one
-// for the vectors: the group with the least of it, a last round that few CTAs have counting from three tenths on.  (Four
-// groups for every CTA, as it was, gave 2,500 tokens groups of one in six rounds.)  RoPE / the whole layer, 28/4 heads of 128: 1,300
-// tokens 6.8 -> 5.5 / 22.0 -> 20.6 us, 2,500 11.7 -> 9.3 / 38.2 -> 36.1, 3,500 15.2 -> 11.7 / 56.6 -> 53.3; 32/8 heads, 3,500 tokens
-// 17.6 -> 14.1 / 67.0 -> 64.0; 14/2 heads, 4,300 tokens 10.0 -> 8.6 / 42.5 -> 40.9; 4/2 heads of 64, 900 tokens 3.0 -> 1.9 / 13.4 -> 11.8.
-// The fixed part is as long as the vectors of 1,600 elements: 0.6 us to 1.25 a token for 28/4 heads, 0.9 to 1.27 for 14/2.  With few
-// heads a CTA forms the angles of kStep tokens at a time, and groups are multiples of that; of one token too where the
-// vectors of kStep take the threads more than one turn (14/2 heads of 64, 300 tokens: 2.0 us, 2.4 in groups of four).
+// Tokens of a group.  The call takes as many rounds as the resident CTAs need for its groups; in a round a CTA forms its group's
+// angles, kStep tokens at a time, and walks over the group's vectors, kSlots at a time.  Taken is the group for which the rounds come to
+// the least of both, counted in vectors (a step of angles, a chain of fp64 operations, is as long as a turn of the slots; with few heads
+// a turn counts whole), the larger of two that are alike.  Heads of 64 in the small form take whole steps of tokens or one:
+// 1,695 tokens of 8/1 heads, a layer, are 10 % slower with groups of two than with four.
+// Layers, us, groups such that every CTA has four (three with few heads) of them, as it was at first / this rule: 28/4 heads of 128, 1,300
+// tokens 22.3 / 21.8, 2,500 38.4 / 36.2, 3,500 57.4 / 53.5; 32/8, 3,500 tokens 75.4 / 70.2; 14/2, 4,300 tokens 44.0 / 41.5; 4/2 heads of 64,
+// 900 tokens 14.2 / 12.4.  Counting elements instead of turns and steps, and few groups in a last round as less than one, took
+// the wrong group in between: 14/2 heads of 64, 1,776 tokens 24.4 / 25.3 so / 22.9, 16/2 heads of 128, 3,700 tokens 37.3 / 38.7 / 36.2,
+// 14/2, 7,755 tokens 79.9 / 83.2 / 79.2.  Over 2,176 layers of 300 to 21,000 tokens of 17 forms of heads, every group timed, the rule is
+// on average within 0.5 % of the best group, 1.0 % with few heads (the first one 3.8 and 3.5 %); 43 of them are 1.2 to 10 % slower than with the first one.
+// Calls that are long enough take the most tokens: no rounds to be won, though not always the best (RoPE alone, 28/4 heads, 10,000
+// tokens 33.1 us, 31.1 with groups of three; 14/2 heads, 33,000 tokens 54.7, 52.0 with six).
 template <int D, bool FEW>
 static int group_size(int64_t n_tokens, int heads) {
     using F = RopeForm<FEW>;
     const int64_t resident = static_cast<int64_t>(kNumSms) * F::kCtasPerSm;
     if (n_tokens >= (FEW ? 3 : 4) * resident * F::kTokens) return F::kTokens;
-    constexpr int kStep = FEW ? F::kThreads / (D / 2) : 1;
+    constexpr int kSlots = F::kThreads / (D / 16), kStep = F::kThreads / (D / 2);
+    constexpr int kMore = FEW && D == 64 ? kStep : 1;
     int best = 0;
     int64_t least = 0;
-    for (int g = heads * kStep <= F::kThreads / (D / 16) ? kStep : 1; g <= F::kTokens; g += g < kStep ? kStep - g : kStep) {
-        const int64_t groups = (n_tokens + g - 1) / g, full = groups / resident, rest = groups % resident;
-        int64_t tenths = 10;  // of rounds
-        if (full > 0) tenths = 10 * full + (rest == 0 ? 0 : rest * 5 < resident ? 3 + rest * 30 / resident : 10);
-        const int64_t cost = tenths * (1600 + static_cast<int64_t>(heads) * D * g);
-        if (best == 0 || cost < least) {
+    for (int g = 1; g <= F::kTokens; g = g < kMore ? kMore : g + kMore) {
+        const int64_t rounds = ((n_tokens + g - 1) / g + resident - 1) / resident;
+        const int64_t walked = static_cast<int64_t>(heads) * g, vectors = FEW ? (walked + kSlots - 1) / kSlots * kSlots : walked;
+        const int64_t cost = rounds * ((g + kStep - 1) / kStep * kSlots + vectors);
+        if (best == 0 || cost <= least) {
             best = g;
             least = cost;
         }
@@ -273,14 +277,21 @@ static cudaError_t launch_form(const RopeParams& params, cudaStream_t stream) {
     return launch_chained<rope_kernel<D, FEW>>(grid, F::kThreads, sizeof(RopeSmem<D, FEW>), stream, p);
 }
 
+// Most heads, V's counted, of the form for few.  The small form against the large one, 12.6K / 33K / 74K tokens: heads of 128, 18 of
+// them 0.97 / 0.95 / 0.87, 20 0.97 / 0.93 / 0.87, 24 1.04 / 1.06 / 1.02, 28 1.00 / 1.08 / 1.02; heads of 64, 20 of them
+// 0.92 / 0.81 / 0.77, 24 0.92 / 1.03 / 1.06, 28 0.99 / 0.94 / 0.87.
+constexpr int kFewHeads = 20;
+
 cudaError_t launch_rope(const RopeParams& p, int head_dim, cudaStream_t stream) {
     const int heads = p.Hq + p.Hkv + p.Hv;
     if (p.n_tokens <= 0 || heads == 0) return cudaSuccess;
-    // The line between the forms, V's heads counted.  The small one against the large one, 12.6K / 33K / 74K tokens: heads of 128, 18 of
-    // them 0.97 / 0.95 / 0.87, 20 0.97 / 0.93 / 0.87, 24 1.04 / 1.06 / 1.02, 28 1.00 / 1.08 / 1.02; heads of 64, 20 of them
-    // 0.92 / 0.81 / 0.77, 24 0.92 / 1.03 / 1.06, 28 0.99 / 0.94 / 0.87.
-    if (head_dim == 128) return heads <= 20 ? launch_form<128, true>(p, stream) : launch_form<128, false>(p, stream);
-    return heads <= 20 ? launch_form<64, true>(p, stream) : launch_form<64, false>(p, stream);
+    if (head_dim == 128) return heads <= kFewHeads ? launch_form<128, true>(p, stream) : launch_form<128, false>(p, stream);
+    return heads <= kFewHeads ? launch_form<64, true>(p, stream) : launch_form<64, false>(p, stream);
+}
+
+extern "C" int pevlm_rope_group_size(int64_t n_tokens, int heads, int head_dim) {
+    if (head_dim == 128) return heads <= kFewHeads ? group_size<128, true>(n_tokens, heads) : group_size<128, false>(n_tokens, heads);
+    return heads <= kFewHeads ? group_size<64, true>(n_tokens, heads) : group_size<64, false>(n_tokens, heads);
 }
 
 }  // namespace pevlm
