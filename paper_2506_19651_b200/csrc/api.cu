@@ -494,8 +494,9 @@ static void add_prefill(AttnParams& p, const pevlm_shape_t* s, bool blocks_only,
         // that run at the same time on few K/V tiles (best for long blocks); short blocks (at most 4 query tiles)
         // run faster when pairs of equal length are handed out together across all blocks, and a segment with few
         // items per SM balances best with single pairs, heaviest first, the sink and a shorter last block too where they are not
-        // short (28/4 heads, whole list of the sink against single pairs: 7 times 784 tokens 103.3 / 98.9 us, a sink of 1,980 before
-        // 272 46.6 / 44.3, of 999 before 80 23.3 / 21.4).  Thresholds from measurements on B200.
+        // short (28/4 heads, whole list of the sink against single pairs, medians in one process: 7 times 784 tokens 111.5 / 108.6 us, a sink of
+        // 1,980 before 272 49.3 / 46.2, of 999 before 80 24.0 / 21.8; of 42 shapes, batches among them, none slower beyond noise).  Thresholds
+        // from measurements on B200.
         int want_pc = sp.pairs;
         if (blocks && sp.tiles <= 4) want_pc = p.G / 2 > 0 ? p.G / 2 : 1;
         else if (sp.tiles > 4 && static_cast<int64_t>(n) * p.Hkv * sp.pairs < 16 * kNumSms) want_pc = 1;
